@@ -30,11 +30,14 @@ constexpr int kRowThreads = 256;
 __device__ __forceinline__ float bf16_at(const uint16_t* p, int64_t i) { return __uint_as_float(uint32_t(p[i]) << 16); }
 __device__ __forceinline__ uint16_t to_bf16(float v) { return static_cast<uint16_t>(pack_bf16x2(v, 0.0f) & 0xFFFFu); }
 
+__device__ __forceinline__ float team_sum(float v, int team) {
+  for (int o = team >> 1; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+
 __device__ __forceinline__ float block_sum(float v, float* red) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  v = team_sum(v, 32);
   const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-  __syncthreads();
   if (l == 0) red[w] = v;
   __syncthreads();
   float t = 0.0f;
@@ -44,117 +47,330 @@ __device__ __forceinline__ float block_sum(float v, float* red) {
 }
 
 // ---------------------------------------------------------------- RMSNorm
-__device__ __forceinline__ float load_act(const uint16_t* p, int64_t i) { return bf16_at(p, i); }
-__device__ __forceinline__ float load_act(const float* p, int64_t i) { return p[i]; }
+// Both directions are bound by HBM: a row's 16-byte vectors (8 elements) are loaded once, kept
+// as loaded (bf16 packed) in registers through the row's sum and unpacked again for the output,
+// so that a thread holds many rows' or vectors' loads in flight.  A row of at most 1024 elements
+// belongs to a team of lanes (16 lanes for a 128-wide attention head, so a warp holds two rows at
+// a time, four times over), a longer one to a CTA; VPL vectors per thread.  On one GB300, against
+// kernels that loaded 2-byte elements twice: backward of 8192 rows of 4096 (fp32 row, two
+// gradients and the residual's, 403 MB) 124 -> 64 us = 6.3 TB/s, forward 76 -> 60 us; backward of
+// 262144 head rows of 128 (201 MB) 64 -> 49 us, forward (134 MB) 47 -> 27 us.
+__device__ __forceinline__ void unpack8(const uint4& v, float (&f)[8]) {
+  const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    f[2 * i] = bf16lo_to_f32(w[i]);
+    f[2 * i + 1] = bf16hi_to_f32(w[i]);
+  }
+}
 
-// One CTA per token row: h = x (+ residual, in fp32, stored unrounded when h_out is given),
-// r = 1 / sqrt(mean(h^2) + eps), z = gamma * h * r.
+__device__ __forceinline__ uint4 pack8(const float (&f)[8]) {
+  return make_uint4(pack_bf16x2(f[0], f[1]), pack_bf16x2(f[2], f[3]), pack_bf16x2(f[4], f[5]),
+                    pack_bf16x2(f[6], f[7]));
+}
+
+// Eight consecutive elements as loaded.
+template <typename T>
+struct Raw8;
+template <>
+struct Raw8<uint16_t> {
+  uint4 q;
+  __device__ __forceinline__ void load(const uint16_t* p) { q = *reinterpret_cast<const uint4*>(p); }
+  __device__ __forceinline__ void zero() { q = make_uint4(0u, 0u, 0u, 0u); }
+  __device__ __forceinline__ void get(float (&f)[8]) const { unpack8(q, f); }
+};
+template <>
+struct Raw8<float> {
+  float4 a, b;
+  __device__ __forceinline__ void load(const float* p) {
+    a = reinterpret_cast<const float4*>(p)[0];
+    b = reinterpret_cast<const float4*>(p)[1];
+  }
+  __device__ __forceinline__ void zero() { a = b = make_float4(0.f, 0.f, 0.f, 0.f); }
+  __device__ __forceinline__ void get(float (&f)[8]) const {
+    f[0] = a.x; f[1] = a.y; f[2] = a.z; f[3] = a.w;
+    f[4] = b.x; f[5] = b.y; f[6] = b.z; f[7] = b.w;
+  }
+};
+
+__device__ __forceinline__ void load8(const uint16_t* p, float (&f)[8]) {
+  unpack8(*reinterpret_cast<const uint4*>(p), f);
+}
+// The norm's weights carry no alignment beyond their type's: GVEC when they are 16-byte aligned.
+template <bool GVEC>
+__device__ __forceinline__ void load_gamma8(const float* p, float (&f)[8]) {
+  if constexpr (GVEC) {
+    Raw8<float> v;
+    v.load(p);
+    v.get(f);
+  } else {
+#pragma unroll
+    for (int i = 0; i < 8; ++i) f[i] = __ldg(p + i);
+  }
+}
+
+// One vector of the forward: h = x (+ residual in fp32, never rounded).
 template <typename TX>
+struct FwdVec {
+  Raw8<TX> x;
+  Raw8<uint16_t> res;
+  __device__ __forceinline__ void load(const TX* xp, const uint16_t* rp, int64_t at) {
+    x.load(xp + at);
+    if (rp) res.load(rp + at);
+  }
+  __device__ __forceinline__ void h(bool with_res, float (&f)[8]) const {
+    x.get(f);
+    if (with_res) {
+      float q[8];
+      res.get(q);
+#pragma unroll
+      for (int i = 0; i < 8; ++i) f[i] += q[i];
+    }
+  }
+  // its squares added to s; h stored when h_out is given
+  __device__ __forceinline__ float sum(bool with_res, float* h_out, int64_t at, float s) const {
+    float f[8];
+    h(with_res, f);
+    if (h_out) {
+      reinterpret_cast<float4*>(h_out + at)[0] = make_float4(f[0], f[1], f[2], f[3]);
+      reinterpret_cast<float4*>(h_out + at)[1] = make_float4(f[4], f[5], f[6], f[7]);
+    }
+#pragma unroll
+    for (int i = 0; i < 8; ++i) s = fmaf(f[i], f[i], s);
+    return s;
+  }
+  // z = gamma * h * r
+  template <bool GVEC>
+  __device__ __forceinline__ void store_z(bool with_res, const float* gamma, int64_t col, float rr, uint16_t* z) const {
+    float f[8], g[8];
+    h(with_res, f);
+    load_gamma8<GVEC>(gamma + col, g);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) f[i] = g[i] * f[i] * rr;
+    *reinterpret_cast<uint4*>(z) = pack8(f);
+  }
+};
+
+// One vector of the backward: dx = r u - h r^3 mean(u h) (+ dres), u = gamma (dy + dy2).
+template <typename TH>
+struct BwdVec {
+  Raw8<TH> x;
+  Raw8<uint16_t> dy, dy2, dres;
+  __device__ __forceinline__ void load(const TH* xp, const uint16_t* d1, const uint16_t* d2, const uint16_t* dr,
+                                       int64_t at) {
+    dy.load(d1 + at);
+    if (d2) dy2.load(d2 + at);
+    x.load(xp + at);
+    if (dr) dres.load(dr + at);
+  }
+  template <bool GVEC>
+  __device__ __forceinline__ void u(bool two, const float* gamma, int64_t col, float (&f)[8]) const {
+    float g[8];
+    dy.get(f);
+    if (two) {
+      float q[8];
+      dy2.get(q);
+#pragma unroll
+      for (int i = 0; i < 8; ++i) f[i] += q[i];
+    }
+    load_gamma8<GVEC>(gamma + col, g);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) f[i] *= g[i];
+  }
+  template <bool GVEC>
+  __device__ __forceinline__ float dot(bool two, const float* gamma, int64_t col, float s) const {
+    float f[8], h[8];
+    u<GVEC>(two, gamma, col, f);
+    x.get(h);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) s = fmaf(f[i], h[i], s);
+    return s;
+  }
+  template <bool GVEC>
+  __device__ __forceinline__ void store_dx(bool two, bool with_res, const float* gamma, int64_t col, float rr, float c,
+                                           uint16_t* dx) const {
+    float f[8], h[8];
+    u<GVEC>(two, gamma, col, f);
+    x.get(h);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) f[i] = rr * f[i] - h[i] * c;
+    if (with_res) {
+      dres.get(h);
+#pragma unroll
+      for (int i = 0; i < 8; ++i) f[i] += h[i];
+    }
+    *reinterpret_cast<uint4*>(dx) = pack8(f);
+  }
+};
+
+// One CTA per row; rows of more than 8 VPL kRowThreads elements load their further vectors
+// twice.
+template <typename TX, bool GVEC, int VPL>
 __global__ void __launch_bounds__(kRowThreads) rmsnorm_fwd_kernel(const TX* __restrict__ x,
                                                                    const uint16_t* __restrict__ res,
                                                                    const float* __restrict__ gamma, int64_t H,
                                                                    float eps, float* __restrict__ h_out,
                                                                    uint16_t* __restrict__ z, float* __restrict__ r) {
   __shared__ float red[kRowThreads / 32];
-  const int64_t t = blockIdx.x;
+  const int64_t t = blockIdx.x, row = t * H;
+  const int nvec = static_cast<int>(H / 8);
+  FwdVec<TX> q[VPL];
   float ss = 0.0f;
-  for (int64_t i = threadIdx.x; i < H; i += kRowThreads) {
-    float h = load_act(x, t * H + i);
-    if (res) h += bf16_at(res, t * H + i);
-    if (h_out) h_out[t * H + i] = h;
-    ss = fmaf(h, h, ss);
+#pragma unroll
+  for (int k = 0; k < VPL; ++k) {
+    const int v = threadIdx.x + k * kRowThreads;
+    if (v < nvec) q[k].load(x, res, row + 8 * v);
+  }
+#pragma unroll
+  for (int k = 0; k < VPL; ++k) {
+    const int v = threadIdx.x + k * kRowThreads;
+    if (v < nvec) ss = q[k].sum(res != nullptr, h_out, row + 8 * v, ss);
+  }
+  for (int v = threadIdx.x + VPL * kRowThreads; v < nvec; v += kRowThreads) {
+    FwdVec<TX> w;
+    w.load(x, res, row + 8 * v);
+    ss = w.sum(res != nullptr, h_out, row + 8 * v, ss);
   }
   const float rr = rsqrtf(block_sum(ss, red) / static_cast<float>(H) + eps);
   if (threadIdx.x == 0) r[t] = rr;
-  for (int64_t i = threadIdx.x; i < H; i += kRowThreads) {
-    float h = load_act(x, t * H + i);
-    if (res) h += bf16_at(res, t * H + i);
-    z[t * H + i] = to_bf16(gamma[i] * h * rr);
+#pragma unroll
+  for (int k = 0; k < VPL; ++k) {
+    const int v = threadIdx.x + k * kRowThreads;
+    if (v < nvec) q[k].template store_z<GVEC>(res != nullptr, gamma, 8 * v, rr, z + row + 8 * v);
+  }
+  for (int v = threadIdx.x + VPL * kRowThreads; v < nvec; v += kRowThreads) {
+    FwdVec<TX> w;
+    w.load(x, res, row + 8 * v);
+    w.template store_z<GVEC>(res != nullptr, gamma, 8 * v, rr, z + row + 8 * v);
   }
 }
 
-// dx = r u - h r^3 mean(u h) (+ dres), u = gamma (dy + dy2).
-template <typename TH>
+// dx may alias dy, dy2 or dres: a thread stores only vectors that it alone loads, after loading
+// them for the last time.
+template <typename TH, bool GVEC, int VPL>
 __global__ void __launch_bounds__(kRowThreads) rmsnorm_bwd_kernel(const TH* __restrict__ x,
                                                                    const float* __restrict__ gamma,
                                                                    const float* __restrict__ r, const uint16_t* dy,
                                                                    const uint16_t* dy2, const uint16_t* dres,
-                                                                   int64_t H, uint16_t* dx) {  // dx may alias
+                                                                   int64_t H, uint16_t* dx) {
   __shared__ float red[kRowThreads / 32];
-  const int64_t t = blockIdx.x;
+  const int64_t t = blockIdx.x, row = t * H;
+  const int nvec = static_cast<int>(H / 8);
+  const bool two = dy2 != nullptr, with_res = dres != nullptr;
+  BwdVec<TH> q[VPL];
+#pragma unroll
+  for (int k = 0; k < VPL; ++k) {
+    const int v = threadIdx.x + k * kRowThreads;
+    if (v < nvec) q[k].load(x, dy, dy2, dres, row + 8 * v);
+  }
   const float rr = r[t];
   float sux = 0.0f;
-  for (int64_t i = threadIdx.x; i < H; i += kRowThreads) {
-    const float g = bf16_at(dy, t * H + i) + (dy2 ? bf16_at(dy2, t * H + i) : 0.0f);
-    sux = fmaf(gamma[i] * g, load_act(x, t * H + i), sux);
+#pragma unroll
+  for (int k = 0; k < VPL; ++k) {
+    const int v = threadIdx.x + k * kRowThreads;
+    if (v < nvec) sux = q[k].template dot<GVEC>(two, gamma, 8 * v, sux);
+  }
+  for (int v = threadIdx.x + VPL * kRowThreads; v < nvec; v += kRowThreads) {
+    BwdVec<TH> w;
+    w.load(x, dy, dy2, nullptr, row + 8 * v);
+    sux = w.template dot<GVEC>(two, gamma, 8 * v, sux);
   }
   const float c = block_sum(sux, red) / static_cast<float>(H) * rr * rr * rr;
-  for (int64_t i = threadIdx.x; i < H; i += kRowThreads) {
-    const float g = bf16_at(dy, t * H + i) + (dy2 ? bf16_at(dy2, t * H + i) : 0.0f);
-    float v = rr * gamma[i] * g - load_act(x, t * H + i) * c;
-    if (dres) v += bf16_at(dres, t * H + i);
-    dx[t * H + i] = to_bf16(v);
+#pragma unroll
+  for (int k = 0; k < VPL; ++k) {
+    const int v = threadIdx.x + k * kRowThreads;
+    if (v < nvec) q[k].template store_dx<GVEC>(two, with_res, gamma, 8 * v, rr, c, dx + row + 8 * v);
+  }
+  for (int v = threadIdx.x + VPL * kRowThreads; v < nvec; v += kRowThreads) {
+    BwdVec<TH> w;
+    w.load(x, dy, dy2, dres, row + 8 * v);
+    w.template store_dx<GVEC>(two, with_res, gamma, 8 * v, rr, c, dx + row + 8 * v);
   }
 }
 
-// Rows of at most 1024 elements (e.g. one attention head, the Qwen3 query/key norm): one warp
-// per row, the same arithmetic as the kernels above.
+// Rows of at most 1024 elements: a team of `team` lanes (a power of two) per row, VPL vectors per
+// lane, U rows of every team of a warp in flight at once.
 constexpr int kRowWarps = kRowThreads / 32;
 
-__device__ __forceinline__ float warp_sum(float v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
-}
-
-template <typename TX>
-__global__ void __launch_bounds__(kRowThreads) rmsnorm_fwd_warp_kernel(const TX* __restrict__ x,
+template <typename TX, bool GVEC, int VPL, int U>
+__global__ void __launch_bounds__(kRowThreads) rmsnorm_fwd_team_kernel(const TX* __restrict__ x,
                                                                         const uint16_t* __restrict__ res,
                                                                         const float* __restrict__ gamma, int64_t T,
-                                                                        int64_t H, float eps,
+                                                                        int32_t H, int32_t team, float eps,
                                                                         float* __restrict__ h_out,
                                                                         uint16_t* __restrict__ z,
                                                                         float* __restrict__ r) {
-  const int lane = threadIdx.x & 31;
-  for (int64_t t = (blockIdx.x * (int64_t)kRowWarps) + (threadIdx.x >> 5); t < T; t += (int64_t)gridDim.x * kRowWarps) {
-    float ss = 0.0f;
-    for (int64_t i = lane; i < H; i += 32) {
-      float h = load_act(x, t * H + i);
-      if (res) h += bf16_at(res, t * H + i);
-      if (h_out) h_out[t * H + i] = h;
-      ss = fmaf(h, h, ss);
+  const int lane = threadIdx.x & 31, sub = lane & (team - 1), nvec = H / 8;
+  const int per_warp = 32 / team;
+  const int64_t t0 =
+      (blockIdx.x * static_cast<int64_t>(kRowWarps) + (threadIdx.x >> 5)) * per_warp * U + lane / team;
+  FwdVec<TX> q[U][VPL];
+#pragma unroll
+  for (int k = 0; k < U; ++k) {
+    const int64_t t = t0 + k * per_warp;
+#pragma unroll
+    for (int u = 0; u < VPL; ++u) {
+      const int v = sub + u * team;
+      if (t < T && v < nvec) q[k][u].load(x, res, t * H + 8 * v);
     }
-    const float rr = rsqrtf(warp_sum(ss) / static_cast<float>(H) + eps);
-    if (lane == 0) r[t] = rr;
-    for (int64_t i = lane; i < H; i += 32) {
-      float h = load_act(x, t * H + i);
-      if (res) h += bf16_at(res, t * H + i);
-      z[t * H + i] = to_bf16(gamma[i] * h * rr);
+  }
+#pragma unroll
+  for (int k = 0; k < U; ++k) {
+    const int64_t t = t0 + k * per_warp;
+    float ss = 0.0f;
+#pragma unroll
+    for (int u = 0; u < VPL; ++u) {
+      const int v = sub + u * team;
+      if (t < T && v < nvec) ss = q[k][u].sum(res != nullptr, h_out, t * H + 8 * v, ss);
+    }
+    const float rr = rsqrtf(team_sum(ss, team) / static_cast<float>(H) + eps);  // every lane of the warp
+    if (t < T && sub == 0) r[t] = rr;
+#pragma unroll
+    for (int u = 0; u < VPL; ++u) {
+      const int v = sub + u * team;
+      if (t < T && v < nvec) q[k][u].template store_z<GVEC>(res != nullptr, gamma, 8 * v, rr, z + t * H + 8 * v);
     }
   }
 }
 
-template <typename TH>
-__global__ void __launch_bounds__(kRowThreads) rmsnorm_bwd_warp_kernel(const TH* __restrict__ x,
+template <typename TH, bool GVEC, int VPL, int U>
+__global__ void __launch_bounds__(kRowThreads) rmsnorm_bwd_team_kernel(const TH* __restrict__ x,
                                                                         const float* __restrict__ gamma,
                                                                         const float* __restrict__ r,
                                                                         const uint16_t* dy, const uint16_t* dy2,
-                                                                        const uint16_t* dres, int64_t T, int64_t H,
-                                                                        uint16_t* dx) {  // dx may alias
-  const int lane = threadIdx.x & 31;
-  for (int64_t t = (blockIdx.x * (int64_t)kRowWarps) + (threadIdx.x >> 5); t < T; t += (int64_t)gridDim.x * kRowWarps) {
-    const float rr = r[t];
-    float sux = 0.0f;
-    for (int64_t i = lane; i < H; i += 32) {
-      const float g = bf16_at(dy, t * H + i) + (dy2 ? bf16_at(dy2, t * H + i) : 0.0f);
-      sux = fmaf(gamma[i] * g, load_act(x, t * H + i), sux);
+                                                                        const uint16_t* dres, int64_t T, int32_t H,
+                                                                        int32_t team, uint16_t* dx) {
+  const int lane = threadIdx.x & 31, sub = lane & (team - 1), nvec = H / 8;
+  const int per_warp = 32 / team;
+  const int64_t t0 =
+      (blockIdx.x * static_cast<int64_t>(kRowWarps) + (threadIdx.x >> 5)) * per_warp * U + lane / team;
+  const bool two = dy2 != nullptr, with_res = dres != nullptr;
+  BwdVec<TH> q[U][VPL];
+  float rr[U];
+#pragma unroll
+  for (int k = 0; k < U; ++k) {
+    const int64_t t = t0 + k * per_warp;
+    rr[k] = t < T ? r[t] : 0.0f;
+#pragma unroll
+    for (int u = 0; u < VPL; ++u) {
+      const int v = sub + u * team;
+      if (t < T && v < nvec) q[k][u].load(x, dy, dy2, dres, t * H + 8 * v);
     }
-    const float c = warp_sum(sux) / static_cast<float>(H) * rr * rr * rr;
-    for (int64_t i = lane; i < H; i += 32) {
-      const float g = bf16_at(dy, t * H + i) + (dy2 ? bf16_at(dy2, t * H + i) : 0.0f);
-      float v = rr * gamma[i] * g - load_act(x, t * H + i) * c;
-      if (dres) v += bf16_at(dres, t * H + i);
-      dx[t * H + i] = to_bf16(v);
+  }
+#pragma unroll
+  for (int k = 0; k < U; ++k) {
+    const int64_t t = t0 + k * per_warp;
+    float sux = 0.0f;
+#pragma unroll
+    for (int u = 0; u < VPL; ++u) {
+      const int v = sub + u * team;
+      if (t < T && v < nvec) sux = q[k][u].template dot<GVEC>(two, gamma, 8 * v, sux);
+    }
+    const float c = team_sum(sux, team) / static_cast<float>(H) * rr[k] * rr[k] * rr[k];
+#pragma unroll
+    for (int u = 0; u < VPL; ++u) {
+      const int v = sub + u * team;
+      if (t < T && v < nvec) q[k][u].template store_dx<GVEC>(two, with_res, gamma, 8 * v, rr[k], c, dx + t * H + 8 * v);
     }
   }
 }
@@ -183,16 +399,35 @@ __global__ void __launch_bounds__(kRowThreads) rope_kernel(uint16_t* __restrict_
 }
 
 // Rows of 8 consecutive elements of d = 16 k (half = 8 k) heads: one thread per (token, 8
-// consecutive i), its 8 angles computed once and applied to every head of the token with
-// 16-byte loads and stores.
+// consecutive i, run of `hpt` heads), its 8 angles computed once and applied to its heads with
+// 16-byte loads and stores.  Bound by HBM (4 bytes an element); the head runs give the launch
+// enough loads in flight (8192 tokens of 32 128-wide heads, 134 MB: 28 us with one thread per
+// token and i over all heads, 23 with runs of 4).
 __global__ void __launch_bounds__(kRowThreads) rope_vec_kernel(uint16_t* __restrict__ x, int64_t T, int64_t S,
                                                                 int32_t nheads, int32_t d, float log2_base,
-                                                                int32_t inverse) {
-  const int32_t half = d / 2, groups = half / 8;
-  const int64_t items = T * groups;
+                                                                int32_t inverse, int32_t hpt) {
+  const int32_t half = d / 2, groups = half / 8, runs = (nheads + hpt - 1) / hpt;
+  const int64_t items = T * groups * runs;
   for (int64_t e = blockIdx.x * (int64_t)kRowThreads + threadIdx.x; e < items; e += (int64_t)gridDim.x * kRowThreads) {
     const int32_t i0 = static_cast<int32_t>(e % groups) * 8;
-    const int64_t t = e / groups;
+    const int64_t tr = e / groups;
+    const int32_t h0 = static_cast<int32_t>(tr % runs) * hpt;
+    const int64_t t = tr / runs;
+    const int32_t h1 = min(h0 + hpt, nheads);
+    // four heads' loads go out before any store, which the compiler could not move them over, and
+    // the first four before the angles, which cover their latency
+    constexpr int kAhead = 4;
+    uint4 av[kAhead], bv[kAhead];
+    auto load = [&](int32_t hb) {
+#pragma unroll
+      for (int u = 0; u < kAhead; ++u)
+        if (hb + u < h1) {
+          const uint16_t* p = x + (t * nheads + hb + u) * d + i0;
+          av[u] = *reinterpret_cast<const uint4*>(p);
+          bv[u] = *reinterpret_cast<const uint4*>(p + half);
+        }
+    };
+    load(h0);
     const float pos = static_cast<float>(t % S);
     float cs[8], sn[8];
 #pragma unroll
@@ -201,21 +436,23 @@ __global__ void __launch_bounds__(kRowThreads) rope_vec_kernel(uint16_t* __restr
       sincosf(pos * inv_freq, &sn[j], &cs[j]);
       if (inverse) sn[j] = -sn[j];
     }
-    for (int32_t h = 0; h < nheads; ++h) {
-      uint16_t* p = x + (t * nheads + h) * d;
-      const uint4 av = *reinterpret_cast<const uint4*>(p + i0), bv = *reinterpret_cast<const uint4*>(p + i0 + half);
-      const uint32_t aw[4] = {av.x, av.y, av.z, av.w}, bw[4] = {bv.x, bv.y, bv.z, bv.w};
-      uint32_t ow[4], qw[4];
+    for (int32_t hb = h0; hb < h1; hb += kAhead) {
+      if (hb > h0) load(hb);
 #pragma unroll
-      for (int w = 0; w < 4; ++w) {
-        const float a0 = bf16lo_to_f32(aw[w]), a1 = bf16hi_to_f32(aw[w]);
-        const float b0 = bf16lo_to_f32(bw[w]), b1 = bf16hi_to_f32(bw[w]);
-        const int j = 2 * w;
-        ow[w] = pack_bf16x2(a0 * cs[j] - b0 * sn[j], a1 * cs[j + 1] - b1 * sn[j + 1]);
-        qw[w] = pack_bf16x2(a0 * sn[j] + b0 * cs[j], a1 * sn[j + 1] + b1 * cs[j + 1]);
-      }
-      *reinterpret_cast<uint4*>(p + i0) = make_uint4(ow[0], ow[1], ow[2], ow[3]);
-      *reinterpret_cast<uint4*>(p + i0 + half) = make_uint4(qw[0], qw[1], qw[2], qw[3]);
+      for (int u = 0; u < kAhead; ++u)
+        if (hb + u < h1) {
+          uint16_t* p = x + (t * nheads + hb + u) * d + i0;
+          float a[8], b[8], o[8], q[8];
+          unpack8(av[u], a);
+          unpack8(bv[u], b);
+#pragma unroll
+          for (int j = 0; j < 8; ++j) {
+            o[j] = a[j] * cs[j] - b[j] * sn[j];
+            q[j] = a[j] * sn[j] + b[j] * cs[j];
+          }
+          *reinterpret_cast<uint4*>(p) = pack8(o);
+          *reinterpret_cast<uint4*>(p + half) = pack8(q);
+        }
     }
   }
 }
@@ -223,20 +460,6 @@ __global__ void __launch_bounds__(kRowThreads) rope_vec_kernel(uint16_t* __restr
 // ---------------------------------------------------------------- SwiGLU
 // Eight elements per thread and iteration (16-byte loads and stores); block 0 takes the tail.
 __device__ __forceinline__ float sigmoidf(float a) { return 1.0f / (1.0f + expf(-a)); }
-
-__device__ __forceinline__ void unpack8(const uint4& v, float (&f)[8]) {
-  const uint32_t w[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    f[2 * i] = bf16lo_to_f32(w[i]);
-    f[2 * i + 1] = bf16hi_to_f32(w[i]);
-  }
-}
-
-__device__ __forceinline__ uint4 pack8(const float (&f)[8]) {
-  return make_uint4(pack_bf16x2(f[0], f[1]), pack_bf16x2(f[2], f[3]), pack_bf16x2(f[4], f[5]),
-                    pack_bf16x2(f[6], f[7]));
-}
 
 __global__ void __launch_bounds__(kRowThreads) swiglu_fwd_kernel(const uint16_t* __restrict__ gt,
                                                                   const uint16_t* __restrict__ u, int64_t n,
@@ -576,25 +799,27 @@ __global__ void __launch_bounds__(kAttnThreads) attn_fwd_kernel(const AttnArgs a
   }
 }
 
-// delta[b, h, s] = sum over the head's columns of dO * O (one warp per token and head).
+// delta[b, h, s] = sum over the head's columns of dO * O.  HD / 8 lanes per row, each one
+// 16-byte vector of O and dO; a CTA takes as many consecutive tokens of one head as it has such
+// teams (16 or 32, which divide S), so that their sums leave as whole sectors.  Bound by HBM:
+// 134 MB of the 8B block's 4 x 2048 tokens in 25 us = 5.3 TB/s (a warp per row with 2-byte loads:
+// 64).
 template <int HD>
 __global__ void __launch_bounds__(kRowThreads) attn_delta_kernel(const AttnArgs a) {
-  const int64_t rows = static_cast<int64_t>(a.B) * a.S * a.nh;
-  const int lane = threadIdx.x & 31;
-  for (int64_t w = (blockIdx.x * (int64_t)kRowThreads + threadIdx.x) >> 5; w < rows;
-       w += ((int64_t)gridDim.x * kRowThreads) >> 5) {
-    const int64_t tok = w / a.nh;
+  constexpr int kTeam = HD / 8, kTok = kRowThreads / kTeam;
+  const int64_t blocks = static_cast<int64_t>(a.B) * (a.S / kTok) * a.nh;
+  const int sub = threadIdx.x % kTeam, row = threadIdx.x / kTeam;
+  for (int64_t w = blockIdx.x; w < blocks; w += gridDim.x) {
     const int h = static_cast<int>(w % a.nh);
-    const uint16_t* o = a.o + tok * a.nh * HD + static_cast<int64_t>(h) * HD;
-    const uint16_t* d = a.dO + tok * a.nh * HD + static_cast<int64_t>(h) * HD;
-    float s = 0.0f;
-    for (int i = lane; i < HD; i += 32) s = fmaf(bf16_at(o, i), bf16_at(d, i), s);
+    const int64_t tok = w / a.nh * kTok + row;
+    const int64_t at = (tok * a.nh + h) * HD + 8 * sub;
+    float o[8], d[8], s = 0.0f;
+    load8(a.o + at, o);
+    load8(a.dO + at, d);
 #pragma unroll
-    for (int o2 = 16; o2 > 0; o2 >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o2);
-    if (lane == 0) {
-      const int64_t b = tok / a.S, sidx = tok % a.S;
-      a.delta[(b * a.nh + h) * a.S + sidx] = s;
-    }
+    for (int i = 0; i < 8; ++i) s = fmaf(o[i], d[i], s);
+    s = team_sum(s, kTeam);
+    if (sub == 0) a.delta[(tok / a.S * a.nh + h) * a.S + tok % a.S] = s;
   }
 }
 
@@ -819,7 +1044,7 @@ cudaError_t attn_launch(const AttnArgs& a, bool backward, cudaStream_t st) {
     return cudaGetLastError();
   }
   const int64_t rows = static_cast<int64_t>(a.B) * a.S * a.nh;
-  attn_delta_kernel<HD><<<elem_grid(rows * 32), kRowThreads, 0, st>>>(a);
+  attn_delta_kernel<HD><<<elem_grid(rows * (HD / 8)), kRowThreads, 0, st>>>(a);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   // 128-wide heads over whole 128-token tiles: dQ and dK/dV on tcgen05 (attn_tc.cu)
@@ -840,27 +1065,84 @@ cudaError_t attn_launch(const AttnArgs& a, bool backward, cudaStream_t st) {
 
 }  // namespace
 
+namespace {
+
+bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
+
+// Lanes per row of the team kernels: one vector per lane up to 256 elements (four rows of a team in
+// flight, two of fp32 input), then 2 or 4 vectors per lane of a whole warp.
+int row_team(int64_t H) {
+  int team = 1;
+  while (team < 32 && team * 8 < H) team *= 2;
+  return team;
+}
+
+unsigned row_grid(int64_t T, int team, int in_flight) {
+  const int64_t rows = static_cast<int64_t>(kRowWarps) * (32 / team) * in_flight;
+  return static_cast<unsigned>((T + rows - 1) / rows);
+}
+
+template <typename TX, bool GVEC>
+cudaError_t run_rmsnorm_fwd(const TX* x, const uint16_t* res, const float* gamma, int64_t T, int64_t H, float eps,
+                            float* h_out, uint16_t* z, float* r, cudaStream_t st) {
+  const int team = row_team(H), h32 = static_cast<int>(H);
+  const unsigned rows = static_cast<unsigned>(T);
+  constexpr int U = sizeof(TX) == 2 ? 4 : 2;
+  if (H <= 256)
+    rmsnorm_fwd_team_kernel<TX, GVEC, 1, U><<<row_grid(T, team, U), kRowThreads, 0, st>>>(x, res, gamma, T, h32, team,
+                                                                                         eps, h_out, z, r);
+  else if (H <= 512)
+    rmsnorm_fwd_team_kernel<TX, GVEC, 2, 1><<<row_grid(T, team, 1), kRowThreads, 0, st>>>(x, res, gamma, T, h32, team,
+                                                                                         eps, h_out, z, r);
+  else if (H <= 1024)
+    rmsnorm_fwd_team_kernel<TX, GVEC, 4, 1><<<row_grid(T, team, 1), kRowThreads, 0, st>>>(x, res, gamma, T, h32, team,
+                                                                                         eps, h_out, z, r);
+  else if (H <= 8 * kRowThreads)
+    rmsnorm_fwd_kernel<TX, GVEC, 1><<<rows, kRowThreads, 0, st>>>(x, res, gamma, H, eps, h_out, z, r);
+  else if (H <= 16 * kRowThreads)
+    rmsnorm_fwd_kernel<TX, GVEC, 2><<<rows, kRowThreads, 0, st>>>(x, res, gamma, H, eps, h_out, z, r);
+  else
+    rmsnorm_fwd_kernel<TX, GVEC, 4><<<rows, kRowThreads, 0, st>>>(x, res, gamma, H, eps, h_out, z, r);
+  return cudaGetLastError();
+}
+
+template <typename TH, bool GVEC>
+cudaError_t run_rmsnorm_bwd(const TH* x, const float* gamma, const float* r, const uint16_t* dy, const uint16_t* dy2,
+                            const uint16_t* dres, int64_t T, int64_t H, uint16_t* dx, cudaStream_t st) {
+  const int team = row_team(H), h32 = static_cast<int>(H);
+  const unsigned rows = static_cast<unsigned>(T);
+  constexpr int U = sizeof(TH) == 2 ? 4 : 2;
+  if (H <= 256)
+    rmsnorm_bwd_team_kernel<TH, GVEC, 1, U><<<row_grid(T, team, U), kRowThreads, 0, st>>>(x, gamma, r, dy, dy2, dres, T,
+                                                                                         h32, team, dx);
+  else if (H <= 512)
+    rmsnorm_bwd_team_kernel<TH, GVEC, 2, 1><<<row_grid(T, team, 1), kRowThreads, 0, st>>>(x, gamma, r, dy, dy2, dres, T,
+                                                                                         h32, team, dx);
+  else if (H <= 1024)
+    rmsnorm_bwd_team_kernel<TH, GVEC, 4, 1><<<row_grid(T, team, 1), kRowThreads, 0, st>>>(x, gamma, r, dy, dy2, dres, T,
+                                                                                         h32, team, dx);
+  else if (H <= 8 * kRowThreads)
+    rmsnorm_bwd_kernel<TH, GVEC, 1><<<rows, kRowThreads, 0, st>>>(x, gamma, r, dy, dy2, dres, H, dx);
+  else if (H <= 16 * kRowThreads)
+    rmsnorm_bwd_kernel<TH, GVEC, 2><<<rows, kRowThreads, 0, st>>>(x, gamma, r, dy, dy2, dres, H, dx);
+  else
+    rmsnorm_bwd_kernel<TH, GVEC, 4><<<rows, kRowThreads, 0, st>>>(x, gamma, r, dy, dy2, dres, H, dx);
+  return cudaGetLastError();
+}
+
+}  // namespace
+
 cudaError_t launch_rmsnorm_fwd(const void* x, bool x_f32, const void* res, const float* gamma, int64_t T, int64_t H,
                                float eps, float* h_out, void* z, float* r, cudaStream_t st) {
   const auto* rp = static_cast<const uint16_t*>(res);
   auto* zp = static_cast<uint16_t*>(z);
-  if (H <= 1024) {
-    const unsigned grid = static_cast<unsigned>(std::min<int64_t>((T + kRowWarps - 1) / kRowWarps, 152 * 16));
-    if (x_f32)
-      rmsnorm_fwd_warp_kernel<float><<<grid, kRowThreads, 0, st>>>(static_cast<const float*>(x), rp, gamma, T, H, eps,
-                                                                   h_out, zp, r);
-    else
-      rmsnorm_fwd_warp_kernel<uint16_t><<<grid, kRowThreads, 0, st>>>(static_cast<const uint16_t*>(x), rp, gamma, T, H,
-                                                                      eps, h_out, zp, r);
-    return cudaGetLastError();
-  }
-  if (x_f32)
-    rmsnorm_fwd_kernel<float><<<static_cast<unsigned>(T), kRowThreads, 0, st>>>(static_cast<const float*>(x), rp, gamma,
-                                                                                H, eps, h_out, zp, r);
-  else
-    rmsnorm_fwd_kernel<uint16_t><<<static_cast<unsigned>(T), kRowThreads, 0, st>>>(static_cast<const uint16_t*>(x), rp,
-                                                                                   gamma, H, eps, h_out, zp, r);
-  return cudaGetLastError();
+  const auto* xf = static_cast<const float*>(x);
+  const auto* xh = static_cast<const uint16_t*>(x);
+  if (aligned16(gamma))
+    return x_f32 ? run_rmsnorm_fwd<float, true>(xf, rp, gamma, T, H, eps, h_out, zp, r, st)
+                 : run_rmsnorm_fwd<uint16_t, true>(xh, rp, gamma, T, H, eps, h_out, zp, r, st);
+  return x_f32 ? run_rmsnorm_fwd<float, false>(xf, rp, gamma, T, H, eps, h_out, zp, r, st)
+               : run_rmsnorm_fwd<uint16_t, false>(xh, rp, gamma, T, H, eps, h_out, zp, r, st);
 }
 
 cudaError_t launch_rmsnorm_bwd(const void* x, bool x_f32, const float* gamma, const float* r, const void* dy,
@@ -869,31 +1151,25 @@ cudaError_t launch_rmsnorm_bwd(const void* x, bool x_f32, const float* gamma, co
   const auto* dy2p = static_cast<const uint16_t*>(dy2);
   const auto* drp = static_cast<const uint16_t*>(dres);
   auto* dxp = static_cast<uint16_t*>(dx);
-  if (H <= 1024) {
-    const unsigned grid = static_cast<unsigned>(std::min<int64_t>((T + kRowWarps - 1) / kRowWarps, 152 * 16));
-    if (x_f32)
-      rmsnorm_bwd_warp_kernel<float><<<grid, kRowThreads, 0, st>>>(static_cast<const float*>(x), gamma, r, dyp, dy2p,
-                                                                   drp, T, H, dxp);
-    else
-      rmsnorm_bwd_warp_kernel<uint16_t><<<grid, kRowThreads, 0, st>>>(static_cast<const uint16_t*>(x), gamma, r, dyp,
-                                                                      dy2p, drp, T, H, dxp);
-    return cudaGetLastError();
-  }
-  if (x_f32)
-    rmsnorm_bwd_kernel<float><<<static_cast<unsigned>(T), kRowThreads, 0, st>>>(static_cast<const float*>(x), gamma, r,
-                                                                                dyp, dy2p, drp, H, dxp);
-  else
-    rmsnorm_bwd_kernel<uint16_t><<<static_cast<unsigned>(T), kRowThreads, 0, st>>>(static_cast<const uint16_t*>(x),
-                                                                                   gamma, r, dyp, dy2p, drp, H, dxp);
-  return cudaGetLastError();
+  const auto* xf = static_cast<const float*>(x);
+  const auto* xh = static_cast<const uint16_t*>(x);
+  if (aligned16(gamma))
+    return x_f32 ? run_rmsnorm_bwd<float, true>(xf, gamma, r, dyp, dy2p, drp, T, H, dxp, st)
+                 : run_rmsnorm_bwd<uint16_t, true>(xh, gamma, r, dyp, dy2p, drp, T, H, dxp, st);
+  return x_f32 ? run_rmsnorm_bwd<float, false>(xf, gamma, r, dyp, dy2p, drp, T, H, dxp, st)
+               : run_rmsnorm_bwd<uint16_t, false>(xh, gamma, r, dyp, dy2p, drp, T, H, dxp, st);
 }
 
 cudaError_t launch_rope(void* x, int64_t T, int64_t S, int32_t nheads, int32_t d, float base, int32_t inverse,
                         cudaStream_t st) {
-  if (d % 16 == 0)
-    rope_vec_kernel<<<elem_grid(T * (d / 16)), kRowThreads, 0, st>>>(static_cast<uint16_t*>(x), T, S, nheads, d,
-                                                                      log2f(base), inverse);
-  else
+  if (d % 16 == 0) {
+    // heads per thread: the longest run (fewest repeated angles) that still gives every SM a full
+    // set of threads
+    int32_t hpt = 8;
+    while (hpt > 1 && T * (d / 16) * ((nheads + hpt - 1) / hpt) < 152 * 2048) hpt /= 2;
+    rope_vec_kernel<<<elem_grid(T * (d / 16) * ((nheads + hpt - 1) / hpt)), kRowThreads, 0, st>>>(
+        static_cast<uint16_t*>(x), T, S, nheads, d, log2f(base), inverse, hpt);
+  } else
     rope_kernel<<<elem_grid(T * nheads * (d / 2)), kRowThreads, 0, st>>>(static_cast<uint16_t*>(x), T, S, nheads, d,
                                                                           log2f(base), inverse);
   return cudaGetLastError();
