@@ -64,13 +64,13 @@ __device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t (&r)[32
 __device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 
 // D[tmem] (+)= A[tmem] * B[smem] (A: M x K bf16 in TMEM, one row per lane, column j holding
-// elements 2j and 2j + 1 of the row).
-__device__ __forceinline__ void umma_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t bdesc, uint32_t idesc,
+// elements 2j and 2j + 1 of the row; B by its descriptor's lower half).
+__device__ __forceinline__ void umma_ts(uint32_t d_tmem, uint32_t a_tmem, uint32_t b_lo, uint32_t idesc,
                                         uint32_t accumulate) {
   asm volatile(
-      "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}" ::"r"(d_tmem),
-      "r"(a_tmem), "l"(bdesc), "r"(idesc), "r"(accumulate)
+      "{\n\t.reg .pred p;\n\t.reg .b64 db;\n\tsetp.ne.b32 p, %4, 0;\n\tmov.b64 db, {%2, %5};\n\t"
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], db, %3, p;\n\t}" ::"r"(d_tmem),
+      "r"(a_tmem), "r"(b_lo), "r"(idesc), "r"(accumulate), "r"(kDescHi)
       : "memory");
 }
 
@@ -84,6 +84,27 @@ __device__ __forceinline__ uint32_t pack2(float lo, float hi) {
   uint32_t r;
   asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi), "f"(lo));
   return r;
+}
+
+// K-major SS products: D = A B^T over d = 128 (A, B: 128 rows x 128 columns, two 64-column boxes
+// each).
+__device__ __forceinline__ void mma_kmajor(uint32_t d_tmem, uint32_t a_smem, uint32_t b_smem, uint32_t idesc) {
+  const uint32_t ad = desc_lo(a_smem, 16), bd = desc_lo(b_smem, 16);
+#pragma unroll
+  for (int kk = 0; kk < kHd / 16; ++kk) {
+    const uint32_t off = ((kk >> 2) * kBox + (kk & 3) * 32) / 16;
+    umma_lo<1>(d_tmem, ad + off, bd + off, idesc, kk > 0 ? 1u : 0u);
+  }
+}
+
+// TS products: D (+)= A[tmem] B[smem] over 128 (A: 128 x 128 bf16 in TMEM, B: the 128-row
+// tile read as K x N with N contiguous).
+__device__ __forceinline__ void mma_ts_tile(uint32_t d_tmem, uint32_t a_tmem, uint32_t b_smem, uint32_t idesc,
+                                            bool accumulate) {
+  const uint32_t bd = desc_lo(b_smem, kBox);
+#pragma unroll
+  for (int kk = 0; kk < 8; ++kk)
+    umma_ts(d_tmem, a_tmem + 8u * kk, bd + kk * (2048 / 16), idesc, (accumulate || kk > 0) ? 1u : 0u);
 }
 
 // Bounded wait for copies or MMAs still in flight when a launch gives up.
@@ -173,59 +194,55 @@ __global__ void __launch_bounds__(kThreadsTc, 1)
       for (int t = g - 2 < 0 ? 0 : g - 2; t < g; ++t) drain(kv_full0 + 8u * (t & 1), (t >> 1) & 1);
     }
   } else if (warp == kMmaWarp) {
-    if (lane == 0) {
-      constexpr uint32_t idesc_s = idesc_bf16_f32(kTq, kTk, false, false);  // Q, K both K-major
-      constexpr uint32_t idesc_o = idesc_bf16_f32(kTq, kHd, false, true);   // V MN-major
-      // S_t = Q K^T of global tile t into score buffer t & 1; after an item's last one, the Q
-      // buffer is released
-      auto issue_s = [&](int t, bool last) -> bool {
-        if (!mbar_wait(kv_full0 + 8u * (t & 1), (t >> 1) & 1, a.wc)) return false;
-        tc_fence_after();
-        const uint32_t kt = base + kOffK + (t & 1) * kTile;
-#pragma unroll
-        for (int kk = 0; kk < kHd / 16; ++kk) {
-          const uint32_t off = (kk >> 2) * kBox + (kk & 3) * 32;
-          umma_bf16<1>(tmem + kColS0 + 128u * (t & 1), smem_desc_sw128(base + kOffQ + off, 16, 1024),
-                       smem_desc_sw128(kt + off, 16, 1024), idesc_s, kk > 0 ? 1u : 0u);
-        }
+    // the whole warp walks the items, one elected lane issues (see elect_one): with 16 to 32 MMAs
+    // a tile, single-lane issue took 1.7 to 3.4 thousand cycles of it (the 8B block's 4 x 2048
+    // tokens: forward 196 -> 187 us, dQ 240 -> 222, dK/dV 358 -> 341)
+    constexpr uint32_t idesc_s = idesc_bf16_f32(kTq, kTk, false, false);  // Q, K both K-major
+    constexpr uint32_t idesc_o = idesc_bf16_f32(kTq, kHd, false, true);   // V MN-major
+    const bool issuer = elect_one();
+    // S_t = Q K^T of global tile t into score buffer t & 1; after an item's last one, the Q
+    // buffer is released
+    auto issue_s = [&](int t, bool last) -> bool {
+      if (!mbar_wait_warp(kv_full0 + 8u * (t & 1), (t >> 1) & 1, a.wc)) return false;
+      tc_fence_after();
+      if (issuer) {
+        mma_kmajor(tmem + kColS0 + 128u * (t & 1), base + kOffQ, base + kOffK + (t & 1) * kTile, idesc_s);
         umma_commit<1>(s_full0 + 8u * (t & 1));
         if (last) umma_commit<1>(q_empty);
-        return true;
-      };
-      int g = 0, li = 0;
-      for (int it = blockIdx.x; ok && it < n_items; it += gridDim.x, ++li) {
-        int qt, h, b;
-        item_of(it, qt, h, b);
-        const int n = qt + 1;
-        const uint32_t ocol = tmem + kColO + 128u * (li & 1);
-        if (!mbar_wait(q_full, li & 1, a.wc) || !issue_s(g, n == 1)) { ok = false; break; }
-        for (int j = 0; ok && j < n; ++j) {
-          const int t = g + j;
-          if (j + 1 < n && !issue_s(t + 1, j + 2 == n)) { ok = false; break; }
-          if (!mbar_wait(p_full, t & 1, a.wc)) { ok = false; break; }
-          // the item's output buffer is free once the epilogue two items back has read it
-          if (j == 0 && li >= 2 && !mbar_wait(o_free0 + 8u * (li & 1), ((li >> 1) & 1) ^ 1, a.wc)) {
-            ok = false;
-            break;
-          }
-          tc_fence_after();
-          const uint32_t vt = base + kOffV + (t & 1) * kTile;
-          const uint32_t pcol = tmem + kColS0 + 128u * (t & 1);
-#pragma unroll
-          for (int kk = 0; kk < kTk / 16; ++kk)
-            umma_ts(ocol, pcol + 8u * kk, smem_desc_sw128(vt + kk * 2048, kBox, 1024), idesc_o,
-                    (j > 0 || kk > 0) ? 1u : 0u);
+      }
+      return true;
+    };
+    int g = 0, li = 0;
+    for (int it = blockIdx.x; ok && it < n_items; it += gridDim.x, ++li) {
+      int qt, h, b;
+      item_of(it, qt, h, b);
+      const int n = qt + 1;
+      const uint32_t ocol = tmem + kColO + 128u * (li & 1);
+      if (!mbar_wait_warp(q_full, li & 1, a.wc) || !issue_s(g, n == 1)) { ok = false; break; }
+      for (int j = 0; ok && j < n; ++j) {
+        const int t = g + j;
+        if (j + 1 < n && !issue_s(t + 1, j + 2 == n)) { ok = false; break; }
+        if (!mbar_wait_warp(p_full, t & 1, a.wc)) { ok = false; break; }
+        // the item's output buffer is free once the epilogue two items back has read it
+        if (j == 0 && li >= 2 && !mbar_wait_warp(o_free0 + 8u * (li & 1), ((li >> 1) & 1) ^ 1, a.wc)) {
+          ok = false;
+          break;
+        }
+        tc_fence_after();
+        if (issuer) {
+          mma_ts_tile(ocol, tmem + kColS0 + 128u * (t & 1), base + kOffV + (t & 1) * kTile, idesc_o, j > 0);
           umma_commit<1>(o_bar);
           umma_commit<1>(kv_empty0 + 8u * (t & 1));
         }
-        if (!ok) break;
-        umma_commit<1>(item_done0 + 8u * (li & 1));
-        g += n;
       }
-      // every MMA has completed before TMEM is released
-      umma_commit<1>(final_bar);
-      drain(final_bar, 0);
+      if (!ok) break;
+      if (issuer) umma_commit<1>(item_done0 + 8u * (li & 1));
+      g += n;
     }
+    // every MMA has completed before TMEM is released
+    if (issuer) umma_commit<1>(final_bar);
+    __syncwarp();
+    drain(final_bar, 0);
   } else {
     // softmax and epilogue: this thread's query row r of each item's tile (TMEM lane r)
     const int r = warp * 32 + lane;
@@ -374,27 +391,6 @@ __device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t (&r)[16
       : "memory");
 }
 
-// K-major SS products of the backward: D (+)= A B^T over d = 128 (A, B: 128 rows x 128
-// columns, two 64-column boxes each).
-__device__ __forceinline__ void mma_kmajor(uint32_t d_tmem, uint32_t a_smem, uint32_t b_smem, uint32_t idesc) {
-#pragma unroll
-  for (int kk = 0; kk < kHd / 16; ++kk) {
-    const uint32_t off = (kk >> 2) * kBox + (kk & 3) * 32;
-    umma_bf16<1>(d_tmem, smem_desc_sw128(a_smem + off, 16, 1024), smem_desc_sw128(b_smem + off, 16, 1024), idesc,
-                 kk > 0 ? 1u : 0u);
-  }
-}
-
-// TS products: D (+)= A[tmem] B[smem] over 128 (A: 128 x 128 bf16 in TMEM, B: the 128-row
-// tile read as K x N with N contiguous).
-__device__ __forceinline__ void mma_ts_tile(uint32_t d_tmem, uint32_t a_tmem, uint32_t b_smem, uint32_t idesc,
-                                            bool accumulate) {
-#pragma unroll
-  for (int kk = 0; kk < 8; ++kk)
-    umma_ts(d_tmem, a_tmem + 8u * kk, smem_desc_sw128(b_smem + kk * 2048, kBox, 1024), idesc,
-            (accumulate || kk > 0) ? 1u : 0u);
-}
-
 // dQ: persistent CTAs over (128-query tile, head, sequence) items (the forward's order), each
 // over the key tiles up to the diagonal.  TMEM: S [0, 128), dP [128, 256), dQ in two buffers
 // [256, 512) (one per item parity, so an item's epilogue overlaps the next item's products);
@@ -477,42 +473,46 @@ __global__ void __launch_bounds__(kThreadsTc, 1)
       for (int t = g - 2 < 0 ? 0 : g - 2; t < g; ++t) drain(kv_full0 + 8u * (t & 1), (t >> 1) & 1);
     }
   } else if (warp == kMmaWarp) {
-    if (lane == 0) {
-      constexpr uint32_t idesc_s = idesc_bf16_f32(kTq, kTk, false, false);
-      constexpr uint32_t idesc_q = idesc_bf16_f32(kTq, kHd, false, true);
-      int g = 0, li = 0;
-      for (int it = blockIdx.x; ok && it < n_items; it += gridDim.x, ++li) {
-        int qt, h, b;
-        item_of(it, qt, h, b);
-        const int n = qt + 1;
-        const uint32_t qcol = tmem + kColQ + 128u * (li & 1);
-        if (!mbar_wait(qd_full, li & 1, a.wc)) { ok = false; break; }
-        for (int j = 0; ok && j < n; ++j) {
-          const int t = g + j;
-          const uint32_t kt = base + kDqOffK + (t & 1) * kTile, vt = base + kDqOffV + (t & 1) * kTile;
-          if (!mbar_wait(kv_full0 + 8u * (t & 1), (t >> 1) & 1, a.wc)) { ok = false; break; }
-          tc_fence_after();
+    constexpr uint32_t idesc_s = idesc_bf16_f32(kTq, kTk, false, false);
+    constexpr uint32_t idesc_q = idesc_bf16_f32(kTq, kHd, false, true);
+    const bool issuer = elect_one();
+    int g = 0, li = 0;
+    for (int it = blockIdx.x; ok && it < n_items; it += gridDim.x, ++li) {
+      int qt, h, b;
+      item_of(it, qt, h, b);
+      const int n = qt + 1;
+      const uint32_t qcol = tmem + kColQ + 128u * (li & 1);
+      if (!mbar_wait_warp(qd_full, li & 1, a.wc)) { ok = false; break; }
+      for (int j = 0; ok && j < n; ++j) {
+        const int t = g + j;
+        const uint32_t kt = base + kDqOffK + (t & 1) * kTile, vt = base + kDqOffV + (t & 1) * kTile;
+        if (!mbar_wait_warp(kv_full0 + 8u * (t & 1), (t >> 1) & 1, a.wc)) { ok = false; break; }
+        tc_fence_after();
+        if (issuer) {
           mma_kmajor(tmem + kColS, base + kDqOffQ, kt, idesc_s);   // S = Q K^T
           mma_kmajor(tmem + kColP, base + kDqOffDo, vt, idesc_s);  // dP = dO V^T
           umma_commit<1>(s_full);
           if (j + 1 == n) umma_commit<1>(qd_empty);
-          if (!mbar_wait(ds_full, t & 1, a.wc)) { ok = false; break; }
-          // the item's dQ buffer is free once the epilogue two items back has read it
-          if (j == 0 && li >= 2 && !mbar_wait(dq_free0 + 8u * (li & 1), ((li >> 1) & 1) ^ 1, a.wc)) {
-            ok = false;
-            break;
-          }
-          tc_fence_after();
+        }
+        if (!mbar_wait_warp(ds_full, t & 1, a.wc)) { ok = false; break; }
+        // the item's dQ buffer is free once the epilogue two items back has read it
+        if (j == 0 && li >= 2 && !mbar_wait_warp(dq_free0 + 8u * (li & 1), ((li >> 1) & 1) ^ 1, a.wc)) {
+          ok = false;
+          break;
+        }
+        tc_fence_after();
+        if (issuer) {
           mma_ts_tile(qcol, tmem + kColS, kt, idesc_q, j > 0);  // dQ += dS K
           umma_commit<1>(kv_empty0 + 8u * (t & 1));
         }
-        if (!ok) break;
-        umma_commit<1>(item_done0 + 8u * (li & 1));
-        g += n;
       }
-      umma_commit<1>(final_bar);
-      drain(final_bar, 0);
+      if (!ok) break;
+      if (issuer) umma_commit<1>(item_done0 + 8u * (li & 1));
+      g += n;
     }
+    if (issuer) umma_commit<1>(final_bar);
+    __syncwarp();
+    drain(final_bar, 0);
   } else {
     const int r = warp * 32 + lane;
     const uint32_t lane_off = static_cast<uint32_t>(warp * 32) << 16;
@@ -670,26 +670,30 @@ __global__ void __launch_bounds__(kThreadsTc, 1)
       for (int t = issued - 2 < 0 ? 0 : issued - 2; t < issued; ++t) drain(st_full0 + 8u * (t & 1), (t >> 1) & 1);
     }
   } else if (warp == kMmaWarp) {
-    if (lane == 0) {
-      constexpr uint32_t idesc_s = idesc_bf16_f32(kTk, kTq, false, false);
-      constexpr uint32_t idesc_g = idesc_bf16_f32(kTk, kHd, false, true);
-      if (!mbar_wait(kv_full, 0, a.wc)) ok = false;
-      for (int t = 0; ok && t < nsteps; ++t) {
-        const uint32_t sb = base + kKvOffStage + (t & 1) * kStageBytes;
-        if (!mbar_wait(st_full0 + 8u * (t & 1), (t >> 1) & 1, a.wc)) { ok = false; break; }
-        tc_fence_after();
+    constexpr uint32_t idesc_s = idesc_bf16_f32(kTk, kTq, false, false);
+    constexpr uint32_t idesc_g = idesc_bf16_f32(kTk, kHd, false, true);
+    const bool issuer = elect_one();
+    if (!mbar_wait_warp(kv_full, 0, a.wc)) ok = false;
+    for (int t = 0; ok && t < nsteps; ++t) {
+      const uint32_t sb = base + kKvOffStage + (t & 1) * kStageBytes;
+      if (!mbar_wait_warp(st_full0 + 8u * (t & 1), (t >> 1) & 1, a.wc)) { ok = false; break; }
+      tc_fence_after();
+      if (issuer) {
         mma_kmajor(tmem + kColS, base + kKvOffK, sb, idesc_s);          // S^T = K Q^T
         mma_kmajor(tmem + kColP, base + kKvOffV, sb + kTile, idesc_s);  // dP^T = V dO^T
         umma_commit<1>(s_full);
-        if (!mbar_wait(pd_full, t & 1, a.wc)) { ok = false; break; }
-        tc_fence_after();
+      }
+      if (!mbar_wait_warp(pd_full, t & 1, a.wc)) { ok = false; break; }
+      tc_fence_after();
+      if (issuer) {
         mma_ts_tile(tmem + kColV, tmem + kColS, sb + kTile, idesc_g, t > 0);  // dV += P^T dO
         mma_ts_tile(tmem + kColK, tmem + kColP, sb, idesc_g, t > 0);          // dK += dS^T Q
         umma_commit<1>(st_empty0 + 8u * (t & 1));
       }
-      umma_commit<1>(final_bar);
-      drain(final_bar, 0);
     }
+    if (issuer) umma_commit<1>(final_bar);
+    __syncwarp();
+    drain(final_bar, 0);
   } else {
     const int rk = warp * 32 + lane;  // key row of the tile (TMEM lane)
     const uint32_t lane_off = static_cast<uint32_t>(warp * 32) << 16;

@@ -120,6 +120,13 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, const W
   }
 }
 
+// mbar_wait by a converged warp: every lane has seen the phase before any goes on (an issuing lane
+// that ran ahead could let the barrier pass a second phase under a lane still polling), and the
+// result is uniform.
+__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, const WaitCtl& w) {
+  return __all_sync(0xffffffffu, mbar_wait(bar, parity, w));
+}
+
 // Bring a contiguous range of global memory (16-byte aligned, a multiple of 16 bytes) into
 // L2 without waiting for it.
 __device__ __forceinline__ void prefetch_l2_bulk(const void* p, uint32_t bytes) {
@@ -333,6 +340,45 @@ __device__ __forceinline__ uint64_t smem_desc_sw128(uint32_t addr, uint32_t lbo,
   d |= (uint64_t)1 << 46;  // descriptor version for tcgen05
   d |= (uint64_t)2 << 61;  // 128-byte swizzle
   return d;
+}
+
+// The same descriptors as 32-bit halves.  The upper half is one constant for every 128-byte-swizzled
+// tile here (stride 1024); in the lower one the 14-bit address field counts 16-byte units, so
+// stepping through a tile is one addition.  (In a cluster a shared-memory address carries the CTA's
+// rank above its 24 bits of offset, which must not reach the descriptor.)
+constexpr uint32_t kDescHi = (1024u >> 4) | (1u << 14) | (2u << 29);
+__device__ __forceinline__ uint32_t desc_lo(uint32_t addr, uint32_t lbo) {
+  return ((addr >> 4) & 0x3FFFu) | ((lbo >> 4) << 16);
+}
+
+// One lane of a converged warp (the same one each time), as a predicate that the compiler knows to
+// be uniform: an MMA warp whose 32 lanes all walk the pipeline and whose elected lane issues keeps its
+// loop and its descriptors in uniform registers, where a single-lane branch moves every operand
+// of every MMA over from vector registers (about 100 cycles an MMA).
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
+  return p != 0;
+}
+
+// D[tmem] (+)= A[smem] * B[smem] with descriptors by their lower halves.
+template <int CG>
+__device__ __forceinline__ void umma_lo(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t idesc,
+                                        uint32_t accumulate) {
+  if constexpr (CG == 1)
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t.reg .b64 da, db;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+        "mov.b64 da, {%1, %5};\n\tmov.b64 db, {%2, %5};\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %3, p;\n\t}" ::"r"(d_tmem),
+        "r"(a_lo), "r"(b_lo), "r"(idesc), "r"(accumulate), "r"(kDescHi)
+        : "memory");
+  else
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t.reg .b64 da, db;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+        "mov.b64 da, {%1, %5};\n\tmov.b64 db, {%2, %5};\n\t"
+        "tcgen05.mma.cta_group::2.kind::f16 [%0], da, db, %3, p;\n\t}" ::"r"(d_tmem),
+        "r"(a_lo), "r"(b_lo), "r"(idesc), "r"(accumulate), "r"(kDescHi)
+        : "memory");
 }
 
 // Instruction descriptor for kind::f16: bf16 A and B, fp32 D, M x N tile.

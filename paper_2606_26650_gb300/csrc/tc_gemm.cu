@@ -552,8 +552,14 @@ __global__ void __launch_bounds__(FusedCfg<CG, PAIRS>::kThreads, 1)
     }
   } else if (warp == kMmaWarp) {
     // ------------------------------------------------------------ MMA issuer (even CTA of each pair)
-    if (cta == 0 && lane == 0) {
+    // The whole warp walks the pipeline and one elected lane issues (see elect_one): with every
+    // operand in uniform registers a stage's 8 MMAs issue in about 300 cycles instead of 860,
+    // well inside the 1024 that the tensor cores take for them.  1999 x 6144 x 2048: forward 80 ->
+    // 74 us, dX 58 -> 53; 128 experts' 65536 x 4096 x 1536: 833 -> 789 and 884 -> 845 us.
+    if (cta == 0) {
       constexpr uint32_t idesc = idesc_bf16_f32(Cfg::kRowsPerAcc, BN, false, B_MN);
+      constexpr uint32_t kStepB = (B_MN ? 2048 : 32) / 16;  // descriptor units per 16-deep step
+      const bool issuer = elect_one();
       const int T = args.num_k_blocks;
       // Accumulators drain and refill separately, so the epilogue overlaps the MMAs: a tile's
       // last J stages run accumulator 0 first (the epilogue drains it while accumulator 1
@@ -564,26 +570,31 @@ __global__ void __launch_bounds__(FusedCfg<CG, PAIRS>::kThreads, 1)
       bool ok = true;
       auto stage_in = [&](uint32_t qq) -> bool {  // wait for stage qq; arm a received slot's next use
         const uint32_t sa = qq % SA, pa = (qq / SA) & 1u, sw = qq % SW, pw = (qq / SW) & 1u;
-        if (!mbar_wait(full_a(sa), pa, wc) || !mbar_wait(full_w(sw), pw, wc)) return false;
-        if (PAIRS == 2 && (qq & 1u) != pair) mbar_arrive_expect_tx(full_w(sw), Cfg::kWBytes);
+        if (!mbar_wait_warp(full_a(sa), pa, wc) || !mbar_wait_warp(full_w(sw), pw, wc)) return false;
+        if (PAIRS == 2 && (qq & 1u) != pair && issuer) mbar_arrive_expect_tx(full_w(sw), Cfg::kWBytes);
         tc_fence_after();
         return true;
       };
       // An accumulator whose rows all lie past the tile's last row (an expert's short last M
       // block, or a ragged M) gets no MMAs; the epilogue stores nothing from it.
       bool live[NACC] = {};
-      auto issue = [&](uint32_t qq, int acc, bool first) {  // one accumulator's MMAs of stage qq
-        if (!live[acc]) return;
-        const uint32_t aa = a_base + (qq % SA) * Cfg::kABytes, ww = w_base + (qq % SW) * Cfg::kWBytes;
+      // accumulators acc0 .. acc1 - 1 of stage qq
+      auto issue = [&](uint32_t qq, int acc0, int acc1, bool first) {
+        const uint32_t ad = desc_lo(a_base + (qq % SA) * Cfg::kABytes, 16);
+        const uint32_t bd = desc_lo(w_base + (qq % SW) * Cfg::kWBytes, B_MN ? 8192 : 16);
+        if (issuer) {
 #pragma unroll
-        for (int kk = 0; kk < BK / 16; ++kk) {
-          const uint64_t bdesc = B_MN ? smem_desc_sw128(ww + kk * 2048, 8192, 1024)
-                                      : smem_desc_sw128(ww + kk * 32, 16, 1024);
-          const uint64_t adesc = smem_desc_sw128(aa + acc * (128 * BK * 2) + kk * 32, 16, 1024);
-          umma_bf16<CG>(tmem_base + acc * BN, adesc, bdesc, idesc, (first && kk == 0) ? 0u : 1u);
+          for (int acc = 0; acc < NACC; ++acc) {
+            if (acc < acc0 || acc >= acc1 || !live[acc]) continue;
+#pragma unroll
+            for (int kk = 0; kk < BK / 16; ++kk)
+              umma_lo<CG>(tmem_base + acc * BN, ad + acc * (128 * BK * 2 / 16) + kk * 2, bd + kk * kStepB, idesc,
+                          (first && kk == 0) ? 0u : 1u);
+          }
         }
       };
       auto release = [&](uint32_t qq) {  // both accumulators are done with stage qq
+        if (!issuer) return;
         if constexpr (PAIRS == 1) {
           umma_commit<CG>(empty_a(qq % SA));
           umma_commit<CG>(empty_w(qq % SW));
@@ -593,6 +604,7 @@ __global__ void __launch_bounds__(FusedCfg<CG, PAIRS>::kThreads, 1)
         }
       };
       auto full = [&](int acc) {
+        if (!issuer) return;
         if constexpr (PAIRS == 1) umma_commit<CG>(tmem_full0 + 8u * acc);
         else umma_commit_pair_mask(tmem_full0 + 8u * acc, pair_mask);
       };
@@ -605,24 +617,23 @@ __global__ void __launch_bounds__(FusedCfg<CG, PAIRS>::kThreads, 1)
         }
         const uint32_t ep = (it & 1u) ^ 1u;  // the epilogue has drained the previous tile's accumulator
         // head: accumulator 0 over stages 0 .. J-1
-        if (!mbar_wait(tmem_empty0, ep, wc)) break;
+        if (!mbar_wait_warp(tmem_empty0, ep, wc)) break;
         tc_fence_after();
         for (int h = 0; ok && h < J; ++h) {
           if (!stage_in(q + h)) { ok = false; break; }
-          issue(q + h, 0, h == 0);
+          issue(q + h, 0, 1, h == 0);
         }
-        if (!ok || !mbar_wait(tmem_empty0 + 8u * (NACC - 1), ep, wc)) break;
+        if (!ok || !mbar_wait_warp(tmem_empty0 + 8u * (NACC - 1), ep, wc)) break;
         tc_fence_after();
         for (int h = 0; h < J; ++h) {
-          issue(q + h, 1, h == 0);
+          issue(q + h, 1, 2, h == 0);
           release(q + h);
         }
         q += J;
         // body: both accumulators per stage
         for (int kb = J; kb < T - J; ++kb, ++q) {
           if (!stage_in(q)) { ok = false; break; }
-          issue(q, 0, kb == 0);
-          issue(q, 1, kb == 0);
+          issue(q, 0, 2, kb == 0);
           release(q);
         }
         if (!ok) break;
@@ -630,21 +641,24 @@ __global__ void __launch_bounds__(FusedCfg<CG, PAIRS>::kThreads, 1)
         // accumulator 1 finishes them
         for (int h = 0; ok && h < J; ++h) {
           if (!stage_in(q + h)) { ok = false; break; }
-          issue(q + h, 0, false);
+          issue(q + h, 0, 1, false);
         }
         if (!ok) break;
         full(0);
         for (int h = 0; h < J; ++h) {
-          issue(q + h, 1, false);
+          issue(q + h, 1, 2, false);
           release(q + h);
         }
         q += J;
         full(1);
       }
-      if constexpr (PAIRS == 1) umma_commit<CG>(final_bar);
-      else umma_commit_pair_mask(final_bar, pair_mask);
+      if (issuer) {
+        if constexpr (PAIRS == 1) umma_commit<CG>(final_bar);
+        else umma_commit_pair_mask(final_bar, pair_mask);
+      }
+      __syncwarp();
       mbar_wait_drain(final_bar, 0);
-    } else if (PAIRS == 2 && cta == 1 && lane == 0) {
+    } else if (PAIRS == 2 && lane == 0) {
       // ---------------------------------------------------------- odd CTA: received stages
       // Once this CTA's half of a received stage has landed, arm the slot's next use and
       // report the half to the pair's MMA.
@@ -1036,34 +1050,36 @@ __global__ void __launch_bounds__(DwCfg<CG>::kThreads, 1)
           if (issued_mask & (1u << s)) mbar_wait_drain(full(s), (issued_phase >> s) & 1u);
     }
   } else if (warp == kMma) {
-    if (cta == 0 && lane == 0) {
+    if (cta == 0) {  // the whole warp walks the pipeline, one elected lane issues (see elect_one)
       constexpr uint32_t idesc = idesc_bf16_f32(Cfg::kTileRows, BN, true, true);
+      const bool issuer = elect_one();
       uint32_t stage = 0, phase = 0, it = 0;
       bool ok = true;
       for (int t = cluster; ok && t < num_tiles; t += nclusters, ++it) {
         int kb0, kb1;
         kb_range(t, kb0, kb1);
         const uint32_t buf = it & 1u;
-        if (!mbar_wait(tmem_empty0 + 8u * buf, ((it >> 1) & 1u) ^ 1u, wc)) break;
+        if (!mbar_wait_warp(tmem_empty0 + 8u * buf, ((it >> 1) & 1u) ^ 1u, wc)) break;
         tc_fence_after();
         // Stages arrive in the TMA's order (forwards or, on odd iterations, backwards over M);
         // the sum does not depend on it, and the tile's first stage clears the accumulator.
         for (int j = 0; j < kb1 - kb0; ++j) {
-          if (!mbar_wait(full(stage), phase, wc)) { ok = false; break; }
+          if (!mbar_wait_warp(full(stage), phase, wc)) { ok = false; break; }
           tc_fence_after();
-          const uint32_t sa = base + stage * Cfg::kStageBytes, sb = sa + Cfg::kABytes;
+          const uint32_t ad = desc_lo(base + stage * Cfg::kStageBytes, 8192);
+          if (issuer) {
 #pragma unroll
-          for (int kk = 0; kk < BK / 16; ++kk) {
-            const uint64_t adesc = smem_desc_sw128(sa + kk * 2048, 8192, 1024);
-            const uint64_t bdesc = smem_desc_sw128(sb + kk * 2048, 8192, 1024);
-            umma_bf16<CG>(tmem_base + buf * BN, adesc, bdesc, idesc, (j > 0 || kk > 0) ? 1u : 0u);
+            for (int kk = 0; kk < BK / 16; ++kk)
+              umma_lo<CG>(tmem_base + buf * BN, ad + kk * (2048 / 16), ad + (Cfg::kABytes + kk * 2048) / 16, idesc,
+                          (j > 0 || kk > 0) ? 1u : 0u);
+            umma_commit<CG>(empty(stage));
           }
-          umma_commit<CG>(empty(stage));
           if (++stage == S) { stage = 0; phase ^= 1u; }
         }
-        if (ok) umma_commit<CG>(tmem_full0 + 8u * buf);
+        if (ok && issuer) umma_commit<CG>(tmem_full0 + 8u * buf);
       }
-      umma_commit<CG>(final_bar);
+      if (issuer) umma_commit<CG>(final_bar);
+      __syncwarp();
       mbar_wait_drain(final_bar, 0);
     }
   } else {
