@@ -117,14 +117,14 @@ typedef struct {
   const float* d_alpha; /* [G] learnable factor d_alpha (Eq. 3), > 0 */
   const float* d_delta; /* [G] learnable factor d_delta (§2.2), > 0 */
   /* [4*G] fp32 ([5*G] when recon is CATQ_RECON_ALPHA_T_MU), 16-byte aligned; required for
-   * bf16 layers by the forward and by a backward that computes dX, ignored otherwise.  Each
-   * such call first writes here the four per-group constants of its schedule point that
-   * turn a weight into its Eq. 6 operand (SOFT: s/alpha, -s mu/alpha, s Delta,
+   * bf16 layers by the forward and by a backward that computes dX, ignored otherwise.  Scratch of
+   * such a call, whose larger shapes first write here the four per-group constants of its schedule
+   * point that turn a weight into its Eq. 6 operand (SOFT: s/alpha, -s mu/alpha, s Delta,
    * alpha/(2 tanh s); HARD: 1/alpha, -mu/alpha, Delta, alpha), as float4 in
    * group-column-major order [K/g][N], then (CATQ_RECON_ALPHA_T_MU only) the G group offsets
    * mu in the same order; the fused GEMMs read one 16-byte vector (and one mu) per group
-   * and row.  Contents are overwritten by every call, so two calls on one layer must not
-   * overlap on the GPU. */
+   * and row.  (Smaller shapes form them in shared memory and leave it alone.)  Two calls on one
+   * layer must not overlap on the GPU. */
   float* op_const;
   int32_t recon;    /* catq_recon */
   int32_t reserved; /* must be 0 */

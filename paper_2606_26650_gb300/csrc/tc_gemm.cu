@@ -14,7 +14,11 @@
 //                    and reduces each row's columns into per-group partial sums.  G is never
 //                    written to memory.
 //
-// CG = 1: one CTA per tile (MMA M = 128).  CG = 2: a CTA pair (cluster of 2) computes one
+// fused_narrow_kernel  the fused contraction for launches whose 512-row tiles would leave most SMs
+//                    idle: one CTA per tile of up to 512 rows x 64 or 128 columns and share of
+//                    the contraction, the shares added up through distributed shared memory.
+//
+// CG = 1 (dw_kernel, narrow layers): one CTA per tile (MMA M = 128).  CG = 2: a CTA pair (cluster of 2) computes one
 // tile with tcgen05 cta_group::2 (MMA M = 256), each CTA holding half of the operand
 // columns; only the even CTA issues MMAs.
 //
@@ -29,6 +33,7 @@
 #include <mutex>
 #include <numeric>
 #include <type_traits>
+#include <algorithm>
 
 #include "launch.h"
 #include "ptx_sm100.cuh"
@@ -53,19 +58,19 @@ constexpr int gcd_c(int a, int b) { return b == 0 ? a : gcd_c(b, a % b); }
 // against the same produced operand tiles; each pair produces every other stage and sends
 // its transformed half-tiles to the other pair's CTAs through distributed shared memory,
 // which halves the per-SM transform work.
-template <int CG, int PAIRS = 1>
+template <int PAIRS>
 struct FusedCfg {
-  static_assert(PAIRS == 1 || CG == 2, "pairs of pairs need CTA pairs");
+  static constexpr int CG = 2;  // CTAs per pair
   static constexpr int kClusterCtas = CG * PAIRS;
   static constexpr int kRowsPerAcc = 128 * CG;          // MMA M
   static constexpr int kTileRows = kRowsPerAcc * NACC;  // rows of C per pair per tile
   static constexpr int kBRows = BN / CG;                // 128-byte operand rows per CTA per stage
   static constexpr int kABytes = NACC * 128 * BK * 2;   // this CTA's A rows per stage
   static constexpr int kWBytes = kBRows * BK * 2;       // this CTA's operand rows per stage
-  static constexpr int kStagesA = CG == 1 ? 3 : 4;      // A ring: TMA -> MMA
+  static constexpr int kStagesA = 4;                    // A ring: TMA -> MMA
   // W ring: TMA -> producers (in place) -> MMA.  Even with two pairs, so every slot is always
   // produced by the same pair (and received by the other).
-  static constexpr int kStagesW = PAIRS == 2 ? 6 : (CG == 1 ? 3 : 5);
+  static constexpr int kStagesW = PAIRS == 2 ? 6 : 5;
   static constexpr int kEpiWarps = 4;
   // Two groups of 8 producer warps take alternate stages (of the ones this CTA produces), so
   // each group has two stage periods per operand tile and the groups' MUFU work interleaves.
@@ -73,7 +78,7 @@ struct FusedCfg {
   static constexpr int kGroupWarps = 8;
   static constexpr int kProdWarps = kProdGroups * kGroupWarps;
   static constexpr int kGroupThreads = 32 * kGroupWarps;
-  static constexpr int kThreadsPerRow = kGroupThreads / kBRows;  // 1 (CG 1) or 2 (CG 2)
+  static constexpr int kThreadsPerRow = kGroupThreads / kBRows;  // 2
   static constexpr int kChunksPerThread = 8 / kThreadsPerRow;    // 16-byte chunks of a 128-byte row
   static constexpr int kThreads = 32 * (kEpiWarps + 2 + kProdWarps);
   // Stage q lands on the raw-W barrier of its producer group and slot; that barrier sees one
@@ -335,9 +340,9 @@ __device__ __forceinline__ void load_yref_bf16x16(const uint16_t* Yr, int64_t nc
 // CTA's tile sequence) and tracks which W row, K chunk and group its 128-byte operand row
 // holds, the group as its index into the [K/g][N] operand-constant array.  Divisions happen
 // once per tile; each stage step is a few integer adds.
-template <int CG, bool B_MN, int PAIRS>
+template <bool B_MN, int PAIRS>
 struct OperandRowIter {
-  using Cfg = FusedCfg<CG, PAIRS>;
+  using Cfg = FusedCfg<PAIRS>;
   int t, kb;      // tile index, k block
   int64_t n, kc;  // W row (within its expert), first K column of the 64-element chunk
   int64_t ci;     // operand-constant index of (n, kc): (kc / g) * N + n, in float4 units from
@@ -407,12 +412,12 @@ struct OperandRowIter {
 // kernel carries none of its work).  EPI: 0 stores C in bf16; 1 is the general epilogue
 // (row scale, fp32 C, fused loss), a separate instantiation so the plain forward and dX
 // keep their register allocation.
-template <int CG, bool B_MN, int PAIRS, bool MU, int EPI = 0>
-__global__ void __launch_bounds__(FusedCfg<CG, PAIRS>::kThreads, 1)
+template <bool B_MN, int PAIRS, bool MU, int EPI = 0>
+__global__ void __launch_bounds__(FusedCfg<PAIRS>::kThreads, 1)
     fused_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmW,
                       const FusedArgs args) {
-  using Cfg = FusedCfg<CG, PAIRS>;
-  constexpr int SA = Cfg::kStagesA, SW = Cfg::kStagesW;
+  using Cfg = FusedCfg<PAIRS>;
+  constexpr int SA = Cfg::kStagesA, SW = Cfg::kStagesW, CG = Cfg::CG;
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw_addr = smem_u32(smem_raw);
   const uint32_t base = (raw_addr + 1023u) & ~1023u;
@@ -435,12 +440,12 @@ __global__ void __launch_bounds__(FusedCfg<CG, PAIRS>::kThreads, 1)
       reinterpret_cast<uint32_t*>(base_ptr + (bars - base) + 8 * (2 * SA + RB + 3 * SW + 2 * NACC + 1));
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const uint32_t rank = CG == 2 ? cluster_ctarank() : 0u;
+  const uint32_t rank = cluster_ctarank();
   const uint32_t cta = rank & 1u;                // half of the pair
   const uint32_t pair = rank >> 1;               // pair within the cluster (PAIRS 2)
   const uint32_t leader = rank & ~1u;            // the pair's MMA-issuing CTA
-  const uint32_t cluster = CG == 2 ? cluster_id_x() : blockIdx.x;
-  const uint32_t nclusters = CG == 2 ? num_clusters_x() : gridDim.x;
+  const uint32_t cluster = cluster_id_x();
+  const uint32_t nclusters = num_clusters_x();
   const WaitCtl& wc = args.wc;
   const int num_tiles = args.num_m_tiles * args.num_n_tiles;
   constexpr int kTmaWarp = Cfg::kEpiWarps, kMmaWarp = Cfg::kEpiWarps + 1;
@@ -479,13 +484,13 @@ __global__ void __launch_bounds__(FusedCfg<CG, PAIRS>::kThreads, 1)
     prefetch_tmap(&tmW);
   }
   tc_fence_before();
-  if constexpr (CG == 2) cluster_sync_all(); else __syncthreads();
+  cluster_sync_all();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
   // Barriers a whole pair signals live in the pair's even CTA.
-  const uint32_t leader_full_a0 = CG == 2 ? mapa_shared(full_a(0), leader) : full_a(0);
-  const uint32_t leader_full_w0 = CG == 2 ? mapa_shared(full_w(0), leader) : full_w(0);
-  const uint32_t leader_tmem_empty0 = CG == 2 ? mapa_shared(tmem_empty0, leader) : tmem_empty0;
+  const uint32_t leader_full_a0 = mapa_shared(full_a(0), leader);
+  const uint32_t leader_full_w0 = mapa_shared(full_w(0), leader);
+  const uint32_t leader_tmem_empty0 = mapa_shared(tmem_empty0, leader);
   const uint16_t pair_mask = static_cast<uint16_t>(3u << (2 * pair));
   const uint16_t all_mask = static_cast<uint16_t>((1u << Cfg::kClusterCtas) - 1u);
 
@@ -508,8 +513,7 @@ __global__ void __launch_bounds__(FusedCfg<CG, PAIRS>::kThreads, 1)
 #pragma unroll
           for (int acc = 0; acc < NACC; ++acc) {
             const int32_t row = m0 + acc * Cfg::kRowsPerAcc + cta * 128;
-            if constexpr (CG == 1) tma_load_2d_hint(dst + acc * (128 * BK * 2), &tmA, fb, kb * BK, row, pol_a);
-            else tma_load_2d_pair_hint(dst + acc * (128 * BK * 2), &tmA, fb, kb * BK, row, pol_a);
+            tma_load_2d_pair_hint(dst + acc * (128 * BK * 2), &tmA, fb, kb * BK, row, pol_a);
           }
           issued_mask |= 1u << s;
           issued_phase = (issued_phase & ~(1u << s)) | (ph << s);
@@ -799,7 +803,7 @@ __global__ void __launch_bounds__(FusedCfg<CG, PAIRS>::kThreads, 1)
     }
   } else {
     // ------------------------------------------------------------ operand producers
-    // Within its group, each thread owns one row (CG 1) or half a row (CG 2) of the stage's
+    // Within its group, each thread owns half a row of the stage's
     // raw W tile and rewrites it in place as the Eq. 6 weight.  A row holds 64 consecutive K
     // elements of one W row, so it lies in one group (g is a multiple of 64).  Rows outside
     // W were zero-filled by the copy and stay 0.  The CTA's produced stages are
@@ -825,7 +829,7 @@ __global__ void __launch_bounds__(FusedCfg<CG, PAIRS>::kThreads, 1)
     // `cur` is the stage being produced; `ahead` runs two of this thread's stages ahead and
     // requests that stage's operand constants (one 16-byte vector, precomputed per call), so
     // an L2 round trip is hidden behind two stages.
-    OperandRowIter<CG, B_MN, PAIRS> cur, ahead;
+    OperandRowIter<B_MN, PAIRS> cur, ahead;
     cur.init(args, cta, row, cluster, 0);
     cur.step(args, cta, row, nclusters, q0);
     ahead = cur;
@@ -834,7 +838,7 @@ __global__ void __launch_bounds__(FusedCfg<CG, PAIRS>::kThreads, 1)
     float m0 = 0.0f, m1 = 0.0f;
     int64_t j0 = -1, j1 = -1;
     constexpr bool with_mu = MU;
-    auto request = [&](const OperandRowIter<CG, B_MN, PAIRS>& it, float4& dst, float& dm, int64_t& jd,
+    auto request = [&](const OperandRowIter<B_MN, PAIRS>& it, float4& dst, float& dm, int64_t& jd,
                        const float4& other, float om, int64_t jo) {
       if (transform && it.live(args, num_tiles) && it.valid(args)) {
         if (jo == it.ci) {
@@ -909,10 +913,378 @@ __global__ void __launch_bounds__(FusedCfg<CG, PAIRS>::kThreads, 1)
   }
 
   tc_fence_before();
-  if constexpr (CG == 2) cluster_sync_all(); else __syncthreads();
+  cluster_sync_all();
   if (warp == kMmaWarp) {
     tc_fence_after();
     tmem_dealloc<CG>(tmem_base, kTmemCols);
+  }
+}
+
+// ============================================================================ narrow kernel
+
+// fused_narrow_kernel: the same contraction and operand as fused_gemm_kernel for launches whose
+// tiles would leave most SMs idle (few rows or few columns).  A CTA computes one tile of
+// 128 nacc rows x BN columns over its share of the contraction; the `splits` CTAs of a cluster
+// hold one tile's partial sums, which meet through distributed shared memory in rank order
+// (deterministic).  The operand constants of the CTA's share come from the six per-group arrays
+// into a shared-memory table at the start (no launch writes op_const, and no global load is in
+// flight at the producers' proxy fences, which would wait for it).
+struct NarrowPlan {
+  int32_t bn, nacc, splits;    // columns, 128-row accumulators, CTAs per tile
+  int32_t stages_a, stages_w;  // ring depths; stages_w is even (a slot belongs to one producer group)
+  int32_t entries;             // table entries: (row, group) pairs of one CTA's share, at most
+};
+
+constexpr int kNarrowProdWarps = 16, kNarrowGroupWarps = 8;
+constexpr int kNarrowRoleWarps = 3;  // A copies, MMA, W copies
+constexpr int kNarrowThreads = 32 * (kNarrowRoleWarps + kNarrowProdWarps);
+constexpr int kNarrowMaxStages = 8;
+constexpr int kNarrowBarBytes = 8 * (5 * kNarrowMaxStages + 1) + 16;
+constexpr int kNarrowABytes = 128 * BK * 2;  // one accumulator's A rows per stage
+constexpr int kNarrowSmemMax = 227 * 1024;
+
+// Shared memory: rings, table (float4, then mu), barriers, 1 KB of alignment slack.
+__host__ __device__ constexpr int narrow_smem(int bn, int nacc, int sa, int sw, int entries, bool mu) {
+  return sa * nacc * kNarrowABytes + sw * bn * BK * 2 + entries * (mu ? 20 : 16) + kNarrowBarBytes + 16 + 1024;
+}
+
+__device__ __forceinline__ float4 ld_cluster_f4(uint32_t cluster_addr) {
+  float4 v;
+  asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
+               : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+               : "r"(cluster_addr)
+               : "memory");
+  return v;
+}
+
+// The options of the general epilogue for 8 consecutive finished columns of one row.
+__device__ __forceinline__ void narrow_emit(const FusedArgs& a, int64_t row, int64_t col, float (&y)[8], Sum2& lacc) {
+  if (a.row_scale) {
+    const float rs = __ldg(a.row_scale + row);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) y[i] *= rs;
+  }
+  const int64_t at = row * a.ncols + col;
+  auto pack = [](const float (&f)[8]) {
+    return make_uint4(pack_bf16x2(f[0], f[1]), pack_bf16x2(f[2], f[3]), pack_bf16x2(f[4], f[5]),
+                      pack_bf16x2(f[6], f[7]));
+  };
+  if (a.C) {
+    if (a.c_f32) {
+      float4* c = reinterpret_cast<float4*>(static_cast<float*>(a.C) + at);
+      c[0] = make_float4(y[0], y[1], y[2], y[3]);
+      c[1] = make_float4(y[4], y[5], y[6], y[7]);
+    } else {
+      *reinterpret_cast<uint4*>(static_cast<uint16_t*>(a.C) + at) = pack(y);
+    }
+  }
+  if (!a.yref) return;
+  if (a.yref_f32) {
+    const float4* q = reinterpret_cast<const float4*>(static_cast<const float*>(a.yref) + at);
+    const float4 r0 = __ldg(q), r1 = __ldg(q + 1);
+    y[0] -= r0.x; y[1] -= r0.y; y[2] -= r0.z; y[3] -= r0.w;
+    y[4] -= r1.x; y[5] -= r1.y; y[6] -= r1.z; y[7] -= r1.w;
+  } else {
+    const uint4 q = __ldg(reinterpret_cast<const uint4*>(static_cast<const uint16_t*>(a.yref) + at));
+    const uint32_t w[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      y[2 * i] -= bf16lo_to_f32(w[i]);
+      y[2 * i + 1] -= bf16hi_to_f32(w[i]);
+    }
+  }
+  float s = 0.0f;
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    s = fmaf(y[i], y[i], s);
+    y[i] *= a.dscale;
+  }
+  sum2_add(lacc, s);
+  *reinterpret_cast<uint4*>(a.dY + at) = pack(y);
+}
+
+template <int BNN, bool B_MN, bool MU>
+__global__ void __launch_bounds__(kNarrowThreads, 1)
+    fused_narrow_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmW,
+                        const __grid_constant__ FusedArgs args, const NarrowPlan np) {
+  constexpr int kWBytes = BNN * BK * 2;
+  extern __shared__ uint8_t smem_raw[];
+  __shared__ Sum2 red[kNarrowProdWarps];
+  const uint32_t raw_addr = smem_u32(smem_raw);
+  const uint32_t base = (raw_addr + 1023u) & ~1023u;
+  uint8_t* base_ptr = smem_raw + (base - raw_addr);
+  const int SA = np.stages_a, SW = np.stages_w, S = np.splits;
+  const uint32_t a_stage = np.nacc * kNarrowABytes;
+  const uint32_t w_base = base + SA * a_stage;
+  float4* const tab = reinterpret_cast<float4*>(base_ptr + (w_base - base) + SW * kWBytes);
+  float* const tab_mu = reinterpret_cast<float*>(tab + np.entries);
+  const uint32_t bars = (w_base + SW * kWBytes + np.entries * (MU ? 20u : 16u) + 15u) & ~15u;
+  auto full_a = [&](int s) { return bars + 8u * s; };
+  auto empty_a = [&](int s) { return bars + 8u * (kNarrowMaxStages + s); };
+  auto raw_w = [&](int s) { return bars + 8u * (2 * kNarrowMaxStages + s); };
+  auto full_w = [&](int s) { return bars + 8u * (3 * kNarrowMaxStages + s); };
+  auto empty_w = [&](int s) { return bars + 8u * (4 * kNarrowMaxStages + s); };
+  const uint32_t done = bars + 8u * (5 * kNarrowMaxStages);
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(base_ptr + (done - base) + 8);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const uint32_t rank = S > 1 ? cluster_ctarank() : 0u;
+  const WaitCtl& wc = args.wc;
+  const TileInfo ti = tile_info(args, blockIdx.x / S, 128 * np.nacc);
+  const int T = args.num_k_blocks;
+  const int kb0 = static_cast<int>(static_cast<int64_t>(T) * rank / S);
+  const int kb1 = static_cast<int>(static_cast<int64_t>(T) * (rank + 1) / S);
+  const int nk = kb1 - kb0;
+  const int live = static_cast<int>(min(static_cast<int64_t>(np.nacc), (ti.row_end - ti.row0 + 127) / 128));
+  const int64_t col0 = static_cast<int64_t>(ti.n_blk) * BNN;
+  uint32_t tmem_cols = 32;
+  while (tmem_cols < static_cast<uint32_t>(np.nacc * BNN)) tmem_cols *= 2;
+
+  if (threadIdx.x < 5 * kNarrowMaxStages + 1)  // one thread per barrier; full_w counts a producer group's warps
+    mbar_init(bars + 8u * threadIdx.x, threadIdx.x / kNarrowMaxStages == 3 ? kNarrowGroupWarps : 1);
+  fence_mbar_init_cluster();
+  if (warp == 0 && lane == 0) {
+    prefetch_tmap(&tmA);
+    prefetch_tmap(&tmW);
+  }
+  if (warp == 1) tmem_alloc<1>(smem_u32(tmem_slot), tmem_cols);
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = *tmem_slot;
+
+  if (warp == 0) {
+    if (lane == 0) {
+      // -------------------------------------------------------------- TMA: A tiles
+      int s = 0, issued = 0;
+      uint32_t ph = 1;
+      for (int i = 0; i < nk; ++i) {
+        if (!mbar_wait(empty_a(s), ph, wc)) break;
+        mbar_arrive_expect_tx(full_a(s), live * kNarrowABytes);
+        for (int acc = 0; acc < live; ++acc)
+          tma_load_2d(base + s * a_stage + acc * kNarrowABytes, &tmA, full_a(s), (kb0 + i) * BK,
+                      static_cast<int32_t>(ti.row0) + acc * 128);
+        issued = i + 1;
+        if (++s == SA) { s = 0; ph ^= 1u; }
+      }
+      for (int i = max(0, issued - SA); i < issued; ++i) mbar_wait_drain(full_a(i % SA), (i / SA) & 1);
+    }
+  } else if (warp == 2) {
+    if (lane == 0) {
+      // -------------------------------------------------------------- TMA: raw W tiles (a warp of its
+      // own: two lanes of one warp that both wait hold each other up)
+      const int32_t wrow = static_cast<int32_t>(ti.e * args.L.N), n0 = static_cast<int32_t>(col0);
+      int s = 0, issued = 0;
+      uint32_t ph = 1;
+      for (int i = 0; i < nk; ++i) {
+        if (!mbar_wait(empty_w(s), ph, wc)) break;
+        mbar_arrive_expect_tx(raw_w(s), kWBytes);
+        const uint32_t dst = w_base + s * kWBytes;
+        if constexpr (!B_MN) {
+          tma_load_2d(dst, &tmW, raw_w(s), (kb0 + i) * BK, wrow + n0);
+        } else {
+#pragma unroll
+          for (int b = 0; b < BNN / 64; ++b)
+            tma_load_2d(dst + b * 8192, &tmW, raw_w(s), n0 + 64 * b, wrow + (kb0 + i) * BK);
+        }
+        issued = i + 1;
+        if (++s == SW) { s = 0; ph ^= 1u; }
+      }
+      for (int i = max(0, issued - SW); i < issued; ++i) mbar_wait_drain(raw_w(i % SW), (i / SW) & 1);
+    }
+  } else if (warp == 1) {
+    // ---------------------------------------------------------------- MMA issuer (see elect_one)
+    constexpr uint32_t idesc = idesc_bf16_f32(128, BNN, false, B_MN);
+    constexpr uint32_t kStepB = (B_MN ? 2048 : 32) / 16;
+    const bool issuer = elect_one();
+    int sa = 0, sw = 0;
+    uint32_t pa = 0, pw = 0;
+    for (int i = 0; i < nk; ++i) {
+      if (!mbar_wait_warp(full_a(sa), pa, wc) || !mbar_wait_warp(full_w(sw), pw, wc)) break;
+      tc_fence_after();
+      const uint32_t ad = desc_lo(base + sa * a_stage, 16), bd = desc_lo(w_base + sw * kWBytes, B_MN ? 8192 : 16);
+      if (issuer) {
+        for (int acc = 0; acc < live; ++acc) {
+#pragma unroll
+          for (int kk = 0; kk < BK / 16; ++kk)
+            umma_lo<1>(tmem + acc * BNN, ad + acc * (kNarrowABytes / 16) + kk * 2, bd + kk * kStepB, idesc,
+                       (i > 0 || kk > 0) ? 1u : 0u);
+        }
+        umma_commit<1>(empty_a(sa));
+        umma_commit<1>(empty_w(sw));
+      }
+      if (++sa == SA) { sa = 0; pa ^= 1u; }
+      if (++sw == SW) { sw = 0; pw ^= 1u; }
+    }
+    if (issuer) umma_commit<1>(done);
+    __syncwarp();
+    mbar_wait_drain(done, 0);
+  } else {
+    // ---------------------------------------------------------------- operand producers
+    // As in fused_gemm_kernel: two groups of 8 warps take alternate stages; a thread rewrites
+    // kChunks 16-byte chunks of one 128-byte row in place.
+    constexpr int kThreadsPerRow = 32 * kNarrowGroupWarps / BNN;
+    constexpr int kChunks = 8 / kThreadsPerRow;
+    const int pw = warp - kNarrowRoleWarps, grp = pw / kNarrowGroupWarps;
+    const int tt = threadIdx.x - 32 * kNarrowRoleWarps - grp * 32 * kNarrowGroupWarps;
+    const int row = tt / kThreadsPerRow, c_begin = (tt % kThreadsPerRow) * kChunks;
+    const LayerDev& L = args.L;
+    const int32_t phase_t = args.sc.phase;
+    const bool transform = phase_t != PHASE_TEACHER;
+    // The table: operand constants of (W row, group column) pairs, stored [group][row].  Forward: the
+    // tile's BN rows x the groups of the share's columns; dX: the share's rows x the groups of the
+    // tile's columns.
+    const int64_t first_n = B_MN ? static_cast<int64_t>(kb0) * BK : col0;
+    const int rows = B_MN ? nk * BK : BNN;
+    const int64_t c_lo = B_MN ? col0 : static_cast<int64_t>(kb0) * BK;
+    const int64_t c_hi = min(B_MN ? col0 + BNN : static_cast<int64_t>(kb1) * BK, L.K);
+    const int64_t g_lo = c_lo / L.g;
+    const int groups = static_cast<int>((c_hi - 1) / L.g - g_lo) + 1;
+    if (transform) {
+      const int64_t jbase = ti.e * (L.N * L.groups_per_row) + g_lo;
+      for (int e = threadIdx.x - 32 * kNarrowRoleWarps; e < rows * groups; e += 32 * kNarrowProdWarps) {
+        const int r = e / groups, c = e - r * groups;  // a row's groups are contiguous in memory
+        const int64_t n = first_n + r;
+        if (n < L.N) {
+          const GroupConst gc = group_const(L, jbase + n * L.groups_per_row + c);
+          tab[c * rows + r] = operand_const_vec(gc, args.sc.s, args.sc.inv_2tanh_s, phase_t);
+          if constexpr (MU) tab_mu[c * rows + r] = gc.mu;
+        }
+      }
+    }
+    asm volatile("bar.sync 1, %0;" ::"n"(32 * kNarrowProdWarps) : "memory");  // the producer warps
+    bool ok = true;
+    int s = grp;
+    uint32_t ph = 0;
+    for (int i = grp; ok && i < nk; i += 2) {
+      bool live_row;
+      int at;
+      if constexpr (!B_MN) {
+        live_row = col0 + row < L.N;
+        at = static_cast<int>(static_cast<int64_t>(kb0 + i) * BK / L.g - g_lo) * rows + row;
+      } else {
+        const int64_t kc = col0 + 64 * (row >> 6);
+        live_row = static_cast<int64_t>(kb0 + i) * BK + (row & 63) < L.N && kc < L.K;
+        at = static_cast<int>(kc / L.g - g_lo) * rows + i * BK + (row & 63);
+      }
+      ProducerConst pc{};
+      if (transform && live_row) pc = producer_const_from(tab[at], MU ? tab_mu[at] : 0.0f);
+      if (!mbar_wait(raw_w(s), ph, wc)) {
+        ok = false;
+        break;
+      }
+      if (transform && live_row) {
+        uint8_t* rowp = base_ptr + (w_base - base) + s * kWBytes + row * 128;
+        auto run = [&](auto kind_tag) {
+          constexpr int KIND = decltype(kind_tag)::value;
+          uint4 v[kChunks];
+#pragma unroll
+          for (int c = 0; c < kChunks; ++c)
+            v[c] = *reinterpret_cast<const uint4*>(rowp + (((c_begin + c) ^ (row & 7)) * 16));
+#pragma unroll
+          for (int c = 0; c < kChunks; ++c)
+            *reinterpret_cast<uint4*>(rowp + (((c_begin + c) ^ (row & 7)) * 16)) = transform_chunk<KIND>(v[c], pc);
+        };
+        constexpr int kMu = MU ? XF_MU : 0;
+        switch (transform_kind(pc, phase_t, MU ? 1 : 0)) {
+          case XF_SOFT1 | kMu: run(std::integral_constant<int, XF_SOFT1 | kMu>{}); break;
+          case XF_SOFT2 | kMu: run(std::integral_constant<int, XF_SOFT2 | kMu>{}); break;
+          case XF_HARD | kMu: run(std::integral_constant<int, XF_HARD | kMu>{}); break;
+          default: break;
+        }
+        fence_proxy_async_smem();
+      }
+      __syncwarp();
+      if (lane == 0) mbar_arrive_local(full_w(s));
+      s += 2;  // SW is even: a group keeps to its slots
+      if (s >= SW) { s -= SW; ph ^= 1u; }
+    }
+  }
+
+  // ------------------------------------------------------------------ partial sums and epilogue
+  // Every MMA has completed (or the launch gave up: the waits fail at once and the rounds below
+  // pass garbage through the same barriers).  One round per accumulator: each CTA puts its 128 x
+  // BN fp32 partial into its (now idle) rings, 16-byte chunks xor-swizzled by the row, then adds
+  // its share of the rows of every CTA's partial in rank order and stores them.
+  mbar_wait(done, 0, wc);
+  __syncwarp();
+  __syncthreads();
+  tc_fence_after();
+  Sum2 lacc{0.f, 0.f};
+  for (int acc = 0; acc < live; ++acc) {
+    if (warp >= kNarrowRoleWarps) {
+      const int q = warp & 3, cq = (warp - kNarrowRoleWarps) >> 2;  // TMEM lane quarter, column quarter
+      const int r = q * 32 + lane;
+      float* rowp = reinterpret_cast<float*>(base_ptr + static_cast<size_t>(r) * BNN * 4);
+      const uint32_t src = tmem + (static_cast<uint32_t>(q * 32) << 16) + acc * BNN;
+      constexpr int kCols = BNN / 4;
+#pragma unroll
+      for (int c0 = 0; c0 < kCols; c0 += 16) {
+        uint32_t v[16];
+        tmem_ld16(src + cq * kCols + c0, v);
+        tmem_ld_wait();
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+          const int chunk = (cq * kCols + c0) / 4 + c;
+          *reinterpret_cast<uint4*>(rowp + 4 * (chunk ^ (r & 7))) =
+              make_uint4(v[4 * c], v[4 * c + 1], v[4 * c + 2], v[4 * c + 3]);
+        }
+      }
+    }
+    if (S > 1) cluster_sync_all(); else __syncthreads();
+    if (warp >= kNarrowRoleWarps) {
+      auto reduce = [&](auto splits_tag) {
+        constexpr int SP = decltype(splits_tag)::value;
+        constexpr int kUnits = 128 * (BNN / 8);
+        const int u1 = kUnits * (static_cast<int>(rank) + 1) / SP;
+        for (int u = kUnits * static_cast<int>(rank) / SP + threadIdx.x - 32 * kNarrowRoleWarps; u < u1; u += 32 * kNarrowProdWarps) {
+          const int r = u / (BNN / 8), c8 = u % (BNN / 8);
+          const int64_t row = ti.row0 + acc * 128 + r, col = col0 + 8 * c8;
+          if (row >= ti.row_end || col >= args.ncols) continue;
+          const uint32_t at0 = base + static_cast<uint32_t>(r * BNN * 4 + 16 * ((2 * c8) ^ (r & 7)));
+          const uint32_t at1 = base + static_cast<uint32_t>(r * BNN * 4 + 16 * ((2 * c8 + 1) ^ (r & 7)));
+          float4 v0[SP], v1[SP];  // every CTA's partial on its way before the first is added
+#pragma unroll
+          for (int p = 0; p < SP; ++p) {
+            if constexpr (SP > 1) {
+              v0[p] = ld_cluster_f4(mapa_shared(at0, p));
+              v1[p] = ld_cluster_f4(mapa_shared(at1, p));
+            } else {
+              v0[p] = *reinterpret_cast<const float4*>(base_ptr + (at0 - base));
+              v1[p] = *reinterpret_cast<const float4*>(base_ptr + (at1 - base));
+            }
+          }
+          float y[8] = {v0[0].x, v0[0].y, v0[0].z, v0[0].w, v1[0].x, v1[0].y, v1[0].z, v1[0].w};
+#pragma unroll
+          for (int p = 1; p < SP; ++p) {
+            y[0] += v0[p].x; y[1] += v0[p].y; y[2] += v0[p].z; y[3] += v0[p].w;
+            y[4] += v1[p].x; y[5] += v1[p].y; y[6] += v1[p].z; y[7] += v1[p].w;
+          }
+          narrow_emit(args, row, col, y, lacc);
+        }
+      };
+      if (S == 1) reduce(std::integral_constant<int, 1>{});
+      else if (S == 2) reduce(std::integral_constant<int, 2>{});
+      else if (S == 4) reduce(std::integral_constant<int, 4>{});
+      else reduce(std::integral_constant<int, 8>{});
+      __syncwarp();
+    }
+    if (S > 1) cluster_sync_all(); else __syncthreads();
+  }
+  if (args.yref) {
+    lacc = sum2_team(lacc, 32);
+    if (warp >= kNarrowRoleWarps && lane == 0) red[warp - kNarrowRoleWarps] = lacc;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      Sum2 t = red[0];
+      for (int w = 1; w < kNarrowProdWarps; ++w) t = sum2_merge(t, red[w]);
+      args.loss_part[blockIdx.x] = sum2_value(t);
+    }
+  }
+  tc_fence_before();
+  __syncthreads();
+  if (warp == 1) {
+    tc_fence_after();
+    tmem_dealloc<1>(tmem, tmem_cols);
   }
 }
 
@@ -1330,27 +1702,9 @@ int max_active_clusters(Kern kern, int cluster_ctas, int threads, int smem, int 
   return n;
 }
 
-// Tile shape by M: pairs of pairs (1024 rows per cluster tile) once M fills both pairs,
-// CTA pairs (512 rows) from 512 rows, single CTAs below.
-int fused_variant_for(int64_t M) { return M >= 1024 ? 4 : (M >= 512 ? 2 : 1); }
-
-// grp (nullable): a grouped launch over grp->E experts whose weights are stacked from L.W on
-// and whose rows of A and C are expert-sorted (host offsets grp->off).
-template <int CG, bool B_MN, int PAIRS, bool MU, int EPI = 0>
-cudaError_t run_fused(const LayerDev& L, StepScalars sc, const void* A, int64_t M, int64_t depth, void* C,
-                      int64_t ncols, cudaStream_t st, const GroupSpec* grp = nullptr, const EpiOpts* opts = nullptr) {
-  using Cfg = FusedCfg<CG, PAIRS>;
-  DeviceInfo& d = device_info();
-  if (!d.ok) return cudaErrorInvalidDevice;
-  const int64_t wrows = grp ? grp->E * L.N : L.N;
-  CUtensorMap ta, tw;
-  if (!make_tmap(&ta, A, depth, M, BK, 128)) return cudaErrorInvalidValue;
-  if constexpr (!B_MN) {
-    if (!make_tmap(&tw, L.W, L.K, wrows, BK, Cfg::kBRows)) return cudaErrorInvalidValue;
-  } else {
-    if (!make_tmap(&tw, L.W, L.K, wrows, 64, BK)) return cudaErrorInvalidValue;
-  }
-  FusedArgs args;
+// The launch arguments that do not depend on the tile shape.
+void fill_fused_args(FusedArgs& args, const LayerDev& L, StepScalars sc, void* C, int64_t M, int64_t depth,
+                     int64_t ncols, const EpiOpts* opts) {
   args.L = L;
   args.sc = sc;
   args.C = C;
@@ -1364,9 +1718,50 @@ cudaError_t run_fused(const LayerDev& L, StepScalars sc, const void* A, int64_t 
   if (opts && opts->n_parts) *opts->n_parts = 0;
   args.M = M;
   args.ncols = ncols;
+  args.num_k_blocks = static_cast<int32_t>((depth + BK - 1) / BK);
+  args.E = 0;
+  args.const_stride = 0;
+}
+
+// The tile table of a grouped launch (at most kMaxGroupExperts experts): returns its tile count.
+int64_t fill_groups(FusedArgs& args, const GroupSpec& grp, int64_t rows_per_tile) {
+  args.E = grp.E;
+  args.const_stride = grp.const_stride;
+  int64_t t = 0;
+  for (int e = 0; e <= grp.E; ++e) {
+    args.tile0[e] = static_cast<int32_t>(t);
+    args.row0[e] = static_cast<int32_t>(grp.off[e]);
+    if (e < grp.E) t += (grp.off[e + 1] - grp.off[e] + rows_per_tile - 1) / rows_per_tile * args.num_n_tiles;
+  }
+  return t;
+}
+
+// grp (nullable): a grouped launch over grp->E experts whose weights are stacked from L.W on
+// and whose rows of A and C are expert-sorted (host offsets grp->off).
+template <bool B_MN, int PAIRS, bool MU, int EPI = 0>
+cudaError_t run_fused(const LayerDev& L, StepScalars sc, const void* A, int64_t M, int64_t depth, void* C,
+                      int64_t ncols, cudaStream_t st, const GroupSpec* grp = nullptr, const EpiOpts* opts = nullptr) {
+  using Cfg = FusedCfg<PAIRS>;
+  DeviceInfo& d = device_info();
+  if (!d.ok) return cudaErrorInvalidDevice;
+  if (grp && (grp->E < 1 || grp->E > kMaxGroupExperts)) return cudaErrorInvalidValue;
+  if (sc.phase != PHASE_TEACHER) {
+    const cudaError_t e = grp ? launch_operand_consts_grouped(L, sc, grp->E, grp->const_stride, st)
+                              : launch_operand_consts(L, sc, st);
+    if (e != cudaSuccess) return e;
+  }
+  const int64_t wrows = grp ? grp->E * L.N : L.N;
+  CUtensorMap ta, tw;
+  if (!make_tmap(&ta, A, depth, M, BK, 128)) return cudaErrorInvalidValue;
+  if constexpr (!B_MN) {
+    if (!make_tmap(&tw, L.W, L.K, wrows, BK, Cfg::kBRows)) return cudaErrorInvalidValue;
+  } else {
+    if (!make_tmap(&tw, L.W, L.K, wrows, 64, BK)) return cudaErrorInvalidValue;
+  }
+  FusedArgs args;
+  fill_fused_args(args, L, sc, C, M, depth, ncols, opts);
   args.num_m_tiles = static_cast<int32_t>((M + Cfg::kTileRows * PAIRS - 1) / (Cfg::kTileRows * PAIRS));
   args.num_n_tiles = static_cast<int32_t>((ncols + BN - 1) / BN);
-  args.num_k_blocks = static_cast<int32_t>((depth + BK - 1) / BK);
   args.group_m = std::min(4, args.num_m_tiles);
   {
     // A rows of one raster group: kept in L2 when they take at most a third of it (dense
@@ -1375,25 +1770,13 @@ cudaError_t run_fused(const LayerDev& L, StepScalars sc, const void* A, int64_t 
     args.a_keep = (!grp && std::min<int64_t>(group_rows, M) * depth * 2 <= (int64_t(40) << 20)) ? 1 : 0;
   }
   args.wc = make_wait_ctl(d);
-  args.E = 0;
-  args.const_stride = 0;
   int tiles = args.num_m_tiles * args.num_n_tiles;
   if (grp) {
-    if (grp->E < 1 || grp->E > kMaxGroupExperts) return cudaErrorInvalidValue;
-    args.E = grp->E;
-    args.const_stride = grp->const_stride;
-    const int64_t rows_per_tile = Cfg::kTileRows * PAIRS;
-    int64_t t = 0;
-    for (int e = 0; e <= grp->E; ++e) {
-      args.tile0[e] = static_cast<int32_t>(t);
-      args.row0[e] = static_cast<int32_t>(grp->off[e]);
-      if (e < grp->E) t += (grp->off[e + 1] - grp->off[e] + rows_per_tile - 1) / rows_per_tile * args.num_n_tiles;
-    }
-    tiles = static_cast<int>(t);
-    args.num_m_tiles = static_cast<int32_t>(t / args.num_n_tiles);  // the kernel's tile count is M x N blocks
+    tiles = static_cast<int>(fill_groups(args, *grp, Cfg::kTileRows * PAIRS));
+    args.num_m_tiles = tiles / args.num_n_tiles;  // the kernel's tile count is M x N blocks
     if (tiles == 0) return cudaSuccess;
   }
-  auto kern = fused_gemm_kernel<CG, B_MN, PAIRS, MU, EPI>;
+  auto kern = fused_gemm_kernel<B_MN, PAIRS, MU, EPI>;
   const int fit = max_active_clusters(kern, Cfg::kClusterCtas, Cfg::kThreads, Cfg::kSmemBytes,
                                       d.sm_count / Cfg::kClusterCtas);
   const int clusters = std::min(tiles, fit);
@@ -1498,52 +1881,174 @@ cudaError_t run_dw_grouped(const LayerDev& L0, StepScalars sc, const void* X, co
   return cudaSuccess;
 }
 
-// Tile shape by M, and the W ~ alpha T + mu instantiation for such layers outside TEACHER.
-// Tile shape by rows (M, or a grouped launch's mean rows per expert) and the W ~ alpha T + mu
-// instantiation for such layers outside TEACHER; the general epilogue (EPI 1) for a forward
-// with epilogue options.
+// ---------------------------------------------------------------- narrow launches
+
+template <int BNN, bool B_MN, bool MU>
+cudaError_t run_narrow(const LayerDev& L, StepScalars sc, const void* A, int64_t M, int64_t depth, void* C,
+                       int64_t ncols, const NarrowPlan& np, cudaStream_t st, const GroupSpec* grp,
+                       const EpiOpts* opts) {
+  DeviceInfo& d = device_info();
+  if (!d.ok) return cudaErrorInvalidDevice;
+  CUtensorMap ta, tw;
+  if (!make_tmap(&ta, A, depth, M, BK, 128)) return cudaErrorInvalidValue;
+  const int64_t wrows = grp ? grp->E * L.N : L.N;
+  if (!make_tmap(&tw, L.W, L.K, wrows, 64, B_MN ? BK : BNN)) return cudaErrorInvalidValue;
+  FusedArgs args;
+  fill_fused_args(args, L, sc, C, M, depth, ncols, opts);
+  args.num_n_tiles = static_cast<int32_t>((ncols + BNN - 1) / BNN);
+  args.num_m_tiles = static_cast<int32_t>((M + 128 * np.nacc - 1) / (128 * np.nacc));
+  args.group_m = args.num_m_tiles;
+  args.a_keep = 0;
+  args.wc = make_wait_ctl(d);
+  int64_t tiles = static_cast<int64_t>(args.num_m_tiles) * args.num_n_tiles;
+  if (grp) tiles = fill_groups(args, *grp, 128 * np.nacc);
+  if (tiles == 0) return cudaSuccess;
+  const int grid = static_cast<int>(tiles) * np.splits;
+  if (opts && opts->n_parts) *opts->n_parts = grid;
+  // at least half an SM's shared memory: two CTAs on one SM, each holding tensor memory that the
+  // other's cluster peers wait for, could wait for ever
+  const int smem = std::max(116 * 1024, narrow_smem(BNN, np.nacc, np.stages_a, np.stages_w, np.entries, MU));
+  void* params[4] = {&ta, &tw, &args, const_cast<NarrowPlan*>(&np)};
+  return launch_persistent(fused_narrow_kernel<BNN, B_MN, MU>, np.splits, grid, kNarrowThreads, smem, st, params);
+}
+
+template <bool B_MN, bool MU>
+cudaError_t dispatch_narrow(const LayerDev& L, StepScalars sc, const void* A, int64_t M, int64_t depth, void* C,
+                            int64_t ncols, const NarrowPlan& np, cudaStream_t st, const GroupSpec* grp,
+                            const EpiOpts* opts) {
+  if (np.bn == 64) return run_narrow<64, B_MN, MU>(L, sc, A, M, depth, C, ncols, np, st, grp, opts);
+  return run_narrow<128, B_MN, MU>(L, sc, A, M, depth, C, ncols, np, st, grp, opts);
+}
+
+// Table entries of a CTA's share of nk contraction blocks (see fused_narrow_kernel).
+int64_t narrow_entries(int bn, int64_t nk, int32_t g, bool b_mn) {
+  if (!b_mn) return bn * ((nk * BK + 2 * g - BK - 1) / g);  // a share starts at any multiple of BK
+  const int64_t cols = g % bn == 0 ? 1 : (bn % g == 0 ? bn / g : (bn - 1) / g + 2);
+  return nk * BK * cols;
+}
+
+// Tiles of `rows` rows x `cols` columns.
+int64_t count_tiles(int64_t M, int64_t ncols, const GroupSpec* grp, int64_t rows, int64_t cols) {
+  int64_t m = 0;
+  if (grp)
+    for (int e = 0; e < grp->E; ++e) m += (grp->off[e + 1] - grp->off[e] + rows - 1) / rows;
+  else
+    m = (M + rows - 1) / rows;
+  return m * ((ncols + cols - 1) / cols);
+}
+
+// How a fused launch is cut: pairs of pairs (4 CTAs, 1024 rows), pairs (2, 512 rows) or narrow (1).
+// Each form's time is estimated from what it measured per contraction block on one GB300 (g = 128,
+// SOFT; microseconds), and the least is taken:
+//   pairs       8 + waves (0.62 T + 2), plus 3.5 for the launch that writes op_const,
+//   narrow      7 + rounds (S = 1) or 6 + 3 rounds (S > 1: two cluster barriers each), and nk blocks of
+//               0.38 / 0.48 / 0.54 / 0.68 (64 columns, 1 to 4 accumulators) or 0.56 / 0.72 / 0.95 /
+//               1.2 (128 columns), per wave; W from HBM at no more than 1.95 TB/s.
+// T contraction blocks of 64, nk a share's, rounds the accumulators with rows.  Forward of M x K x N,
+// before (single CTAs below 512 rows) and now: 8 x 2048 x 1024 40 -> 10 us, 128 x 2048 x 2048 41 -> 12,
+// 300 x 2048 x 1024 42 -> 14, 512 x 6144 x 2048 69 -> 33, 1000 x 2048 x 2048 31 -> 23; as pairs
+// instead of single CTAs or pairs of pairs: 64 x 4096 x 14336 77 -> 46, 1100 x 4096 x 14336 173 -> 134,
+// dX of 1500 x 6144 x 2048 51 -> 30.  Pairs of pairs are 3 to 5 % faster than pairs at equal waves,
+// and transform each weight half as often under the power cap: kept up to 10 % more.
+struct FusedPlan {
+  int pairs;      // 2, 1, or 0: narrow
+  NarrowPlan np;
+};
+
+FusedPlan plan_fused(int64_t M, int64_t depth, int64_t ncols, int32_t g, bool b_mn, bool mu, const GroupSpec* grp,
+                     bool loss, bool teacher, int sm_count) {
+  const int64_t T = (depth + BK - 1) / BK;
+  auto waves = [](int64_t tiles, int64_t fit) { return static_cast<double>((tiles + fit - 1) / fit); };
+  const int64_t clusters2 = std::max(1, sm_count / 2), clusters4 = std::max(1, sm_count / 4 - 2);
+  const double per_tile = 0.62 * T + 2.0, consts = teacher ? 0.0 : 3.5;
+  const double t2 = 8.0 + consts + waves(count_tiles(M, ncols, grp, 512, BN), clusters2) * per_tile;
+  const double t4 = 8.0 + consts + waves(count_tiles(M, ncols, grp, 1024, BN), clusters4) * per_tile;
+  FusedPlan p{};
+  const int64_t rows = grp ? M / grp->E : M;  // grouped: by the mean rows of an expert
+  p.pairs = rows >= 1024 && t4 <= 1.1 * t2 ? 2 : 1;
+  double best = 0.92 * (p.pairs == 2 ? t4 : t2);  // the estimates' own error
+  static constexpr double kBlock[2][4] = {{0.38, 0.48, 0.54, 0.68}, {0.56, 0.72, 0.95, 1.2}};
+  const double w_us = static_cast<double>(grp ? grp->E : 1) * depth * ncols * 2 / 1.95e6;
+  for (int bi = 0; bi < 2; ++bi)
+    for (int nacc = 1; nacc <= 4; ++nacc) {
+      if (nacc > 1 && 128 * (nacc - 1) >= M) break;
+      const int bn = 64 << bi;
+      const int64_t tiles = count_tiles(M, ncols, grp, 128 * nacc, bn);
+      for (int s = 1; s <= 8; s *= 2) {
+        // clusters of s CTAs, one per SM, that a GPC layout leaves room for
+        const int64_t fit = s == 8 ? sm_count / 8 - 5 : (s == 4 ? sm_count / 4 - 2 : sm_count / s);
+        if (s > T || fit < 1 || (loss && tiles * s > sm_count * FusedCfg<1>::kEpiWarps)) continue;
+        const int64_t nk = (T + s - 1) / s;
+        const double over = s == 1 ? 7.0 + nacc : 6.0 + 3.0 * nacc;
+        const double t = std::max(waves(tiles, fit) * (over + nk * kBlock[bi][nacc - 1]), 6.0 + w_us);
+        if (t >= best) continue;
+        NarrowPlan np{};
+        np.bn = bn;
+        np.nacc = nacc;
+        np.splits = s;
+        np.entries = static_cast<int32_t>(std::min<int64_t>((narrow_entries(bn, nk, g, b_mn) + 3) / 4 * 4, 1 << 20));
+        // the deepest pair of rings that fits beside the table
+        int depth_best = 0;
+        for (int sw = kNarrowMaxStages; sw >= 2; sw -= 2) {
+          const int64_t left = kNarrowSmemMax - narrow_smem(bn, nacc, 0, sw, np.entries, mu);
+          const int sa = static_cast<int>(std::min<int64_t>(kNarrowMaxStages, left / (nacc * kNarrowABytes)));
+          if (left > 0 && std::min(sa, sw) > depth_best) {
+            depth_best = std::min(sa, sw);
+            np.stages_w = sw;
+            np.stages_a = sa;
+          }
+        }
+        if (depth_best < 2) continue;
+        best = t;
+        p.pairs = 0;
+        p.np = np;
+      }
+    }
+  return p;
+}
+
+// The planned form, with the W ~ alpha T + mu instantiation for such layers outside TEACHER and the
+// general epilogue (EPI 1) for a forward with epilogue options.
 template <bool B_MN, int EPI>
-cudaError_t dispatch_fused_epi(const LayerDev& L, StepScalars sc, const void* A, int64_t M, int64_t tile_rows,
-                               int64_t depth, void* C, int64_t ncols, cudaStream_t st, const GroupSpec* grp,
-                               const EpiOpts* opts) {
-  const bool mu = L.recon != 0 && sc.phase != PHASE_TEACHER;
-  switch (fused_variant_for(tile_rows) * 2 + (mu ? 1 : 0)) {
-    case 8: return run_fused<2, B_MN, 2, false, EPI>(L, sc, A, M, depth, C, ncols, st, grp, opts);
-    case 9: return run_fused<2, B_MN, 2, true, EPI>(L, sc, A, M, depth, C, ncols, st, grp, opts);
-    case 4: return run_fused<2, B_MN, 1, false, EPI>(L, sc, A, M, depth, C, ncols, st, grp, opts);
-    case 5: return run_fused<2, B_MN, 1, true, EPI>(L, sc, A, M, depth, C, ncols, st, grp, opts);
-    case 3: return run_fused<1, B_MN, 1, true, EPI>(L, sc, A, M, depth, C, ncols, st, grp, opts);
-    default: return run_fused<1, B_MN, 1, false, EPI>(L, sc, A, M, depth, C, ncols, st, grp, opts);
-  }
+cudaError_t dispatch_fused_epi(const LayerDev& L, StepScalars sc, const void* A, int64_t M, int64_t depth, void* C,
+                               int64_t ncols, cudaStream_t st, const GroupSpec* grp, const EpiOpts* opts) {
+  if (grp && (grp->E < 1 || grp->E > kMaxGroupExperts)) return cudaErrorInvalidValue;
+  const DeviceInfo& d = device_info();
+  if (!d.ok) return cudaErrorInvalidDevice;
+  const bool teacher = sc.phase == PHASE_TEACHER, mu = L.recon != 0 && !teacher;
+  const FusedPlan p = plan_fused(M, depth, ncols, L.g, B_MN, mu, grp, opts && opts->yref, teacher, d.sm_count);
+  if (p.pairs == 0)
+    return mu ? dispatch_narrow<B_MN, true>(L, sc, A, M, depth, C, ncols, p.np, st, grp, opts)
+              : dispatch_narrow<B_MN, false>(L, sc, A, M, depth, C, ncols, p.np, st, grp, opts);
+  if (p.pairs == 2)
+    return mu ? run_fused<B_MN, 2, true, EPI>(L, sc, A, M, depth, C, ncols, st, grp, opts)
+              : run_fused<B_MN, 2, false, EPI>(L, sc, A, M, depth, C, ncols, st, grp, opts);
+  return mu ? run_fused<B_MN, 1, true, EPI>(L, sc, A, M, depth, C, ncols, st, grp, opts)
+            : run_fused<B_MN, 1, false, EPI>(L, sc, A, M, depth, C, ncols, st, grp, opts);
 }
 
 template <bool B_MN>
 cudaError_t dispatch_fused(const LayerDev& L, StepScalars sc, const void* A, int64_t M, int64_t depth, void* C,
                            int64_t ncols, cudaStream_t st, const EpiOpts* opts = nullptr) {
   if constexpr (!B_MN)
-    if (opts) return dispatch_fused_epi<false, 1>(L, sc, A, M, M, depth, C, ncols, st, nullptr, opts);
-  return dispatch_fused_epi<B_MN, 0>(L, sc, A, M, M, depth, C, ncols, st, nullptr, nullptr);
+    if (opts) return dispatch_fused_epi<false, 1>(L, sc, A, M, depth, C, ncols, st, nullptr, opts);
+  return dispatch_fused_epi<B_MN, 0>(L, sc, A, M, depth, C, ncols, st, nullptr, nullptr);
 }
 
-// Grouped: the tile shape by the mean rows per expert.
 template <bool B_MN>
 cudaError_t dispatch_fused_grouped(const LayerDev& L, StepScalars sc, const void* A, int64_t depth, void* C,
                                    int64_t ncols, const GroupSpec& grp, cudaStream_t st,
                                    const EpiOpts* opts = nullptr) {
   const int64_t R = grp.off[grp.E];
   if constexpr (!B_MN)
-    if (opts) return dispatch_fused_epi<false, 1>(L, sc, A, R, R / grp.E, depth, C, ncols, st, &grp, opts);
-  return dispatch_fused_epi<B_MN, 0>(L, sc, A, R, R / grp.E, depth, C, ncols, st, &grp, nullptr);
+    if (opts) return dispatch_fused_epi<false, 1>(L, sc, A, R, depth, C, ncols, st, &grp, opts);
+  return dispatch_fused_epi<B_MN, 0>(L, sc, A, R, depth, C, ncols, st, &grp, nullptr);
 }
 
 }  // namespace
 
 cudaError_t launch_tc_fwd_grouped(const LayerDev& L0, StepScalars sc, const void* X, const GroupSpec& grp, void* Y,
                                   cudaStream_t st, const EpiOpts* opts) {
-  if (sc.phase != PHASE_TEACHER) {
-    const cudaError_t e = launch_operand_consts_grouped(L0, sc, grp.E, grp.const_stride, st);
-    if (e != cudaSuccess) return e;
-  }
   return dispatch_fused_grouped<false>(L0, sc, X, L0.K, Y, L0.N, grp, st, opts);
 }
 
@@ -1551,10 +2056,6 @@ int fused_loss_max_parts(int sm_count) { return (sm_count > 0 ? sm_count : 1) * 
 
 cudaError_t launch_tc_dx_grouped(const LayerDev& L0, StepScalars sc, const void* dY, const GroupSpec& grp, void* dX,
                                  cudaStream_t st) {
-  if (sc.phase != PHASE_TEACHER) {
-    const cudaError_t e = launch_operand_consts_grouped(L0, sc, grp.E, grp.const_stride, st);
-    if (e != cudaSuccess) return e;
-  }
   return dispatch_fused_grouped<true>(L0, sc, dY, L0.N, dX, L0.K, grp, st);
 }
 
@@ -1584,18 +2085,10 @@ TcPlan tc_plan_bwd(const LayerDev& L, int64_t M, int sm_count) {
 
 cudaError_t launch_tc_fwd(const LayerDev& L, StepScalars sc, const void* X, int64_t M, void* Y, cudaStream_t st,
                          const EpiOpts* opts) {
-  if (sc.phase != PHASE_TEACHER) {
-    const cudaError_t e = launch_operand_consts(L, sc, st);
-    if (e != cudaSuccess) return e;
-  }
   return dispatch_fused<false>(L, sc, X, M, L.K, Y, L.N, st, opts);
 }
 
 cudaError_t launch_tc_dx(const LayerDev& L, StepScalars sc, const void* dY, int64_t M, void* dX, cudaStream_t st) {
-  if (sc.phase != PHASE_TEACHER) {
-    const cudaError_t e = launch_operand_consts(L, sc, st);
-    if (e != cudaSuccess) return e;
-  }
   return dispatch_fused<true>(L, sc, dY, M, L.N, dX, L.K, st);
 }
 

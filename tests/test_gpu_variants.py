@@ -70,3 +70,57 @@ def test_rope_head_runs(device, T, S, nh, d):
     xd = U.to_device(x, "bf16", device)
     C.catq_rope(xd, S, nh, d, 500000.0)
     assert U.fro_rel(_f64(xd), O.rope(x, S, nh, d, 500000.0)) <= 4e-3
+
+
+# The fused contraction's narrow form: 64- and 128-column tiles, 1 to 4 accumulators of 128 rows, the
+# contraction cut into 1 to 8 shares (of unequal length where their number does not divide it), groups
+# that straddle a tile's columns (192), rows and columns past the matrix, every phase, the options
+# of the general epilogue; and pairs of CTAs on fewer than 512 rows (400 x 2048 x 8192).  The bf16 bar.
+@pytest.mark.parametrize("M,N,K,g,recon,phase,s,fused", [
+    (1, 8, 64, 64, 0, O.PHASE_SOFT, 30.0, False), (3, 72, 1408, 128, 0, O.PHASE_SOFT, 3.75, True),
+    (127, 328, 960, 192, 1, O.PHASE_SOFT, 30.0, True), (129, 136, 4032, 64, 0, O.PHASE_HARD, 30.0, False),
+    (300, 1024, 2048, 2048, 0, O.PHASE_SOFT, 7.5, False), (513, 264, 1152, 384, 1, O.PHASE_HARD, 15.0, False),
+    (1000, 520, 704, 64, 0, O.PHASE_SOFT, 30.0, True), (400, 8192, 2048, 128, 0, O.PHASE_SOFT, 30.0, False)])
+def test_linear_narrow_forms(device, M, N, K, g, recon, phase, s, fused):
+    r = syn.rng(302, f"narrow/{M}/{N}/{K}")
+    W, X = _bf16(r, (N, K), 0.02), _bf16(r, (M, K))
+    fac = syn.factors(N * K // g, 3, f"narrow/{N}/{K}", perturbed=True)
+    got = U.gpu_step(W, X, g, fac, O.THR_HALF, phase, s, "bf16", device, recon=recon, fused=fused)
+    ref = O.calibration_step(X, W, g, O.group_stats(W, g, O.THR_HALF), fac, phase, s, with_mu=bool(recon))
+    errs = {k: U.fro_rel(got[k], ref[k]) for k in ("Y", "dY", "dX")}
+    errs["loss"] = abs(got["loss"] - ref["loss"]) / ref["loss"]
+    bad = {k: v for k, v in errs.items() if not v <= U.TOL_BF16}
+    assert not bad, (bad, errs)
+
+
+# Grouped launches in the narrow form: experts of 0, 1, 130 and 257 rows, and the same rows expert by
+# expert as dense layers give the same sums (both cut the contraction, in fp32: 1e-2 in bf16).
+def test_grouped_narrow_matches_dense(device):
+    import torch
+
+    from paper_2606_26650_gb300 import catq as C
+    E, N, K, g, rows = 5, 192, 1024, 128, [130, 0, 1, 257, 40]
+    off = [0] + [int(v) for v in np.cumsum(rows)]
+    r = syn.rng(303, "grouped narrow")
+    W = U.to_device(_bf16(r, (E * N, K), 0.02), "bf16", device).view(E, N, K)
+    X = U.to_device(_bf16(r, (off[-1], K)), "bf16", device)
+    dY = U.to_device(_bf16(r, (off[-1], N)), "bf16", device)
+    fac = [torch.from_numpy(f).to(device) for f in syn.factors(E * N * K // g, 3, "grouped narrow", perturbed=True)]
+    layer = C.GroupedLayer.create(W, g, *fac)
+    C.catq_group_stats(layer.dense)
+    sched = C.schedule(C.PHASE_SOFT, 30.0)
+    Y, dX = torch.empty(off[-1], N, dtype=X.dtype, device=device), torch.empty_like(X)
+    C.catq_grouped_soft_ternary_linear_fwd(layer, sched, X, off, Y)
+    C.catq_grouped_soft_ternary_linear_bwd(layer, sched, X, dY, off, dX)
+    per = N * K // g
+    for e in range(E):
+        a, b = off[e], off[e + 1]
+        if a == b:
+            continue
+        one = C.Layer.create(W[e], g, *(f[e * per:(e + 1) * per].clone() for f in fac))
+        C.catq_group_stats(one)
+        y, dx = torch.empty(b - a, N, dtype=X.dtype, device=device), torch.empty(b - a, K, dtype=X.dtype, device=device)
+        C.catq_soft_ternary_linear_fwd(one, sched, X[a:b], y)
+        C.catq_soft_ternary_linear_bwd(one, sched, X[a:b], dY[a:b], dx)
+        assert U.fro_rel(_f64(Y[a:b]), _f64(y)) <= 1e-2
+        assert U.fro_rel(_f64(dX[a:b]), _f64(dx)) <= 1e-2
