@@ -124,3 +124,20 @@ def test_grouped_narrow_matches_dense(device):
         C.catq_soft_ternary_linear_bwd(one, sched, X[a:b], dY[a:b], dx)
         assert U.fro_rel(_f64(Y[a:b]), _f64(y)) <= 1e-2
         assert U.fro_rel(_f64(dX[a:b]), _f64(dx)) <= 1e-2
+
+
+# The fp32 path: tiles of 32, 128 and 256 rows with remainders, an output width that is no multiple of
+# 4, groups of 4 to 512, contractions shared by 1 to 8 CTAs, a single slice.  The fp32 bar.
+@pytest.mark.parametrize("M,N,K,g,recon,phase,s", [
+    (1, 17, 4, 4, 0, O.PHASE_SOFT, 30.0), (13, 342, 640, 64, 1, O.PHASE_SOFT, 7.5), (33, 36, 1024, 16, 0, O.PHASE_HARD, 30.0),
+    (129, 130, 96, 32, 0, O.PHASE_SOFT, 3.75), (300, 64, 520, 8, 1, O.PHASE_SOFT, 30.0), (700, 511, 512, 512, 0, O.PHASE_SOFT, 30.0)])
+def test_linear_fp32_tiles(device, M, N, K, g, recon, phase, s):
+    r = syn.rng(304, f"fp32/{M}/{N}/{K}")
+    W, X = (r.standard_normal((N, K)) * 0.02).astype(np.float32), r.standard_normal((M, K)).astype(np.float32)
+    fac = syn.factors(N * K // g, 3, f"fp32/{N}/{K}", perturbed=True)
+    got = U.gpu_step(W, X, g, fac, O.THR_HALF, phase, s, "f32", device, recon=recon)
+    ref = O.calibration_step(X, W, g, O.group_stats(W, g, O.THR_HALF), fac, phase, s, with_mu=bool(recon))
+    errs = {k: U.max_rel(got[k], ref[k]) for k in ("Y_ref", "Y", "dY", "dX", "g_dmu", "g_dalpha", "g_ddelta")}
+    errs["loss"] = abs(got["loss"] - ref["loss"]) / ref["loss"]
+    bad = {k: v for k, v in errs.items() if not v <= U.TOL_F32}
+    assert not bad, (bad, errs)
