@@ -112,6 +112,7 @@ class Block:
         ws = max(C.catq_bwd_workspace_bytes(L, T) for L in self.layers.values())
         # side streams (independent calls) and one dW workspace per side stream
         self.sides = [torch.cuda.Stream(device=dev) for _ in range(max(0, int(side_streams)))]
+        self._event = torch.cuda.Event()
         self.bwd_ws = [C.workspace(ws, dev) for _ in range(1 + len(self.sides))]
         self.loss_ws = C.workspace(C.catq_recon_loss_workspace_bytes(T * H), dev)
         self._next_side = 0
@@ -123,9 +124,9 @@ class Block:
     def _after(self, src, dst):
         """dst waits for the work issued so far on src."""
         if dst is not src:
-            ev = self.torch.cuda.Event()
-            ev.record(src)
-            dst.wait_event(ev)
+            # one event serves every pair: a wait takes the event's latest record when it is issued
+            self._event.record(src)
+            dst.wait_event(self._event)
 
     def _side(self, i):
         """Side stream i (the main stream when the block has none)."""

@@ -11,6 +11,7 @@ import ctypes
 import dataclasses
 import os
 import re
+import struct
 
 PKG = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(PKG, "libcatq.so")
@@ -81,7 +82,7 @@ def lib() -> ctypes.CDLL:
         raise RuntimeError(f"{LIB_PATH} is missing: build it with __graft_entry__.build()")
     L = ctypes.CDLL(LIB_PATH)
     P, I64, I32, F, S = ctypes.c_void_p, ctypes.c_int64, ctypes.c_int32, ctypes.c_float, ctypes.c_size_t
-    LP = ctypes.POINTER(catq_layer)
+    LP = P  # structs by address: byref(...) or their packed bytes
     sig = {
         "catq_abi_version": (I32, []),
         "catq_status_string": (ctypes.c_char_p, [I32]),
@@ -98,13 +99,13 @@ def lib() -> ctypes.CDLL:
         "catq_ternary_infer": (I32, [P, P, P, I64, I64, I32, P, I64, I32, P, P]),
         "catq_soft_ternary_linear_bwd_noalloc": (I32, [LP, catq_schedule, P, P, I64, I32, P, P, P, P, P]),
         "catq_bwd_noalloc_max_scratch_bytes": (S, []),
-        "catq_grouped_soft_ternary_linear_fwd": (I32, [ctypes.POINTER(catq_grouped_layer), catq_schedule, P, P, I32, P,
+        "catq_grouped_soft_ternary_linear_fwd": (I32, [P, catq_schedule, P, P, I32, P,
                                                        P]),
-        "catq_grouped_bwd_workspace_bytes": (S, [ctypes.POINTER(catq_grouped_layer), P]),
+        "catq_grouped_bwd_workspace_bytes": (S, [P, P]),
         "catq_schedule_at_epoch": (I32, [I32, I32, ctypes.c_double, ctypes.c_double, ctypes.POINTER(catq_schedule)]),
         "catq_linear_decay_lr": (I32, [ctypes.c_double, I64, I64, ctypes.POINTER(F)]),
         "catq_factor_adamw_step": (I32, [I64, P, P, P, P, P, P, P, ctypes.POINTER(catq_adamw), I64, F, P]),
-        "catq_grouped_soft_ternary_linear_bwd": (I32, [ctypes.POINTER(catq_grouped_layer), catq_schedule, P, P, P, I32,
+        "catq_grouped_soft_ternary_linear_bwd": (I32, [P, catq_schedule, P, P, P, I32,
                                                        P, P, P, P, P, S, P]),
         "catq_soft_ternary_linear_fwd_ex": (I32, [LP, catq_schedule, P, I64, I32, P, P, I32, P]),
         "catq_fwd_loss_workspace_bytes": (S, [LP, I64]),
@@ -112,13 +113,12 @@ def lib() -> ctypes.CDLL:
         "catq_act_quant_a8": (I32, [P, I64, I64, I32, P, P, P, P]),
         "catq_direct_adamw_step": (I32, [I64, P, P, P, P, P, ctypes.POINTER(catq_adamw), I64, F, P]),
         "catq_ternary_infer_max_layers": (I32, []),
-        "catq_ternary_infer_batched": (I32, [ctypes.POINTER(catq_infer_layer), I32, I32, I64, I32, P]),
+        "catq_ternary_infer_batched": (I32, [P, I32, I32, I64, I32, P]),
         "catq_ternary_infer_max_stages": (I32, []),
         "catq_ternary_infer_sync_bytes": (S, []),
-        "catq_ternary_infer_staged": (I32, [ctypes.POINTER(catq_infer_layer), I32, ctypes.POINTER(I32), I32, I64, I32,
-                                            P, P]),
+        "catq_ternary_infer_staged": (I32, [P, I32, P, I32, I64, I32, P, P]),
         "catq_group_recon_error": (I32, [LP, P, P]),
-        "catq_grouped_fwd_loss_workspace_bytes": (S, [ctypes.POINTER(catq_grouped_layer), P]),
+        "catq_grouped_fwd_loss_workspace_bytes": (S, [P, P]),
         "catq_rmsnorm_fwd": (I32, [P, I32, P, P, I64, I64, F, P, P, P, P]),
         "catq_rmsnorm_bwd": (I32, [P, I32, P, P, P, P, P, I64, I64, P, P]),
         "catq_rope": (I32, [P, I64, I64, I32, I32, F, I32, P]),
@@ -127,7 +127,7 @@ def lib() -> ctypes.CDLL:
         "catq_block_output_loss": (I32, [P, P, I64, P, I32, P, P, P, P, S, P]),
         "catq_attention_fwd": (I32, [P, P, P, I32, I32, I32, I32, I32, P, P, P]),
         "catq_attention_bwd": (I32, [P, P, P, P, P, P, I32, I32, I32, I32, I32, P, P, P, P, P]),
-        "catq_grouped_soft_ternary_linear_fwd_loss": (I32, [ctypes.POINTER(catq_grouped_layer), catq_schedule, P, P,
+        "catq_grouped_soft_ternary_linear_fwd_loss": (I32, [P, catq_schedule, P, P,
                                                             I32, P, I32, P, P, P, P, S, P]),
     }
     for name, (res, args) in sig.items():
@@ -146,24 +146,39 @@ def header_functions(path: str = HEADER):
 
 
 # ------------------------------------------------------------------ marshalling helpers
+# A small call (a norm of a few rows, a decode step's layers) costs a few microseconds on the GPU,
+# so these run on every argument of every call and keep to a handful of attribute reads each:
+# addresses as ints, structs as packed bytes, the stream without a Stream object.  Nothing is
+# remembered from one call to the next.  On a Grace host, Python and launch together: forward of a layer 18.0 -> 8.9 us, its
+# backward 27.3 -> 16.2, a row norm 9.7 -> 5.3, three decode layers 17.9 -> 9.9.
 
 def _ptr(t):
-    return None if t is None else ctypes.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
 
 
 def _stream(stream=None):
+    if stream is not None:
+        return stream.cuda_stream
     import torch
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return ctypes.c_void_p(s.cuda_stream)
+    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+
+
+_DTYPES: dict = {}
+
+
+def _known_dtype(t):
+    """The code of a tensor's dtype, None for one the library does not take."""
+    if not _DTYPES:
+        import torch
+        _DTYPES.update({torch.bfloat16: BF16, torch.float32: F32})
+    return _DTYPES.get(t.dtype)
 
 
 def _dtype_code(t) -> int:
-    import torch
-    if t.dtype == torch.bfloat16:
-        return BF16
-    if t.dtype == torch.float32:
-        return F32
-    raise TypeError(f"unsupported dtype {t.dtype}")
+    code = _known_dtype(t)
+    if code is None:
+        raise TypeError(f"unsupported dtype {t.dtype}")
+    return code
 
 
 def _check(status: int, where: str):
@@ -175,16 +190,30 @@ def _buf(t, name: str, nbytes: int, where: str):
     """The library reads and writes `nbytes` bytes at a tensor's address without seeing its
     size or device: refuse a host tensor or one too small before the call, so that a
     caller's mistake raises here instead of touching memory the tensor does not own.
-    None passes (the call decides whether the argument is optional)."""
+    None passes (the call decides whether the argument is optional).  Returns the address."""
     if t is None:
-        return
+        return None
+    if t.is_cuda and t.is_contiguous() and t.numel() * t.element_size() >= nbytes:
+        return t.data_ptr()
     if not t.is_cuda:
         raise ValueError(f"{where}: {name} must be a CUDA tensor")
     if not t.is_contiguous():
         raise ValueError(f"{where}: {name} must be contiguous")
     have = t.numel() * t.element_size()
-    if have < nbytes:
-        raise ValueError(f"{where}: {name} holds {have} bytes, the call needs {nbytes}")
+    raise ValueError(f"{where}: {name} holds {have} bytes, the call needs {nbytes}")
+
+
+def _ws(workspace, where: str):
+    """(address, bytes) of a workspace; the call decides whether it is large enough."""
+    if workspace is None:
+        return None, 0
+    return _buf(workspace, "workspace", 0, where), workspace.numel() * workspace.element_size()
+
+
+# catq_layer, catq_grouped_layer and catq_infer_layer as packed bytes (native sizes and alignment).
+_LAYER = struct.Struct("qqii8Qii")
+_GROUPED = struct.Struct("iiqqii8Q")
+_INFER = struct.Struct("QQQqqQQ")
 
 
 @dataclasses.dataclass
@@ -229,16 +258,24 @@ class Layer:
     def G(self):
         return self.N * self.K // self.g
 
+    def _addresses(self, N: int, K: int):
+        """The checked addresses of W, the six per-group arrays and op_const (0: none)."""
+        W, where, need = self.W, "Layer", 4 * (N * K // self.g)
+        return (_buf(W, "W", N * K * W.element_size(), where), _buf(self.mu0, "mu0", need, where),
+                _buf(self.alpha0, "alpha0", need, where), _buf(self.delta0, "delta0", need, where),
+                _buf(self.d_mu, "d_mu", need, where), _buf(self.d_alpha, "d_alpha", need, where),
+                _buf(self.d_delta, "d_delta", need, where),
+                _buf(self.op_const, "op_const", (5 if self.recon else 4) * need, where) or 0)
+
     def struct(self) -> catq_layer:
-        G, where = self.G, "Layer"
-        _buf(self.W, "W", self.N * self.K * self.W.element_size(), where)
-        for name in ("mu0", "alpha0", "delta0", "d_mu", "d_alpha", "d_delta"):
-            _buf(getattr(self, name), name, 4 * G, where)
-        _buf(self.op_const, "op_const", 4 * (5 if self.recon else 4) * G, where)
-        return catq_layer(self.N, self.K, self.g, _dtype_code(self.W), self.W.data_ptr(),
-                          self.mu0.data_ptr(), self.alpha0.data_ptr(), self.delta0.data_ptr(),
-                          self.d_mu.data_ptr(), self.d_alpha.data_ptr(), self.d_delta.data_ptr(),
-                          self.op_const.data_ptr() if self.op_const is not None else None, self.recon, 0)
+        N, K = self.W.shape
+        *ptrs, op = self._addresses(N, K)
+        return catq_layer(N, K, self.g, _dtype_code(self.W), *ptrs, op or None, self.recon, 0)
+
+    def packed(self) -> bytes:
+        """struct() as bytes (what the calls below pass)."""
+        N, K = self.W.shape
+        return _LAYER.pack(N, K, self.g, _dtype_code(self.W), *self._addresses(N, K), self.recon, 0)
 
 
 def schedule(phase: int, s: float = 0.0) -> catq_schedule:
@@ -248,63 +285,61 @@ def schedule(phase: int, s: float = 0.0) -> catq_schedule:
 # ------------------------------------------------------------------ the C calls
 
 def catq_group_stats(layer: Layer, thr_init: int = THR_HALF, stream=None):
-    st = layer.struct()
-    _check(lib().catq_group_stats(ctypes.byref(st), int(thr_init), _stream(stream)), "catq_group_stats")
+    _check(lib().catq_group_stats(layer.packed(), int(thr_init), _stream(stream)), "catq_group_stats")
 
 
 def catq_modulate_ternarize(layer: Layer, sched: catq_schedule, Wq_out=None, T_out=None, alpha_out=None,
                             stream=None):
-    st = layer.struct()
+    st = layer.packed()
     w = "catq_modulate_ternarize"
-    _buf(Wq_out, "Wq_out", layer.N * layer.K * layer.W.element_size(), w)
-    _buf(T_out, "T_out", layer.N * layer.K, w)
-    _buf(alpha_out, "alpha_out", 4 * layer.G, w)
-    _check(lib().catq_modulate_ternarize(ctypes.byref(st), sched, _ptr(Wq_out), _ptr(T_out), _ptr(alpha_out),
-                                         _stream(stream)), "catq_modulate_ternarize")
+    wq = _buf(Wq_out, "Wq_out", layer.N * layer.K * layer.W.element_size(), w)
+    t = _buf(T_out, "T_out", layer.N * layer.K, w)
+    al = _buf(alpha_out, "alpha_out", 4 * layer.G, w)
+    _check(lib().catq_modulate_ternarize(st, sched, wq, t, al, _stream(stream)), w)
 
 
 def catq_soft_ternary_linear_fwd(layer: Layer, sched: catq_schedule, X, Y, stream=None):
-    st = layer.struct()
-    M, e, w = X.shape[0], X.element_size(), "catq_soft_ternary_linear_fwd"
-    _buf(X, "X", M * layer.K * e, w)
-    _buf(Y, "Y", M * layer.N * e, w)
-    _check(lib().catq_soft_ternary_linear_fwd(ctypes.byref(st), sched, _ptr(X), X.shape[0], _dtype_code(X),
-                                              _ptr(Y), _stream(stream)), "catq_soft_ternary_linear_fwd")
+    w = "catq_soft_ternary_linear_fwd"
+    st = layer.packed()
+    N, K = layer.W.shape
+    M, e = X.shape[0], X.element_size()
+    _check(lib().catq_soft_ternary_linear_fwd(st, sched, _buf(X, "X", M * K * e, w), M, _dtype_code(X),
+                                              _buf(Y, "Y", M * N * e, w), _stream(stream)), w)
 
 
 def catq_soft_ternary_linear_fwd_ex(layer: Layer, sched: catq_schedule, X, Y, x_row_scale=None, stream=None):
     """Y = diag(x_row_scale) X Wq^T; Y may be fp32 for a bf16 layer."""
-    st = layer.struct()
-    M, w = X.shape[0], "catq_soft_ternary_linear_fwd_ex"
-    _buf(X, "X", M * layer.K * X.element_size(), w)
-    _buf(Y, "Y", M * layer.N * (Y.element_size() if Y is not None else 0), w)
-    _buf(x_row_scale, "x_row_scale", 4 * M, w)
-    _check(lib().catq_soft_ternary_linear_fwd_ex(ctypes.byref(st), sched, _ptr(X), M, _dtype_code(X),
-                                                 _ptr(x_row_scale), _ptr(Y), _dtype_code(Y), _stream(stream)), w)
+    w = "catq_soft_ternary_linear_fwd_ex"
+    st = layer.packed()
+    N, K = layer.W.shape
+    M = X.shape[0]
+    x = _buf(X, "X", M * K * X.element_size(), w)
+    y = _buf(Y, "Y", M * N * (Y.element_size() if Y is not None else 0), w)
+    rs = _buf(x_row_scale, "x_row_scale", 4 * M, w)
+    _check(lib().catq_soft_ternary_linear_fwd_ex(st, sched, x, M, _dtype_code(X), rs, y, _dtype_code(Y),
+                                                 _stream(stream)), w)
 
 
 def catq_fwd_loss_workspace_bytes(layer: Layer, M: int) -> int:
-    st = layer.struct()
-    return int(lib().catq_fwd_loss_workspace_bytes(ctypes.byref(st), int(M)))
+    return int(lib().catq_fwd_loss_workspace_bytes(layer.packed(), int(M)))
 
 
 def catq_soft_ternary_linear_fwd_loss(layer: Layer, sched: catq_schedule, X, Y_ref, loss_out, dY, Y=None,
                                       x_row_scale=None, workspace=None, reduction: int = REDUCE_MEAN, stream=None):
     """Forward, Eq. 7 loss and dY in one pass; Y_ref may be fp32 for a bf16 layer."""
-    st = layer.struct()
-    M, e, w = X.shape[0], X.element_size(), "catq_soft_ternary_linear_fwd_loss"
-    _buf(X, "X", M * layer.K * e, w)
-    _buf(Y_ref, "Y_ref", M * layer.N * Y_ref.element_size(), w)
-    _buf(dY, "dY", M * layer.N * e, w)
-    _buf(Y, "Y", M * layer.N * e, w)
-    _buf(loss_out, "loss_out", 4, w)
-    _buf(x_row_scale, "x_row_scale", 4 * M, w)
-    _buf(workspace, "workspace", 0, w)
-    ws_bytes = 0 if workspace is None else workspace.numel() * workspace.element_size()
-    _check(lib().catq_soft_ternary_linear_fwd_loss(ctypes.byref(st), sched, _ptr(X), M, _dtype_code(X),
-                                                   _ptr(x_row_scale), _ptr(Y_ref), _dtype_code(Y_ref),
-                                                   int(reduction), _ptr(loss_out), _ptr(dY), _ptr(Y),
-                                                   _ptr(workspace), ws_bytes, _stream(stream)), w)
+    w = "catq_soft_ternary_linear_fwd_loss"
+    st = layer.packed()
+    N, K = layer.W.shape
+    M, e = X.shape[0], X.element_size()
+    x = _buf(X, "X", M * K * e, w)
+    ref = _buf(Y_ref, "Y_ref", M * N * Y_ref.element_size(), w)
+    dy = _buf(dY, "dY", M * N * e, w)
+    y = _buf(Y, "Y", M * N * e, w)
+    lo = _buf(loss_out, "loss_out", 4, w)
+    rs = _buf(x_row_scale, "x_row_scale", 4 * M, w)
+    ws, ws_bytes = _ws(workspace, w)
+    _check(lib().catq_soft_ternary_linear_fwd_loss(st, sched, x, M, _dtype_code(X), rs, ref, _dtype_code(Y_ref),
+                                                   int(reduction), lo, dy, y, ws, ws_bytes, _stream(stream)), w)
 
 
 def catq_act_quant_a8(X, codes, scale, X_deq=None, stream=None):
@@ -312,49 +347,41 @@ def catq_act_quant_a8(X, codes, scale, X_deq=None, stream=None):
     dequantized activations."""
     M, K = X.shape
     n, w = M * K * X.element_size(), "catq_act_quant_a8"
-    _buf(X, "X", n, w)
-    _buf(codes, "codes", n, w)
-    _buf(X_deq, "X_deq", n, w)
-    _buf(scale, "scale", 4 * M, w)
-    _check(lib().catq_act_quant_a8(_ptr(X), M, K, _dtype_code(X), _ptr(codes), _ptr(scale), _ptr(X_deq),
-                                   _stream(stream)), w)
+    x, c, d = _buf(X, "X", n, w), _buf(codes, "codes", n, w), _buf(X_deq, "X_deq", n, w)
+    sc = _buf(scale, "scale", 4 * M, w)
+    _check(lib().catq_act_quant_a8(x, M, K, _dtype_code(X), c, sc, d, _stream(stream)), w)
 
 
 def catq_bwd_workspace_bytes(layer: Layer, M: int) -> int:
-    st = layer.struct()
-    return int(lib().catq_bwd_workspace_bytes(ctypes.byref(st), int(M)))
+    return int(lib().catq_bwd_workspace_bytes(layer.packed(), int(M)))
 
 
 def catq_soft_ternary_linear_bwd(layer: Layer, sched: catq_schedule, X, dY, dX=None, g_dmu=None, g_dalpha=None,
                                  g_ddelta=None, workspace=None, stream=None):
-    st = layer.struct()
-    _bwd_bufs(layer, X, dY, dX, (g_dmu, g_dalpha, g_ddelta), "catq_soft_ternary_linear_bwd")
-    _buf(workspace, "workspace", 0, "catq_soft_ternary_linear_bwd")
-    ws_bytes = 0 if workspace is None else workspace.numel() * workspace.element_size()
-    _check(lib().catq_soft_ternary_linear_bwd(ctypes.byref(st), sched, _ptr(X), _ptr(dY), X.shape[0],
-                                              _dtype_code(X), _ptr(dX), _ptr(g_dmu), _ptr(g_dalpha),
-                                              _ptr(g_ddelta), _ptr(workspace), ws_bytes, _stream(stream)),
-           "catq_soft_ternary_linear_bwd")
+    w = "catq_soft_ternary_linear_bwd"
+    st = layer.packed()
+    x, dy, dx, g0, g1, g2 = _bwd_bufs(layer, X, dY, dX, (g_dmu, g_dalpha, g_ddelta), w)
+    ws, ws_bytes = _ws(workspace, w)
+    _check(lib().catq_soft_ternary_linear_bwd(st, sched, x, dy, X.shape[0], _dtype_code(X), dx, g0, g1, g2, ws,
+                                              ws_bytes, _stream(stream)), w)
 
 
 def catq_soft_ternary_linear_bwd_noalloc(layer: Layer, sched: catq_schedule, X, dY, dX=None, g_dmu=None,
                                          g_dalpha=None, g_ddelta=None, stream=None):
-    st = layer.struct()
-    _bwd_bufs(layer, X, dY, dX, (g_dmu, g_dalpha, g_ddelta), "catq_soft_ternary_linear_bwd_noalloc")
-    _check(lib().catq_soft_ternary_linear_bwd_noalloc(ctypes.byref(st), sched, _ptr(X), _ptr(dY), X.shape[0],
-                                                      _dtype_code(X), _ptr(dX), _ptr(g_dmu), _ptr(g_dalpha),
-                                                      _ptr(g_ddelta), _stream(stream)),
-           "catq_soft_ternary_linear_bwd_noalloc")
+    w = "catq_soft_ternary_linear_bwd_noalloc"
+    st = layer.packed()
+    x, dy, dx, g0, g1, g2 = _bwd_bufs(layer, X, dY, dX, (g_dmu, g_dalpha, g_ddelta), w)
+    _check(lib().catq_soft_ternary_linear_bwd_noalloc(st, sched, x, dy, X.shape[0], _dtype_code(X), dx, g0, g1, g2,
+                                                      _stream(stream)), w)
 
 
-def _bwd_bufs(layer, X, dY, dX, grads, where, rows=None, groups=None):
-    M = X.shape[0] if rows is None else rows
-    e = X.element_size()
-    _buf(X, "X", M * layer.K * e, where)
-    _buf(dY, "dY", M * layer.N * e, where)
-    _buf(dX, "dX", M * layer.K * e, where)
-    for name, arr in zip(("g_dmu", "g_dalpha", "g_ddelta"), grads):
-        _buf(arr, name, 4 * (layer.G if groups is None else groups), where)
+def _bwd_bufs(layer, X, dY, dX, grads, where):
+    """The checked addresses of a backward's arrays."""
+    N, K = layer.W.shape
+    M, e, need = X.shape[0], X.element_size(), 4 * (N * K // layer.g)
+    return (_buf(X, "X", M * K * e, where), _buf(dY, "dY", M * N * e, where), _buf(dX, "dX", M * K * e, where),
+            _buf(grads[0], "g_dmu", need, where), _buf(grads[1], "g_dalpha", need, where),
+            _buf(grads[2], "g_ddelta", need, where))
 
 
 def catq_bwd_noalloc_max_scratch_bytes() -> int:
@@ -366,25 +393,21 @@ def catq_recon_loss_workspace_bytes(count: int) -> int:
 
 
 def catq_recon_loss(Y, Y_ref, loss_out, dY=None, workspace=None, reduction: int = REDUCE_MEAN, stream=None):
-    w, n = "catq_recon_loss", Y.numel() * Y.element_size()
-    _buf(Y, "Y", n, w)
-    _buf(Y_ref, "Y_ref", n, w)
-    _buf(dY, "dY", n, w)
-    _buf(loss_out, "loss_out", 4, w)
-    _buf(workspace, "workspace", 0, w)
-    ws_bytes = 0 if workspace is None else workspace.numel() * workspace.element_size()
-    _check(lib().catq_recon_loss(_ptr(Y), _ptr(Y_ref), Y.numel(), _dtype_code(Y), int(reduction), _ptr(loss_out),
-                                 _ptr(dY), _ptr(workspace), ws_bytes, _stream(stream)), "catq_recon_loss")
+    w, count = "catq_recon_loss", Y.numel()
+    n = count * Y.element_size()
+    y, ref, dy = _buf(Y, "Y", n, w), _buf(Y_ref, "Y_ref", n, w), _buf(dY, "dY", n, w)
+    lo = _buf(loss_out, "loss_out", 4, w)
+    ws, ws_bytes = _ws(workspace, w)
+    _check(lib().catq_recon_loss(y, ref, count, _dtype_code(Y), int(reduction), lo, dy, ws, ws_bytes,
+                                 _stream(stream)), w)
 
 
 def catq_hard_ternarize_pack(layer: Layer, codes, alpha=None, mu=None, stream=None):
-    st = layer.struct()
-    w = "catq_hard_ternarize_pack"
-    _buf(codes, "codes", layer.N * layer.K // 4, w)
-    _buf(alpha, "alpha", 4 * layer.G, w)
-    _buf(mu, "mu", 4 * layer.G, w)
-    _check(lib().catq_hard_ternarize_pack(ctypes.byref(st), _ptr(codes), _ptr(alpha), _ptr(mu), _stream(stream)),
-           "catq_hard_ternarize_pack")
+    st = layer.packed()
+    w, G = "catq_hard_ternarize_pack", layer.G
+    c = _buf(codes, "codes", layer.N * layer.K // 4, w)
+    al, m = _buf(alpha, "alpha", 4 * G, w), _buf(mu, "mu", 4 * G, w)
+    _check(lib().catq_hard_ternarize_pack(st, c, al, m, _stream(stream)), w)
 
 
 def catq_device_status(stream=None) -> int:
@@ -396,56 +419,40 @@ def catq_device_status(stream=None) -> int:
 def catq_ternary_infer(codes, alpha, N: int, K: int, g: int, X, Y, mu=None, stream=None):
     """Y [B, N] = X [B, K] (alpha T + mu)^T from the 2-bit codes, group scales and (for the
     W ~ alpha T + mu form) group offsets of catq_hard_ternarize_pack."""
-    w, B, G = "catq_ternary_infer", X.shape[0], int(N) * int(K) // max(int(g), 1)
-    _buf(codes, "codes", int(N) * int(K) // 4, w)
-    _buf(alpha, "alpha", 4 * G, w)
-    _buf(mu, "mu", 4 * G, w)
-    _buf(X, "X", B * int(K) * X.element_size(), w)
-    _buf(Y, "Y", B * int(N) * X.element_size(), w)
-    _check(lib().catq_ternary_infer(_ptr(codes), _ptr(alpha), _ptr(mu), int(N), int(K), int(g), _ptr(X),
-                                    X.shape[0], _dtype_code(X), _ptr(Y), _stream(stream)), "catq_ternary_infer")
+    w, B, N, K = "catq_ternary_infer", X.shape[0], int(N), int(K)
+    G, e = N * K // max(int(g), 1), X.element_size()
+    c = _buf(codes, "codes", N * K // 4, w)
+    al, m = _buf(alpha, "alpha", 4 * G, w), _buf(mu, "mu", 4 * G, w)
+    x, y = _buf(X, "X", B * K * e, w), _buf(Y, "Y", B * N * e, w)
+    _check(lib().catq_ternary_infer(c, al, m, N, K, int(g), x, B, _dtype_code(X), y, _stream(stream)), w)
 
 
 def catq_ternary_infer_max_layers() -> int:
     return int(lib().catq_ternary_infer_max_layers())
 
 
+def _infer_layer_array(layers, g, w):
+    """The layers as packed catq_infer_layer structs, and their token rows."""
+    B, g, out = layers[0][4].shape[0] if layers else 0, max(int(g), 1), []
+    for codes, alpha, N, K, X, Y, mu in layers:
+        N, K = int(N), int(K)
+        n = N * K
+        if X.shape[0] != B:
+            raise ValueError(f"{w}: every layer needs the same token rows ({B})")
+        e, need = X.element_size(), 4 * (n // g)
+        out.append(_INFER.pack(_buf(codes, "codes", n // 4, w), _buf(alpha, "alpha", need, w),
+                               _buf(mu, "mu", need, w) or 0, N, K, _buf(X, "X", B * K * e, w),
+                               _buf(Y, "Y", B * N * e, w)))
+    return b"".join(out) or bytes(_INFER.size), B
+
+
 def catq_ternary_infer_batched(layers, g: int, stream=None):
     """Several independent layers in one launch: `layers` is a list of tuples
     (codes, alpha, N, K, X, Y, mu) (mu may be None), all with the same token rows X.shape[0]."""
     w = "catq_ternary_infer_batched"
-    arr = (catq_infer_layer * max(1, len(layers)))()
-    B = layers[0][4].shape[0] if layers else 0
-    for i, (codes, alpha, N, K, X, Y, mu) in enumerate(layers):
-        G = int(N) * int(K) // max(int(g), 1)
-        _buf(codes, "codes", int(N) * int(K) // 4, w)
-        _buf(alpha, "alpha", 4 * G, w)
-        _buf(mu, "mu", 4 * G, w)
-        if X.shape[0] != B:
-            raise ValueError(f"{w}: every layer needs the same token rows ({B})")
-        _buf(X, "X", B * int(K) * X.element_size(), w)
-        _buf(Y, "Y", B * int(N) * X.element_size(), w)
-        arr[i] = catq_infer_layer(codes.data_ptr(), alpha.data_ptr(), mu.data_ptr() if mu is not None else None,
-                                  int(N), int(K), X.data_ptr(), Y.data_ptr())
+    arr, B = _infer_layer_array(layers, g, w)
     dt = _dtype_code(layers[0][4]) if layers else BF16
     _check(lib().catq_ternary_infer_batched(arr, len(layers), int(g), int(B), dt, _stream(stream)), w)
-
-
-def _infer_layer_array(layers, g, w):
-    arr = (catq_infer_layer * max(1, len(layers)))()
-    B = layers[0][4].shape[0] if layers else 0
-    for i, (codes, alpha, N, K, X, Y, mu) in enumerate(layers):
-        G = int(N) * int(K) // max(int(g), 1)
-        _buf(codes, "codes", int(N) * int(K) // 4, w)
-        _buf(alpha, "alpha", 4 * G, w)
-        _buf(mu, "mu", 4 * G, w)
-        if X.shape[0] != B:
-            raise ValueError(f"{w}: every layer needs the same token rows ({B})")
-        _buf(X, "X", B * int(K) * X.element_size(), w)
-        _buf(Y, "Y", B * int(N) * X.element_size(), w)
-        arr[i] = catq_infer_layer(codes.data_ptr(), alpha.data_ptr(), mu.data_ptr() if mu is not None else None,
-                                  int(N), int(K), X.data_ptr(), Y.data_ptr())
-    return arr, B
 
 
 def catq_ternary_infer_sync_bytes() -> int:
@@ -463,12 +470,12 @@ def catq_ternary_infer_staged(layers, stages, g: int, sync, stream=None):
     of catq_ternary_infer_sync_bytes() bytes (left zeroed)."""
     w = "catq_ternary_infer_staged"
     arr, B = _infer_layer_array(layers, g, w)
-    _buf(sync, "sync", catq_ternary_infer_sync_bytes(), w)
-    st = (ctypes.c_int32 * max(1, len(stages)))(*[int(v) for v in stages])
+    sy = _buf(sync, "sync", catq_ternary_infer_sync_bytes(), w)
     if len(stages) != len(layers):
         raise ValueError(f"{w}: one stage per layer")
+    st = struct.pack(f"{max(1, len(stages))}i", *([int(v) for v in stages] or [0]))
     dt = _dtype_code(layers[0][4]) if layers else BF16
-    _check(lib().catq_ternary_infer_staged(arr, len(layers), st, int(g), int(B), dt, _ptr(sync), _stream(stream)), w)
+    _check(lib().catq_ternary_infer_staged(arr, len(layers), st, int(g), int(B), dt, sy, _stream(stream)), w)
 
 
 def catq_schedule_at_epoch(e: int, m: int = 60, gamma: float = 0.8, s0: float = 30.0) -> catq_schedule:
@@ -496,13 +503,11 @@ def catq_factor_adamw_step(d_mu, d_alpha, d_delta, g_dmu, g_dalpha, g_ddelta, mo
     """One AdamW update of the factors [G] in place from their gradients; moments [6 * G]
     (zero before the first update) is the optimizer state."""
     G, w = d_mu.numel(), "catq_factor_adamw_step"
-    for name, arr in zip(("d_mu", "d_alpha", "d_delta", "g_dmu", "g_dalpha", "g_ddelta"),
-                         (d_mu, d_alpha, d_delta, g_dmu, g_dalpha, g_ddelta)):
-        _buf(arr, name, 4 * G, w)
-    _buf(moments, "moments", 4 * 6 * G, w)
-    _check(lib().catq_factor_adamw_step(d_mu.numel(), _ptr(d_mu), _ptr(d_alpha), _ptr(d_delta), _ptr(g_dmu),
-                                        _ptr(g_dalpha), _ptr(g_ddelta), _ptr(moments), ctypes.byref(hp), int(t),
-                                        float(lr), _stream(stream)), "catq_factor_adamw_step")
+    n = 4 * G
+    _check(lib().catq_factor_adamw_step(
+        G, _buf(d_mu, "d_mu", n, w), _buf(d_alpha, "d_alpha", n, w), _buf(d_delta, "d_delta", n, w),
+        _buf(g_dmu, "g_dmu", n, w), _buf(g_dalpha, "g_dalpha", n, w), _buf(g_ddelta, "g_ddelta", n, w),
+        _buf(moments, "moments", 6 * n, w), ctypes.byref(hp), int(t), float(lr), _stream(stream)), w)
 
 
 def catq_direct_adamw_step(d_alpha, d_delta, g_dalpha, g_ddelta, moments, hp: catq_adamw, t: int, lr: float,
@@ -518,9 +523,8 @@ def catq_direct_adamw_step(d_alpha, d_delta, g_dalpha, g_ddelta, moments, hp: ca
 
 def catq_group_recon_error(layer: Layer, err, stream=None):
     """err [G] = per-group mean of (W - Wq)^2 for the hard reconstruction."""
-    st = layer.struct()
-    _buf(err, "err", 4 * layer.G, "catq_group_recon_error")
-    _check(lib().catq_group_recon_error(ctypes.byref(st), _ptr(err), _stream(stream)), "catq_group_recon_error")
+    w = "catq_group_recon_error"
+    _check(lib().catq_group_recon_error(layer.packed(), _buf(err, "err", 4 * layer.G, w), _stream(stream)), w)
 
 
 def catq_selftest_wait_timeout(timeout_ns: int, stream=None):
@@ -552,177 +556,171 @@ class GroupedLayer:
     def E(self):
         return self.W.shape[0]
 
-    def struct(self) -> catq_grouped_layer:
+    def _fields(self):
         E, N, K = self.W.shape
         d = self.dense
-        d.struct()  # checks the stacked weights and the [E * G] per-group arrays
-        return catq_grouped_layer(E, self.g, N, K, _dtype_code(self.W), d.recon, self.W.data_ptr(), d.mu0.data_ptr(),
-                                  d.alpha0.data_ptr(), d.delta0.data_ptr(), d.d_mu.data_ptr(), d.d_alpha.data_ptr(),
-                                  d.d_delta.data_ptr(), d.op_const.data_ptr() if d.op_const is not None else None)
+        # the stacked weights and the [E * G] per-group arrays, checked as one dense layer
+        ptrs = d._addresses(*d.W.shape)
+        return (E, self.g, N, K, _dtype_code(self.W), d.recon, self.W.data_ptr()) + ptrs[1:]
+
+    def struct(self) -> catq_grouped_layer:
+        f = self._fields()
+        return catq_grouped_layer(*f[:-1], f[-1] or None)
+
+    def packed(self) -> bytes:
+        """struct() as bytes (what the calls below pass)."""
+        return _GROUPED.pack(*self._fields())
 
 
 def _offsets(row_offsets):
-    arr = (ctypes.c_int64 * len(row_offsets))(*[int(v) for v in row_offsets])
-    return arr
+    return struct.pack(f"{len(row_offsets)}q", *[int(v) for v in row_offsets])
 
 
 def _grouped_bufs(layer, row_offsets, where, X=None, Y=None, dY=None, dX=None, grads=()):
-    """The library reads E + 1 row offsets and rows 0 .. R-1 of the row-indexed arrays."""
+    """The library reads E + 1 row offsets and rows 0 .. R-1 of the row-indexed arrays: the checked
+    addresses of X, Y, dY, dX and the gradients."""
     E, N, K = layer.W.shape
     if len(row_offsets) != E + 1:
         raise ValueError(f"{where}: row_offsets has {len(row_offsets)} entries, the layer's {E} experts need {E + 1}")
     R = int(row_offsets[-1])
     e = X.element_size() if X is not None else 2
-    _buf(X, "X", R * K * e, where)
-    _buf(Y, "Y", R * N * e, where)
-    _buf(dY, "dY", R * N * e, where)
-    _buf(dX, "dX", R * K * e, where)
-    for name, arr in zip(("g_dmu", "g_dalpha", "g_ddelta"), grads):
-        _buf(arr, name, 4 * E * (N * K // layer.g), where)
+    return (_buf(X, "X", R * K * e, where), _buf(Y, "Y", R * N * e, where), _buf(dY, "dY", R * N * e, where),
+            _buf(dX, "dX", R * K * e, where)) + tuple(
+                _buf(arr, name, 4 * E * (N * K // layer.g), where)
+                for name, arr in zip(("g_dmu", "g_dalpha", "g_ddelta"), grads))
 
 
 def catq_grouped_soft_ternary_linear_fwd(layer: GroupedLayer, sched: catq_schedule, X, row_offsets, Y, stream=None):
-    st = layer.struct()
-    _grouped_bufs(layer, row_offsets, "catq_grouped_soft_ternary_linear_fwd", X=X, Y=Y)
-    off = _offsets(row_offsets)
-    _check(lib().catq_grouped_soft_ternary_linear_fwd(ctypes.byref(st), sched, _ptr(X), off, _dtype_code(X), _ptr(Y),
-                                                      _stream(stream)), "catq_grouped_soft_ternary_linear_fwd")
+    w = "catq_grouped_soft_ternary_linear_fwd"
+    st = layer.packed()
+    x, y, _, _ = _grouped_bufs(layer, row_offsets, w, X=X, Y=Y)
+    _check(lib().catq_grouped_soft_ternary_linear_fwd(st, sched, x, _offsets(row_offsets), _dtype_code(X), y,
+                                                      _stream(stream)), w)
 
 
 def catq_grouped_bwd_workspace_bytes(layer: GroupedLayer, row_offsets) -> int:
-    st = layer.struct()
+    st = layer.packed()
     _grouped_bufs(layer, row_offsets, "catq_grouped_bwd_workspace_bytes")
-    return int(lib().catq_grouped_bwd_workspace_bytes(ctypes.byref(st), _offsets(row_offsets)))
+    return int(lib().catq_grouped_bwd_workspace_bytes(st, _offsets(row_offsets)))
 
 
 def catq_grouped_soft_ternary_linear_bwd(layer: GroupedLayer, sched: catq_schedule, X, dY, row_offsets, dX=None,
                                          g_dmu=None, g_dalpha=None, g_ddelta=None, workspace=None, stream=None):
-    st = layer.struct()
-    _grouped_bufs(layer, row_offsets, "catq_grouped_soft_ternary_linear_bwd", X=X, dY=dY, dX=dX,
-                  grads=(g_dmu, g_dalpha, g_ddelta))
-    _buf(workspace, "workspace", 0, "catq_grouped_soft_ternary_linear_bwd")
-    ws_bytes = 0 if workspace is None else workspace.numel() * workspace.element_size()
-    _check(lib().catq_grouped_soft_ternary_linear_bwd(ctypes.byref(st), sched, _ptr(X), _ptr(dY),
-                                                      _offsets(row_offsets), _dtype_code(X), _ptr(dX), _ptr(g_dmu),
-                                                      _ptr(g_dalpha), _ptr(g_ddelta), _ptr(workspace), ws_bytes,
-                                                      _stream(stream)), "catq_grouped_soft_ternary_linear_bwd")
+    w = "catq_grouped_soft_ternary_linear_bwd"
+    st = layer.packed()
+    x, _, dy, dx, g0, g1, g2 = _grouped_bufs(layer, row_offsets, w, X=X, dY=dY, dX=dX,
+                                             grads=(g_dmu, g_dalpha, g_ddelta))
+    ws, ws_bytes = _ws(workspace, w)
+    _check(lib().catq_grouped_soft_ternary_linear_bwd(st, sched, x, dy, _offsets(row_offsets), _dtype_code(X), dx, g0,
+                                                      g1, g2, ws, ws_bytes, _stream(stream)), w)
 
 
 def catq_grouped_fwd_loss_workspace_bytes(layer: GroupedLayer, row_offsets) -> int:
-    st = layer.struct()
+    st = layer.packed()
     _grouped_bufs(layer, row_offsets, "catq_grouped_fwd_loss_workspace_bytes")
-    return int(lib().catq_grouped_fwd_loss_workspace_bytes(ctypes.byref(st), _offsets(row_offsets)))
+    return int(lib().catq_grouped_fwd_loss_workspace_bytes(st, _offsets(row_offsets)))
 
 
 def catq_grouped_soft_ternary_linear_fwd_loss(layer: GroupedLayer, sched: catq_schedule, X, row_offsets, Y_ref,
                                               loss_out, dY, Y=None, workspace=None, reduction: int = REDUCE_MEAN,
                                               stream=None):
-    st = layer.struct()
     w = "catq_grouped_soft_ternary_linear_fwd_loss"
-    _grouped_bufs(layer, row_offsets, w, X=X, Y=Y, dY=dY)
-    _grouped_bufs(layer, row_offsets, w, Y=Y_ref)
-    _buf(loss_out, "loss_out", 4, w)
-    _buf(workspace, "workspace", 0, w)
-    ws_bytes = 0 if workspace is None else workspace.numel() * workspace.element_size()
-    _check(lib().catq_grouped_soft_ternary_linear_fwd_loss(ctypes.byref(st), sched, _ptr(X), _offsets(row_offsets),
-                                                           _dtype_code(X), _ptr(Y_ref), int(reduction),
-                                                           _ptr(loss_out), _ptr(dY), _ptr(Y), _ptr(workspace),
-                                                           ws_bytes, _stream(stream)), w)
+    st = layer.packed()
+    x, y, dy, _ = _grouped_bufs(layer, row_offsets, w, X=X, Y=Y, dY=dY)
+    ref = _grouped_bufs(layer, row_offsets, w, Y=Y_ref)[1]
+    lo = _buf(loss_out, "loss_out", 4, w)
+    ws, ws_bytes = _ws(workspace, w)
+    _check(lib().catq_grouped_soft_ternary_linear_fwd_loss(st, sched, x, _offsets(row_offsets), _dtype_code(X), ref,
+                                                           int(reduction), lo, dy, y, ws, ws_bytes,
+                                                           _stream(stream)), w)
 
 
 # ------------------------------------------------------------------ decoder-block layers
 # bf16 activations [T, *] (tokens t = b S + s); fp32 gamma, r, lse, delta.
 
-def _bf16_bufs(where, nbytes, **bufs):
-    import torch
-    for name, t in bufs.items():
-        if t is not None and t.dtype != torch.bfloat16:
-            raise ValueError(f"{where}: {name} must be bfloat16")
-        _buf(t, name, nbytes, where)
+def _bf16(t, name: str, nbytes: int, where: str):
+    if t is not None and _known_dtype(t) != BF16:
+        raise ValueError(f"{where}: {name} must be bfloat16")
+    return _buf(t, name, nbytes, where)
+
+
+def _f32(t, name: str, nbytes: int, where: str):
+    if t is not None and _known_dtype(t) != F32:
+        raise ValueError(f"{where}: {name} must be float32")
+    return _buf(t, name, nbytes, where)
 
 
 def catq_rmsnorm_fwd(X, gamma, Z, r, eps, residual=None, h_out=None, stream=None):
     """Z = gamma * h / rms(h), h = X (+ residual, in fp32, stored into h_out); r [T] = 1 / rms(h).
     X bf16 or fp32; residual, Z bf16; h_out fp32."""
-    import torch
     T, H = X.shape
-    w = "catq_rmsnorm_fwd"
-    _buf(X, "X", T * H * X.element_size(), w)
-    _bf16_bufs(w, 2 * T * H, residual=residual, Z=Z)
-    if h_out is not None and h_out.dtype != torch.float32:
-        raise ValueError(f"{w}: h_out must be float32")
-    _buf(h_out, "h_out", 4 * T * H, w)
-    _buf(gamma, "gamma", 4 * H, w)
-    _buf(r, "r", 4 * T, w)
-    _check(lib().catq_rmsnorm_fwd(_ptr(X), _dtype_code(X), _ptr(residual), _ptr(gamma), T, H, float(eps),
-                                  _ptr(h_out), _ptr(Z), _ptr(r), _stream(stream)), w)
+    n, w = T * H, "catq_rmsnorm_fwd"
+    x = _buf(X, "X", n * X.element_size(), w)
+    res, z = _bf16(residual, "residual", 2 * n, w), _bf16(Z, "Z", 2 * n, w)
+    h = _f32(h_out, "h_out", 4 * n, w)
+    ga, rr = _buf(gamma, "gamma", 4 * H, w), _buf(r, "r", 4 * T, w)
+    _check(lib().catq_rmsnorm_fwd(x, _dtype_code(X), res, ga, T, H, float(eps), h, z, rr, _stream(stream)), w)
 
 
 def catq_rmsnorm_bwd(h, gamma, r, dZ, dX, dZ2=None, d_residual=None, stream=None):
     """dX of catq_rmsnorm_fwd at h (bf16 or fp32); dZ, dZ2, d_residual, dX bf16."""
     T, H = h.shape
-    w = "catq_rmsnorm_bwd"
-    _buf(h, "h", T * H * h.element_size(), w)
-    _bf16_bufs(w, 2 * T * H, dZ=dZ, dZ2=dZ2, d_residual=d_residual, dX=dX)
-    _buf(gamma, "gamma", 4 * H, w)
-    _buf(r, "r", 4 * T, w)
-    _check(lib().catq_rmsnorm_bwd(_ptr(h), _dtype_code(h), _ptr(gamma), _ptr(r), _ptr(dZ), _ptr(dZ2),
-                                  _ptr(d_residual), T, H, _ptr(dX), _stream(stream)), w)
+    n, w = T * H, "catq_rmsnorm_bwd"
+    hp = _buf(h, "h", n * h.element_size(), w)
+    dz, dz2 = _bf16(dZ, "dZ", 2 * n, w), _bf16(dZ2, "dZ2", 2 * n, w)
+    dr, dx = _bf16(d_residual, "d_residual", 2 * n, w), _bf16(dX, "dX", 2 * n, w)
+    ga, rr = _buf(gamma, "gamma", 4 * H, w), _buf(r, "r", 4 * T, w)
+    _check(lib().catq_rmsnorm_bwd(hp, _dtype_code(h), ga, rr, dz, dz2, dr, T, H, dx, _stream(stream)), w)
 
 
 def catq_rope(X, S, n_heads, d, base, inverse=False, stream=None):
     T = X.shape[0]
     w = "catq_rope"
-    _bf16_bufs(w, 2 * T * n_heads * d, X=X)
-    _check(lib().catq_rope(_ptr(X), T, int(S), int(n_heads), int(d), float(base), int(bool(inverse)),
-                           _stream(stream)), w)
+    x = _bf16(X, "X", 2 * T * n_heads * d, w)
+    _check(lib().catq_rope(x, T, int(S), int(n_heads), int(d), float(base), int(bool(inverse)), _stream(stream)), w)
 
 
 def catq_swiglu_fwd(gate, up, M, stream=None):
-    n = gate.numel()
-    _bf16_bufs("catq_swiglu_fwd", 2 * n, gate=gate, up=up, M=M)
-    _check(lib().catq_swiglu_fwd(_ptr(gate), _ptr(up), n, _ptr(M), _stream(stream)), "catq_swiglu_fwd")
+    n, w = gate.numel(), "catq_swiglu_fwd"
+    a, b, m = _bf16(gate, "gate", 2 * n, w), _bf16(up, "up", 2 * n, w), _bf16(M, "M", 2 * n, w)
+    _check(lib().catq_swiglu_fwd(a, b, n, m, _stream(stream)), w)
 
 
 def catq_swiglu_bwd(gate, up, dM, d_gate, d_up, stream=None):
-    n = gate.numel()
-    _bf16_bufs("catq_swiglu_bwd", 2 * n, gate=gate, up=up, dM=dM, d_gate=d_gate, d_up=d_up)
-    _check(lib().catq_swiglu_bwd(_ptr(gate), _ptr(up), _ptr(dM), n, _ptr(d_gate), _ptr(d_up), _stream(stream)),
-           "catq_swiglu_bwd")
+    n, w = gate.numel(), "catq_swiglu_bwd"
+    a, b, m = _bf16(gate, "gate", 2 * n, w), _bf16(up, "up", 2 * n, w), _bf16(dM, "dM", 2 * n, w)
+    da, db = _bf16(d_gate, "d_gate", 2 * n, w), _bf16(d_up, "d_up", 2 * n, w)
+    _check(lib().catq_swiglu_bwd(a, b, m, n, da, db, _stream(stream)), w)
 
 
 def catq_block_output_loss(h, branch, out_ref=None, loss_out=None, d_out=None, out=None, workspace=None,
                            reduction: int = REDUCE_MEAN, stream=None):
     """out = h + branch in fp32; with out_ref, Eq. 7's loss into loss_out and d_out (bf16)."""
-    import torch
     n, w = h.numel(), "catq_block_output_loss"
-    for name, t in (("h", h), ("out_ref", out_ref), ("out", out)):
-        if t is not None and t.dtype != torch.float32:
-            raise ValueError(f"{w}: {name} must be float32")
-        _buf(t, name, 4 * n, w)
-    _bf16_bufs(w, 2 * n, branch=branch, d_out=d_out)
-    _buf(loss_out, "loss_out", 4, w)
-    _buf(workspace, "workspace", 0, w)
-    ws_bytes = 0 if workspace is None else workspace.numel() * workspace.element_size()
-    _check(lib().catq_block_output_loss(_ptr(h), _ptr(branch), n, _ptr(out_ref), int(reduction), _ptr(loss_out),
-                                        _ptr(d_out), _ptr(out), _ptr(workspace), ws_bytes, _stream(stream)), w)
+    hp, ref, o = _f32(h, "h", 4 * n, w), _f32(out_ref, "out_ref", 4 * n, w), _f32(out, "out", 4 * n, w)
+    br, do = _bf16(branch, "branch", 2 * n, w), _bf16(d_out, "d_out", 2 * n, w)
+    lo = _buf(loss_out, "loss_out", 4, w)
+    ws, ws_bytes = _ws(workspace, w)
+    _check(lib().catq_block_output_loss(hp, br, n, ref, int(reduction), lo, do, o, ws, ws_bytes, _stream(stream)), w)
 
 
 def catq_attention_fwd(Q, K, V, O, lse, B, S, n_heads, n_kv_heads, d, stream=None):
     w = "catq_attention_fwd"
-    _bf16_bufs(w, 2 * B * S * n_heads * d, Q=Q, O=O)
-    _bf16_bufs(w, 2 * B * S * n_kv_heads * d, K=K, V=V)
-    _buf(lse, "lse", 4 * B * n_heads * S, w)
-    _check(lib().catq_attention_fwd(_ptr(Q), _ptr(K), _ptr(V), int(B), int(S), int(n_heads), int(n_kv_heads),
-                                    int(d), _ptr(O), _ptr(lse), _stream(stream)), w)
+    nq, nk = 2 * B * S * n_heads * d, 2 * B * S * n_kv_heads * d
+    q, o = _bf16(Q, "Q", nq, w), _bf16(O, "O", nq, w)
+    k, v = _bf16(K, "K", nk, w), _bf16(V, "V", nk, w)
+    ls = _buf(lse, "lse", 4 * B * n_heads * S, w)
+    _check(lib().catq_attention_fwd(q, k, v, int(B), int(S), int(n_heads), int(n_kv_heads), int(d), o, ls,
+                                    _stream(stream)), w)
 
 
 def catq_attention_bwd(Q, K, V, O, dO, lse, delta, dQ, dK, dV, B, S, n_heads, n_kv_heads, d, stream=None):
     w = "catq_attention_bwd"
-    _bf16_bufs(w, 2 * B * S * n_heads * d, Q=Q, O=O, dO=dO, dQ=dQ)
-    _bf16_bufs(w, 2 * B * S * n_kv_heads * d, K=K, V=V, dK=dK, dV=dV)
-    _buf(lse, "lse", 4 * B * n_heads * S, w)
-    _buf(delta, "delta", 4 * B * n_heads * S, w)
-    _check(lib().catq_attention_bwd(_ptr(Q), _ptr(K), _ptr(V), _ptr(O), _ptr(dO), _ptr(lse), int(B), int(S),
-                                    int(n_heads), int(n_kv_heads), int(d), _ptr(delta), _ptr(dQ), _ptr(dK),
-                                    _ptr(dV), _stream(stream)), w)
+    nq, nk, ns = 2 * B * S * n_heads * d, 2 * B * S * n_kv_heads * d, 4 * B * n_heads * S
+    q, o = _bf16(Q, "Q", nq, w), _bf16(O, "O", nq, w)
+    do, dq = _bf16(dO, "dO", nq, w), _bf16(dQ, "dQ", nq, w)
+    k, v = _bf16(K, "K", nk, w), _bf16(V, "V", nk, w)
+    dk, dv = _bf16(dK, "dK", nk, w), _bf16(dV, "dV", nk, w)
+    ls, de = _buf(lse, "lse", ns, w), _buf(delta, "delta", ns, w)
+    _check(lib().catq_attention_bwd(q, k, v, o, do, ls, int(B), int(S), int(n_heads), int(n_kv_heads), int(d), de, dq,
+                                    dk, dv, _stream(stream)), w)
