@@ -2,19 +2,8 @@
 // block-output reconstruction step (§2.4, Eq. 7 over a window of one block): RMSNorm (with the
 // residual add fused into the forward, and the residual and second upstream gradient fused
 // into the backward; one CTA per long row, one warp per short row such as an attention head),
-// rotary position embedding, SwiGLU, the fp32 block output with the loss on it, and causal
-// grouped-query attention (forward, and a deterministic backward in two kernels).
-//
-// Attention with 128-wide heads over whole 128-token tiles runs on tcgen05 (attn_tc.cu); the
-// kernels here serve the other shapes (d = 64, or S a multiple of 64 only) on the tensor pipe
-// with mma.sync m16n8k16 (bf16 in, fp32 accumulate): blocks of 64 queries (four warps of 16) against blocks of 64 keys, which stream through two
-// shared-memory buffers by cp.async; an online softmax in fp32 with the probabilities fed back
-// as the A operand of P V straight from the score accumulators, and operand fragments read
-// from shared memory with ldmatrix (transposed where the contraction runs along rows).  The
-// backward recomputes the probabilities from the forward's log-sum-exp: one kernel per query
-// block accumulates dQ; one per key block accumulates dK and dV (32 queries per step) over
-// every query head that shares the key/value head, so no atomics are needed and the result is
-// deterministic.
+// rotary position embedding, SwiGLU, the fp32 block output with the loss on it, and the row sums
+// the attention backward needs.  The attention itself runs on tcgen05 (attn_tc.cu).
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -566,238 +555,11 @@ __global__ void __launch_bounds__(kRowThreads) block_output_loss_kernel(const fl
 }
 
 // ---------------------------------------------------------------- attention
-constexpr int kBlk = 64;          // queries / keys per block
-constexpr int kAttnThreads = 128; // four warps of 16 rows
-
-__device__ __forceinline__ void ldsm_x4(uint32_t addr, uint32_t& r0, uint32_t& r1, uint32_t& r2, uint32_t& r3) {
-  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
-               : "=r"(r0), "=r"(r1), "=r"(r2), "=r"(r3)
-               : "r"(addr));
-}
-__device__ __forceinline__ void ldsm_x4_t(uint32_t addr, uint32_t& r0, uint32_t& r1, uint32_t& r2, uint32_t& r3) {
-  asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];"
-               : "=r"(r0), "=r"(r1), "=r"(r2), "=r"(r3)
-               : "r"(addr));
-}
-__device__ __forceinline__ void mma_bf16_16816(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3,
-                                               uint32_t b0, uint32_t b1) {
-  asm volatile(
-      "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, "
-      "{%0, %1, %2, %3};"
-      : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-      : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
-}
-
-// A shared-memory tile of 64 rows x HD bf16, rows padded by 16 bytes (conflict-free ldmatrix).
-template <int HD>
-struct Tile {
-  static constexpr int kStride = HD + 8;  // elements per row
-  static constexpr int kBytes = kBlk * kStride * 2;
+struct DeltaArgs {
+  const uint16_t *o, *dO;
+  float* delta;
+  int32_t B, S, nh;
 };
-
-// Rows row0.. row0 + 63 of a [rows, ld] bf16 matrix, columns col0 .. col0 + HD - 1, into a tile.
-template <int HD>
-__device__ __forceinline__ void load_tile(uint16_t* tile, const uint16_t* src, int64_t row0, int64_t ld,
-                                          int64_t col0) {
-  constexpr int kChunks = kBlk * HD / 8;  // 16-byte chunks
-  for (int c = threadIdx.x; c < kChunks; c += kAttnThreads) {
-    const int r = c / (HD / 8), k = (c % (HD / 8)) * 8;
-    *reinterpret_cast<uint4*>(tile + r * Tile<HD>::kStride + k) =
-        *reinterpret_cast<const uint4*>(src + (row0 + r) * ld + col0 + k);
-  }
-}
-
-__device__ __forceinline__ void cp_async16(uint32_t dst, const void* src) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
-}
-__device__ __forceinline__ void cp_async4(uint32_t dst, const void* src) {
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst), "l"(src) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cp_async_wait() {
-  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
-}
-
-// load_tile through cp.async (16-byte copies that complete with the thread's next wait).
-template <int HD>
-__device__ __forceinline__ void load_tile_async(uint32_t tile, const uint16_t* src, int64_t row0, int64_t ld,
-                                                int64_t col0) {
-  constexpr int kChunks = kBlk * HD / 8;
-  for (int c = threadIdx.x; c < kChunks; c += kAttnThreads) {
-    const int r = c / (HD / 8), k = (c % (HD / 8)) * 8;
-    cp_async16(tile + static_cast<uint32_t>((r * Tile<HD>::kStride + k) * 2), src + (row0 + r) * ld + col0 + k);
-  }
-}
-
-// Address of the row that this lane supplies to an ldmatrix.x4 of a 16 x 16 fragment at
-// (row0, col0) of a tile: matrix m = lane / 8 covers rows + (m & 1) 8 when `row_from_bit0`
-// (A operands and transposed B operands), else + (m >> 1) 8 (B operands stored n-major), and
-// columns + the other bit times 8.
-template <int HD>
-__device__ __forceinline__ uint32_t frag_addr(uint32_t tile, int row0, int col0, bool row_from_bit0) {
-  const int lane = threadIdx.x & 31, m = lane >> 3, r = lane & 7;
-  const int dr = row_from_bit0 ? (m & 1) * 8 : (m >> 1) * 8;
-  const int dc = row_from_bit0 ? (m >> 1) * 8 : (m & 1) * 8;
-  return tile + static_cast<uint32_t>(((row0 + dr + r) * Tile<HD>::kStride + col0 + dc) * 2);
-}
-
-// Scores of this warp's 16 rows of A (tile rows a_row0..) against the 64 rows of B (an
-// n-major tile of keys), over HD columns: acc[n-tile 0..7][4].
-template <int HD>
-__device__ __forceinline__ void scores_16x64(float (&acc)[8][4], uint32_t a_tile, int a_row0, uint32_t b_tile) {
-#pragma unroll
-  for (int nt = 0; nt < 8; ++nt)
-#pragma unroll
-    for (int e = 0; e < 4; ++e) acc[nt][e] = 0.0f;
-#pragma unroll
-  for (int kk = 0; kk < HD / 16; ++kk) {
-    uint32_t a0, a1, a2, a3;
-    ldsm_x4(frag_addr<HD>(a_tile, a_row0, kk * 16, true), a0, a1, a2, a3);
-#pragma unroll
-    for (int p = 0; p < 4; ++p) {
-      uint32_t b0, b1, b2, b3;
-      ldsm_x4(frag_addr<HD>(b_tile, p * 16, kk * 16, false), b0, b1, b2, b3);
-      mma_bf16_16816(acc[2 * p], a0, a1, a2, a3, b0, b1);
-      mma_bf16_16816(acc[2 * p + 1], a0, a1, a2, a3, b2, b3);
-    }
-  }
-}
-
-// acc[d-tile 0 .. HD/8)[4] += P (16 x 64, as bf16 A fragments from fp32 values p[n-tile][4])
-// times the 64 x HD tile (rows = the contraction), read transposed.
-template <int HD>
-__device__ __forceinline__ void accum_pv(float (&acc)[HD / 8][4], const float (&p)[8][4], uint32_t v_tile) {
-#pragma unroll
-  for (int ks = 0; ks < 4; ++ks) {
-    const uint32_t a0 = pack_bf16x2(p[2 * ks][0], p[2 * ks][1]);
-    const uint32_t a1 = pack_bf16x2(p[2 * ks][2], p[2 * ks][3]);
-    const uint32_t a2 = pack_bf16x2(p[2 * ks + 1][0], p[2 * ks + 1][1]);
-    const uint32_t a3 = pack_bf16x2(p[2 * ks + 1][2], p[2 * ks + 1][3]);
-#pragma unroll
-    for (int dp = 0; dp < HD / 16; ++dp) {
-      uint32_t b0, b1, b2, b3;
-      ldsm_x4_t(frag_addr<HD>(v_tile, ks * 16, dp * 16, true), b0, b1, b2, b3);
-      mma_bf16_16816(acc[2 * dp], a0, a1, a2, a3, b0, b1);
-      mma_bf16_16816(acc[2 * dp + 1], a0, a1, a2, a3, b2, b3);
-    }
-  }
-}
-
-struct AttnArgs {
-  const uint16_t *q, *k, *v, *o, *dO;
-  uint16_t *out, *dq, *dk, *dv;
-  float *lse, *delta;
-  int32_t B, S, nh, nkv;
-  float scale_log2;  // log2(e) / sqrt(d)
-  float scale;       // 1 / sqrt(d)
-};
-
-// Forward: one CTA per (query block, head, sequence).  Rows g and g + 8 of the warp's 16 are
-// the thread's (lane / 4); its columns within each 8-wide n-tile are 2 (lane % 4) + {0, 1}.
-// Key/value blocks stream through two shared-memory buffers: block kb + 1's copies are in
-// flight while block kb is computed.
-template <int HD>
-__global__ void __launch_bounds__(kAttnThreads) attn_fwd_kernel(const AttnArgs a) {
-  extern __shared__ __align__(16) uint8_t smem[];
-  uint16_t* Qs = reinterpret_cast<uint16_t*>(smem);
-  const uint32_t qa = smem_u32(Qs);
-  const uint32_t kv0 = qa + Tile<HD>::kBytes;  // buffer b: K at kv0 + 2 b tile, V after it
-  const int nqb = a.S / kBlk;
-  const int qb = nqb - 1 - static_cast<int>(blockIdx.x);  // the longest rows first
-  const int h = blockIdx.y, b = blockIdx.z, hk = h / (a.nh / a.nkv);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t4 = lane & 3;
-  const int64_t tok0 = static_cast<int64_t>(b) * a.S;
-  const int64_t ldq = static_cast<int64_t>(a.nh) * HD, ldk = static_cast<int64_t>(a.nkv) * HD;
-  auto load_kv = [&](int kb) {
-    const uint32_t kt = kv0 + static_cast<uint32_t>((kb & 1) * 2 * Tile<HD>::kBytes);
-    load_tile_async<HD>(kt, a.k, tok0 + kb * kBlk, ldk, static_cast<int64_t>(hk) * HD);
-    load_tile_async<HD>(kt + Tile<HD>::kBytes, a.v, tok0 + kb * kBlk, ldk, static_cast<int64_t>(hk) * HD);
-  };
-  load_tile_async<HD>(qa, a.q, tok0 + qb * kBlk, ldq, static_cast<int64_t>(h) * HD);
-  load_kv(0);
-  cp_async_commit();
-  float o[HD / 8][4];
-#pragma unroll
-  for (int i = 0; i < HD / 8; ++i)
-#pragma unroll
-    for (int e = 0; e < 4; ++e) o[i][e] = 0.0f;
-  float mrow[2] = {-INFINITY, -INFINITY}, lrow[2] = {0.0f, 0.0f};
-  for (int kb = 0; kb <= qb; ++kb) {
-    if (kb < qb) {
-      load_kv(kb + 1);
-      cp_async_commit();
-      cp_async_wait<1>();
-    } else {
-      cp_async_wait<0>();
-    }
-    __syncthreads();
-    const uint32_t ka = kv0 + static_cast<uint32_t>((kb & 1) * 2 * Tile<HD>::kBytes), va = ka + Tile<HD>::kBytes;
-    float s[8][4];
-    scores_16x64<HD>(s, qa, warp * 16, ka);
-    float mx[2] = {-INFINITY, -INFINITY};
-#pragma unroll
-    for (int nt = 0; nt < 8; ++nt)
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        float v = s[nt][e] * a.scale_log2;
-        if (kb == qb) {
-          const int key = nt * 8 + 2 * t4 + (e & 1), qry = warp * 16 + g + (e >> 1) * 8;
-          if (key > qry) v = -INFINITY;
-        }
-        s[nt][e] = v;
-        mx[e >> 1] = fmaxf(mx[e >> 1], v);
-      }
-#pragma unroll
-    for (int i = 0; i < 2; ++i) {
-      mx[i] = fmaxf(mx[i], __shfl_xor_sync(0xffffffffu, mx[i], 1));
-      mx[i] = fmaxf(mx[i], __shfl_xor_sync(0xffffffffu, mx[i], 2));
-    }
-    float corr[2], ls[2] = {0.0f, 0.0f};
-#pragma unroll
-    for (int i = 0; i < 2; ++i) {
-      const float mn = fmaxf(mrow[i], mx[i]);
-      corr[i] = mrow[i] == -INFINITY ? 0.0f : exp2f(mrow[i] - mn);
-      mrow[i] = mn;
-    }
-#pragma unroll
-    for (int nt = 0; nt < 8; ++nt)
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        const float p = exp2f(s[nt][e] - mrow[e >> 1]);
-        s[nt][e] = p;
-        ls[e >> 1] += p;
-      }
-#pragma unroll
-    for (int i = 0; i < 2; ++i) lrow[i] = lrow[i] * corr[i] + ls[i];
-#pragma unroll
-    for (int dn = 0; dn < HD / 8; ++dn) {
-      o[dn][0] *= corr[0];
-      o[dn][1] *= corr[0];
-      o[dn][2] *= corr[1];
-      o[dn][3] *= corr[1];
-    }
-    accum_pv<HD>(o, s, va);
-    __syncthreads();  // buffer kb & 1 is refilled with block kb + 2 next
-  }
-#pragma unroll
-  for (int i = 0; i < 2; ++i) {
-    lrow[i] += __shfl_xor_sync(0xffffffffu, lrow[i], 1);
-    lrow[i] += __shfl_xor_sync(0xffffffffu, lrow[i], 2);
-  }
-  const float inv[2] = {1.0f / lrow[0], 1.0f / lrow[1]};
-#pragma unroll
-  for (int i = 0; i < 2; ++i) {
-    const int64_t tok = tok0 + qb * kBlk + warp * 16 + g + 8 * i;
-    uint16_t* orow = a.out + tok * ldq + static_cast<int64_t>(h) * HD;
-#pragma unroll
-    for (int dn = 0; dn < HD / 8; ++dn)
-      *reinterpret_cast<uint32_t*>(orow + dn * 8 + 2 * t4) = pack_bf16x2(o[dn][2 * i] * inv[i], o[dn][2 * i + 1] * inv[i]);
-    if (t4 == 0)  // natural log-sum-exp of the scaled scores
-      a.lse[(static_cast<int64_t>(b) * a.nh + h) * a.S + qb * kBlk + warp * 16 + g + 8 * i] =
-          (mrow[i] + log2f(lrow[i])) * 0.69314718055994531f;
-  }
-}
 
 // delta[b, h, s] = sum over the head's columns of dO * O.  HD / 8 lanes per row, each one
 // 16-byte vector of O and dO; a CTA takes as many consecutive tokens of one head as it has such
@@ -805,7 +567,7 @@ __global__ void __launch_bounds__(kAttnThreads) attn_fwd_kernel(const AttnArgs a
 // 134 MB of the 8B block's 4 x 2048 tokens in 25 us = 5.3 TB/s (a warp per row with 2-byte loads:
 // 64).
 template <int HD>
-__global__ void __launch_bounds__(kRowThreads) attn_delta_kernel(const AttnArgs a) {
+__global__ void __launch_bounds__(kRowThreads) attn_delta_kernel(const DeltaArgs a) {
   constexpr int kTeam = HD / 8, kTok = kRowThreads / kTeam;
   const int64_t blocks = static_cast<int64_t>(a.B) * (a.S / kTok) * a.nh;
   const int sub = threadIdx.x % kTeam, row = threadIdx.x / kTeam;
@@ -823,244 +585,11 @@ __global__ void __launch_bounds__(kRowThreads) attn_delta_kernel(const AttnArgs 
   }
 }
 
-// dQ: one CTA per (query block, head, sequence), over the key blocks up to the diagonal,
-// which stream through two buffers as in the forward.
-template <int HD>
-__global__ void __launch_bounds__(kAttnThreads) attn_bwd_dq_kernel(const AttnArgs a) {
-  extern __shared__ __align__(16) uint8_t smem[];
-  const uint32_t qa = smem_u32(smem), da = qa + Tile<HD>::kBytes;  // Q, dO
-  const uint32_t kv0 = da + Tile<HD>::kBytes;                       // buffer b: K, V at kv0 + 2 b tile
-  const int nqb = a.S / kBlk;
-  const int qb = nqb - 1 - static_cast<int>(blockIdx.x);
-  const int h = blockIdx.y, b = blockIdx.z, hk = h / (a.nh / a.nkv);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t4 = lane & 3;
-  const int64_t tok0 = static_cast<int64_t>(b) * a.S;
-  const int64_t ldq = static_cast<int64_t>(a.nh) * HD, ldk = static_cast<int64_t>(a.nkv) * HD;
-  auto load_kv = [&](int kb) {
-    const uint32_t kt = kv0 + static_cast<uint32_t>((kb & 1) * 2 * Tile<HD>::kBytes);
-    load_tile_async<HD>(kt, a.k, tok0 + kb * kBlk, ldk, static_cast<int64_t>(hk) * HD);
-    load_tile_async<HD>(kt + Tile<HD>::kBytes, a.v, tok0 + kb * kBlk, ldk, static_cast<int64_t>(hk) * HD);
-  };
-  load_tile_async<HD>(qa, a.q, tok0 + qb * kBlk, ldq, static_cast<int64_t>(h) * HD);
-  load_tile_async<HD>(da, a.dO, tok0 + qb * kBlk, ldq, static_cast<int64_t>(h) * HD);
-  load_kv(0);
-  cp_async_commit();
-  float lse2[2], dl[2];  // this thread's two rows: log-sum-exp in log2 units, and delta
-#pragma unroll
-  for (int i = 0; i < 2; ++i) {
-    const int64_t idx = (static_cast<int64_t>(b) * a.nh + h) * a.S + qb * kBlk + warp * 16 + g + 8 * i;
-    lse2[i] = a.lse[idx] * 1.4426950408889634f;
-    dl[i] = a.delta[idx];
-  }
-  float dq[HD / 8][4];
-#pragma unroll
-  for (int i = 0; i < HD / 8; ++i)
-#pragma unroll
-    for (int e = 0; e < 4; ++e) dq[i][e] = 0.0f;
-  for (int kb = 0; kb <= qb; ++kb) {
-    if (kb < qb) {
-      load_kv(kb + 1);
-      cp_async_commit();
-      cp_async_wait<1>();
-    } else {
-      cp_async_wait<0>();
-    }
-    __syncthreads();
-    const uint32_t ka = kv0 + static_cast<uint32_t>((kb & 1) * 2 * Tile<HD>::kBytes), va = ka + Tile<HD>::kBytes;
-    float s[8][4], dp[8][4];
-    scores_16x64<HD>(s, qa, warp * 16, ka);   // Q K^T
-    scores_16x64<HD>(dp, da, warp * 16, va);  // dO V^T
-#pragma unroll
-    for (int nt = 0; nt < 8; ++nt)
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        float p = exp2f(s[nt][e] * a.scale_log2 - lse2[e >> 1]);
-        if (kb == qb) {
-          const int key = nt * 8 + 2 * t4 + (e & 1), qry = warp * 16 + g + (e >> 1) * 8;
-          if (key > qry) p = 0.0f;
-        }
-        s[nt][e] = p * (dp[nt][e] - dl[e >> 1]);  // dS
-      }
-    accum_pv<HD>(dq, s, ka);  // dS K
-    __syncthreads();
-  }
-#pragma unroll
-  for (int i = 0; i < 2; ++i) {
-    const int64_t tok = tok0 + qb * kBlk + warp * 16 + g + 8 * i;
-    uint16_t* row = a.dq + tok * ldq + static_cast<int64_t>(h) * HD;
-#pragma unroll
-    for (int dn = 0; dn < HD / 8; ++dn)
-      *reinterpret_cast<uint32_t*>(row + dn * 8 + 2 * t4) = pack_bf16x2(dq[dn][2 * i] * a.scale, dq[dn][2 * i + 1] * a.scale);
-  }
-}
-
-// dK, dV: one CTA per (key block, key/value head, sequence), over every query head of the
-// group and the query blocks from the diagonal on (one stream of (head, query block) pairs
-// through two buffers of Q, dO and their rows' log-sum-exp and delta), 32 queries at a time.
-// Scores are formed transposed (keys as rows) so that P^T and dS^T feed the A operand from
-// registers.
-template <int HD>
-__global__ void __launch_bounds__(kAttnThreads) attn_bwd_dkdv_kernel(const AttnArgs a) {
-  extern __shared__ __align__(16) uint8_t smem[];
-  const uint32_t ka = smem_u32(smem), va = ka + Tile<HD>::kBytes;
-  const uint32_t qd0 = va + Tile<HD>::kBytes;  // buffer b: Q at qd0 + 2 b tile, dO after it
-  float* const lsd0 = reinterpret_cast<float*>(smem + 6 * Tile<HD>::kBytes);  // buffer b: lse [64], delta [64]
-  const int nqb = a.S / kBlk;
-  const int kb = static_cast<int>(blockIdx.x);  // the most query blocks first
-  const int hk = blockIdx.y, b = blockIdx.z, rep = a.nh / a.nkv;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t4 = lane & 3;
-  const int64_t tok0 = static_cast<int64_t>(b) * a.S;
-  const int64_t ldq = static_cast<int64_t>(a.nh) * HD, ldk = static_cast<int64_t>(a.nkv) * HD;
-  const int per_head = nqb - kb, n_it = rep * per_head;  // (head, query block) pairs
-  auto load_q = [&](int it) {
-    const int h = hk * rep + it / per_head, qb = kb + it % per_head;
-    const uint32_t qt = qd0 + static_cast<uint32_t>((it & 1) * 2 * Tile<HD>::kBytes);
-    load_tile_async<HD>(qt, a.q, tok0 + qb * kBlk, ldq, static_cast<int64_t>(h) * HD);
-    load_tile_async<HD>(qt + Tile<HD>::kBytes, a.dO, tok0 + qb * kBlk, ldq, static_cast<int64_t>(h) * HD);
-    if (threadIdx.x < kBlk) {
-      const int64_t idx = (static_cast<int64_t>(b) * a.nh + h) * a.S + qb * kBlk + threadIdx.x;
-      float* l = lsd0 + (it & 1) * 2 * kBlk;
-      cp_async4(smem_u32(l + threadIdx.x), a.lse + idx);
-      cp_async4(smem_u32(l + kBlk + threadIdx.x), a.delta + idx);
-    }
-  };
-  load_tile_async<HD>(ka, a.k, tok0 + kb * kBlk, ldk, static_cast<int64_t>(hk) * HD);
-  load_tile_async<HD>(va, a.v, tok0 + kb * kBlk, ldk, static_cast<int64_t>(hk) * HD);
-  load_q(0);
-  cp_async_commit();
-  float dk[HD / 8][4], dv[HD / 8][4];
-#pragma unroll
-  for (int i = 0; i < HD / 8; ++i)
-#pragma unroll
-    for (int e = 0; e < 4; ++e) dk[i][e] = dv[i][e] = 0.0f;
-  for (int it = 0; it < n_it; ++it) {
-    if (it + 1 < n_it) {
-      load_q(it + 1);
-      cp_async_commit();
-      cp_async_wait<1>();
-    } else {
-      cp_async_wait<0>();
-    }
-    __syncthreads();
-    const int qb = kb + it % per_head;
-    const uint32_t qa = qd0 + static_cast<uint32_t>((it & 1) * 2 * Tile<HD>::kBytes), da = qa + Tile<HD>::kBytes;
-    const float* lse_s = lsd0 + (it & 1) * 2 * kBlk;
-    const float* dl_s = lse_s + kBlk;
-#pragma unroll 1
-    for (int qs = 0; qs < kBlk / 32; ++qs) {
-      // S^T and dP^T of the warp's 16 keys against 32 queries: four n-tiles each
-      float st[4][4], dpt[4][4];
-#pragma unroll
-      for (int nt = 0; nt < 4; ++nt)
-#pragma unroll
-        for (int e = 0; e < 4; ++e) st[nt][e] = dpt[nt][e] = 0.0f;
-#pragma unroll
-      for (int kk = 0; kk < HD / 16; ++kk) {
-        uint32_t a0, a1, a2, a3, b0, b1, b2, b3;
-        ldsm_x4(frag_addr<HD>(ka, warp * 16, kk * 16, true), a0, a1, a2, a3);
-#pragma unroll
-        for (int hq = 0; hq < 2; ++hq) {
-          ldsm_x4(frag_addr<HD>(qa, qs * 32 + hq * 16, kk * 16, false), b0, b1, b2, b3);
-          mma_bf16_16816(st[2 * hq], a0, a1, a2, a3, b0, b1);
-          mma_bf16_16816(st[2 * hq + 1], a0, a1, a2, a3, b2, b3);
-        }
-        ldsm_x4(frag_addr<HD>(va, warp * 16, kk * 16, true), a0, a1, a2, a3);
-#pragma unroll
-        for (int hq = 0; hq < 2; ++hq) {
-          ldsm_x4(frag_addr<HD>(da, qs * 32 + hq * 16, kk * 16, false), b0, b1, b2, b3);
-          mma_bf16_16816(dpt[2 * hq], a0, a1, a2, a3, b0, b1);
-          mma_bf16_16816(dpt[2 * hq + 1], a0, a1, a2, a3, b2, b3);
-        }
-      }
-      uint32_t pk[2][4], sk[2][4];  // P^T and dS^T as bf16 A fragments, one per 16 queries
-#pragma unroll
-      for (int hq = 0; hq < 2; ++hq) {
-        float pt[2][4], dst[2][4];
-#pragma unroll
-        for (int j = 0; j < 2; ++j)
-#pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            const int nt = 2 * hq + j;
-            const int qry = qs * 32 + nt * 8 + 2 * t4 + (e & 1);  // within the query block
-            const int key = warp * 16 + g + (e >> 1) * 8;          // within the key block
-            float p = exp2f((st[nt][e] * a.scale - lse_s[qry]) * 1.4426950408889634f);
-            if (qb == kb && key > qry) p = 0.0f;
-            pt[j][e] = p;
-            dst[j][e] = p * (dpt[nt][e] - dl_s[qry]);
-          }
-        pk[hq][0] = pack_bf16x2(pt[0][0], pt[0][1]);
-        pk[hq][1] = pack_bf16x2(pt[0][2], pt[0][3]);
-        pk[hq][2] = pack_bf16x2(pt[1][0], pt[1][1]);
-        pk[hq][3] = pack_bf16x2(pt[1][2], pt[1][3]);
-        sk[hq][0] = pack_bf16x2(dst[0][0], dst[0][1]);
-        sk[hq][1] = pack_bf16x2(dst[0][2], dst[0][3]);
-        sk[hq][2] = pack_bf16x2(dst[1][0], dst[1][1]);
-        sk[hq][3] = pack_bf16x2(dst[1][2], dst[1][3]);
-      }
-      // dV += P^T dO and dK += dS^T Q over these 32 queries (two k-steps)
-#pragma unroll
-      for (int hq = 0; hq < 2; ++hq)
-#pragma unroll
-        for (int dp = 0; dp < HD / 16; ++dp) {
-          uint32_t b0, b1, b2, b3;
-          ldsm_x4_t(frag_addr<HD>(da, qs * 32 + hq * 16, dp * 16, true), b0, b1, b2, b3);
-          mma_bf16_16816(dv[2 * dp], pk[hq][0], pk[hq][1], pk[hq][2], pk[hq][3], b0, b1);
-          mma_bf16_16816(dv[2 * dp + 1], pk[hq][0], pk[hq][1], pk[hq][2], pk[hq][3], b2, b3);
-          ldsm_x4_t(frag_addr<HD>(qa, qs * 32 + hq * 16, dp * 16, true), b0, b1, b2, b3);
-          mma_bf16_16816(dk[2 * dp], sk[hq][0], sk[hq][1], sk[hq][2], sk[hq][3], b0, b1);
-          mma_bf16_16816(dk[2 * dp + 1], sk[hq][0], sk[hq][1], sk[hq][2], sk[hq][3], b2, b3);
-        }
-    }
-    __syncthreads();  // buffer it & 1 is refilled with pair it + 2 next
-  }
-#pragma unroll
-  for (int i = 0; i < 2; ++i) {
-    const int64_t tok = tok0 + kb * kBlk + warp * 16 + g + 8 * i;
-    uint16_t* krow = a.dk + tok * ldk + static_cast<int64_t>(hk) * HD;
-    uint16_t* vrow = a.dv + tok * ldk + static_cast<int64_t>(hk) * HD;
-#pragma unroll
-    for (int dn = 0; dn < HD / 8; ++dn) {
-      *reinterpret_cast<uint32_t*>(krow + dn * 8 + 2 * t4) = pack_bf16x2(dk[dn][2 * i] * a.scale, dk[dn][2 * i + 1] * a.scale);
-      *reinterpret_cast<uint32_t*>(vrow + dn * 8 + 2 * t4) = pack_bf16x2(dv[dn][2 * i], dv[dn][2 * i + 1]);
-    }
-  }
-}
-
 int elem_grid(int64_t n) {
   int64_t b = (n + kRowThreads - 1) / kRowThreads;
   if (b < 1) b = 1;
   if (b > 152 * 16) b = 152 * 16;
   return static_cast<int>(b);
-}
-
-template <int HD>
-cudaError_t attn_launch(const AttnArgs& a, bool backward, cudaStream_t st) {
-  const dim3 grid(static_cast<unsigned>(a.S / kBlk), static_cast<unsigned>(a.nh), static_cast<unsigned>(a.B));
-  if (!backward) {
-    const int smem = 5 * Tile<HD>::kBytes;
-    cudaError_t e = cudaFuncSetAttribute(attn_fwd_kernel<HD>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (e != cudaSuccess) return e;
-    attn_fwd_kernel<HD><<<grid, kAttnThreads, smem, st>>>(a);
-    return cudaGetLastError();
-  }
-  const int64_t rows = static_cast<int64_t>(a.B) * a.S * a.nh;
-  attn_delta_kernel<HD><<<elem_grid(rows * (HD / 8)), kRowThreads, 0, st>>>(a);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  // 128-wide heads over whole 128-token tiles: dQ and dK/dV on tcgen05 (attn_tc.cu)
-  if (attention_fwd_tc_supported(a.S, HD))
-    return launch_attention_bwd_tc(a.q, a.k, a.v, a.dO, a.lse, a.delta, a.dq, a.dk, a.dv, a.B, a.S, a.nh, a.nkv, st);
-  const int smem_q = 6 * Tile<HD>::kBytes;
-  e = cudaFuncSetAttribute(attn_bwd_dq_kernel<HD>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_q);
-  if (e != cudaSuccess) return e;
-  attn_bwd_dq_kernel<HD><<<grid, kAttnThreads, smem_q, st>>>(a);
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  const int smem_k = 6 * Tile<HD>::kBytes + 4 * kBlk * static_cast<int>(sizeof(float));
-  e = cudaFuncSetAttribute(attn_bwd_dkdv_kernel<HD>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_k);
-  if (e != cudaSuccess) return e;
-  const dim3 gk(static_cast<unsigned>(a.S / kBlk), static_cast<unsigned>(a.nkv), static_cast<unsigned>(a.B));
-  attn_bwd_dkdv_kernel<HD><<<gk, kAttnThreads, smem_k, st>>>(a);
-  return cudaGetLastError();
 }
 
 }  // namespace
@@ -1203,28 +732,16 @@ cudaError_t launch_block_output_loss(const float* h, const void* branch, const f
 
 cudaError_t launch_attention(const AttnIo& io, int32_t B, int32_t S, int32_t nh, int32_t nkv, int32_t d, bool backward,
                              cudaStream_t st) {
-  AttnArgs a{};
-  a.q = static_cast<const uint16_t*>(io.q);
-  a.k = static_cast<const uint16_t*>(io.k);
-  a.v = static_cast<const uint16_t*>(io.v);
-  a.o = static_cast<const uint16_t*>(io.o);
-  a.dO = static_cast<const uint16_t*>(io.dO);
-  a.out = static_cast<uint16_t*>(io.out);
-  a.dq = static_cast<uint16_t*>(io.dq);
-  a.dk = static_cast<uint16_t*>(io.dk);
-  a.dv = static_cast<uint16_t*>(io.dv);
-  a.lse = io.lse;
-  a.delta = io.delta;
-  a.B = B;
-  a.S = S;
-  a.nh = nh;
-  a.nkv = nkv;
-  a.scale = 1.0f / sqrtf(static_cast<float>(d));
-  a.scale_log2 = a.scale * 1.4426950408889634f;
-  // the forward of 128-wide heads over whole 128-token tiles runs on tcgen05 (attn_tc.cu)
-  if (!backward && attention_fwd_tc_supported(S, d))
-    return launch_attention_fwd_tc(io.q, io.k, io.v, io.out, io.lse, B, S, nh, nkv, st);
-  return d == 128 ? attn_launch<128>(a, backward, st) : attn_launch<64>(a, backward, st);
+  if (!backward) return launch_attention_fwd_tc(io.q, io.k, io.v, io.out, io.lse, B, S, nh, nkv, d, st);
+  const DeltaArgs a{static_cast<const uint16_t*>(io.o), static_cast<const uint16_t*>(io.dO), io.delta, B, S, nh};
+  const int64_t rows = static_cast<int64_t>(B) * S * nh;
+  if (d == 128)
+    attn_delta_kernel<128><<<elem_grid(rows * 16), kRowThreads, 0, st>>>(a);
+  else
+    attn_delta_kernel<64><<<elem_grid(rows * 8), kRowThreads, 0, st>>>(a);
+  const cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return e;
+  return launch_attention_bwd_tc(io.q, io.k, io.v, io.dO, io.lse, io.delta, io.dq, io.dk, io.dv, B, S, nh, nkv, d, st);
 }
 
 }  // namespace catq

@@ -141,3 +141,31 @@ def test_linear_fp32_tiles(device, M, N, K, g, recon, phase, s):
     errs["loss"] = abs(got["loss"] - ref["loss"]) / ref["loss"]
     bad = {k: v for k, v in errs.items() if not v <= U.TOL_F32}
     assert not bad, (bad, errs)
+
+
+# Attention tiles of 128 tokens with a last one of 64, for both head widths: one tile, a half tile alone,
+# odd numbers of 64-token blocks, query heads in groups of 1, 2, 3 and 5; log-sum-exp and delta on
+# 4-byte alignment.  Two sequences, so that what lies past the first one's end is the second.  bf16
+# operands and probabilities: the bf16 bar.
+@pytest.mark.parametrize("S,nh,nkv,d", [(64, 3, 1, 64), (192, 2, 2, 64), (320, 5, 1, 128), (64, 2, 1, 128),
+                                        (448, 4, 2, 128), (128, 6, 2, 64), (832, 2, 1, 64)])
+def test_attention_ragged_tiles(device, S, nh, nkv, d):
+    import torch
+
+    from paper_2606_26650_gb300 import catq as C
+    B = 2
+    r = syn.rng(305, f"attn/{S}/{nh}/{d}")
+    q, k, v, do = (_bf16(r, (B * S, n * d)) for n in (nh, nkv, nkv, nh))
+    qd, kd, vd, dod = (U.to_device(t, "bf16", device) for t in (q, k, v, do))
+    o, dq, dk, dv = (torch.full_like(t, float("nan")) for t in (qd, qd, kd, vd))
+    rows = B * nh * S
+    lse = torch.zeros(rows + 1, dtype=torch.float32, device=device)[1:]
+    delta = torch.zeros(rows + 1, dtype=torch.float32, device=device)[1:]
+    C.catq_attention_fwd(qd, kd, vd, o, lse, B, S, nh, nkv, d)
+    C.catq_attention_bwd(qd, kd, vd, o, dod, lse, delta, dq, dk, dv, B, S, nh, nkv, d)
+    assert C.catq_device_status() == 0
+    o_ref, p = O.attention(q, k, v, B, S, nh, nkv, d)
+    dq_ref, dk_ref, dv_ref = (t.reshape(B * S, -1) for t in O.attention_bwd(q, k, v, p, do, B, S, nh, nkv, d))
+    assert np.abs(_f64(lse).reshape(B, nh, S) - O.attention_logsumexp(q, k, B, S, nh, nkv, d)).max() <= 1e-4
+    for name, got, want in (("o", o, o_ref.reshape(B * S, -1)), ("dq", dq, dq_ref), ("dk", dk, dk_ref), ("dv", dv, dv_ref)):
+        assert U.fro_rel(_f64(got), want) <= U.TOL_BF16, name
