@@ -26,21 +26,30 @@
 // its B rows are the activations of exactly those columns.
 //
 // A launch covers one or several layers (independent of each other).  Its work items are
-// blocks of 16 R rows of a layer; a persistent CTA of 8 warps takes every gridDim-th item and
-// streams their codes, in K slabs, through two shared-memory buffers by bulk copies, the next
-// slab (of this item or the next) on its way while the current one is computed.  The warps
-// split each slab into contiguous K ranges, and their partial sums meet in shared memory in a
-// fixed order (deterministic).  Token rows are taken 8 at a time (the MMA's N); all
-// arithmetic after the MMAs is fp32, with one rounding of Y.
+// blocks of 16 R rows of a layer; a persistent CTA of 8 computing and 2 copying warps takes every
+// gridDim-th item.  The copying warps stream the items' codes and group scales, in K slabs, through a
+// ring of shared-memory buffers (asynchronous 16-byte copies: bulk copies of one row each are issued
+// one after the other, 150 to 260 cycles a row), beside a few words on what the slab is, so that the
+// computing warps touch neither the layer table nor any weight in global memory.  Those split each
+// slab into contiguous K ranges, and their partial sums meet in shared memory in a fixed
+// order (deterministic), summed while the next item's products run.  Token rows are taken 8 at a
+// time (the MMA's N); all arithmetic after the MMAs is fp32, with one rounding of Y.
 //
 // A staged launch runs a chain of such layer sets in one cooperative launch (the layers of a
 // decode step in dependency order: stage s + 1 may read what stage s wrote).  The work items
 // of all stages form one stream; before its first item of a stage, a CTA arrives at the
 // barriers of the stages it is done with and waits (bounded) until every CTA has arrived at
-// the previous stage's.  The code slabs of the next items do not depend on earlier stages,
+// the previous stage's.  The weights of the next items do not depend on earlier stages,
 // so their copies are issued before the wait and the HBM stream does not drain at a stage
-// boundary.  Activations of a staged launch are read through L2 (ld.global.cg), since a
-// previous stage of the same launch may have written them.
+// boundary.
+//
+// What bounds it: the multiply-adds of a 128-column super-chunk (24 MMAs at 8 cycles and about 190
+// other instructions for 32 rows) run at some 70 % of the MMA rate while they run; a third of
+// the time goes to the ends of items, stages and launches.  Two 8B blocks (109 MB of codes, 18 us at the
+// HBM rate), as eight launches in a graph / one staged call (with scales fetched where they are
+// used and row-wise bulk copies, in parentheses): groups of 128, 1 token 80 us (84) / 96 (119), 8 tokens
+// 87 (94) / 101 (139); groups of 64 with offsets, 1 token 91 (108) / 101 (144).  Four 1.7B blocks, 6
+// tokens, groups of 64 with offsets, staged: 87 us (133).
 #include <algorithm>
 #include <cstdint>
 #include <type_traits>
@@ -51,7 +60,10 @@
 namespace catq {
 namespace {
 
-constexpr int kMmaWarps = 8;
+constexpr int kMmaWarps = 8;                       // computing warps
+constexpr int kCopyWarps = 2;                      // copying warps
+constexpr int kThreads = (kMmaWarps + kCopyWarps) * 32;
+constexpr int kMaxBufs = 4;                        // slab buffers
 constexpr uint32_t kMagic = 0x43004300u;  // bf16 128.0 in both halves
 
 // D += A B for one m16n8k16 tile (A row-major 16 x 16, B column-major 16 x 8, bf16).
@@ -101,6 +113,34 @@ __device__ __forceinline__ uint32_t code_pair(const Shifted& s) {
   return d;
 }
 
+// 16 or 4 bytes from global to shared memory, asynchronously (in this thread's open group of copies).
+__device__ __forceinline__ void copy16_async(uint32_t dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+}
+__device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
+__device__ __forceinline__ void copy4_async(uint32_t dst, const float* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst), "l"(src) : "memory");
+}
+// The thread's arrival at an mbarrier, once all its copies so far have landed.
+__device__ __forceinline__ void copies_arrive(uint32_t bar) {
+  asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(bar) : "memory");
+}
+__device__ __forceinline__ void copies_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
+// 32 bytes (aligned) of global memory.
+__device__ __forceinline__ void ld_global_32(const void* p, uint4& lo, uint4& hi) {
+  asm volatile("ld.global.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+               : "=r"(lo.x), "=r"(lo.y), "=r"(lo.z), "=r"(lo.w), "=r"(hi.x), "=r"(hi.y), "=r"(hi.z), "=r"(hi.w)
+               : "l"(p)
+               : "memory");
+}
+
+__device__ __forceinline__ float ld_shared_f32(uint32_t addr) {
+  float v;
+  asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(addr));
+  return v;
+}
+
 // An opaque copy of the magic constant (kept in a register instead of being folded into
 // each logic operation as a second immediate).
 __device__ __forceinline__ uint32_t magic_reg() {
@@ -136,13 +176,6 @@ __device__ __forceinline__ void word_mma(float (&d)[4], const Shifted& r0, const
             xb[2 * J], xb[2 * J + 1]);
 }
 
-// Bounded wait for copies already issued, used when a launch gives up.
-__device__ __forceinline__ void drain_wait(uint32_t bar, uint32_t parity) {
-  const uint64_t t0 = globaltimer_ns();
-  while (!mbar_try_wait(bar, parity))
-    if (globaltimer_ns() - t0 > 200000000ull) return;
-}
-
 // One layer of a launch: its buffers, shape and code slabs (KS columns per slab, nslabs per
 // token block), its group count per row, and its first work item.
 struct InferLayer {
@@ -155,6 +188,9 @@ struct InferLayer {
   int32_t gpr;     // groups per row, K / g
   int32_t KS;      // code columns per slab (a multiple of 64 VW)
   int32_t nslabs;  // slabs per token block
+  int32_t csh, ssh;  // log2 of the lanes that copy a row's codes, its scales
+  int32_t wide;    // scales per copy, 4 or 1
+  int32_t sld;     // row stride of a slab's scales in shared memory, words (4 times an odd number)
   int32_t item0;   // first work item of this layer
 };
 
@@ -171,9 +207,11 @@ struct InferArgs {
   InferLayer L[kMaxInferLayers];
 };
 
-// Staged launches: arrive at a stage barrier (after every thread's stores, by one thread).
-__device__ __forceinline__ void counter_arrive(uint32_t* ctr) {
-  asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(ctr) : "memory");
+// Staged launches: arrive at stage barriers from, ..., to - 1 (one thread, after a CTA barrier that
+// follows every thread's stores): one fence for all of them.
+__device__ __forceinline__ void counters_arrive(uint32_t* ctr, int32_t from, int32_t to) {
+  __threadfence();
+  for (int32_t b = from; b < to; ++b) asm volatile("red.relaxed.gpu.global.add.u32 [%0], 1;" ::"l"(ctr + b) : "memory");
 }
 
 __device__ __forceinline__ uint32_t counter_load(const uint32_t* ctr) {
@@ -188,7 +226,7 @@ __device__ __forceinline__ bool counter_wait(const uint32_t* ctr, uint32_t targe
   if (counter_load(ctr) >= target) return true;
   const uint64_t t0 = globaltimer_ns();
   for (;;) {
-    __nanosleep(128);
+    __nanosleep(20);
     if (counter_load(ctr) >= target) return true;
     if (aborted(w)) return false;
     if (globaltimer_ns() - t0 > w.timeout_ns) {
@@ -205,19 +243,13 @@ struct Cursor {
   int64_t b0;
 };
 
+// Move to item t, which lies in layer c.l or a later one.
 __device__ __forceinline__ void cursor_at(Cursor& c, int32_t t, const InferArgs& a) {
   c.t = t;
   c.slab = 0;
   c.b0 = 0;
-  c.l = 0;
   if (t >= a.total_items) return;
-  int lo = 0, hi = a.n_layers;  // last layer whose first item is <= t
-  while (hi - lo > 1) {
-    const int mid = (lo + hi) >> 1;
-    if (a.L[mid].item0 <= t) lo = mid;
-    else hi = mid;
-  }
-  c.l = lo;
+  while (c.l + 1 < a.n_layers && t >= a.L[c.l + 1].item0) ++c.l;
 }
 
 __device__ __forceinline__ void cursor_next(Cursor& c, const InferArgs& a) {
@@ -229,290 +261,446 @@ __device__ __forceinline__ void cursor_next(Cursor& c, const InferArgs& a) {
   cursor_at(c, c.t + static_cast<int32_t>(gridDim.x), a);
 }
 
+// What the computing warps need to know of a slab, written beside it by a copying warp: the layer's
+// parameters and the arithmetic on them cost each computing warp some 1,000 cycles an item.
+struct __align__(16) SlabInfo {
+  const uint16_t* X;  // the first token's activations of the slab's first column
+  uint16_t* Y;        // the first token's output of the item's first row
+  int32_t ldx, ldy;   // their row strides (K, N)
+  int32_t nb;         // token rows of the block, 1 .. 8
+  int32_t rows;       // output rows of the item
+  int32_t n_sc;       // super-chunks of the slab; 0: no slab, the stream has ended
+  int32_t row_bytes;  // row stride of its codes in shared memory
+  int32_t sld;        // row stride of its scales, bytes
+  int32_t sc0;        // super-chunks between the start of its first group and its first column
+  int32_t stage;
+  int32_t place;      // 1: the token block's first slab, 2: its last
+};
+static_assert(sizeof(SlabInfo) == 64, "read as four 16-byte words");
+
 // R: 16-row tiles per work item.  VW: code words per thread per super-chunk (a super-chunk is
 // 64 VW columns and lies in one group).  MU: add mu times each group's activation sum.
-// A persistent CTA walks its work items (over every layer of the launch) as one stream of
-// code slabs through two shared-memory buffers: once every warp has passed slab c + 1's
-// barrier (so slab c is consumed), warp 0 issues the bulk copies of slab c + 2 into slab c's
-// buffer, whichever item and layer it belongs to, so the next item's codes are on their way
-// while this one finishes its slabs and its reduction.  Each row's copy lands at a stride
-// padded by 16 VW bytes, so the fragment reads (four lanes per row, eight rows per
-// instruction) are free of bank conflicts.  Two CTA barriers per slab or item: the slab's
-// landing (which also frees the slab before it) and the partial sums' hand-over.
+// A persistent CTA of 8 computing and 2 copying warps walks its work items (over every layer of
+// the launch) as one stream of code slabs through `nbuf` shared-memory buffers: the copying warps
+// run ahead by that many slabs, whichever item, layer or stage they belong to, and the computing
+// warps only wait for a slab to land and hand it back.  Each row's copy lands at a stride padded by
+// 16 VW bytes, so the fragment reads (four lanes per row, eight rows per instruction) are free
+// of bank conflicts; its groups' scales (and offsets) land beside it, since fetched where they are
+// used each cost a trip to HBM.  One CTA barrier per work item: the partial sums' hand-over, in two
+// alternating arrays.
 template <int R, int VW, bool MU, bool STAGED>
-__global__ void __launch_bounds__(kMmaWarps * 32, 2) ternary_mma_kernel(const __grid_constant__ InferArgs a,
-                                                                     int32_t buf_bytes, const WaitCtl wc) {
+__global__ void __launch_bounds__(kThreads, 2) ternary_mma_kernel(const __grid_constant__ InferArgs a,
+                                                                 int32_t buf_bytes, int32_t nbuf, int32_t toks,
+                                                                 const WaitCtl wc) {
   constexpr int ROWS = 16 * R;
-  extern __shared__ __align__(128) uint8_t ring[];
-  __shared__ float red[kMmaWarps][8][ROWS];
-  __shared__ __align__(8) uint64_t full_bar[2];
+  constexpr int NX = VW == 1 ? 4 : 2;
+  constexpr int LDR = ROWS + 4;  // row stride of the partial sums: a warp's stores hit 32 banks
+  extern __shared__ __align__(128) uint8_t ring[];  // nbuf slab buffers, then red[2][kMmaWarps][toks][LDR]
+  __shared__ __align__(8) uint64_t bars[3 * kMaxBufs + 2];
+  __shared__ SlabInfo infos[kMaxBufs];
+  __shared__ SlabInfo handed[2];  // of the work items (token blocks) handed over
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int gid = lane >> 2, q = lane & 3;
   const uint32_t ring_base = smem_u32(ring);
-  const uint32_t bar0 = smem_u32(&full_bar[0]);
-  const int32_t sc_per_group = a.g / (64 * VW);
+  const uint32_t full = smem_u32(&bars[0]), empty = smem_u32(&bars[kMaxBufs]), info = smem_u32(&bars[2 * kMaxBufs]);
+  const uint32_t summed = smem_u32(&bars[3 * kMaxBufs]);
+  float* const red = reinterpret_cast<float*>(ring + nbuf * buf_bytes);
   if (threadIdx.x == 0) {
-    mbar_init(bar0, 1);
-    mbar_init(bar0 + 8, 1);
+    for (int i = 0; i < nbuf; ++i) {
+      mbar_init(info + 8 * i, 1);                // the slab's SlabInfo is written
+      mbar_init(full + 8 * i, 32 * kCopyWarps);  // the copying warps' lanes
+      mbar_init(empty + 8 * i, kMmaWarps);       // the computing warps
+    }
+    mbar_init(summed, kMmaWarps);
+    mbar_init(summed + 8, kMmaWarps);
     fence_mbar_init_cluster();
   }
-  __syncthreads();
-  const uint32_t magic = magic_reg();
-
-  // Warp 0 issues the bulk copies of the slab at cursor c into buffer `buf`.
-  auto issue = [&](const Cursor& c, int buf) {
-    const InferLayer& L = a.L[c.l];
-    const int64_t n0 = static_cast<int64_t>(c.t - L.item0) * ROWS;
-    const int64_t k0 = static_cast<int64_t>(c.slab) * L.KS;
-    const uint32_t bytes = static_cast<uint32_t>((L.K - k0 < L.KS ? L.K - k0 : L.KS) / 4);
-    const uint32_t row_bytes = static_cast<uint32_t>(L.KS / 4 + 16 * VW);
-    const int nvalid = static_cast<int>(L.N - n0 < ROWS ? L.N - n0 : ROWS);
-    const uint32_t bar = bar0 + 8u * buf;
-    if (lane == 0) mbar_arrive_expect_tx(bar, bytes * nvalid);
-    __syncwarp();
-    for (int r = lane; r < nvalid; r += 32)
-      bulk_load_g2s(ring_base + buf * buf_bytes + r * row_bytes, L.codes + (n0 + r) * (L.K / 4) + k0 / 4, bytes,
-                    bar);
-  };
-
   // The next kernel of the stream may launch now (it waits for this one before it touches
-  // anything this one writes).  The codes, scales and offsets are weights that inference
-  // never writes, so the first slabs' copies go out before waiting for the previous kernel,
-  // whose output may be this launch's X (or whose input may alias this launch's Y).
+  // anything this one writes).
   grid_launch_dependents();
-  Cursor iss, con;
-  cursor_at(iss, blockIdx.x, a);
-  cursor_at(con, blockIdx.x, a);
-  uint32_t issued = 0;  // slabs issued (tracked by warp 0, which issues them)
-  if (warp == 0) {
-    for (int b = 0; b < 2 && iss.t < a.total_items; ++b) {
-      issue(iss, b);
-      cursor_next(iss, a);
-      ++issued;
+  __syncthreads();
+
+  if (warp >= kMmaWarps) {
+    // codes of the slab at c: 16-byte pieces, 1 << csh lanes a row
+    const int pw = warp - kMmaWarps;
+    auto codes = [&](const Cursor& c, uint32_t base, auto hint) {
+      constexpr bool kHint = decltype(hint)::value;
+      const InferLayer& L = a.L[c.l];
+      const int64_t n0 = static_cast<int64_t>(c.t - L.item0) * ROWS;
+      const int32_t KS = L.KS, k0 = c.slab * KS, pieces = min(static_cast<int32_t>(L.K) - k0, KS) / 64;
+      const int32_t nvalid = static_cast<int32_t>(min(L.N - n0, static_cast<int64_t>(ROWS)));
+      const int32_t step = 1 << L.csh, rs = (kCopyWarps * 32) >> L.csh;
+      const int32_t r0 = (lane >> L.csh) * kCopyWarps + pw;
+      const int64_t ld = L.K / 4, row_step = rs * ld;
+      const uint32_t row_bytes = static_cast<uint32_t>(KS / 4 + 16 * VW), dst_step = rs * row_bytes;
+      const uint8_t* src = L.codes + (n0 + r0) * ld + k0 / 4;
+      const uint32_t dst = base + r0 * row_bytes;
+      for (int32_t j = lane & (step - 1); j < pieces; j += step) {
+        if (kHint && (j & 1) != 0) continue;  // 32-byte sectors
+        const uint8_t* p = src + 16 * j;
+        uint32_t d = dst + 16 * j;
+#pragma unroll 4
+        for (int32_t r = r0; r < nvalid; r += rs) {
+          if constexpr (kHint) prefetch_l2(p);
+          else copy16_async(d, p);
+          p += row_step;
+          d += dst_step;
+        }
+      }
+    };
+    // the scales (and offsets) of the groups it touches, 1 << ssh lanes a row: 16-byte pieces where every
+    // row's start on such a boundary, otherwise 4-byte pieces
+    struct Scales {
+      const float *alpha, *mu;  // of the lane's first row
+      uint32_t dst;
+      int32_t ng, nvalid, r0, rs, src_step, j0, j_step, wide, sld;
+    };
+    auto scales_of = [&](const Cursor& c, uint32_t base) {
+      const InferLayer& L = a.L[c.l];
+      const int64_t n0 = static_cast<int64_t>(c.t - L.item0) * ROWS;
+      const int32_t KS = L.KS, k0 = c.slab * KS, cols = min(static_cast<int32_t>(L.K) - k0, KS);
+      Scales f;
+      const int32_t g0 = k0 / a.g;
+      f.ng = (k0 + cols - 1) / a.g + 1 - g0;
+      f.nvalid = static_cast<int32_t>(min(L.N - n0, static_cast<int64_t>(ROWS)));
+      f.wide = L.wide;
+      f.sld = L.sld;
+      f.rs = (kCopyWarps * 32) >> L.ssh;
+      f.r0 = (lane >> L.ssh) * kCopyWarps + pw;
+      f.j0 = (lane & ((1 << L.ssh) - 1)) * f.wide;
+      f.j_step = f.wide << L.ssh;
+      f.src_step = f.rs * L.gpr;
+      const int64_t src = (n0 + f.r0) * L.gpr + g0;
+      f.alpha = L.alpha + src;
+      f.mu = MU ? L.mu + src : nullptr;
+      f.dst = base + ROWS * static_cast<uint32_t>(KS / 4 + 16 * VW) + f.r0 * f.sld * 4;
+      return f;
+    };
+    auto scales = [&](const Scales& f, auto hint) {
+      constexpr bool kHint = decltype(hint)::value;
+      for (int32_t j = f.j0; j < f.ng; j += f.j_step) {
+        if (kHint && (j & 7) != 0 && j + f.wide < f.ng) continue;  // 32-byte sectors, wherever they start
+        const float* p = f.alpha + j;
+        const float* m = f.mu + j;
+        uint32_t d = f.dst + 4 * j;
+#pragma unroll 4
+        for (int32_t r = f.r0; r < f.nvalid; r += f.rs) {
+          if constexpr (kHint) {
+            prefetch_l2(p);
+            if constexpr (MU) prefetch_l2(m);
+          } else if (f.wide == 4) {
+            copy16_async(d, p);
+            if constexpr (MU) copy16_async(d + ROWS * f.sld * 4, m);
+          } else {
+            copy4_async(d, p);
+            if constexpr (MU) copy4_async(d + ROWS * f.sld * 4, m);
+          }
+          p += f.src_step;
+          m += f.src_step;
+          d += f.rs * f.sld * 4;
+        }
+      }
+    };
+    int32_t stage = 0;
+    auto describe = [&](const Cursor& c, int slot) {
+      if (warp != kMmaWarps || lane != 0) return;
+      SlabInfo f{};
+      if (c.t < a.total_items) {
+        const InferLayer& L = a.L[c.l];
+        const int64_t n0 = static_cast<int64_t>(c.t - L.item0) * ROWS;
+        const int32_t k0 = c.slab * L.KS;
+        if constexpr (STAGED)
+          while (c.t >= a.stage_end[stage]) ++stage;
+        f.X = L.X + c.b0 * L.K + k0;
+        f.Y = L.Y + c.b0 * L.N + n0;
+        f.ldx = static_cast<int32_t>(L.K);
+        f.ldy = static_cast<int32_t>(L.N);
+        f.nb = static_cast<int32_t>(min(L.B - c.b0, static_cast<int64_t>(8)));
+        f.rows = static_cast<int32_t>(min(L.N - n0, static_cast<int64_t>(ROWS)));
+        f.n_sc = min(f.ldx - k0, L.KS) / (64 * VW);
+        f.row_bytes = L.KS / 4 + 16 * VW;
+        f.sld = L.sld * 4;
+        f.sc0 = a.g == 64 * VW ? 0 : k0 % a.g / (64 * VW);
+        f.stage = stage;
+        f.place = (c.slab == 0 ? 1 : 0) | (c.slab + 1 == L.nslabs ? 2 : 0);
+      }
+      infos[slot] = f;
+      mbar_arrive_local(info + 8 * slot);
+    };
+    constexpr std::false_type kCopy{};
+    constexpr std::true_type kAsk{};
+    // The codes are weights that inference never writes, so the first slab's copy goes out before
+    // waiting for the previous kernel (whose output may be this launch's X); its scales and the other
+    // buffers' slabs are on their way to L2 meanwhile.
+    Cursor c{};
+    cursor_at(c, blockIdx.x, a);
+    Scales first{};
+    const bool any = c.t < a.total_items;
+    if (any) {
+      codes(c, ring_base, kCopy);
+      first = scales_of(c, ring_base);
+      scales(first, kAsk);
+      describe(c, 0);
+      Cursor n = c;
+      cursor_next(n, a);
+      for (int i = 1; i < nbuf && n.t < a.total_items; ++i, cursor_next(n, a)) {
+        codes(n, 0, kAsk);
+        scales(scales_of(n, 0), kAsk);
+      }
     }
+    grid_dependency_wait();
+    int slot = 0;
+    uint32_t phase = 0;
+    if (any) {
+      scales(first, kCopy);
+      copies_arrive(full);
+      slot = 1;  // (at least two buffers)
+      cursor_next(c, a);
+    }
+    for (;;) {
+      // a buffer's first use needs no wait: the phase before a barrier's first counts as passed
+      if (!mbar_wait_warp(empty + 8 * slot, phase ^ 1u, wc)) break;
+      if (c.t >= a.total_items) {
+        describe(c, slot);
+        break;
+      }
+      const uint32_t base = ring_base + slot * buf_bytes;
+      codes(c, base, kCopy);
+      describe(c, slot);
+      scales(scales_of(c, base), kCopy);
+      copies_arrive(full + 8 * slot);
+      if (++slot == nbuf) {
+        slot = 0;
+        phase ^= 1u;
+      }
+      cursor_next(c, a);
+    }
+    copies_wait_all();
+    return;
   }
+
   grid_dependency_wait();
-  uint32_t qn = 0;  // slabs consumed
-  bool ok = true;
-  int32_t goff[R][2];
-  const uint16_t* xrow = nullptr;
-  float acc[R][4], d[R][4], da[4];
+  const int gid = lane >> 2, q = lane & 3;
+  const uint32_t magic = magic_reg();
+  const int32_t sc_per_group = a.g / (64 * VW);
+  int slot = 0;
+  uint32_t phase = 0;
+  float acc[R][4];
   int32_t stage = 0, arrived = 0;  // staged: stage of the current item, barriers arrived at
 
-  while (ok && con.t < a.total_items) {
-    if constexpr (STAGED) {
-      if (con.slab == 0 && con.b0 == 0) {
-        int32_t st = stage;
-        while (con.t >= a.stage_end[st]) ++st;
-        if (st > stage) {
-          // This CTA has no items left in stages before st (items run in order): its outputs
-          // there are stored.  Arrive at those stages' barriers, then wait until every CTA has
-          // arrived at stage st - 1's.
-          __syncthreads();
-          bool good = true;
-          if (threadIdx.x == 0) {
-            __threadfence();
-            for (int32_t b = arrived; b < st; ++b) counter_arrive(a.sync + b);
-            good = counter_wait(a.sync + (st - 1), gridDim.x, wc);
-          }
-          arrived = st;
-          stage = st;
-          if (!__syncthreads_and(good)) {
-            if (threadIdx.x == 0) {
-              // copies of this CTA's next slabs may be in flight
-              if (issued > qn) drain_wait(bar0 + 8u * (qn & 1u), (qn >> 1) & 1u);
-              if (issued > qn + 1) drain_wait(bar0 + 8u * ((qn + 1) & 1u), ((qn + 1) >> 1) & 1u);
-            }
-            __syncthreads();
-            ok = false;
-            break;
-          }
-        }
-      }
+  // Hand-overs: the warps' partial sums of a token block meet in shared memory, in a fixed order, and
+  // are summed and stored only when the next block's products are done (or the stream or the
+  // stage ends), so that no warp waits for the slowest one of the same block.  Two arrays suffice: a
+  // warp writes the one of two blocks before once it has seen every warp hand over the block before,
+  // which each did after its share of that sum.
+  uint32_t given = 0, taken = 0;  // token blocks handed over, summed
+  auto take = [&]() -> bool {
+    if (taken == given) return true;
+    const uint32_t p = taken & 1u;
+    if (!mbar_wait_warp(summed + 8 * p, (taken >> 1) & 1u, wc)) return false;
+    ++taken;
+    const SlabInfo& h = handed[p];
+    const float* const part = red + static_cast<int>(p) * kMmaWarps * toks * LDR;
+    const int row = threadIdx.x % ROWS;
+    for (int tok = threadIdx.x / ROWS; tok < h.nb; tok += kMmaWarps * 32 / ROWS) {
+      float s = 0.0f;
+#pragma unroll
+      for (int w = 0; w < kMmaWarps; ++w) s += part[(w * toks + tok) * LDR + row];
+      if (row < h.rows)
+        h.Y[static_cast<int64_t>(tok) * h.ldy + row] = static_cast<uint16_t>(pack_bf16x2(s, 0.0f) & 0xFFFFu);
     }
-    const InferLayer& L = a.L[con.l];
-    const int64_t n0 = static_cast<int64_t>(con.t - L.item0) * ROWS;
-    if (con.slab == 0) {
-      // a new token block of this item: group offsets of the thread's rows (rows past N take
-      // row N - 1's and are not stored), accumulators, and the activation row (token columns
-      // past B read token b0's activations: their sums are computed and never stored)
-#pragma unroll
-      for (int r = 0; r < R; ++r)
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          const int64_t n = n0 + 16 * r + gid + 8 * h;
-          goff[r][h] = static_cast<int32_t>((n < L.N ? n : L.N - 1) * L.gpr);
-        }
-      xrow = L.X + (con.b0 + gid < L.B ? con.b0 + gid : con.b0) * L.K;
-#pragma unroll
-      for (int r = 0; r < R; ++r)
-#pragma unroll
-        for (int e = 0; e < 4; ++e) acc[r][e] = d[r][e] = 0.0f;
-#pragma unroll
-      for (int e = 0; e < 4; ++e) da[e] = 0.0f;
-    }
-    const int buf = qn & 1;
-    const bool landed = mbar_wait(bar0 + 8u * buf, (qn >> 1) & 1u, wc);
-    if (!__syncthreads_and(landed)) {
-      // copies into this buffer, and the next slab's into the other, may still be in flight
-      if (threadIdx.x == 0) {
-        drain_wait(bar0 + 8u * buf, (qn >> 1) & 1u);
-        if (issued > qn + 1) drain_wait(bar0 + 8u * (buf ^ 1), ((qn + 1) >> 1) & 1u);
-      }
-      __syncthreads();
-      ok = false;
+    return true;
+  };
+
+  // Waits are bounded: a warp whose wait gives up tells the others at the CTA barrier that they reach
+  // next, whichever it is, and all leave (a warp waiting for its hand-over gives up too).
+  for (;;) {
+    if (!mbar_wait_warp(info + 8 * slot, phase, wc)) {
+      bar_all(1, kMmaWarps * 32, false);
       break;
     }
-    // Every warp is past this slab's barrier, so it is done with the slab before: that buffer
-    // takes the slab after this one (the first two went out at the start).
-    if (warp == 0 && issued < qn + 2 && iss.t < a.total_items) {
-      issue(iss, buf ^ 1);
-      cursor_next(iss, a);
-      ++issued;
+    const SlabInfo& f = infos[slot];
+    const int32_t n_sc = f.n_sc;
+    if (n_sc == 0) {
+      bar_all(1, kMmaWarps * 32, take());
+      break;
     }
-    {
-      // this warp's contiguous range of the slab's super-chunks, and the group it starts in
-      const int32_t sc_per_slab = L.KS / (64 * VW);
-      const int32_t k0 = con.slab * L.KS;
-      const int32_t n_sc = static_cast<int32_t>(((L.K - k0 < L.KS) ? L.K - k0 : L.KS) / (64 * VW));
-      const int32_t lo = n_sc * warp / kMmaWarps, hi = n_sc * (warp + 1) / kMmaWarps;
-      int32_t grp = (con.slab * sc_per_slab + lo) / sc_per_group;
-      int32_t left = (grp + 1) * sc_per_group - (con.slab * sc_per_slab + lo);  // super-chunks to its end
-      const uint32_t row_bytes = static_cast<uint32_t>(L.KS / 4 + 16 * VW);
-      const uint32_t tile = ring_base + buf * buf_bytes;
-      uint32_t rowa[R][2];  // shared-memory address of the thread's words in each of its rows
+    if constexpr (STAGED) {
+      const int32_t st = f.stage;
+      if (st > stage) {
+        // This CTA has no items left in stages before st (items run in order).  Store its last
+        // outputs there, arrive at those stages' barriers, then wait until every CTA has
+        // arrived at stage st - 1's.
+        if (!bar_all(1, kMmaWarps * 32, take())) break;
+        bool good = true;
+        if (threadIdx.x == 0) {
+          counters_arrive(a.sync, arrived, st);
+          good = counter_wait(a.sync + (st - 1), gridDim.x, wc);
+        }
+        arrived = st;
+        stage = st;
+        if (!bar_all(1, kMmaWarps * 32, good)) break;
+      }
+    }
+    // this warp's contiguous range of the slab's super-chunks, and its first activations (token columns
+    // past the block's rows read the first row's: their sums are computed and never stored, as are
+    // those of rows past the layer's last, whose codes and scales are whatever lay there)
+    const int32_t lo = n_sc * warp / kMmaWarps, hi = n_sc * (warp + 1) / kMmaWarps;
+    const int32_t nb = f.nb, place = f.place;
+    const uint4* const xbase =
+        reinterpret_cast<const uint4*>(f.X + static_cast<int64_t>(gid < nb ? gid : 0) * f.ldx + 16 * VW * q);
+    // (32 bytes at a time where X allows: half the passes through L1, which a load of eight token rows
+    // at 16 bytes a lane keeps busy; two 8B blocks, 8 tokens: 97 -> 87 us, staged 129 -> 101.  A staged
+    // launch's X may be an earlier stage's Y: plain loads, after the stage's acquire, or through L2 for
+    // a single token, whose row is not read twice: 96 -> 92.)
+    const bool x32 = (reinterpret_cast<uintptr_t>(xbase) & 31u) == 0 && (!STAGED || nb > 1);
+    auto load_x = [&](int32_t sc, uint4 (&xv)[2 * VW]) {
+      const uint4* xp = xbase + sc * (8 * VW);
+      if (x32) {
+#pragma unroll
+        for (int i = 0; i < VW; ++i) ld_global_32(xp + 2 * i, xv[2 * i], xv[2 * i + 1]);
+        return;
+      }
+#pragma unroll
+      for (int i = 0; i < 2 * VW; ++i) xv[i] = STAGED ? __ldcg(xp + i) : __ldg(xp + i);
+    };
+    uint4 xs[NX][2 * VW];  // activations, up to NX super-chunks ahead
+#pragma unroll
+    for (int j = 0; j < NX; ++j)
+      if (lo + j < hi) load_x(lo + j, xs[j]);
+    if (place & 1) {
 #pragma unroll
       for (int r = 0; r < R; ++r)
 #pragma unroll
-        for (int h = 0; h < 2; ++h) rowa[r][h] = tile + (16 * r + gid + 8 * h) * row_bytes + VW * q * 4;
-      const uint4* xbase = reinterpret_cast<const uint4*>(xrow + k0 + 16 * VW * q);
-      const bool every_sc = sc_per_group == 1;  // each super-chunk is a whole group
-      const float* alpha = L.alpha;
-      const float* mu = L.mu;
-      auto load_x = [&](int32_t sc, uint4 (&xv)[2 * VW]) {
-        const uint4* xp = xbase + sc * (8 * VW);
-#pragma unroll
-        for (int i = 0; i < 2 * VW; ++i) xv[i] = STAGED ? __ldcg(xp + i) : __ldg(xp + i);
-      };
-      // one super-chunk: this thread's code words from shared memory, its activations xv
-      auto step = [&](int32_t sc, const uint4 (&xv)[2 * VW]) {
-        const uint32_t woff = static_cast<uint32_t>(sc * 16 * VW);
-        // The group (or this warp's range) ends with this super-chunk: its scales (and offsets)
-        // are requested before the MMAs, which then cover their latency.
-        const bool ends = every_sc || left == 1 || sc + 1 == hi;
-        float av[R][2], mv[R][2];
-        if (ends) {
-#pragma unroll
-          for (int r = 0; r < R; ++r) {
-            av[r][0] = __ldg(alpha + goff[r][0] + grp);
-            av[r][1] = __ldg(alpha + goff[r][1] + grp);
-            if constexpr (MU) {
-              mv[r][0] = __ldg(mu + goff[r][0] + grp);
-              mv[r][1] = __ldg(mu + goff[r][1] + grp);
-            }
-          }
-        }
-        uint32_t cw[R][2][VW];  // the thread's code words of rows gid and gid + 8 of each tile
-#pragma unroll
-        for (int r = 0; r < R; ++r) {
-          ld_shared_words<VW>(rowa[r][0] + woff, cw[r][0]);
-          ld_shared_words<VW>(rowa[r][1] + woff, cw[r][1]);
-        }
-#pragma unroll
-        for (int v = 0; v < VW; ++v) {
-          uint32_t xb[8];
-          const uint4 h0 = xv[2 * v], h1 = xv[2 * v + 1];
-          xb[0] = act_pair<0>(h0, h1);
-          xb[1] = act_pair<1>(h0, h1);
-          xb[2] = act_pair<2>(h0, h1);
-          xb[3] = act_pair<3>(h0, h1);
-          xb[4] = act_pair<4>(h0, h1);
-          xb[5] = act_pair<5>(h0, h1);
-          xb[6] = act_pair<6>(h0, h1);
-          xb[7] = act_pair<7>(h0, h1);
-          // rows 0..7 of the constant tile: the correction sums; rows 8..15: activation sums
-          mma_16816(da, pos_corr(0), pos_unit(0), pos_corr(1), pos_unit(1), xb[0], xb[1]);
-          mma_16816(da, pos_corr(2), pos_unit(2), pos_corr(3), pos_unit(3), xb[2], xb[3]);
-          mma_16816(da, pos_corr(4), pos_unit(4), pos_corr(5), pos_unit(5), xb[4], xb[5]);
-          mma_16816(da, pos_corr(6), pos_unit(6), pos_corr(7), pos_unit(7), xb[6], xb[7]);
-#pragma unroll
-          for (int r = 0; r < R; ++r) {
-            const Shifted s0 = shifted(cw[r][0][v], magic), s1 = shifted(cw[r][1][v], magic);
-            word_mma<0>(d[r], s0, s1, xb);
-            word_mma<1>(d[r], s0, s1, xb);
-            word_mma<2>(d[r], s0, s1, xb);
-            word_mma<3>(d[r], s0, s1, xb);
-          }
-        }
-        if (ends) {
-#pragma unroll
-          for (int r = 0; r < R; ++r) {
-            acc[r][0] = fmaf(av[r][0], d[r][0] - da[0], acc[r][0]);
-            acc[r][1] = fmaf(av[r][0], d[r][1] - da[1], acc[r][1]);
-            acc[r][2] = fmaf(av[r][1], d[r][2] - da[0], acc[r][2]);
-            acc[r][3] = fmaf(av[r][1], d[r][3] - da[1], acc[r][3]);
-            if constexpr (MU) {
-              acc[r][0] = fmaf(mv[r][0], da[2], acc[r][0]);
-              acc[r][1] = fmaf(mv[r][0], da[3], acc[r][1]);
-              acc[r][2] = fmaf(mv[r][1], da[2], acc[r][2]);
-              acc[r][3] = fmaf(mv[r][1], da[3], acc[r][3]);
-            }
-#pragma unroll
-            for (int e = 0; e < 4; ++e) d[r][e] = 0.0f;
-          }
-#pragma unroll
-          for (int e = 0; e < 4; ++e) da[e] = 0.0f;
-        }
-        if (every_sc) {
-          ++grp;
-        } else if (--left == 0) {
-          ++grp;
-          left = sc_per_group;
-        }
-      };
-      // activations one super-chunk ahead, in two alternating register sets
-      uint4 xa[2 * VW], xc[2 * VW];
-      if (lo < hi) load_x(lo, xa);
-      for (int32_t sc = lo; sc < hi; sc += 2) {
-        if (sc + 1 < hi) load_x(sc + 1, xc);
-        step(sc, xa);
-        if (sc + 1 >= hi) break;
-        if (sc + 2 < hi) load_x(sc + 2, xa);
-        step(sc + 1, xc);
-      }
+        for (int e = 0; e < 4; ++e) acc[r][e] = 0.0f;
     }
-    ++qn;
-    if (con.slab + 1 == L.nslabs) {
-      // the token block's last slab: its partial sums meet in shared memory, in a fixed order
-      // D fragment: (row gid, tokens 2q, 2q + 1) and (row gid + 8, the same tokens)
+    const uint32_t row_bytes = static_cast<uint32_t>(f.row_bytes), sld = static_cast<uint32_t>(f.sld);
+    const uint32_t tile = ring_base + slot * buf_bytes;
+    // shared-memory address of the thread's words in row gid, and of that row's scale in the group
+    // that the warp's range starts in; the super-chunks to the group's end
+    const uint32_t rowa = tile + gid * row_bytes + VW * q * 4;
+    uint32_t scale = tile + ROWS * row_bytes + gid * sld;
+    int32_t left = 1;
+    if (sc_per_group == 1) {
+      scale += lo * 4;
+    } else {
+      const int32_t at = f.sc0 + lo, grp = at / sc_per_group;
+      left = (grp + 1) * sc_per_group - at;
+      scale += grp * 4;
+    }
+    if (!mbar_wait_warp(full + 8 * slot, phase, wc)) {
+      bar_all(1, kMmaWarps * 32, false);
+      break;
+    }
+    // one super-chunk: this thread's code words from shared memory, its activations xv
+    auto step = [&](int32_t sc, const uint4 (&xv)[2 * VW]) {
+      const uint32_t woff = static_cast<uint32_t>(sc * 16 * VW);
+      float d[R][4], da[4];
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        da[e] = 0.0f;
+#pragma unroll
+        for (int r = 0; r < R; ++r) d[r][e] = 0.0f;
+      }
+      uint32_t cw[R][2][VW];  // the thread's code words of rows gid and gid + 8 of each tile
 #pragma unroll
       for (int r = 0; r < R; ++r) {
-        red[warp][2 * q][16 * r + gid] = acc[r][0];
-        red[warp][2 * q + 1][16 * r + gid] = acc[r][1];
-        red[warp][2 * q][16 * r + gid + 8] = acc[r][2];
-        red[warp][2 * q + 1][16 * r + gid + 8] = acc[r][3];
+        ld_shared_words<VW>(rowa + (16 * r) * row_bytes + woff, cw[r][0]);
+        ld_shared_words<VW>(rowa + (16 * r + 8) * row_bytes + woff, cw[r][1]);
       }
-      __syncthreads();
-      for (int e = threadIdx.x; e < 8 * ROWS; e += kMmaWarps * 32) {
-        const int tok = e / ROWS, row = e % ROWS;
-        float s = 0.0f;
 #pragma unroll
-        for (int w = 0; w < kMmaWarps; ++w) s += red[w][tok][row];
-        if (con.b0 + tok < L.B && n0 + row < L.N)
-          L.Y[(con.b0 + tok) * L.N + n0 + row] = static_cast<uint16_t>(pack_bf16x2(s, 0.0f) & 0xFFFFu);
+      for (int v = 0; v < VW; ++v) {
+        uint32_t xb[8];
+        const uint4 h0 = xv[2 * v], h1 = xv[2 * v + 1];
+        xb[0] = act_pair<0>(h0, h1);
+        xb[1] = act_pair<1>(h0, h1);
+        xb[2] = act_pair<2>(h0, h1);
+        xb[3] = act_pair<3>(h0, h1);
+        xb[4] = act_pair<4>(h0, h1);
+        xb[5] = act_pair<5>(h0, h1);
+        xb[6] = act_pair<6>(h0, h1);
+        xb[7] = act_pair<7>(h0, h1);
+        // rows 0..7 of the constant tile: the correction sums; rows 8..15: activation sums
+        mma_16816(da, pos_corr(0), pos_unit(0), pos_corr(1), pos_unit(1), xb[0], xb[1]);
+        mma_16816(da, pos_corr(2), pos_unit(2), pos_corr(3), pos_unit(3), xb[2], xb[3]);
+        mma_16816(da, pos_corr(4), pos_unit(4), pos_corr(5), pos_unit(5), xb[4], xb[5]);
+        mma_16816(da, pos_corr(6), pos_unit(6), pos_corr(7), pos_unit(7), xb[6], xb[7]);
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+          const Shifted s0 = shifted(cw[r][0][v], magic), s1 = shifted(cw[r][1][v], magic);
+          word_mma<0>(d[r], s0, s1, xb);
+          word_mma<1>(d[r], s0, s1, xb);
+          word_mma<2>(d[r], s0, s1, xb);
+          word_mma<3>(d[r], s0, s1, xb);
+        }
       }
-      // red is written again only after the next slab's barrier, which every thread reaches
-      // after this loop
+      // a super-chunk lies in one group: scale (and offset) its sums
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        const float a0 = ld_shared_f32(scale + (16 * r) * sld);
+        const float a1 = ld_shared_f32(scale + (16 * r + 8) * sld);
+        acc[r][0] = fmaf(a0, d[r][0] - da[0], acc[r][0]);
+        acc[r][1] = fmaf(a0, d[r][1] - da[1], acc[r][1]);
+        acc[r][2] = fmaf(a1, d[r][2] - da[0], acc[r][2]);
+        acc[r][3] = fmaf(a1, d[r][3] - da[1], acc[r][3]);
+        if constexpr (MU) {
+          const float m0 = ld_shared_f32(scale + (ROWS + 16 * r) * sld);
+          const float m1 = ld_shared_f32(scale + (ROWS + 16 * r + 8) * sld);
+          acc[r][0] = fmaf(m0, da[2], acc[r][0]);
+          acc[r][1] = fmaf(m0, da[3], acc[r][1]);
+          acc[r][2] = fmaf(m1, da[2], acc[r][2]);
+          acc[r][3] = fmaf(m1, da[3], acc[r][3]);
+        }
+      }
+      if (--left == 0) {
+        scale += 4;
+        left = sc_per_group;
+      }
+    };
+    for (int32_t sc = lo; sc < hi; sc += NX) {
+#pragma unroll
+      for (int j = 0; j < NX; ++j) {
+        if (sc + j >= hi) break;
+        step(sc + j, xs[j]);
+        if (sc + j + NX < hi) load_x(sc + j + NX, xs[j]);
+      }
     }
-    cursor_next(con, a);
+    if (place & 2) {
+      // the token block's last slab: sum the block before, hand this one over
+      // D fragment: (row gid, tokens 2q, 2q + 1) and (row gid + 8, the same tokens)
+      if (!take()) {
+        bar_all(1, kMmaWarps * 32, false);
+        break;
+      }
+      const uint32_t p = given & 1u;
+      float* const part = red + (static_cast<int>(p) * kMmaWarps + warp) * toks * LDR;
+#pragma unroll
+      for (int e = 0; e < 2; ++e)
+        if (2 * q + e < nb) {
+          float* const to = part + (2 * q + e) * LDR + gid;
+#pragma unroll
+          for (int r = 0; r < R; ++r) {
+            to[16 * r] = acc[r][e];
+            to[16 * r + 8] = acc[r][2 + e];
+          }
+        }
+      if (threadIdx.x == 0) handed[p] = f;
+      __syncwarp();
+      if (lane == 0) mbar_arrive_local(summed + 8 * p);
+      ++given;
+    }
+    __syncwarp();
+    if (lane == 0) mbar_arrive_local(empty + 8 * slot);
+    if (++slot == nbuf) {
+      slot = 0;
+      phase ^= 1u;
+    }
   }
   if constexpr (STAGED) {
-    // Arrive at the barriers still owed, then leave; the last CTA to leave (every other one has
-    // passed all its waits by then) zeroes the counters for the next launch.
-    __syncthreads();
+    // Arrive at the barriers still owed (every thread's stores came before the last CTA barrier), then
+    // leave; the last CTA to leave (every other one has passed all its waits by then) zeroes the
+    // counters for the next launch.
     if (threadIdx.x == 0) {
-      __threadfence();
-      for (int32_t b = arrived; b < a.n_stages - 1; ++b) counter_arrive(a.sync + b);
+      counters_arrive(a.sync, arrived, a.n_stages - 1);
       const uint32_t prev = atomicAdd(a.sync + kMaxInferStages, 1u);
       if (prev == gridDim.x - 1) {
         for (int32_t b = 0; b < a.n_stages - 1; ++b) a.sync[b] = 0u;
@@ -523,20 +711,37 @@ __global__ void __launch_bounds__(kMmaWarps * 32, 2) ternary_mma_kernel(const __
   }
 }
 
-// One slab buffer: two per CTA plus the reduction array fit twice in an SM's shared memory.
-constexpr int64_t kBufBytes = 46 * 1024;
+// Dynamic shared memory of a CTA: half of an SM's, less its reserve and the static arrays.
+constexpr int64_t kDynBytes = 112 * 1024;
+// More than two slab buffers only up to this much of it: the rest caches activations (the layers of
+// two 8B blocks, 8 tokens, as one staged call: 121 us so, 141 us with a third buffer instead).
+constexpr int64_t kRingBytes = 80 * 1024;
 
-// Bytes of one slab buffer for KS columns: 16 R rows of codes, each padded by 16 VW bytes.
-int64_t slab_bytes(int64_t KS, int R, int VW) { return 16 * R * (KS / 4 + 16 * VW); }
+// log2 of the lanes that share n pieces of a row: the power of two up to a warp that covers them.
+int32_t lanes_log2(int64_t n) {
+  int32_t s = 0;
+  while (s < 5 && (int64_t(1) << s) < n) ++s;
+  return s;
+}
+
+// Row stride of a slab's scales, words: the groups that KS columns can touch, up to 4 times an odd
+// number, so that 16-byte copies fit and the eight rows that a warp reads lie in different banks.
+int64_t scale_stride(int64_t KS, int64_t g) { return (((KS % g == 0 ? KS / g : KS / g + 2) + 3) / 4 | 1) * 4; }
+
+// Bytes of one slab buffer for KS columns: 16 R rows of codes, each padded by 16 VW bytes, and their
+// groups' scales (and offsets).
+int64_t slab_bytes(int64_t KS, int R, int VW, int64_t g, bool mu) {
+  return 16 * R * (KS / 4 + 16 * VW + scale_stride(KS, g) * 4 * (mu ? 2 : 1));
+}
 
 // Code columns per slab for K: all of K when it fits one buffer, else the fewest equal slabs
 // (multiples of 64 VW columns) that do.
-int64_t slab_cols(int64_t K, int R, int VW) {
+int64_t slab_cols(int64_t K, int R, int VW, int64_t g, bool mu, int64_t cap) {
   const int64_t unit = 64 * VW;
-  if (slab_bytes(K, R, VW) <= kBufBytes) return K;
-  const int64_t cap = ((kBufBytes / (16 * R) - 16 * VW) * 4) / unit * unit;
-  const int64_t nslabs = (K + cap - 1) / cap;
-  return ((K + nslabs - 1) / nslabs + unit - 1) / unit * unit;
+  for (int64_t nslabs = 1;; ++nslabs) {
+    const int64_t KS = ((K + nslabs - 1) / nslabs + unit - 1) / unit * unit;
+    if (KS == unit || slab_bytes(KS, R, VW, g, mu) <= cap) return KS;
+  }
 }
 
 // stage_of (nullable): the stage of each layer (non-decreasing from 0 in steps of 1); sync: the
@@ -551,6 +756,9 @@ cudaError_t launch_mma(const InferDesc* ls, int n, int32_t g, bool with_mu, cons
   a.g = g;
   a.n_stages = stage_of ? stage_of[n - 1] + 1 : 1;
   a.sync = sync;
+  const int64_t toks = std::min<int64_t>(ls[0].B, 8);  // (the layers of a launch share B)
+  const int64_t red_bytes = 2 * kMmaWarps * toks * (16 * R + 4) * 4;
+  const int64_t cap = (kDynBytes - red_bytes) / 2 / 128 * 128;  // of a slab buffer
   int64_t items = 0, max_buf = 0;
   for (int i = 0; i < n; ++i) {
     InferLayer& L = a.L[i];
@@ -563,12 +771,17 @@ cudaError_t launch_mma(const InferDesc* ls, int n, int32_t g, bool with_mu, cons
     L.K = ls[i].K;
     L.B = ls[i].B;
     L.gpr = static_cast<int32_t>(ls[i].K / g);
-    const int64_t KS = slab_cols(L.K, R, VW);
+    const int64_t KS = slab_cols(L.K, R, VW, g, with_mu, cap);
     L.KS = static_cast<int32_t>(KS);
+    L.csh = lanes_log2(KS / 64);
+    const bool al16 = (reinterpret_cast<uintptr_t>(L.alpha) & 15u) == 0 && (reinterpret_cast<uintptr_t>(L.mu) & 15u) == 0;
+    L.wide = al16 && L.gpr % 4 == 0 && (KS >= L.K || KS % (4 * g) == 0) ? 4 : 1;
+    L.ssh = lanes_log2(((KS % g == 0 ? KS / g : KS / g + 2) + L.wide - 1) / L.wide);
+    L.sld = static_cast<int32_t>(scale_stride(KS, g));
     L.nslabs = static_cast<int32_t>((L.K + KS - 1) / KS);
     L.item0 = static_cast<int32_t>(items);
     items += (L.N + 16 * R - 1) / (16 * R);
-    max_buf = std::max<int64_t>(max_buf, slab_bytes(KS, R, VW));
+    max_buf = std::max<int64_t>(max_buf, slab_bytes(KS, R, VW, g, with_mu));
     if (stage_of) a.stage_end[stage_of[i]] = static_cast<int32_t>(std::min<int64_t>(items, INT32_MAX));
   }
   if (items >= (int64_t(1) << 31)) return cudaErrorInvalidValue;
@@ -579,7 +792,9 @@ cudaError_t launch_mma(const InferDesc* ls, int n, int32_t g, bool with_mu, cons
   for (int32_t s = 0, prev = 0; s < a.n_stages; prev = a.stage_end[s], ++s)
     widest = std::max<int64_t>(widest, a.stage_end[s] - prev);
   const int buf_bytes = static_cast<int>((max_buf + 127) / 128 * 128);
-  const int smem = 2 * buf_bytes;
+  const int nbuf = static_cast<int>(
+      std::max<int64_t>(2, std::min<int64_t>(kMaxBufs, (kRingBytes - red_bytes) / buf_bytes)));
+  const int smem = nbuf * buf_bytes + static_cast<int>(red_bytes);
   int sm = 152;
   int dev = 0;
   if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sm, cudaDevAttrMultiProcessorCount, dev);
@@ -595,7 +810,7 @@ cudaError_t launch_mma(const InferDesc* ls, int n, int32_t g, bool with_mu, cons
     // every CTA must be resident at once (they wait on each other): a cooperative launch of
     // at most the co-resident CTAs, and no more than the widest stage has items
     int per_sm = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kMmaWarps * 32, static_cast<size_t>(smem));
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kThreads, static_cast<size_t>(smem));
     if (e != cudaSuccess) return e;
     if (per_sm < 1) return cudaErrorInvalidConfiguration;
     blocks = std::min<int64_t>(widest, static_cast<int64_t>(per_sm) * sm);
@@ -608,12 +823,12 @@ cudaError_t launch_mma(const InferDesc* ls, int n, int32_t g, bool with_mu, cons
     attr[0].val.programmaticStreamSerializationAllowed = 1;
   }
   cfg.gridDim = dim3(static_cast<unsigned>(blocks));
-  cfg.blockDim = dim3(kMmaWarps * 32);
+  cfg.blockDim = dim3(kThreads);
   cfg.dynamicSmemBytes = static_cast<size_t>(smem);
   cfg.stream = st;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kern, a, buf_bytes, wc);
+  return cudaLaunchKernelEx(&cfg, kern, a, buf_bytes, nbuf, static_cast<int32_t>(toks), wc);
 }
 
 template <int R>

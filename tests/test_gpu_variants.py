@@ -169,3 +169,41 @@ def test_attention_ragged_tiles(device, S, nh, nkv, d):
     assert np.abs(_f64(lse).reshape(B, nh, S) - O.attention_logsumexp(q, k, B, S, nh, nkv, d)).max() <= 1e-4
     for name, got, want in (("o", o, o_ref.reshape(B * S, -1)), ("dq", dq, dq_ref), ("dk", dk, dk_ref), ("dv", dv, dv_ref)):
         assert U.fro_rel(_f64(got), want) <= U.TOL_BF16, name
+
+
+# Inference on packed codes: one super-chunk for eight warps, groups longer and shorter than a slab, several
+# slabs with a remainder, both item heights with remainders, two token blocks, scales and
+# activations at their least alignment (no 16-byte scale copies, no 32-byte activation loads).
+@pytest.mark.parametrize("N,K,g,B,mu,shift", [
+    (33, 64, 64, 1, False, 0), (40, 192, 192, 9, True, 1), (16, 20480, 256, 8, False, 0), (48, 24576, 24576, 3, True, 0),
+    (9744, 256, 128, 2, False, 1), (9744, 640, 64, 8, True, 0), (31, 17408, 128, 5, False, 1)])
+def test_ternary_infer_slabs(device, N, K, g, B, mu, shift):
+    import torch
+
+    from paper_2606_26650_gb300 import catq as C
+    r = syn.rng(306, f"infer/{N}/{K}/{g}")
+    c = r.integers(0, 3, (N * K // 4, 4)).astype(np.uint8)
+    packed = (c[:, 0] | c[:, 1] << 2 | c[:, 2] << 4 | c[:, 3] << 6).astype(np.uint8)
+    G = N * K // g
+    alpha = r.uniform(0.5, 1.5, G).astype(np.float32) / np.sqrt(K).astype(np.float32)
+    off = r.uniform(-0.1, 0.1, G).astype(np.float32) / np.sqrt(K).astype(np.float32) if mu else None
+    X = _bf16(r, (B, K))
+
+    def at(a, dtype, skip):  # on the device, `skip` elements into its buffer
+        buf = torch.zeros(a.size + skip, dtype=dtype, device=device)
+        buf[skip:] = torch.from_numpy(np.ascontiguousarray(a).reshape(-1)).to(device).to(dtype)
+        return buf[skip:].view(a.shape)
+
+    codes, al = at(packed, torch.uint8, 0), at(alpha, torch.float32, shift)
+    m = at(off, torch.float32, shift) if mu else None
+    x, y = at(X, torch.bfloat16, 8 * shift), torch.full((B, N), float("nan"), dtype=torch.bfloat16, device=device)
+    want = O.ternary_infer(packed, alpha, N, K, g, X, mu=off)
+    for _ in range(2):
+        C.catq_ternary_infer_batched([(codes, al, N, K, x, y, m)], g)
+        assert C.catq_device_status() == 0
+        assert U.fro_rel(_f64(y), want) <= U.TOL_BF16
+    sync = torch.zeros(C.catq_ternary_infer_sync_bytes() // 4, dtype=torch.int32, device=device)
+    y2 = torch.full_like(y, float("nan"))
+    C.catq_ternary_infer_staged([(codes, al, N, K, x, y, m), (codes, al, N, K, x, y2, m)], [0, 1], g, sync)
+    assert C.catq_device_status() == 0
+    assert torch.equal(y, y2) and not sync.any()
