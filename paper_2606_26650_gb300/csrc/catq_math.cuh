@@ -123,6 +123,33 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
   return d;
 }
 
+// Two fp32 values in one 64-bit register pair: one instruction for both (each result rounded as the
+// scalar instruction's).
+using f32x2 = uint64_t;
+__device__ __forceinline__ f32x2 pack_f32x2(float lo, float hi) {
+  f32x2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+  return r;
+}
+__device__ __forceinline__ void unpack_f32x2(f32x2 v, float& lo, float& hi) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+}
+__device__ __forceinline__ f32x2 fma_f32x2(f32x2 a, f32x2 b, f32x2 c) {
+  f32x2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+__device__ __forceinline__ f32x2 mul_f32x2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f32x2 add_f32x2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+
 // Per-row constants of the bf16 operand producer for one group.
 //   SOFT: u = s What = fma(w, A, B), D = s Delta, C = alpha / (2 tanh s);
 //         `one_tanh` when D >= 6: for u >= 0 the term tanh(u + D) >= tanh 6 = 1 - 1.2e-5 is
@@ -388,38 +415,81 @@ __device__ __forceinline__ float times_sign_of_neg(float a, float x) {
   return __int_as_float(__float_as_int(a) ^ (~__float_as_int(x) & 0x80000000));
 }
 
-// CLAMP caps the exponent at 126; a group needs it only when its largest exponent, c2 (at
-// x = 0), is above that.
-template <bool MU, bool SOFT, bool CLAMP>
-__device__ __forceinline__ void grad_element_logistic(float G, float w, const GroupConst& c, const OneExp& oe,
-                                                      LogiSums& acc, float inv_k) {
-  const float x = what(w, c);
-  float y = fmaf(fabsf(x), oe.c1, oe.c2);
-  if constexpr (CLAMP) y = fminf(y, 126.0f);
-  const float e = ex2_approx(y);
-  const float p = rcp_approx(fmaf(e, 0.5f, 0.5f));
-  const float a = G * (p * p * e);
-  acc.smu += MU ? fmaf(-G, inv_k, a) : a;
-  acc.sxs = fmaf(x, a, acc.sxs);
-  acc.st = fmaf(G, SOFT ? copysignf(p, x) : hard_q(x, c.delta), acc.st);
-  acc.sdelta += times_sign_of_neg(a, x);
+// LogiSums of the even and of the odd elements of a row.
+struct LogiSums2 {
+  f32x2 smu, st, sxs, sdelta;
+};
+__device__ __forceinline__ LogiSums logi_total(const LogiSums2& a) {
+  LogiSums t;
+  float lo, hi;
+  unpack_f32x2(a.smu, lo, hi);
+  t.smu = lo + hi;
+  unpack_f32x2(a.st, lo, hi);
+  t.st = lo + hi;
+  unpack_f32x2(a.sxs, lo, hi);
+  t.sxs = lo + hi;
+  unpack_f32x2(a.sdelta, lo, hi);
+  t.sdelta = lo + hi;
+  return t;
 }
 
-// 32 consecutive elements of one row: fp32 accumulator values g[0..31] and the bf16 weights
-// packed two per word in w[0..3].
+__device__ __forceinline__ LogiSums2 logi_add(const LogiSums2& a, const LogiSums& b) {
+  return LogiSums2{add_f32x2(a.smu, pack_f32x2(b.smu, 0.0f)), add_f32x2(a.st, pack_f32x2(b.st, 0.0f)),
+                   add_f32x2(a.sxs, pack_f32x2(b.sxs, 0.0f)), add_f32x2(a.sdelta, pack_f32x2(b.sdelta, 0.0f))};
+}
+
+// grad_element_onexp's form of two neighbouring elements, w2 their bf16 weights.  CLAMP caps the
+// exponent at 126; a group needs it only when its largest exponent, c2 (at x = 0), is above that.
 template <bool MU, bool SOFT, bool CLAMP>
-__device__ __forceinline__ void grad_chunk_logistic(const uint32_t (&g)[32], const uint4 (&w)[4], const GroupConst& c,
-                                                    const OneExp& oe, LogiSums& acc, float inv_k) {
+__device__ __forceinline__ void grad_pair_logistic(float g0, float g1, uint32_t w2, const GroupConst& c,
+                                                   const OneExp& oe, LogiSums2& acc, float inv_k) {
+  const f32x2 G = pack_f32x2(g0, g1);
+  const f32x2 x2 = fma_f32x2(pack_f32x2(bf16lo_to_f32(w2), bf16hi_to_f32(w2)), pack_f32x2(c.r, c.r),
+                             pack_f32x2(c.b, c.b));
+  float x0, x1;
+  unpack_f32x2(x2, x0, x1);
+  float y0 = fmaf(fabsf(x0), oe.c1, oe.c2), y1 = fmaf(fabsf(x1), oe.c1, oe.c2);
+  if constexpr (CLAMP) {
+    y0 = fminf(y0, 126.0f);
+    y1 = fminf(y1, 126.0f);
+  }
+  const f32x2 e2 = pack_f32x2(ex2_approx(y0), ex2_approx(y1)), half = pack_f32x2(0.5f, 0.5f);
+  float d0, d1;
+  unpack_f32x2(fma_f32x2(e2, half, half), d0, d1);
+  const float p0 = rcp_approx(d0), p1 = rcp_approx(d1);
+  const f32x2 p2 = pack_f32x2(p0, p1);
+  const f32x2 a2 = mul_f32x2(G, mul_f32x2(mul_f32x2(p2, p2), e2));
+  acc.smu = add_f32x2(acc.smu, MU ? fma_f32x2(G, pack_f32x2(-inv_k, -inv_k), a2) : a2);
+  acc.sxs = fma_f32x2(x2, a2, acc.sxs);
+  const f32x2 t2 = SOFT ? pack_f32x2(copysignf(p0, x0), copysignf(p1, x1))
+                        : pack_f32x2(hard_q(x0, c.delta), hard_q(x1, c.delta));
+  acc.st = fma_f32x2(G, t2, acc.st);
+  float a0, a1;
+  unpack_f32x2(a2, a0, a1);
+  acc.sdelta = add_f32x2(acc.sdelta, pack_f32x2(times_sign_of_neg(a0, x0), times_sign_of_neg(a1, x1)));
+}
+
+// 8 consecutive elements of one row: fp32 accumulator values g[at..at + 7] and the bf16 weights packed
+// two per word.
+template <bool MU, bool SOFT, bool CLAMP, int N>
+__device__ __forceinline__ void grad_eight_logistic(const uint32_t (&g)[N], int at, const uint4& w, const GroupConst& c,
+                                                    const OneExp& oe, LogiSums2& acc, float inv_k) {
+  const uint32_t w4[4] = {w.x, w.y, w.z, w.w};
 #pragma unroll
-  for (int v = 0; v < 4; ++v) {
-    const uint32_t w4[4] = {w[v].x, w[v].y, w[v].z, w[v].w};
+  for (int e = 0; e < 4; ++e)
+    grad_pair_logistic<MU, SOFT, CLAMP>(__uint_as_float(g[at + 2 * e]), __uint_as_float(g[at + 2 * e + 1]), w4[e], c, oe,
+                                        acc, inv_k);
+}
+
+// The same in the two-exponential form.
+template <bool MU, int N>
+__device__ __forceinline__ void grad_eight_sums(const uint32_t (&g)[N], int at, const uint4& w, const GroupConst& c,
+                                                float s, int32_t phase, LogiSums& acc, float inv_k) {
+  const uint32_t w4[4] = {w.x, w.y, w.z, w.w};
 #pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      grad_element_logistic<MU, SOFT, CLAMP>(__uint_as_float(g[8 * v + 2 * e]), bf16lo_to_f32(w4[e]), c, oe, acc,
-                                             inv_k);
-      grad_element_logistic<MU, SOFT, CLAMP>(__uint_as_float(g[8 * v + 2 * e + 1]), bf16hi_to_f32(w4[e]), c, oe,
-                                             acc, inv_k);
-    }
+  for (int e = 0; e < 4; ++e) {
+    grad_element_sums<MU>(__uint_as_float(g[at + 2 * e]), bf16lo_to_f32(w4[e]), c, s, phase, acc, inv_k);
+    grad_element_sums<MU>(__uint_as_float(g[at + 2 * e + 1]), bf16hi_to_f32(w4[e]), c, s, phase, acc, inv_k);
   }
 }
 

@@ -96,7 +96,8 @@ struct FusedCfg {
   static constexpr int kHold = (kStagesA < kStagesW ? kStagesA : kStagesW) - 1;
 };
 
-template <int CG>
+// GROUPED: the W tile of the epilogue comes through shared memory by TMA (see the epilogue).
+template <int CG, bool GROUPED>
 struct DwCfg {
   static constexpr int kRowsPerCta = 128;    // G rows (n) per CTA
   static constexpr int kTileRows = 128 * CG; // MMA M
@@ -104,11 +105,19 @@ struct DwCfg {
   static constexpr int kABytes = 128 * BK * 2;
   static constexpr int kBBytes = kBCols * BK * 2;
   static constexpr int kStageBytes = kABytes + kBBytes;
-  static constexpr int kStages = CG == 1 ? 4 : 6;
-  static constexpr int kEpiWarps = 8;        // two warps per TMEM lane quarter (column halves)
-  static constexpr int kThreads = 32 * (kEpiWarps + 2);
-  static constexpr int kBarBytes = 8 * (2 * kStages + 5) + 16;
-  static constexpr int kSmemBytes = kStages * kStageBytes + 1024 + kBarBytes;
+  static constexpr int kStages = GROUPED ? (CG == 1 ? 2 : 4) : (CG == 1 ? 4 : 6);
+  static constexpr int kWBox = 128 * 128;    // 64 columns of the CTA's 128 W rows, bytes
+  static constexpr int kWBoxes = GROUPED ? 4 : 0;
+  // two warps per TMEM lane quarter (column halves), four in a grouped launch (column quarters)
+  static constexpr int kEpiWarps = GROUPED ? 16 : 8;
+  static constexpr int kThreads = 32 * (kEpiWarps + 2 + (GROUPED ? 2 : 0));
+  static constexpr int kBarBytes = (8 * (2 * kStages + 5 + 2 * kWBoxes + (GROUPED ? 4 : 0)) + 16 + 15) / 16 * 16;
+  // sums that pairs of epilogue warps add up, two buffers
+  static constexpr int kPairBytes = GROUPED ? 2 * (kEpiWarps / 2) * 32 * 16 : 0;
+  // group constants of a tile's rows and boxes, and where the tile is, two buffers
+  static constexpr int kConstBytes = GROUPED ? 2 * (kWBoxes * 128 * 16 + 16) : 0;
+  static constexpr int kSmemBytes =
+      kStages * kStageBytes + kWBoxes * kWBox + 1024 + kBarBytes + kPairBytes + kConstBytes;
 };
 
 // Experts of one grouped launch (stacked expert weights, expert-sorted rows).
@@ -1303,24 +1312,32 @@ __global__ void wait_probe_kernel(const WaitCtl wc) {
 
 // ============================================================================ dW kernel
 
-// NE > 1: a grouped launch over gm's experts (tmDY, tmX unused).
+// NE > 1: a grouped launch over gm's experts (tmDY: the stacked W in boxes of 64 columns x 128 rows, tmX
+// unused).
 template <int CG, bool MU, int NE>
-__global__ void __launch_bounds__(DwCfg<CG>::kThreads, 1)
+__global__ void __launch_bounds__(DwCfg<CG, (NE > 1)>::kThreads, 1)
     dw_kernel(const __grid_constant__ CUtensorMap tmDY, const __grid_constant__ CUtensorMap tmX, const DwArgs args,
               const __grid_constant__ DwMaps<NE> gm) {
-  using Cfg = DwCfg<CG>;
+  constexpr bool GROUPED = NE > 1;
+  using Cfg = DwCfg<CG, GROUPED>;
   constexpr int S = Cfg::kStages;
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw_addr = smem_u32(smem_raw);
   const uint32_t base = (raw_addr + 1023u) & ~1023u;
   uint8_t* base_ptr = smem_raw + (base - raw_addr);
-  const uint32_t bars = base + S * Cfg::kStageBytes;
+  const uint32_t w_base = base + S * Cfg::kStageBytes;   // grouped: [kWBoxes][kWBox]
+  const uint32_t bars = w_base + Cfg::kWBoxes * Cfg::kWBox;
   auto full = [&](int s) { return bars + 8u * s; };
   auto empty = [&](int s) { return bars + 8u * (S + s); };
   const uint32_t tmem_full0 = bars + 8u * (2 * S);      // [2]
   const uint32_t tmem_empty0 = tmem_full0 + 16;         // [2]
   const uint32_t final_bar = tmem_full0 + 32;
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(base_ptr + (bars - base) + 8 * (2 * S + 5));
+  auto w_full = [&](int b) { return final_bar + 8u + 8u * b; };
+  auto w_empty = [&](int b) { return final_bar + 8u + 8u * (Cfg::kWBoxes + b); };
+  auto c_full = [&](int b) { return final_bar + 8u + 8u * (2 * Cfg::kWBoxes + b); };
+  auto c_empty = [&](int b) { return final_bar + 8u + 8u * (2 * Cfg::kWBoxes + 2 + b); };
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(base_ptr + (bars - base) +
+                                                    8 * (2 * S + 5 + 2 * Cfg::kWBoxes + (GROUPED ? 4 : 0)));
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t cta = CG == 2 ? cluster_ctarank() : 0u;
@@ -1353,6 +1370,15 @@ __global__ void __launch_bounds__(DwCfg<CG>::kThreads, 1)
       mbar_init(tmem_empty0 + 8u * b, Cfg::kEpiWarps * CG);
     }
     mbar_init(final_bar, 1);
+    for (int b = 0; b < Cfg::kWBoxes; ++b) {
+      mbar_init(w_full(b), 1);
+      mbar_init(w_empty(b), 4);  // the box's four row quarters
+    }
+    if constexpr (GROUPED)
+      for (int b = 0; b < 2; ++b) {
+        mbar_init(c_full(b), 1);
+        mbar_init(c_empty(b), Cfg::kEpiWarps);
+      }
     fence_mbar_init_cluster();
   }
   if (warp == kMma) tmem_alloc<CG>(smem_u32(tmem_slot), kTmemCols);
@@ -1454,11 +1480,199 @@ __global__ void __launch_bounds__(DwCfg<CG>::kThreads, 1)
       __syncwarp();
       mbar_wait_drain(final_bar, 0);
     }
+  } else if (GROUPED && warp == Cfg::kEpiWarps + 2) {
+    // ------------------------------------------------------------ TMA: the epilogue's W tiles (grouped)
+    if (lane == 0) {
+      const uint64_t pol_w = l2_policy_evict_first();  // W is read once per launch
+      uint32_t it = 0, issued = 0, issued_phase = 0;
+      bool ok = true;
+      for (int t = cluster; ok && t < num_tiles; t += nclusters, ++it) {
+        int k_blk, n_blk;
+        dw_tile(args, t % tiles_per_split, n_blk, k_blk);
+        const int32_t row = static_cast<int32_t>(gm.expert[t / tiles_per_split] * args.L.N) +
+                            n_blk * Cfg::kTileRows + static_cast<int32_t>(cta) * 128;
+        for (int b = 0; b < Cfg::kWBoxes; ++b) {
+          if (!mbar_wait(w_empty(b), (it & 1u) ^ 1u, wc)) { ok = false; break; }
+          mbar_arrive_expect_tx(w_full(b), Cfg::kWBox);
+          tma_load_2d_hint(w_base + b * Cfg::kWBox, &tmDY, w_full(b), k_blk * BN + 64 * b, row, pol_w);
+          issued |= 1u << b;
+          issued_phase = (issued_phase & ~(1u << b)) | ((it & 1u) << b);
+        }
+      }
+      for (int b = 0; b < Cfg::kWBoxes; ++b)
+        if (issued & (1u << b)) mbar_wait_drain(w_full(b), (issued_phase >> b) & 1u);
+    }
+  } else if (GROUPED && warp == Cfg::kEpiWarps + 3) {
+    // ------------------------------------------------------------ the epilogue's group constants (grouped)
+    // A tile ahead, once for all the warps that need them.
+    const bool paired = args.P == 128;
+    const LayerDev& L = args.L;
+    float4* const consts = reinterpret_cast<float4*>(base_ptr + (bars - base) + Cfg::kBarBytes + Cfg::kPairBytes);
+    int4* const where = reinterpret_cast<int4*>(consts + 2 * Cfg::kWBoxes * 128);
+    uint32_t it = 0;
+    for (int t = cluster; t < num_tiles; t += nclusters, ++it) {
+      const int buf = it & 1;
+      int k_blk, n_blk;
+      dw_tile(args, t % tiles_per_split, n_blk, k_blk);
+      const int64_t e = gm.expert[t / tiles_per_split];
+      const int64_t n0 = static_cast<int64_t>(n_blk) * Cfg::kTileRows + cta * 128 + lane;
+      const int32_t b_step = paired ? 2 : 1;
+      bool ok = true;
+#pragma unroll 1
+      for (int b0 = 0; ok && b0 < Cfg::kWBoxes; b0 += 2 * b_step) {  // two boxes' loads in flight
+        GroupRaw raw[2][4] = {};
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+          const uint32_t k = static_cast<uint32_t>(k_blk) * BN + 64 * (b0 + i * b_step);
+          const int64_t j0 = (e * L.N + n0) * L.groups_per_row + k / static_cast<uint32_t>(L.g);
+#pragma unroll
+          for (int r = 0; r < 4; ++r)
+            if (n0 + 32 * r < L.N && k < L.K)
+              raw[i][r] = group_raw(L, j0 + static_cast<int64_t>(32 * r) * L.groups_per_row);
+        }
+        if (b0 == 0) ok = mbar_wait_warp(c_empty(buf), ((it >> 1) & 1u) ^ 1u, wc);
+#pragma unroll
+        for (int i = 0; i < 2; ++i)
+#pragma unroll
+          for (int r = 0; r < 4; ++r) {
+            const GroupConst c = group_const(raw[i][r]);  // (zeros past the layer's edges: alpha 0)
+            if (ok) consts[(buf * Cfg::kWBoxes + b0 + i * b_step) * 128 + 32 * r + lane] = make_float4(c.r, c.b, c.delta, c.alpha);
+          }
+      }
+      if (!ok) break;
+      if (lane == 0) where[buf] = make_int4(static_cast<int>(e), n_blk, k_blk, 0);
+      __syncwarp();
+      if (lane == 0) mbar_arrive_local(c_full(buf));
+    }
+  } else if constexpr (GROUPED) {
+    // ------------------------------------------------------------ factor-gradient epilogue, grouped
+    // An expert has few rows to contract over, so a launch is bound by this work on all of its weights.
+    // Warp w has the tile's rows 32 (w % 4).. (its TMEM lanes) and 64 of its columns, which lie in one
+    // group of each row (P, g and K are multiples of 64); the weights arrive a whole tile at a
+    // time, and move to registers at once, so that the next tile's are on their way during the
+    // arithmetic; its group constants come from a warp that works a tile ahead.  A tile takes about 7,000
+    // cycles, 5,000 of them arithmetic (4,096 is what its exponentials and reciprocals take).  128 experts'
+    // 1536 x 4096, 65536 rows: 945 us, against 1255 with 8 warps that loaded weights and group factors
+    // by the row and found them by 64-bit divisions.
+    const int q = warp & 3;
+    const int box = warp >> 2;  // the tile's 64-column box
+    const int p_log2 = args.P == 128 ? 7 : 6;
+    const int64_t cpr = args.L.K >> p_log2;
+    const int64_t plane = args.L.N * cpr;
+    const float k_sc = args.sc.s * args.sc.inv_2tanh_s;
+    const float inv_k = (MU && k_sc > 0.0f) ? 1.0f / k_sc : 0.0f;
+    const bool soft = args.sc.phase == PHASE_SOFT;
+    // P = 128: the two warps of a row's 128-column block add up through shared memory
+    const bool paired = args.P == 128;
+    const int pair = (box >> 1) * 4 + q;
+    float4* const pair_sums = reinterpret_cast<float4*>(base_ptr + (bars - base) + Cfg::kBarBytes) + pair * 32 + lane;
+    const LayerDev& L = args.L;
+    const uint4* const wrow = reinterpret_cast<const uint4*>(base_ptr + (w_base - base) + box * Cfg::kWBox + (q * 32 + lane) * 128);
+    const float4* const consts =
+        reinterpret_cast<const float4*>(base_ptr + (bars - base) + Cfg::kBarBytes + Cfg::kPairBytes);
+    const int4* const where = reinterpret_cast<const int4*>(consts + 2 * Cfg::kWBoxes * 128);
+    uint32_t it = 0;
+    for (int t = cluster; t < num_tiles; t += nclusters, ++it) {
+      const uint32_t buf = it & 1u;
+      bool ok = mbar_wait_warp(c_full(buf), (it >> 1) & 1u, wc);
+      const float4 cv = consts[(buf * Cfg::kWBoxes + (paired ? box & ~1 : box)) * 128 + q * 32 + lane];
+      const int4 at = where[buf];
+      __syncwarp();
+      if (lane == 0) mbar_arrive_local(c_empty(buf));
+      GroupConst gc{};
+      gc.r = cv.x;
+      gc.b = cv.y;
+      gc.delta = cv.z;
+      gc.alpha = cv.w;
+      const bool live = gc.alpha != 0.0f;
+      const float D = args.sc.s * gc.delta;
+      const OneExp oe = one_exp_consts(args.sc.s, D);
+      LogiSums2 lacc{0, 0, 0, 0};
+      ok = ok && mbar_wait_warp(w_full(box), buf, wc);
+      uint4 w[8];
+      if (ok) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) w[i] = wrow[i ^ (lane & 7)];
+      }
+      // the reads are done before the box is handed back: the next tile's copy writes it through the
+      // async proxy, which the barrier alone does not order after them
+      fence_proxy_async_smem();
+      __syncwarp();
+      if (lane == 0) mbar_arrive_local(w_empty(box));
+      ok = ok && mbar_wait_warp(tmem_full0 + 8u * buf, (it >> 1) & 1u, wc);
+      tc_fence_after();
+      if (ok) {
+        const uint32_t src = tmem_base + (static_cast<uint32_t>(q * 32) << 16) + buf * BN + 64 * box;
+        auto run = [&](auto body) {
+#pragma unroll
+          for (int c = 0; c < 4; ++c) {
+            uint32_t rg[16];
+            tmem_ld16(src + 16 * c, rg);
+            tmem_ld_wait();
+            if (c == 3) {  // the accumulator is read
+              tc_fence_before();
+              __syncwarp();
+              if (lane == 0) mbar_arrive_cluster(leader_tmem_empty0 + 8u * buf);
+            }
+            if (live) {
+              body(rg, 0, w[2 * c]);
+              body(rg, 8, w[2 * c + 1]);
+            }
+          }
+        };
+        // One exponential per weight where the far tanh term is 1 to fp32 resolution; the first form
+        // where it serves all the warp's rows.
+        const bool one = D >= kOneExpD;
+        if (soft && __all_sync(0xffffffffu, !live || (one && oe.c2 <= 126.0f))) {
+          run([&](const uint32_t (&rg)[16], int at, const uint4& v) {
+            grad_eight_logistic<MU, true, false>(rg, at, v, gc, oe, lacc, inv_k);
+          });
+        } else {
+          run([&](const uint32_t (&rg)[16], int at, const uint4& v) {
+            if (one && soft) {
+              grad_eight_logistic<MU, true, true>(rg, at, v, gc, oe, lacc, inv_k);
+            } else if (one) {
+              grad_eight_logistic<MU, false, true>(rg, at, v, gc, oe, lacc, inv_k);
+            } else {
+              LogiSums l{0.f, 0.f, 0.f, 0.f};
+              grad_eight_sums<MU>(rg, at, v, gc, args.sc.s, args.sc.phase, l, inv_k);
+              lacc = logi_add(lacc, l);
+            }
+          });
+        }
+      }
+      LogiSums sum = logi_total(lacc);
+      if (paired) {
+        // two alternating buffers: one is written again two tiles on, past the next tile's barrier
+        float4* const slot = pair_sums + buf * (Cfg::kEpiWarps / 2 * 32);
+        if (box & 1) *slot = make_float4(sum.smu, sum.st, sum.sxs, sum.sdelta);
+        if (!bar_all(1 + pair, 64, ok)) break;
+        if (!(box & 1)) {
+          const float4 o = *slot;
+          sum.smu += o.x;
+          sum.st += o.y;
+          sum.sxs += o.z;
+          sum.sdelta += o.w;
+        }
+      } else if (!ok) {
+        break;
+      }
+      const int64_t n = static_cast<int64_t>(at.y) * Cfg::kTileRows + cta * 128 + q * 32 + lane;
+      const int32_t k = at.z * BN + 64 * box;
+      if (n < L.N && k < L.K && !(paired && (box & 1))) {
+        const int64_t to = at.x * 3 * plane + n * cpr + (k >> p_log2);
+        const GradSums acc = grad_sums(sum, soft, args.sc.inv_2tanh_s, k_sc);
+        args.part[to] = acc.smu;
+        args.part[to + plane] = acc.salpha;
+        args.part[to + 2 * plane] = acc.sdelta;
+      }
+    }
   } else {
     // ------------------------------------------------------------ factor-gradient epilogue
     const int q = warp & 3;        // TMEM lane quarter
     const int half = warp >> 2;    // column half of the tile
-    const int64_t cpr = args.L.K / args.P;
+    const int p_log2 = args.P == 128 ? 7 : 6;
+    const int64_t cpr = args.L.K >> p_log2;
     const int64_t plane = args.L.N * cpr;
     const float k_sc = args.sc.s * args.sc.inv_2tanh_s;
     const float inv_k = (MU && k_sc > 0.0f) ? 1.0f / k_sc : 0.0f;
@@ -1485,7 +1699,7 @@ __global__ void __launch_bounds__(DwCfg<CG>::kThreads, 1)
       const int64_t n = (int64_t)n_blk * Cfg::kTileRows + cta * 128 + q * 32 + lane;
       const bool row_ok = n < L.N;
       float* out = args.part + slab * 3 * plane;
-      LogiSums lacc{0.f, 0.f, 0.f, 0.f};
+      LogiSums2 lacc{0, 0, 0, 0};
       const bool soft = args.sc.phase == PHASE_SOFT;
       constexpr int kChunks = (BN / 2) / 32;
       const int64_t k0 = (int64_t)k_blk * BN + half * (BN / 2);
@@ -1506,7 +1720,7 @@ __global__ void __launch_bounds__(DwCfg<CG>::kThreads, 1)
       int64_t cur_j = -1;
       GroupRaw graw{};
       if (row_ok && k0 < L.K) {
-        cur_j = n * L.groups_per_row + k0 / L.g;
+        cur_j = n * L.groups_per_row + static_cast<uint32_t>(k0) / static_cast<uint32_t>(L.g);
         graw = group_raw(L, jbase + cur_j);
       }
       if (!mbar_wait(tmem_full0 + 8u * buf, (it >> 1) & 1u, wc)) break;
@@ -1521,42 +1735,37 @@ __global__ void __launch_bounds__(DwCfg<CG>::kThreads, 1)
         tmem_ld_wait();
         const int64_t k = k0 + c * 32;
         if (row_ok && k < L.K) {
-          const int64_t j = n * L.groups_per_row + k / L.g;
-          if (j != cur_j) {
-            gc = group_const(L, jbase + j);
-            cur_j = j;
+          if (c == 2) {  // a group holds whole 64-column blocks
+            const int64_t j = n * L.groups_per_row + static_cast<uint32_t>(k) / static_cast<uint32_t>(L.g);
+            if (j != cur_j) {
+              gc = group_const(L, jbase + j);
+              cur_j = j;
+            }
           }
           const float D = args.sc.s * gc.delta;
           if (gc.alpha != 0.0f && D >= kOneExpD) {
             // one exponential per weight (the far tanh term is 1 to fp32 resolution)
             const OneExp oe = one_exp_consts(args.sc.s, D);
-            if (oe.c2 <= 126.0f) {
-              if (soft) grad_chunk_logistic<MU, true, false>(rg, wcur, gc, oe, lacc, inv_k);
-              else grad_chunk_logistic<MU, false, false>(rg, wcur, gc, oe, lacc, inv_k);
-            } else {
-              if (soft) grad_chunk_logistic<MU, true, true>(rg, wcur, gc, oe, lacc, inv_k);
-              else grad_chunk_logistic<MU, false, true>(rg, wcur, gc, oe, lacc, inv_k);
-            }
-          } else if (gc.alpha != 0.0f) {
+            const bool clamp = oe.c2 > 126.0f;
 #pragma unroll
             for (int v = 0; v < 4; ++v) {
-              const uint32_t w4[4] = {wcur[v].x, wcur[v].y, wcur[v].z, wcur[v].w};
-#pragma unroll
-              for (int e = 0; e < 4; ++e) {
-                grad_element_sums<MU>(__uint_as_float(rg[8 * v + 2 * e]), bf16lo_to_f32(w4[e]), gc, args.sc.s,
-                                      args.sc.phase, lacc, inv_k);
-                grad_element_sums<MU>(__uint_as_float(rg[8 * v + 2 * e + 1]), bf16hi_to_f32(w4[e]), gc, args.sc.s,
-                                      args.sc.phase, lacc, inv_k);
-              }
+              if (soft && !clamp) grad_eight_logistic<MU, true, false>(rg, 8 * v, wcur[v], gc, oe, lacc, inv_k);
+              else if (soft) grad_eight_logistic<MU, true, true>(rg, 8 * v, wcur[v], gc, oe, lacc, inv_k);
+              else grad_eight_logistic<MU, false, true>(rg, 8 * v, wcur[v], gc, oe, lacc, inv_k);
             }
+          } else if (gc.alpha != 0.0f) {
+            LogiSums l{0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+            for (int v = 0; v < 4; ++v) grad_eight_sums<MU>(rg, 8 * v, wcur[v], gc, args.sc.s, args.sc.phase, l, inv_k);
+            lacc = logi_add(lacc, l);
           }
-          if (((k + 32) % args.P) == 0 || k + 32 >= L.K) {
-            const GradSums acc = grad_sums(lacc, soft, args.sc.inv_2tanh_s, k_sc);
-            const int64_t idx = n * cpr + k / args.P;
+          if ((static_cast<int32_t>(k + 32) & (args.P - 1)) == 0) {  // (K is a multiple of P)
+            const GradSums acc = grad_sums(logi_total(lacc), soft, args.sc.inv_2tanh_s, k_sc);
+            const int64_t idx = n * cpr + (k >> p_log2);
             out[idx] = acc.smu;
             out[plane + idx] = acc.salpha;
             out[2 * plane + idx] = acc.sdelta;
-            lacc = LogiSums{0.f, 0.f, 0.f, 0.f};
+            lacc = LogiSums2{0, 0, 0, 0};
           }
         }
 #pragma unroll
@@ -1798,7 +2007,7 @@ template <int CG, bool MU>
 cudaError_t run_dw(const LayerDev& L, StepScalars sc, const void* X, const void* dY, int64_t M, const TcPlan& plan,
                    float* part, cudaStream_t st) {
   static DwMaps<1> unused_maps;  // the dense kernel's (unread) grouped-map parameter
-  using Cfg = DwCfg<CG>;
+  using Cfg = DwCfg<CG, false>;
   DeviceInfo& d = device_info();
   if (!d.ok) return cudaErrorInvalidDevice;
   CUtensorMap tdy, tx;
@@ -1833,13 +2042,14 @@ cudaError_t run_dw(const LayerDev& L, StepScalars sc, const void* X, const void*
 template <int CG, bool MU>
 cudaError_t run_dw_grouped(const LayerDev& L0, StepScalars sc, const void* X, const void* dY, const GroupSpec& grp,
                            int32_t P, float* part, cudaStream_t st) {
-  using Cfg = DwCfg<CG>;
+  using Cfg = DwCfg<CG, true>;
   DeviceInfo& d = device_info();
   if (!d.ok) return cudaErrorInvalidDevice;
   static std::mutex mu;  // the parameter block below is reused per call
   std::lock_guard<std::mutex> lock(mu);
   static DwMaps<kDwGroupExperts> gm;
-  CUtensorMap unused{};
+  CUtensorMap unused{}, tw;
+  if (!make_tmap(&tw, L0.W, L0.K, static_cast<uint64_t>(grp.E) * L0.N, 64, 128)) return cudaErrorInvalidValue;
   DwArgs args;
   args.L = L0;
   args.sc = sc;
@@ -1873,7 +2083,7 @@ cudaError_t run_dw_grouped(const LayerDev& L0, StepScalars sc, const void* X, co
     args.wc = make_wait_ctl(d);
     const int tiles = args.num_n_tiles * args.num_k_tiles * n;
     const int clusters = std::min(tiles, d.sm_count / CG);
-    void* params[4] = {&unused, &unused, &args, &gm};
+    void* params[4] = {&tw, &unused, &args, &gm};
     const cudaError_t err = launch_persistent(dw_kernel<CG, MU, kDwGroupExperts>, CG, clusters * CG, Cfg::kThreads,
                                               Cfg::kSmemBytes, st, params);
     if (err != cudaSuccess) return err;

@@ -126,6 +126,44 @@ def test_grouped_narrow_matches_dense(device):
         assert U.fro_rel(_f64(dX[a:b]), _f64(dx)) <= 1e-2
 
 
+# Grouped dW: one CTA per tile and pairs, rows and columns short of a tile, groups of 64 (a partial sum per
+# 64 columns), 128 and more, both phases and reconstructions, experts of no and of few rows (tiles
+# whose weights follow each other closely; three runs, the same bits).  Against the oracle.
+@pytest.mark.parametrize("N,K,g,recon,phase,s", [
+    (120, 448, 64, 0, O.PHASE_SOFT, 30.0), (392, 640, 128, 1, O.PHASE_SOFT, 7.5), (768, 2048, 128, 0, O.PHASE_SOFT, 30.0),
+    (264, 768, 384, 0, O.PHASE_HARD, 30.0), (512, 1024, 512, 0, O.PHASE_SOFT, 3.75)])
+def test_grouped_dw(device, N, K, g, recon, phase, s):
+    import torch
+
+    from paper_2606_26650_gb300 import catq as C
+    rows = [3, 0, 300, 1, 64, 17, 130, 5]
+    E, per, off = len(rows), N * K // g, [0] + [int(v) for v in np.cumsum(rows)]
+    r = syn.rng(307, f"grouped dw/{N}/{K}")
+    W, X, dY = _bf16(r, (E, N, K), 0.02), _bf16(r, (off[-1], K)), _bf16(r, (off[-1], N))
+    fac = syn.factors(E * per, 3, f"grouped dw/{N}/{K}", perturbed=True)
+    layer = C.GroupedLayer.create(U.to_device(W.reshape(E * N, K), "bf16", device).view(E, N, K), g,
+                                  *(torch.from_numpy(f).to(device) for f in fac), recon=recon)
+    C.catq_group_stats(layer.dense)
+    x, dy = U.to_device(X, "bf16", device), U.to_device(dY, "bf16", device)
+    first, ws = None, C.workspace(C.catq_grouped_bwd_workspace_bytes(layer, off), device)
+    for _ in range(3):
+        got = [torch.full((E * per,), float("nan"), device=device) for _ in range(3)]
+        C.catq_grouped_soft_ternary_linear_bwd(layer, C.schedule(phase, s), x, dy, off, torch.empty_like(x), *got,
+                                               workspace=ws)
+        assert C.catq_device_status() == 0
+        first = first or got
+        assert all(torch.equal(a, b) for a, b in zip(first, got))
+    want = [np.zeros(E * per) for _ in range(3)]
+    for e in range(E):
+        at, grp = slice(off[e], off[e + 1]), slice(e * per, (e + 1) * per)
+        ref = O.linear_bwd(X[at], dY[at], W[e], g, O.group_stats(W[e], g, O.THR_HALF), tuple(f[grp] for f in fac), phase, s,
+                           with_mu=bool(recon))
+        for dst, src in zip(want, ref[1:]):
+            dst[grp] = src
+    for name, a, b in zip(("g_dmu", "g_dalpha", "g_ddelta"), first, want):
+        assert U.fro_rel(_f64(a), b) <= U.TOL_BF16, name
+
+
 # The fp32 path: tiles of 32, 128 and 256 rows with remainders, an output width that is no multiple of
 # 4, groups of 4 to 512, contractions shared by 1 to 8 CTAs, a single slice.  The fp32 bar.
 @pytest.mark.parametrize("M,N,K,g,recon,phase,s", [
