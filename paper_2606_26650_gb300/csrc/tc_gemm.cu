@@ -80,7 +80,7 @@ struct FusedCfg {
   static constexpr int kGroupThreads = 32 * kGroupWarps;
   static constexpr int kThreadsPerRow = kGroupThreads / kBRows;  // 2
   static constexpr int kChunksPerThread = 8 / kThreadsPerRow;    // 16-byte chunks of a 128-byte row
-  static constexpr int kThreads = 32 * (kEpiWarps + 2 + kProdWarps);
+  static constexpr int kThreads = 32 * (kEpiWarps + 3 + kProdWarps);
   // Stage q lands on the raw-W barrier of its producer group and slot; that barrier sees one
   // stage in every kRawPeriod, so each group waits on its own barriers strictly in phase
   // order (one barrier per slot shared by the groups would let a group running a full phase
@@ -458,6 +458,7 @@ __global__ void __launch_bounds__(FusedCfg<PAIRS>::kThreads, 1)
   const WaitCtl& wc = args.wc;
   const int num_tiles = args.num_m_tiles * args.num_n_tiles;
   constexpr int kTmaWarp = Cfg::kEpiWarps, kMmaWarp = Cfg::kEpiWarps + 1;
+  constexpr int kWTmaWarp = Cfg::kEpiWarps + 2 + Cfg::kProdWarps;
   // does this CTA produce stage q (PAIRS 1: always)
   auto produces = [&](uint32_t q) { return PAIRS == 1 || (q & 1u) == pair; };
 
@@ -531,8 +532,11 @@ __global__ void __launch_bounds__(FusedCfg<PAIRS>::kThreads, 1)
       if (cta == 0)
         for (int s = 0; s < SA; ++s)
           if (issued_mask & (1u << s)) mbar_wait_drain(full_a(s), (issued_phase >> s) & 1u);
-    } else if (lane == 1) {
+    }
+  } else if (warp == kWTmaWarp) {
+    if (lane == 0) {
       // ---------------------------------------------------------- TMA: raw W tiles this CTA produces
+      // (a warp of its own: two lanes of one warp that wait on barriers hold each other up)
       // (a W tile serves the raster group's M blocks at about the same time, then is done)
       const uint64_t pol_w = args.a_keep ? l2_policy_evict_first() : l2_policy_evict_normal();
       uint32_t q = 0, issued_mask = 0, issued_phase = 0;
