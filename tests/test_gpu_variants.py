@@ -245,3 +245,29 @@ def test_ternary_infer_slabs(device, N, K, g, B, mu, shift):
     C.catq_ternary_infer_staged([(codes, al, N, K, x, y, m), (codes, al, N, K, x, y2, m)], [0, 1], g, sync)
     assert C.catq_device_status() == 0
     assert torch.equal(y, y2) and not sync.any()
+
+
+# 8-bit activations: rows in a warp's registers (2 and 8 vectors a lane) and in a block's (2, 4 and 8 a thread),
+# at both ends of each and past the last; a row of zeros, the largest element first and last.
+# Scales and codes are the oracle's, bit for bit.
+@pytest.mark.parametrize("dtype,V", [("bf16", 8), ("f32", 4)])
+@pytest.mark.parametrize("nvec", [1, 64, 65, 256, 257, 512, 513, 1024, 1025, 2048, 2049])
+def test_act_quant_rows(device, dtype, V, nvec):
+    import torch
+
+    from paper_2606_26650_gb300 import catq as C
+    M, K = 19, nvec * V
+    X = (syn.rng(308, f"a8/{nvec}").standard_normal((M, K)) * 3.0).astype(np.float32)
+    X[7] = 0.0
+    X[11, -1], X[12, 0] = 40.0, -50.0
+    X = syn.round_bf16(X) if dtype == "bf16" else X
+    x = U.to_device(X, dtype, device)
+    codes, deq = torch.full_like(x, float("nan")), torch.full_like(x, float("nan"))
+    scale = torch.full((M,), float("nan"), device=device)
+    C.catq_act_quant_a8(x, codes, scale, deq)
+    q, s = O.act_quant_a8(X)
+    np.testing.assert_array_equal(U.to_host(scale), s)
+    np.testing.assert_array_equal(_f64(codes), q)
+    C.catq_act_quant_a8(x, codes, scale)
+    np.testing.assert_array_equal(_f64(codes), q)
+    assert U.err(_f64(deq), q * s.astype(np.float64)[:, None], dtype) <= (3e-3 if dtype == "bf16" else 1e-6)
