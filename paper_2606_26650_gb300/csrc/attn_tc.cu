@@ -425,6 +425,12 @@ __global__ void __launch_bounds__(kThreadsTc, 1)
           }
         }
         if (raise) m = mx;
+        // A chain that has seen only scores of -inf has no maximum yet: 0 in its place gives them weight 0.
+        // And from 2^24 on the fused product's unrounded part could exceed the exponent's range (the
+        // maximum is a rounded product): the products are then rounded first, like it.
+        const float mb = m == -INFINITY ? 0.0f : m;
+        const bool far = __any_sync(0xffffffffu, fabsf(mb) >= 16777216.0f);
+        const float p_scale = far ? 1.0f : a.scale_log2, p_base = far ? 0.0f : mb;
         // P_j in bf16, each half over its own scores (the second half is still in registers)
         float ls[8];
 #pragma unroll
@@ -432,13 +438,20 @@ __global__ void __launch_bounds__(kThreadsTc, 1)
 #pragma unroll
         for (int hf = 1; hf >= 0; --hf) {
           if (hf == 0) load_half(0);
+          if (far) {
+#pragma unroll
+            for (int u = 0; u < 2; ++u)
+#pragma unroll
+              for (int i = 0; i < 32; ++i)
+                sr[u][i] = __float_as_uint(__fsub_rn(__fmul_rn(__uint_as_float(sr[u][i]), a.scale_log2), mb));
+          }
 #pragma unroll
           for (int u = 0; u < 2; ++u) {
             uint32_t pk[16];
 #pragma unroll
             for (int i = 0; i < 32; i += 2) {
-              const float p0 = fast_exp2(fmaf(__uint_as_float(sr[u][i]), a.scale_log2, -m));
-              const float p1 = fast_exp2(fmaf(__uint_as_float(sr[u][i + 1]), a.scale_log2, -m));
+              const float p0 = fast_exp2(fmaf(__uint_as_float(sr[u][i]), p_scale, -p_base));
+              const float p1 = fast_exp2(fmaf(__uint_as_float(sr[u][i + 1]), p_scale, -p_base));
               ls[(i >> 1) & 7] += p0 + p1;
               pk[i / 2] = pack2(p0, p1);
             }

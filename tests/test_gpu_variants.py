@@ -271,3 +271,33 @@ def test_act_quant_rows(device, dtype, V, nvec):
     C.catq_act_quant_a8(x, codes, scale)
     np.testing.assert_array_equal(_f64(codes), q)
     assert U.err(_f64(deq), q * s.astype(np.float64)[:, None], dtype) <= (3e-3 if dtype == "bf16" else 1e-6)
+
+
+# Scores of -inf, and of the type's lowest value, in the online softmax's two chains of key tiles: whole tiles
+# of such keys first, second and last in their chain, and single ones; a query that sees one such
+# key alone in a tile (128 in tile 1).  -inf keys weigh nothing; rows whose every key is lowest weigh
+# them alike.  Outputs to the bf16 bar, log-sum-exp to 1e-5 of its value (fp32) or 1e-4.
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("S,keys,value", [
+    (576, [(128, 256)], -np.inf), (576, [(128, 129), (300, 301), (575, 576)], -np.inf),
+    (576, [(128, 384), (512, 576)], -np.inf), (576, [(0, 128)], -3.38e38), (576, [(128, 256), (384, 512)], -3.38e38),
+    (320, [(0, 320)], -3.38e38), (192, [(1, 64), (128, 130)], -np.inf)])
+def test_attention_masking_scores(device, S, keys, value, d):
+    import torch
+
+    from paper_2606_26650_gb300 import catq as C
+    B, nh, nkv = 2, 3, 1
+    r = syn.rng(309, f"mask/{S}/{d}/{len(keys)}")
+    q, k, v = (_bf16(r, (B * S, n * d)) for n in (nh, nkv, nkv))
+    q.reshape(B * S, nh, d)[:, :, 0] = 1.0  # the first column carries the mask
+    for a, b in keys:
+        k.reshape(B, S, nkv * d)[:, a:b, 0] = syn.round_bf16(np.array([value], np.float32))[0]
+    qd, kd, vd = (U.to_device(t, "bf16", device) for t in (q, k, v))
+    o, lse = torch.full_like(qd, float("nan")), torch.full((B * nh * S,), float("nan"), device=device)
+    C.catq_attention_fwd(qd, kd, vd, o, lse, B, S, nh, nkv, d)
+    assert C.catq_device_status() == 0
+    want, _ = O.attention(q, k, v, B, S, nh, nkv, d)
+    l_ref = O.attention_logsumexp(q, k, B, S, nh, nkv, d)
+    assert np.isfinite(want).all() and np.isfinite(l_ref).all()
+    assert U.fro_rel(_f64(o), want.reshape(B * S, -1)) <= U.TOL_BF16
+    assert (np.abs(_f64(lse).reshape(B, nh, S) - l_ref) <= 1e-4 + 1e-5 * np.abs(l_ref)).all()
