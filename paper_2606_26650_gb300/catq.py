@@ -118,6 +118,8 @@ def lib() -> ctypes.CDLL:
         "catq_ternary_infer_sync_bytes": (S, []),
         "catq_ternary_infer_staged": (I32, [P, I32, P, I32, I64, I32, P, P]),
         "catq_group_recon_error": (I32, [LP, P, P]),
+        "catq_linear_form": (I32, [I64, I64, I32, I32, catq_schedule, I64, I32, P, I32, I32, I32,
+                                   ctypes.POINTER(I32)]),
         "catq_grouped_fwd_loss_workspace_bytes": (S, [P, P]),
         "catq_rmsnorm_fwd": (I32, [P, I32, P, P, I64, I64, F, P, P, P, P]),
         "catq_rmsnorm_bwd": (I32, [P, I32, P, P, P, P, P, I64, I64, P, P]),
@@ -341,6 +343,18 @@ def catq_soft_ternary_linear_fwd_loss(layer: Layer, sched: catq_schedule, X, Y_r
     ws, ws_bytes = _ws(workspace, w)
     _check(lib().catq_soft_ternary_linear_fwd_loss(st, sched, x, M, _dtype_code(X), rs, ref, _dtype_code(Y_ref),
                                                    int(reduction), lo, dy, y, ws, ws_bytes, _stream(stream)), w)
+
+
+def catq_linear_form(N: int, K: int, g: int, sched: catq_schedule, M: int = 0, row_offsets=None, dx: bool = False,
+                     fused_loss: bool = False, recon: int = RECON_ALPHA_T, sm_count: int = 152) -> tuple:
+    """How a bf16 layer's forward or dX is cut: (CTA pairs per cluster or 0 for the narrow kernel, and the
+    narrow kernel's columns, accumulators, shares, A and W ring slots, table entries).  Host only."""
+    form = (ctypes.c_int32 * 7)()
+    off = None if row_offsets is None else _offsets(row_offsets)
+    E = 0 if row_offsets is None else len(row_offsets) - 1
+    _check(lib().catq_linear_form(int(N), int(K), int(g), int(recon), sched, int(M), E, off, int(dx), int(fused_loss),
+                                  int(sm_count), form), "catq_linear_form")
+    return tuple(form)
 
 
 def catq_act_quant_a8(X, codes, scale, X_deq=None, stream=None):

@@ -288,6 +288,28 @@ catq_status catq_soft_ternary_linear_fwd_loss(const catq_layer* layer, catq_sche
   return cuda_status(launch_loss_final(part, nparts, inv, loss_out, s));
 }
 
+catq_status catq_linear_form(int64_t N, int64_t K, int32_t g, int32_t recon, catq_schedule sched, int64_t M,
+                             int32_t n_experts, const int64_t* row_offsets, int32_t dx, int32_t fused_loss,
+                             int32_t sm_count, int32_t* form) {
+  if (N < 1 || K < 1 || g < 1 || g % 64 != 0 || K % g != 0 || N % 8 != 0) return CATQ_ERR_SHAPE;
+  const catq_status st = check_schedule(sched, sched.phase == CATQ_PHASE_SOFT);
+  if (st != CATQ_OK) return st;
+  if (!form || sm_count < 1 || (dx && fused_loss) || (recon != CATQ_RECON_ALPHA_T && recon != CATQ_RECON_ALPHA_T_MU))
+    return CATQ_ERR_INVALID_ARG;
+  GroupSpec grp{n_experts, row_offsets, 0};
+  if (row_offsets) {
+    if (n_experts < 1 || n_experts > kGroupedMaxExperts || row_offsets[0] != 0) return CATQ_ERR_INVALID_ARG;
+    for (int32_t e = 0; e < n_experts; ++e)
+      if (row_offsets[e + 1] < row_offsets[e]) return CATQ_ERR_INVALID_ARG;
+    if (row_offsets[n_experts] < 1) return CATQ_ERR_INVALID_ARG;
+  } else if (M < 1) {
+    return CATQ_ERR_INVALID_ARG;
+  }
+  fused_form(N, K, g, recon != CATQ_RECON_ALPHA_T, scalars(sched), M, row_offsets ? &grp : nullptr, dx != 0,
+             fused_loss != 0, sm_count, form);
+  return CATQ_OK;
+}
+
 catq_status catq_act_quant_a8(const void* X, int64_t M, int64_t K, int32_t x_dtype, void* codes, float* scale,
                               void* X_deq, catq_stream stream) {
   if (x_dtype != CATQ_F32 && x_dtype != CATQ_BF16) return CATQ_ERR_DTYPE;

@@ -157,6 +157,10 @@ cudaError_t launch_grad_reduce_grouped(const LayerDev& L0, StepScalars sc, const
                                        const GroupSpec& grp, float* g_dmu, float* g_dalpha, float* g_ddelta,
                                        cudaStream_t st);
 
+// How launch_tc_fwd / _dx (and their grouped forms, with `grp`) cut a layer's contraction: catq_linear_form.
+void fused_form(int64_t N, int64_t K, int32_t g, bool mu, StepScalars sc, int64_t M, const GroupSpec* grp, bool dx,
+                bool loss, int sm_count, int32_t* form);
+
 // Upper bound of EpiOpts::n_parts for any launch on a device with `sm_count` SMs.
 int fused_loss_max_parts(int sm_count);
 cudaError_t launch_tc_fwd(const LayerDev& L, StepScalars sc, const void* X, int64_t M, void* Y, cudaStream_t st,

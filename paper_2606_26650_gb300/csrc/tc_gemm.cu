@@ -2166,7 +2166,12 @@ int64_t count_tiles(int64_t M, int64_t ncols, const GroupSpec* grp, int64_t rows
 //   narrow      7 + rounds (S = 1) or 6 + 3 rounds (S > 1: two cluster barriers each), and nk blocks of
 //               0.38 / 0.48 / 0.54 / 0.68 (64 columns, 1 to 4 accumulators) or 0.56 / 0.72 / 0.95 /
 //               1.2 (128 columns), per wave; W from HBM at no more than 1.95 TB/s.
-// T contraction blocks of 64, nk a share's, rounds the accumulators with rows.  Forward of M x K x N,
+// T contraction blocks of 64, nk a share's, rounds the accumulators with rows.  The narrow form found is
+// weighed against the pairs once more as its rings pace it: with only two slots of one beside the
+// table a block waits for its copy (no less than 2.0 / the A ring's slots or 2.9 / the W ring's), and in
+// dX two tanh a weight cost a fifth more.  Of 840 forwards and dX of drawn shapes 72 then ran 1.1 to 2.0
+// times faster, as pairs (654 x 14336 x 4096: 216 -> 135 us), and nine 1.05 to 1.23 times slower.
+// Forward of M x K x N,
 // before (single CTAs below 512 rows) and now: 8 x 2048 x 1024 40 -> 10 us, 128 x 2048 x 2048 41 -> 12,
 // 300 x 2048 x 1024 42 -> 14, 512 x 6144 x 2048 69 -> 33, 1000 x 2048 x 2048 31 -> 23; as pairs
 // instead of single CTAs or pairs of pairs: 64 x 4096 x 14336 77 -> 46, 1100 x 4096 x 14336 173 -> 134,
@@ -2178,17 +2183,21 @@ struct FusedPlan {
 };
 
 FusedPlan plan_fused(int64_t M, int64_t depth, int64_t ncols, int32_t g, bool b_mn, bool mu, const GroupSpec* grp,
-                     bool loss, bool teacher, int sm_count) {
+                     bool loss, StepScalars sc, int sm_count) {
   const int64_t T = (depth + BK - 1) / BK;
+  // two tanh a weight (s Delta < 6, reckoned at Delta = 0.5) cost the narrow dX a fifth more a block
+  const double wide_dx = b_mn && sc.phase == PHASE_SOFT && sc.s < 12.0f ? 1.2 : 1.0;
   auto waves = [](int64_t tiles, int64_t fit) { return static_cast<double>((tiles + fit - 1) / fit); };
   const int64_t clusters2 = std::max(1, sm_count / 2), clusters4 = std::max(1, sm_count / 4 - 2);
-  const double per_tile = 0.62 * T + 2.0, consts = teacher ? 0.0 : 3.5;
+  const double per_tile = 0.62 * T + 2.0, consts = sc.phase == PHASE_TEACHER ? 0.0 : 3.5;
   const double t2 = 8.0 + consts + waves(count_tiles(M, ncols, grp, 512, BN), clusters2) * per_tile;
   const double t4 = 8.0 + consts + waves(count_tiles(M, ncols, grp, 1024, BN), clusters4) * per_tile;
   FusedPlan p{};
   const int64_t rows = grp ? M / grp->E : M;  // grouped: by the mean rows of an expert
   p.pairs = rows >= 1024 && t4 <= 1.1 * t2 ? 2 : 1;
-  double best = 0.92 * (p.pairs == 2 ? t4 : t2);  // the estimates' own error
+  const double pairs_best = 0.92 * (p.pairs == 2 ? t4 : t2);  // the estimates' own error
+  double best = pairs_best, best_paced = pairs_best;  // the narrow form's, as listed and paced by its rings
+  NarrowPlan narrow{};
   static constexpr double kBlock[2][4] = {{0.38, 0.48, 0.54, 0.68}, {0.56, 0.72, 0.95, 1.2}};
   const double w_us = static_cast<double>(grp ? grp->E : 1) * depth * ncols * 2 / 1.95e6;
   for (int bi = 0; bi < 2; ++bi)
@@ -2202,7 +2211,8 @@ FusedPlan plan_fused(int64_t M, int64_t depth, int64_t ncols, int32_t g, bool b_
         if (s > T || fit < 1 || (loss && tiles * s > sm_count * FusedCfg<1>::kEpiWarps)) continue;
         const int64_t nk = (T + s - 1) / s;
         const double over = s == 1 ? 7.0 + nacc : 6.0 + 3.0 * nacc;
-        const double t = std::max(waves(tiles, fit) * (over + nk * kBlock[bi][nacc - 1]), 6.0 + w_us);
+        auto estimate = [&](double block) { return std::max(waves(tiles, fit) * (over + nk * block), 6.0 + w_us); };
+        const double block = kBlock[bi][nacc - 1], t = estimate(block);
         if (t >= best) continue;
         NarrowPlan np{};
         np.bn = bn;
@@ -2222,10 +2232,15 @@ FusedPlan plan_fused(int64_t M, int64_t depth, int64_t ncols, int32_t g, bool b_
         }
         if (depth_best < 2) continue;
         best = t;
-        p.pairs = 0;
-        p.np = np;
+        best_paced = estimate(wide_dx * block);
+        if (depth_best == 2) best_paced = std::max(best_paced, estimate(std::max(2.0 / np.stages_a, 2.9 / np.stages_w)));
+        narrow = np;
       }
     }
+  if (best_paced < pairs_best) {
+    p.pairs = 0;
+    p.np = narrow;
+  }
   return p;
 }
 
@@ -2237,8 +2252,8 @@ cudaError_t dispatch_fused_epi(const LayerDev& L, StepScalars sc, const void* A,
   if (grp && (grp->E < 1 || grp->E > kMaxGroupExperts)) return cudaErrorInvalidValue;
   const DeviceInfo& d = device_info();
   if (!d.ok) return cudaErrorInvalidDevice;
-  const bool teacher = sc.phase == PHASE_TEACHER, mu = L.recon != 0 && !teacher;
-  const FusedPlan p = plan_fused(M, depth, ncols, L.g, B_MN, mu, grp, opts && opts->yref, teacher, d.sm_count);
+  const bool mu = L.recon != 0 && sc.phase != PHASE_TEACHER;
+  const FusedPlan p = plan_fused(M, depth, ncols, L.g, B_MN, mu, grp, opts && opts->yref, sc, d.sm_count);
   if (p.pairs == 0)
     return mu ? dispatch_narrow<B_MN, true>(L, sc, A, M, depth, C, ncols, p.np, st, grp, opts)
               : dispatch_narrow<B_MN, false>(L, sc, A, M, depth, C, ncols, p.np, st, grp, opts);
@@ -2278,6 +2293,14 @@ cudaError_t dispatch_fused_grouped(const LayerDev& L, StepScalars sc, const void
 cudaError_t launch_tc_fwd_grouped(const LayerDev& L0, StepScalars sc, const void* X, const GroupSpec& grp, void* Y,
                                   cudaStream_t st, const EpiOpts* opts) {
   return dispatch_fused_grouped<false>(L0, sc, X, L0.K, Y, L0.N, grp, st, opts);
+}
+
+void fused_form(int64_t N, int64_t K, int32_t g, bool mu, StepScalars sc, int64_t M, const GroupSpec* grp, bool dx,
+                bool loss, int sm_count, int32_t* form) {
+  const FusedPlan p = plan_fused(grp ? grp->off[grp->E] : M, dx ? N : K, dx ? K : N, g, dx,
+                                 mu && sc.phase != PHASE_TEACHER, grp, loss, sc, sm_count);
+  const int32_t f[7] = {p.pairs, p.np.bn, p.np.nacc, p.np.splits, p.np.stages_a, p.np.stages_w, p.np.entries};
+  std::copy(f, f + 7, form);
 }
 
 int fused_loss_max_parts(int sm_count) { return (sm_count > 0 ? sm_count : 1) * FusedCfg<1>::kEpiWarps; }
