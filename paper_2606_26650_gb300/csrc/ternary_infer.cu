@@ -47,9 +47,11 @@
 // other instructions for 32 rows) run at some 70 % of the MMA rate while they run; a third of
 // the time goes to the ends of items, stages and launches.  Two 8B blocks (109 MB of codes, 18 us at the
 // HBM rate), as eight launches in a graph / one staged call (with scales fetched where they are
-// used and row-wise bulk copies, in parentheses): groups of 128, 1 token 80 us (84) / 96 (119), 8 tokens
-// 87 (94) / 101 (139); groups of 64 with offsets, 1 token 91 (108) / 101 (144).  Four 1.7B blocks, 6
-// tokens, groups of 64 with offsets, staged: 87 us (133).
+// used and row-wise bulk copies, in parentheses): groups of 128, 1 token 86 us (84) / 95 (119), 8 tokens
+// 92 (94) / 101 (139); groups of 64 with offsets, 1 token 97 (108) / 102 (144).  Four 1.7B blocks, 6
+// tokens, groups of 64 with offsets, staged: 87 us (133).  (The figures in parentheses are of a kernel
+// that copied a launch's first codes before the launch ahead of it had finished, which a pack or a
+// copy just before does not allow: some 0.7 us a launch.)
 #include <algorithm>
 #include <cstdint>
 #include <type_traits>
@@ -428,34 +430,19 @@ __global__ void __launch_bounds__(kThreads, 2) ternary_mma_kernel(const __grid_c
     };
     constexpr std::false_type kCopy{};
     constexpr std::true_type kAsk{};
-    // The codes are weights that inference never writes, so the first slab's copy goes out before
-    // waiting for the previous kernel (whose output may be this launch's X); its scales and the other
-    // buffers' slabs are on their way to L2 meanwhile.
+    // The kernel before may be the one that wrote the codes and scales (a pack, a copy), and its writes
+    // are only sure to be seen past the wait: until then the first slabs are merely asked for in L2.
     Cursor c{};
     cursor_at(c, blockIdx.x, a);
-    Scales first{};
-    const bool any = c.t < a.total_items;
-    if (any) {
-      codes(c, ring_base, kCopy);
-      first = scales_of(c, ring_base);
-      scales(first, kAsk);
-      describe(c, 0);
-      Cursor n = c;
-      cursor_next(n, a);
-      for (int i = 1; i < nbuf && n.t < a.total_items; ++i, cursor_next(n, a)) {
-        codes(n, 0, kAsk);
-        scales(scales_of(n, 0), kAsk);
-      }
+    Cursor n = c;
+    for (int i = 0; i < nbuf && n.t < a.total_items; ++i, cursor_next(n, a)) {
+      if (STAGED && i == 0) continue;  // (no launch to wait for: copied right away)
+      codes(n, 0, kAsk);
+      scales(scales_of(n, 0), kAsk);
     }
     grid_dependency_wait();
     int slot = 0;
     uint32_t phase = 0;
-    if (any) {
-      scales(first, kCopy);
-      copies_arrive(full);
-      slot = 1;  // (at least two buffers)
-      cursor_next(c, a);
-    }
     for (;;) {
       // a buffer's first use needs no wait: the phase before a barrier's first counts as passed
       if (!mbar_wait_warp(empty + 8 * slot, phase ^ 1u, wc)) break;

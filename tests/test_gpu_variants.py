@@ -301,3 +301,38 @@ def test_attention_masking_scores(device, S, keys, value, d):
     assert np.isfinite(want).all() and np.isfinite(l_ref).all()
     assert U.fro_rel(_f64(o), want.reshape(B * S, -1)) <= U.TOL_BF16
     assert (np.abs(_f64(lse).reshape(B, nh, S) - l_ref) <= 1e-4 + 1e-5 * np.abs(l_ref)).all()
+
+
+# A pack, or a copy into the codes, and the inference that reads them, one after the other on a stream with
+# no synchronisation, the same buffers every time: each result is that of its own codes, bit for bit.
+@pytest.mark.parametrize("N,K,g,B", [(64, 256, 64, 1), (1024, 4096, 128, 3), (9744, 2048, 128, 1)])
+def test_inference_follows_its_pack(device, N, K, g, B):
+    import torch
+
+    from paper_2606_26650_gb300 import catq as C
+    r = syn.rng(310, f"pack/{N}/{K}")
+    layers = [C.Layer.create(U.to_device(_bf16(r, (N, K), 0.02), "bf16", device), g) for _ in range(3)]
+    X = U.to_device(_bf16(r, (B, K)), "bf16", device)
+    codes = torch.zeros(N * K // 4, dtype=torch.uint8, device=device)
+    alpha = torch.zeros(N * K // g, device=device)
+    want, kept = [], []
+    for layer in layers:
+        C.catq_group_stats(layer)
+        C.catq_hard_ternarize_pack(layer, codes, alpha)
+        torch.cuda.synchronize()
+        y = torch.empty(B, N, dtype=X.dtype, device=device)
+        C.catq_ternary_infer(codes, alpha, N, K, g, X, y)
+        torch.cuda.synchronize()
+        want.append(y)
+        kept.append((codes.clone(), alpha.clone()))
+    assert not torch.equal(want[0], want[1])
+    got = torch.full((120, B, N), float("nan"), dtype=X.dtype, device=device)
+    for i in range(120):
+        if i % 2:
+            C.catq_hard_ternarize_pack(layers[i % 3], codes, alpha)
+        else:
+            codes.copy_(kept[i % 3][0])
+            alpha.copy_(kept[i % 3][1])
+        C.catq_ternary_infer(codes, alpha, N, K, g, X, got[i])
+    assert C.catq_device_status() == 0
+    assert all(torch.equal(got[i], want[i % 3]) for i in range(120))
