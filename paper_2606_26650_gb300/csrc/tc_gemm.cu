@@ -962,7 +962,7 @@ constexpr int kNarrowThreads = 32 * (kNarrowRoleWarps + kNarrowProdWarps);
 constexpr int kNarrowMaxStages = 8;
 constexpr int kNarrowBarBytes = 8 * (5 * kNarrowMaxStages + 1) + 16;
 constexpr int kNarrowABytes = 128 * BK * 2;  // one accumulator's A rows per stage
-constexpr int kNarrowSmemMax = 227 * 1024;
+constexpr int kNarrowSmemMax = 227 * 1024 - kNarrowProdWarps * static_cast<int>(sizeof(Sum2));  // (beside `red`)
 
 // Shared memory: rings, table (float4, then mu), barriers, 1 KB of alignment slack.
 __host__ __device__ constexpr int narrow_smem(int bn, int nacc, int sa, int sw, int entries, bool mu) {
@@ -1870,10 +1870,12 @@ WaitCtl make_wait_ctl(const DeviceInfo& d) {
   return w;
 }
 
+// smem_limit: the most shared memory that any launch of the kernel asks for.  It is the kernel's own state,
+// which launches from other threads share, so it must not follow one launch's size.
 template <typename Kern>
-cudaError_t launch_persistent(Kern kern, int cg, int grid_ctas, int threads, int smem, cudaStream_t st,
+cudaError_t launch_persistent(Kern kern, int cg, int grid_ctas, int threads, int smem, int smem_limit, cudaStream_t st,
                               void** params) {
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_limit);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3(grid_ctas);
@@ -2004,7 +2006,7 @@ cudaError_t run_fused(const LayerDev& L, StepScalars sc, const void* A, int64_t 
   if (opts && opts->n_parts) *opts->n_parts = clusters * Cfg::kClusterCtas * Cfg::kEpiWarps;
   void* params[3] = {&ta, &tw, &args};
   return launch_persistent(kern, Cfg::kClusterCtas, clusters * Cfg::kClusterCtas, Cfg::kThreads, Cfg::kSmemBytes,
-                           st, params);
+                           Cfg::kSmemBytes, st, params);
 }
 
 // k blocks per raster group of the dW launch: about the square root of the clusters, so that
@@ -2047,7 +2049,8 @@ cudaError_t run_dw(const LayerDev& L, StepScalars sc, const void* X, const void*
   const int tiles = args.num_n_tiles * args.num_k_tiles * args.splits;
   const int clusters = std::min(tiles, d.sm_count / CG);
   void* params[4] = {&tdy, &tx, &args, &unused_maps};
-  return launch_persistent(dw_kernel<CG, MU, 1>, CG, clusters * CG, Cfg::kThreads, Cfg::kSmemBytes, st, params);
+  return launch_persistent(dw_kernel<CG, MU, 1>, CG, clusters * CG, Cfg::kThreads, Cfg::kSmemBytes, Cfg::kSmemBytes, st,
+                           params);
 }
 
 // Grouped dW: every expert with rows, kDwGroupExperts per launch; partials [E][3][N][K/P].
@@ -2097,7 +2100,7 @@ cudaError_t run_dw_grouped(const LayerDev& L0, StepScalars sc, const void* X, co
     const int clusters = std::min(tiles, d.sm_count / CG);
     void* params[4] = {&tw, &unused, &args, &gm};
     const cudaError_t err = launch_persistent(dw_kernel<CG, MU, kDwGroupExperts>, CG, clusters * CG, Cfg::kThreads,
-                                              Cfg::kSmemBytes, st, params);
+                                              Cfg::kSmemBytes, Cfg::kSmemBytes, st, params);
     if (err != cudaSuccess) return err;
   }
   return cudaSuccess;
@@ -2131,7 +2134,8 @@ cudaError_t run_narrow(const LayerDev& L, StepScalars sc, const void* A, int64_t
   // other's cluster peers wait for, could wait for ever
   const int smem = std::max(116 * 1024, narrow_smem(BNN, np.nacc, np.stages_a, np.stages_w, np.entries, MU));
   void* params[4] = {&ta, &tw, &args, const_cast<NarrowPlan*>(&np)};
-  return launch_persistent(fused_narrow_kernel<BNN, B_MN, MU>, np.splits, grid, kNarrowThreads, smem, st, params);
+  return launch_persistent(fused_narrow_kernel<BNN, B_MN, MU>, np.splits, grid, kNarrowThreads, smem, kNarrowSmemMax, st,
+                           params);
 }
 
 template <bool B_MN, bool MU>

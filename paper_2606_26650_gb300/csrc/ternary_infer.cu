@@ -788,7 +788,8 @@ cudaError_t launch_mma(const InferDesc* ls, int n, int32_t g, bool with_mu, cons
   const bool staged = a.n_stages > 1;
   auto kern = staged ? (with_mu ? ternary_mma_kernel<R, VW, true, true> : ternary_mma_kernel<R, VW, false, true>)
                      : (with_mu ? ternary_mma_kernel<R, VW, true, false> : ternary_mma_kernel<R, VW, false, false>);
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  // (the kernel's own state, which launches from other threads share: the most that any asks for)
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kDynBytes));
   if (e != cudaSuccess) return e;
   int64_t blocks = std::min<int64_t>(items, 2 * static_cast<int64_t>(sm));
   cudaLaunchConfig_t cfg{};

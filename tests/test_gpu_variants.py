@@ -336,3 +336,47 @@ def test_inference_follows_its_pack(device, N, K, g, B):
         C.catq_ternary_infer(codes, alpha, N, K, g, X, got[i])
     assert C.catq_device_status() == 0
     assert all(torch.equal(got[i], want[i % 3]) for i in range(120))
+
+
+# Host threads, each with its own stream, layer and buffers, whose two shapes take ring depths of their own in
+# one kernel: what one call asks for in shared memory must not depend on another's.  (Arguments are made
+# beforehand: the calls themselves run side by side, without the interpreter's lock.)
+@pytest.mark.parametrize("what", ["forward", "infer"])
+def test_threads_with_different_shapes(device, what):
+    import threading
+
+    import torch
+
+    from paper_2606_26650_gb300 import catq as C
+    failed = []
+
+    def work(N, K, g):
+        with torch.cuda.stream(torch.cuda.Stream(device)):
+            X, Y = (torch.ones(1, n, dtype=torch.bfloat16, device=device) for n in (K, N))
+            layer = C.Layer.create(torch.randn(N, K, device=device).bfloat16(), g)
+            C.catq_group_stats(layer)
+            codes = torch.zeros(N * K // 4, dtype=torch.uint8, device=device)
+            alpha = torch.ones(N * K // g, device=device)
+            stream = torch.cuda.current_stream()
+            stream.synchronize()
+            if what == "forward":
+                st = layer.struct()
+                call, args = C.lib().catq_soft_ternary_linear_fwd, (
+                    C.ctypes.byref(st), C.schedule(C.PHASE_HARD, 30.0), X.data_ptr(), 1, C.BF16, Y.data_ptr(),
+                    stream.cuda_stream)
+            else:
+                call, args = C.lib().catq_ternary_infer, (codes.data_ptr(), alpha.data_ptr(), None, N, K, g,
+                                                          X.data_ptr(), 1, C.BF16, Y.data_ptr(), stream.cuda_stream)
+            for _ in range(5000):
+                status = call(*args)
+                if status != 0:
+                    failed.append(C.STATUS.get(status, status))
+                    break
+            stream.synchronize()
+
+    threads = [threading.Thread(target=work, args=a) for a in [(64, 64, 64), (64, 16384, 64)] * 2]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not failed and C.catq_device_status() == 0, failed
