@@ -82,7 +82,7 @@ def lib() -> ctypes.CDLL:
         raise RuntimeError(f"{LIB_PATH} is missing: build it with __graft_entry__.build()")
     L = ctypes.CDLL(LIB_PATH)
     P, I64, I32, F, S = ctypes.c_void_p, ctypes.c_int64, ctypes.c_int32, ctypes.c_float, ctypes.c_size_t
-    LP = P  # structs by address: byref(...) or their packed bytes
+    LP, GP, IP = (ctypes.POINTER(t) for t in (catq_layer, catq_grouped_layer, catq_infer_layer))
     sig = {
         "catq_abi_version": (I32, []),
         "catq_status_string": (ctypes.c_char_p, [I32]),
@@ -99,28 +99,26 @@ def lib() -> ctypes.CDLL:
         "catq_ternary_infer": (I32, [P, P, P, I64, I64, I32, P, I64, I32, P, P]),
         "catq_soft_ternary_linear_bwd_noalloc": (I32, [LP, catq_schedule, P, P, I64, I32, P, P, P, P, P]),
         "catq_bwd_noalloc_max_scratch_bytes": (S, []),
-        "catq_grouped_soft_ternary_linear_fwd": (I32, [P, catq_schedule, P, P, I32, P,
-                                                       P]),
-        "catq_grouped_bwd_workspace_bytes": (S, [P, P]),
+        "catq_grouped_soft_ternary_linear_fwd": (I32, [GP, catq_schedule, P, P, I32, P, P]),
+        "catq_grouped_bwd_workspace_bytes": (S, [GP, P]),
         "catq_schedule_at_epoch": (I32, [I32, I32, ctypes.c_double, ctypes.c_double, ctypes.POINTER(catq_schedule)]),
         "catq_linear_decay_lr": (I32, [ctypes.c_double, I64, I64, ctypes.POINTER(F)]),
         "catq_factor_adamw_step": (I32, [I64, P, P, P, P, P, P, P, ctypes.POINTER(catq_adamw), I64, F, P]),
-        "catq_grouped_soft_ternary_linear_bwd": (I32, [P, catq_schedule, P, P, P, I32,
-                                                       P, P, P, P, P, S, P]),
+        "catq_grouped_soft_ternary_linear_bwd": (I32, [GP, catq_schedule, P, P, P, I32, P, P, P, P, P, S, P]),
         "catq_soft_ternary_linear_fwd_ex": (I32, [LP, catq_schedule, P, I64, I32, P, P, I32, P]),
         "catq_fwd_loss_workspace_bytes": (S, [LP, I64]),
         "catq_soft_ternary_linear_fwd_loss": (I32, [LP, catq_schedule, P, I64, I32, P, P, I32, I32, P, P, P, P, S, P]),
         "catq_act_quant_a8": (I32, [P, I64, I64, I32, P, P, P, P]),
         "catq_direct_adamw_step": (I32, [I64, P, P, P, P, P, ctypes.POINTER(catq_adamw), I64, F, P]),
         "catq_ternary_infer_max_layers": (I32, []),
-        "catq_ternary_infer_batched": (I32, [P, I32, I32, I64, I32, P]),
+        "catq_ternary_infer_batched": (I32, [IP, I32, I32, I64, I32, P]),
         "catq_ternary_infer_max_stages": (I32, []),
         "catq_ternary_infer_sync_bytes": (S, []),
-        "catq_ternary_infer_staged": (I32, [P, I32, P, I32, I64, I32, P, P]),
+        "catq_ternary_infer_staged": (I32, [IP, I32, ctypes.POINTER(I32), I32, I64, I32, P, P]),
         "catq_group_recon_error": (I32, [LP, P, P]),
         "catq_linear_form": (I32, [I64, I64, I32, I32, catq_schedule, I64, I32, P, I32, I32, I32,
                                    ctypes.POINTER(I32)]),
-        "catq_grouped_fwd_loss_workspace_bytes": (S, [P, P]),
+        "catq_grouped_fwd_loss_workspace_bytes": (S, [GP, P]),
         "catq_rmsnorm_fwd": (I32, [P, I32, P, P, I64, I64, F, P, P, P, P]),
         "catq_rmsnorm_bwd": (I32, [P, I32, P, P, P, P, P, I64, I64, P, P]),
         "catq_rope": (I32, [P, I64, I64, I32, I32, F, I32, P]),
@@ -129,8 +127,7 @@ def lib() -> ctypes.CDLL:
         "catq_block_output_loss": (I32, [P, P, I64, P, I32, P, P, P, P, S, P]),
         "catq_attention_fwd": (I32, [P, P, P, I32, I32, I32, I32, I32, P, P, P]),
         "catq_attention_bwd": (I32, [P, P, P, P, P, P, I32, I32, I32, I32, I32, P, P, P, P, P]),
-        "catq_grouped_soft_ternary_linear_fwd_loss": (I32, [P, catq_schedule, P, P,
-                                                            I32, P, I32, P, P, P, P, S, P]),
+        "catq_grouped_soft_ternary_linear_fwd_loss": (I32, [GP, catq_schedule, P, P, I32, P, I32, P, P, P, P, S, P]),
     }
     for name, (res, args) in sig.items():
         fn = getattr(L, name)
@@ -150,7 +147,7 @@ def header_functions(path: str = HEADER):
 # ------------------------------------------------------------------ marshalling helpers
 # A small call (a norm of a few rows, a decode step's layers) costs a few microseconds on the GPU,
 # so these run on every argument of every call and keep to a handful of attribute reads each:
-# addresses as ints, structs as packed bytes, the stream without a Stream object.  Nothing is
+# addresses as ints, structs filled in one call, the stream without a Stream object.  Nothing is
 # remembered from one call to the next.  On a Grace host, Python and launch together: forward of a
 # layer 18.0 -> 8.9 us, its backward 27.3 -> 16.2, a row norm 9.7 -> 5.3, three decode layers
 # 17.9 -> 9.9.
@@ -213,7 +210,8 @@ def _ws(workspace, where: str):
     return _buf(workspace, "workspace", 0, where), workspace.numel() * workspace.element_size()
 
 
-# catq_layer, catq_grouped_layer and catq_infer_layer as packed bytes (native sizes and alignment).
+# catq_layer, catq_grouped_layer and catq_infer_layer, to be filled in one call (native sizes and
+# alignment): a ctypes structure sets its fields one by one.
 _LAYER = struct.Struct("qqii8Qii")
 _GROUPED = struct.Struct("iiqqii8Q")
 _INFER = struct.Struct("QQQqqQQ")
@@ -272,13 +270,9 @@ class Layer:
 
     def struct(self) -> catq_layer:
         N, K = self.W.shape
-        *ptrs, op = self._addresses(N, K)
-        return catq_layer(N, K, self.g, _dtype_code(self.W), *ptrs, op or None, self.recon, 0)
-
-    def packed(self) -> bytes:
-        """struct() as bytes (what the calls below pass)."""
-        N, K = self.W.shape
-        return _LAYER.pack(N, K, self.g, _dtype_code(self.W), *self._addresses(N, K), self.recon, 0)
+        st = catq_layer()
+        _LAYER.pack_into(st, 0, N, K, self.g, _dtype_code(self.W), *self._addresses(N, K), self.recon, 0)
+        return st
 
 
 def schedule(phase: int, s: float = 0.0) -> catq_schedule:
@@ -288,12 +282,12 @@ def schedule(phase: int, s: float = 0.0) -> catq_schedule:
 # ------------------------------------------------------------------ the C calls
 
 def catq_group_stats(layer: Layer, thr_init: int = THR_HALF, stream=None):
-    _check(lib().catq_group_stats(layer.packed(), int(thr_init), _stream(stream)), "catq_group_stats")
+    _check(lib().catq_group_stats(layer.struct(), int(thr_init), _stream(stream)), "catq_group_stats")
 
 
 def catq_modulate_ternarize(layer: Layer, sched: catq_schedule, Wq_out=None, T_out=None, alpha_out=None,
                             stream=None):
-    st = layer.packed()
+    st = layer.struct()
     w = "catq_modulate_ternarize"
     wq = _buf(Wq_out, "Wq_out", layer.N * layer.K * layer.W.element_size(), w)
     t = _buf(T_out, "T_out", layer.N * layer.K, w)
@@ -303,7 +297,7 @@ def catq_modulate_ternarize(layer: Layer, sched: catq_schedule, Wq_out=None, T_o
 
 def catq_soft_ternary_linear_fwd(layer: Layer, sched: catq_schedule, X, Y, stream=None):
     w = "catq_soft_ternary_linear_fwd"
-    st = layer.packed()
+    st = layer.struct()
     N, K = layer.W.shape
     M, e = X.shape[0], X.element_size()
     _check(lib().catq_soft_ternary_linear_fwd(st, sched, _buf(X, "X", M * K * e, w), M, _dtype_code(X),
@@ -313,7 +307,7 @@ def catq_soft_ternary_linear_fwd(layer: Layer, sched: catq_schedule, X, Y, strea
 def catq_soft_ternary_linear_fwd_ex(layer: Layer, sched: catq_schedule, X, Y, x_row_scale=None, stream=None):
     """Y = diag(x_row_scale) X Wq^T; Y may be fp32 for a bf16 layer."""
     w = "catq_soft_ternary_linear_fwd_ex"
-    st = layer.packed()
+    st = layer.struct()
     N, K = layer.W.shape
     M = X.shape[0]
     x = _buf(X, "X", M * K * X.element_size(), w)
@@ -324,14 +318,14 @@ def catq_soft_ternary_linear_fwd_ex(layer: Layer, sched: catq_schedule, X, Y, x_
 
 
 def catq_fwd_loss_workspace_bytes(layer: Layer, M: int) -> int:
-    return int(lib().catq_fwd_loss_workspace_bytes(layer.packed(), int(M)))
+    return int(lib().catq_fwd_loss_workspace_bytes(layer.struct(), int(M)))
 
 
 def catq_soft_ternary_linear_fwd_loss(layer: Layer, sched: catq_schedule, X, Y_ref, loss_out, dY, Y=None,
                                       x_row_scale=None, workspace=None, reduction: int = REDUCE_MEAN, stream=None):
     """Forward, Eq. 7 loss and dY in one pass; Y_ref may be fp32 for a bf16 layer."""
     w = "catq_soft_ternary_linear_fwd_loss"
-    st = layer.packed()
+    st = layer.struct()
     N, K = layer.W.shape
     M, e = X.shape[0], X.element_size()
     x = _buf(X, "X", M * K * e, w)
@@ -368,13 +362,13 @@ def catq_act_quant_a8(X, codes, scale, X_deq=None, stream=None):
 
 
 def catq_bwd_workspace_bytes(layer: Layer, M: int) -> int:
-    return int(lib().catq_bwd_workspace_bytes(layer.packed(), int(M)))
+    return int(lib().catq_bwd_workspace_bytes(layer.struct(), int(M)))
 
 
 def catq_soft_ternary_linear_bwd(layer: Layer, sched: catq_schedule, X, dY, dX=None, g_dmu=None, g_dalpha=None,
                                  g_ddelta=None, workspace=None, stream=None):
     w = "catq_soft_ternary_linear_bwd"
-    st = layer.packed()
+    st = layer.struct()
     x, dy, dx, g0, g1, g2 = _bwd_bufs(layer, X, dY, dX, (g_dmu, g_dalpha, g_ddelta), w)
     ws, ws_bytes = _ws(workspace, w)
     _check(lib().catq_soft_ternary_linear_bwd(st, sched, x, dy, X.shape[0], _dtype_code(X), dx, g0, g1, g2, ws,
@@ -384,7 +378,7 @@ def catq_soft_ternary_linear_bwd(layer: Layer, sched: catq_schedule, X, dY, dX=N
 def catq_soft_ternary_linear_bwd_noalloc(layer: Layer, sched: catq_schedule, X, dY, dX=None, g_dmu=None,
                                          g_dalpha=None, g_ddelta=None, stream=None):
     w = "catq_soft_ternary_linear_bwd_noalloc"
-    st = layer.packed()
+    st = layer.struct()
     x, dy, dx, g0, g1, g2 = _bwd_bufs(layer, X, dY, dX, (g_dmu, g_dalpha, g_ddelta), w)
     _check(lib().catq_soft_ternary_linear_bwd_noalloc(st, sched, x, dy, X.shape[0], _dtype_code(X), dx, g0, g1, g2,
                                                       _stream(stream)), w)
@@ -418,7 +412,7 @@ def catq_recon_loss(Y, Y_ref, loss_out, dY=None, workspace=None, reduction: int 
 
 
 def catq_hard_ternarize_pack(layer: Layer, codes, alpha=None, mu=None, stream=None):
-    st = layer.packed()
+    st = layer.struct()
     w, G = "catq_hard_ternarize_pack", layer.G
     c = _buf(codes, "codes", layer.N * layer.K // 4, w)
     al, m = _buf(alpha, "alpha", 4 * G, w), _buf(mu, "mu", 4 * G, w)
@@ -447,18 +441,18 @@ def catq_ternary_infer_max_layers() -> int:
 
 
 def _infer_layer_array(layers, g, w):
-    """The layers as packed catq_infer_layer structs, and their token rows."""
-    B, g, out = layers[0][4].shape[0] if layers else 0, max(int(g), 1), []
-    for codes, alpha, N, K, X, Y, mu in layers:
+    """The layers as an array of catq_infer_layer, and their token rows."""
+    B, g = layers[0][4].shape[0] if layers else 0, max(int(g), 1)
+    arr, size = (catq_infer_layer * max(1, len(layers)))(), _INFER.size
+    for i, (codes, alpha, N, K, X, Y, mu) in enumerate(layers):
         N, K = int(N), int(K)
         n = N * K
         if X.shape[0] != B:
             raise ValueError(f"{w}: every layer needs the same token rows ({B})")
         e, need = X.element_size(), 4 * (n // g)
-        out.append(_INFER.pack(_buf(codes, "codes", n // 4, w), _buf(alpha, "alpha", need, w),
-                               _buf(mu, "mu", need, w) or 0, N, K, _buf(X, "X", B * K * e, w),
-                               _buf(Y, "Y", B * N * e, w)))
-    return b"".join(out) or bytes(_INFER.size), B
+        _INFER.pack_into(arr, i * size, _buf(codes, "codes", n // 4, w), _buf(alpha, "alpha", need, w),
+                         _buf(mu, "mu", need, w) or 0, N, K, _buf(X, "X", B * K * e, w), _buf(Y, "Y", B * N * e, w))
+    return arr, B
 
 
 def catq_ternary_infer_batched(layers, g: int, stream=None):
@@ -488,7 +482,7 @@ def catq_ternary_infer_staged(layers, stages, g: int, sync, stream=None):
     sy = _buf(sync, "sync", catq_ternary_infer_sync_bytes(), w)
     if len(stages) != len(layers):
         raise ValueError(f"{w}: one stage per layer")
-    st = struct.pack(f"{max(1, len(stages))}i", *([int(v) for v in stages] or [0]))
+    st = (ctypes.c_int32 * max(1, len(stages)))(*[int(v) for v in stages])
     dt = _dtype_code(layers[0][4]) if layers else BF16
     _check(lib().catq_ternary_infer_staged(arr, len(layers), st, int(g), int(B), dt, sy, _stream(stream)), w)
 
@@ -539,7 +533,7 @@ def catq_direct_adamw_step(d_alpha, d_delta, g_dalpha, g_ddelta, moments, hp: ca
 def catq_group_recon_error(layer: Layer, err, stream=None):
     """err [G] = per-group mean of (W - Wq)^2 for the hard reconstruction."""
     w = "catq_group_recon_error"
-    _check(lib().catq_group_recon_error(layer.packed(), _buf(err, "err", 4 * layer.G, w), _stream(stream)), w)
+    _check(lib().catq_group_recon_error(layer.struct(), _buf(err, "err", 4 * layer.G, w), _stream(stream)), w)
 
 
 def catq_selftest_wait_timeout(timeout_ns: int, stream=None):
@@ -579,12 +573,9 @@ class GroupedLayer:
         return (E, self.g, N, K, _dtype_code(self.W), d.recon, self.W.data_ptr()) + ptrs[1:]
 
     def struct(self) -> catq_grouped_layer:
-        f = self._fields()
-        return catq_grouped_layer(*f[:-1], f[-1] or None)
-
-    def packed(self) -> bytes:
-        """struct() as bytes (what the calls below pass)."""
-        return _GROUPED.pack(*self._fields())
+        st = catq_grouped_layer()
+        _GROUPED.pack_into(st, 0, *self._fields())
+        return st
 
 
 def _offsets(row_offsets):
@@ -607,14 +598,14 @@ def _grouped_bufs(layer, row_offsets, where, X=None, Y=None, dY=None, dX=None, g
 
 def catq_grouped_soft_ternary_linear_fwd(layer: GroupedLayer, sched: catq_schedule, X, row_offsets, Y, stream=None):
     w = "catq_grouped_soft_ternary_linear_fwd"
-    st = layer.packed()
+    st = layer.struct()
     x, y, _, _ = _grouped_bufs(layer, row_offsets, w, X=X, Y=Y)
     _check(lib().catq_grouped_soft_ternary_linear_fwd(st, sched, x, _offsets(row_offsets), _dtype_code(X), y,
                                                       _stream(stream)), w)
 
 
 def catq_grouped_bwd_workspace_bytes(layer: GroupedLayer, row_offsets) -> int:
-    st = layer.packed()
+    st = layer.struct()
     _grouped_bufs(layer, row_offsets, "catq_grouped_bwd_workspace_bytes")
     return int(lib().catq_grouped_bwd_workspace_bytes(st, _offsets(row_offsets)))
 
@@ -622,7 +613,7 @@ def catq_grouped_bwd_workspace_bytes(layer: GroupedLayer, row_offsets) -> int:
 def catq_grouped_soft_ternary_linear_bwd(layer: GroupedLayer, sched: catq_schedule, X, dY, row_offsets, dX=None,
                                          g_dmu=None, g_dalpha=None, g_ddelta=None, workspace=None, stream=None):
     w = "catq_grouped_soft_ternary_linear_bwd"
-    st = layer.packed()
+    st = layer.struct()
     x, _, dy, dx, g0, g1, g2 = _grouped_bufs(layer, row_offsets, w, X=X, dY=dY, dX=dX,
                                              grads=(g_dmu, g_dalpha, g_ddelta))
     ws, ws_bytes = _ws(workspace, w)
@@ -631,7 +622,7 @@ def catq_grouped_soft_ternary_linear_bwd(layer: GroupedLayer, sched: catq_schedu
 
 
 def catq_grouped_fwd_loss_workspace_bytes(layer: GroupedLayer, row_offsets) -> int:
-    st = layer.packed()
+    st = layer.struct()
     _grouped_bufs(layer, row_offsets, "catq_grouped_fwd_loss_workspace_bytes")
     return int(lib().catq_grouped_fwd_loss_workspace_bytes(st, _offsets(row_offsets)))
 
@@ -640,7 +631,7 @@ def catq_grouped_soft_ternary_linear_fwd_loss(layer: GroupedLayer, sched: catq_s
                                               loss_out, dY, Y=None, workspace=None, reduction: int = REDUCE_MEAN,
                                               stream=None):
     w = "catq_grouped_soft_ternary_linear_fwd_loss"
-    st = layer.packed()
+    st = layer.struct()
     x, y, dy, _ = _grouped_bufs(layer, row_offsets, w, X=X, Y=Y, dY=dY)
     ref = _grouped_bufs(layer, row_offsets, w, Y=Y_ref)[1]
     lo = _buf(loss_out, "loss_out", 4, w)

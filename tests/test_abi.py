@@ -368,3 +368,25 @@ def test_direct_update_validation(lib):
                 C.adamw(margin=0.5)):
         assert du(*args[:6], ctypes.byref(bad), *args[7:]) == 1
     assert du(8, 16, 16, 16, 18, 16, ctypes.byref(hp), 1, 1e-3, None) == 4
+
+
+def test_struct_arguments_are_typed(lib):
+    """A struct of one kind, or bytes, in the place of another's raises before the call."""
+    soft = C.schedule(C.PHASE_SOFT, 30.0)
+    layer, grouped, infer = _layer(), C.catq_grouped_layer(), (C.catq_infer_layer * 2)()
+    calls = {
+        C.catq_layer: [lambda a: lib.catq_group_stats(a, 0, None), lambda a: lib.catq_bwd_workspace_bytes(a, 4),
+                       lambda a: lib.catq_soft_ternary_linear_fwd(a, soft, 16, 4, C.BF16, 16, None)],
+        C.catq_grouped_layer: [lambda a: lib.catq_grouped_bwd_workspace_bytes(a, bytes(16)),
+                               lambda a: lib.catq_grouped_fwd_loss_workspace_bytes(a, bytes(16)),
+                               lambda a: lib.catq_grouped_soft_ternary_linear_fwd(a, soft, 16, bytes(16), C.BF16, 16, None)],
+        C.catq_infer_layer: [lambda a: lib.catq_ternary_infer_batched(a, 1, 128, 1, C.BF16, None)],
+    }
+    for kind, fns in calls.items():
+        others = [o for o in (layer, grouped, infer) if not isinstance(o, kind) and getattr(o, "_type_", None) is not kind]
+        for fn in fns:
+            for wrong in others + [ctypes.byref(o) for o in others[:1]] + [bytes(ctypes.sizeof(kind)), 4096]:
+                with pytest.raises(ctypes.ArgumentError):
+                    fn(wrong)
+    with pytest.raises(ctypes.ArgumentError):
+        lib.catq_ternary_infer_staged(infer, 1, bytes(4), 128, 1, C.BF16, None, None)
