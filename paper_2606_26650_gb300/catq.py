@@ -160,7 +160,10 @@ def _stream(stream=None):
     if stream is not None:
         return stream.cuda_stream
     import torch
-    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+    try:  # (not public: a PyTorch without them takes the public way, 1 us longer)
+        return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+    except AttributeError:
+        return torch.cuda.current_stream().cuda_stream
 
 
 _DTYPES: dict = {}

@@ -134,3 +134,15 @@ def test_wrappers_pass_their_scalars_through(monkeypatch):
     C.catq_soft_ternary_linear_bwd(L, C.schedule(C.PHASE_SOFT, 30.0), X, Y, None,
                                    *(FakeDev(L.G) for _ in range(3)), workspace=FakeDev(256, 1))
     assert seen["catq_soft_ternary_linear_bwd"][4] == M
+
+
+def test_current_stream_without_private_calls(monkeypatch):
+    """Where PyTorch lacks the calls that read the current stream's handle, its public interface serves."""
+    class Stream:
+        cuda_stream = 77
+
+    monkeypatch.setattr(torch.cuda, "current_stream", lambda *a: Stream())
+    for name in ("_cuda_getCurrentRawStream", "_cuda_getDevice"):
+        monkeypatch.delattr(torch._C, name, raising=False)
+    assert C._stream() == 77
+    assert C._stream(Stream()) == 77
