@@ -46,7 +46,7 @@ def test_act_quant_codes_and_scales(device, dtype, M, K):
 
 @pytest.mark.parametrize("wl_name,lin_name,M", [
     ("c2_qwen3_1p7b_block", "q_proj", 300),     # 1% outlier channels x30
-    ("c3_llama3_8b_block", "v_proj", 1100),     # Student-t activations, four-CTA clusters
+    ("c3_llama3_8b_block", "v_proj", 1100),     # Student-t activations, dX by four-CTA clusters
     ("c4_qwen3_14b_block", "k_proj", 700),      # 0.5% outlier channels x50
 ])
 @pytest.mark.parametrize("phase,s", [(O.PHASE_SOFT, 30.0), (O.PHASE_HARD, 30.0)])

@@ -69,7 +69,7 @@ def test_rmsnorm_fwd_with_residual(device, T, H, x_dtype):
 
 @pytest.mark.parametrize("h_dtype,H", [("f32", 1024), ("bf16", 1024), ("f32", 2048), ("bf16", 128)])
 def test_rmsnorm_bwd_two_consumers_and_residual(device, h_dtype, H):
-    """Rows up to 1024 take the warp-per-row kernel, longer ones the CTA-per-row kernel."""
+    """Rows up to 1024 belong to a team of lanes, longer ones to a CTA."""
     import torch
 
     from paper_2606_26650_gb300 import catq as C
@@ -157,7 +157,7 @@ def test_block_output_loss(device, reduction):
 
 # ---------------------------------------------------------------- attention
 
-# d = 128 with S a multiple of 128 takes the tcgen05 forward; the others the mma.sync one
+# both head widths, whole 128-token tiles and a last one of 64
 ATTN_SHAPES = [(2, 128, 4, 2, 128), (1, 192, 4, 1, 64), (1, 64, 2, 2, 128), (3, 256, 8, 8, 64), (2, 512, 8, 2, 128),
                (1, 384, 4, 4, 128)]
 

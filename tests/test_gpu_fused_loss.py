@@ -39,9 +39,9 @@ def _compare(got, W, X, g, fac, thr, phase, s, dtype, reduction=0):
 
 
 CASES = [
-    ("c2_qwen3_1p7b_block", "q_proj", 300),     # single-CTA tiles, ragged tail
-    ("c3_llama3_8b_block", "v_proj", 1100),     # four-CTA clusters, ragged tail
-    ("c4_qwen3_14b_block", "k_proj", 700),      # CTA pairs
+    ("c2_qwen3_1p7b_block", "q_proj", 300),     # narrow kernel, four shares, ragged tail
+    ("c3_llama3_8b_block", "v_proj", 1100),     # narrow forward, dX by four-CTA clusters, ragged tail
+    ("c4_qwen3_14b_block", "k_proj", 700),      # narrow forward, three accumulators
     ("c3_llama3_8b_block", "down_proj", 520),   # K = 14336, CTA pairs, 8-row tail
 ]
 

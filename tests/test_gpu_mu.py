@@ -61,8 +61,8 @@ def test_mu_fp32(device, phase, s):
 
 
 @pytest.mark.parametrize("wl_name,lin_name,M", [
-    ("c2_qwen3_1p7b_block", "q_proj", 300),     # 1-CTA tiles, ragged tail
-    ("c3_llama3_8b_block", "v_proj", 1100),     # 2-CTA tiles over 3 tiles, ragged tail
+    ("c2_qwen3_1p7b_block", "q_proj", 300),     # narrow kernel, four shares, ragged tail
+    ("c3_llama3_8b_block", "v_proj", 1100),     # narrow forward, dX by four-CTA clusters, ragged tail
     ("c4_qwen3_14b_block", "k_proj", 700),
 ])
 @pytest.mark.parametrize("phase,s", [(O.PHASE_SOFT, 30.0), (O.PHASE_SOFT, 0.625), (O.PHASE_HARD, 30.0)])

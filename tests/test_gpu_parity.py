@@ -64,8 +64,8 @@ def test_c1_fp32_full(device, phase, s, perturbed):
 # ---------------------------------------------------------------- bf16 configs, reduced M
 
 BF16_CASES = [
-    # (workload, linear, M): M = 300 runs the 1-CTA tiles with a ragged tail; M = 1100 runs
-    # the 2-CTA tiles (512 rows) over 3 tiles with a ragged tail.
+    # (workload, linear, M): ragged row counts; mostly the narrow kernel, CTA pairs in the 300-row
+    # gate_proj, four-CTA clusters in v_proj's dX (each form on purpose: test_gpu_linear_forms.py).
     ("c2_qwen3_1p7b_block", "q_proj", 300),
     ("c2_qwen3_1p7b_block", "k_proj", 1100),
     ("c2_qwen3_1p7b_block", "down_proj", 300),

@@ -28,7 +28,7 @@ def _near_twn_threshold(W, g):
 
 
 @pytest.mark.parametrize("rule", [O.THR_ABSMEAN, O.THR_TWN_STATIC])
-@pytest.mark.parametrize("N,K,g,M", [(1024, 4096, 128, 1100),   # register (team) kernel, four-CTA GEMMs
+@pytest.mark.parametrize("N,K,g,M", [(1024, 4096, 128, 1100),   # register (team) kernel, dX by four-CTA clusters
                                      (64, 4096, 4096, 300)])     # channel-wise: streaming kernel
 def test_static_rule_stats_and_step(device, rule, N, K, g, M):
     import torch

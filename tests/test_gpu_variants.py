@@ -72,10 +72,10 @@ def test_rope_head_runs(device, T, S, nh, d):
     assert U.fro_rel(_f64(xd), O.rope(x, S, nh, d, 500000.0)) <= 4e-3
 
 
-# The fused contraction's narrow form: 64- and 128-column tiles, 1 to 4 accumulators of 128 rows, the
-# contraction cut into 1 to 8 shares (of unequal length where their number does not divide it), groups
-# that straddle a tile's columns (192), rows and columns past the matrix, every phase, the options
-# of the general epilogue; and pairs of CTAs on fewer than 512 rows (400 x 2048 x 8192).  The bf16 bar.
+# The fused contraction's narrow form at odd sizes: one row, rows and columns past the matrix, the
+# contraction cut into 1 to 8 shares (of unequal length where their number does not divide it), both soft
+# forms and the hard one, the loss in its epilogue; and pairs of CTAs on fewer than 512 rows
+# (400 x 2048 x 8192).  The bf16 bar.  (Every form by its columns and accumulators: test_gpu_linear_forms.py.)
 @pytest.mark.parametrize("M,N,K,g,recon,phase,s,fused", [
     (1, 8, 64, 64, 0, O.PHASE_SOFT, 30.0, False), (3, 72, 1408, 128, 0, O.PHASE_SOFT, 3.75, True),
     (127, 328, 960, 192, 1, O.PHASE_SOFT, 30.0, True), (129, 136, 4032, 64, 0, O.PHASE_HARD, 30.0, False),
@@ -94,7 +94,8 @@ def test_linear_narrow_forms(device, M, N, K, g, recon, phase, s, fused):
 
 
 # Grouped launches in the narrow form: experts of 0, 1, 130 and 257 rows, and the same rows expert by
-# expert as dense layers give the same sums (both cut the contraction, in fp32: 1e-2 in bf16).
+# expert as dense layers, cut otherwise, agree (the contraction's order alone differs, in fp32: 1e-2 in
+# bf16).  Against the oracle: test_gpu_linear_forms.py.
 def test_grouped_narrow_matches_dense(device):
     import torch
 
