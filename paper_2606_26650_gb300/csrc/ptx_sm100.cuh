@@ -266,24 +266,6 @@ __device__ __forceinline__ void tc_fence_after() {
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 }
 
-// D[tmem] (+)= A[smem] * B[smem], bf16 inputs, fp32 accumulation.
-template <int CG>
-__device__ __forceinline__ void umma_bf16(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
-                                          uint32_t accumulate) {
-  if constexpr (CG == 1)
-    asm volatile(
-        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
-        "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
-        : "memory");
-  else
-    asm volatile(
-        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
-        "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
-        : "memory");
-}
-
 // Arrive on `bar` once every tcgen05 operation this thread issued so far has completed.
 // CG == 2: the arrival goes to the barrier at the same offset in both CTAs of the pair.
 template <int CG>
@@ -303,15 +285,6 @@ __device__ __forceinline__ void umma_commit_pair_mask(uint32_t bar, uint16_t cta
   asm volatile(
       "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(bar),
       "h"(cta_mask)
-      : "memory");
-}
-
-// Bulk copy of `bytes` (multiple of 16, both addresses 16-byte aligned) from global memory into
-// this CTA's shared memory; completion is signalled as transaction bytes on `bar`.
-__device__ __forceinline__ void bulk_load_g2s(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
-  asm volatile(
-      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
-      "l"(src), "r"(bytes), "r"(bar)
       : "memory");
 }
 
@@ -351,24 +324,14 @@ __device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.
 
 // ------------------------------------------------------------------ descriptors
 
-// Shared-memory matrix descriptor for a 128-byte-swizzled bf16 operand tile.
-//   K-major  (rows of 64 contiguous K elements): lbo ignored (16), sbo = 1024 (8-row step).
+// Shared-memory matrix descriptor for a 128-byte-swizzled bf16 operand tile, as 32-bit halves.
+//   K-major  (rows of 64 contiguous K elements): lbo ignored (16), 1024 bytes from 8 rows to the next 8.
 //   MN-major (rows of 64 contiguous M/N elements, one row per K index): lbo = byte step
-//            between 64-element M/N column blocks, sbo = 1024 (8 K-row step).
-__device__ __forceinline__ uint64_t smem_desc_sw128(uint32_t addr, uint32_t lbo, uint32_t sbo) {
-  uint64_t d = 0;
-  d |= (uint64_t)((addr >> 4) & 0x3FFFu);
-  d |= (uint64_t)((lbo >> 4) & 0x3FFFu) << 16;
-  d |= (uint64_t)((sbo >> 4) & 0x3FFFu) << 32;
-  d |= (uint64_t)1 << 46;  // descriptor version for tcgen05
-  d |= (uint64_t)2 << 61;  // 128-byte swizzle
-  return d;
-}
-
-// The same descriptors as 32-bit halves.  The upper half is one constant for every 128-byte-swizzled
-// tile here (stride 1024); in the lower one the 14-bit address field counts 16-byte units, so
-// stepping through a tile is one addition.  (In a cluster a shared-memory address carries the CTA's
-// rank above its 24 bits of offset, which must not reach the descriptor.)
+//            between 64-element M/N column blocks, 1024 from 8 K rows to the next 8.
+// The upper half (that stride, the descriptor version for tcgen05, the swizzle) is one constant for every
+// tile here; in the lower one the 14-bit address field counts 16-byte units, so stepping through a tile
+// is one addition.  (In a cluster a shared-memory address carries the CTA's rank above its 24 bits of
+// offset, which must not reach the descriptor.)
 constexpr uint32_t kDescHi = (1024u >> 4) | (1u << 14) | (2u << 29);
 __device__ __forceinline__ uint32_t desc_lo(uint32_t addr, uint32_t lbo) {
   return ((addr >> 4) & 0x3FFFu) | ((lbo >> 4) << 16);

@@ -99,7 +99,6 @@ struct FusedCfg {
 // GROUPED: the W tile of the epilogue comes through shared memory by TMA (see the epilogue).
 template <int CG, bool GROUPED>
 struct DwCfg {
-  static constexpr int kRowsPerCta = 128;    // G rows (n) per CTA
   static constexpr int kTileRows = 128 * CG; // MMA M
   static constexpr int kBCols = BN / CG;     // G columns (k) whose X slice this CTA loads
   static constexpr int kABytes = 128 * BK * 2;
@@ -1694,23 +1693,12 @@ __global__ void __launch_bounds__(DwCfg<CG, (NE > 1)>::kThreads, 1)
       const int split = t / tiles_per_split, r = t % tiles_per_split;
       int k_blk, n_blk;
       dw_tile(args, r, n_blk, k_blk);
-      // the tile's layer: the dense one, or (grouped) its expert's slice of the stacked layer
-      // (grouped: the expert's weights and per-group arrays start e N K elements and e G
-      // groups after expert 0's; its group j is group jbase + j of the stacked arrays)
       const LayerDev& L = args.L;
-      int64_t slab = split;  // which [3][N][K/P] partial block the tile writes
       const uint16_t* W = static_cast<const uint16_t*>(L.W);
-      int64_t jbase = 0;
-      if constexpr (NE > 1) {
-        const int64_t e = gm.expert[split];
-        W += e * L.N * L.K;
-        jbase = e * L.N * L.groups_per_row;
-        slab = e;
-      }
       const uint32_t buf = it & 1u;
       const int64_t n = (int64_t)n_blk * Cfg::kTileRows + cta * 128 + q * 32 + lane;
       const bool row_ok = n < L.N;
-      float* out = args.part + slab * 3 * plane;
+      float* out = args.part + split * 3 * plane;
       LogiSums2 lacc{0, 0, 0, 0};
       const bool soft = args.sc.phase == PHASE_SOFT;
       constexpr int kChunks = (BN / 2) / 32;
@@ -1733,7 +1721,7 @@ __global__ void __launch_bounds__(DwCfg<CG, (NE > 1)>::kThreads, 1)
       GroupRaw graw{};
       if (row_ok && k0 < L.K) {
         cur_j = n * L.groups_per_row + static_cast<uint32_t>(k0) / static_cast<uint32_t>(L.g);
-        graw = group_raw(L, jbase + cur_j);
+        graw = group_raw(L, cur_j);
       }
       if (!mbar_wait(tmem_full0 + 8u * buf, (it >> 1) & 1u, wc)) break;
       tc_fence_after();
@@ -1750,7 +1738,7 @@ __global__ void __launch_bounds__(DwCfg<CG, (NE > 1)>::kThreads, 1)
           if (c == 2) {  // a group holds whole 64-column blocks
             const int64_t j = n * L.groups_per_row + static_cast<uint32_t>(k) / static_cast<uint32_t>(L.g);
             if (j != cur_j) {
-              gc = group_const(L, jbase + j);
+              gc = group_const(L, j);
               cur_j = j;
             }
           }
