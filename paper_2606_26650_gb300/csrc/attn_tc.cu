@@ -165,9 +165,9 @@ __device__ __forceinline__ void warp_arrive(uint32_t bar, int lane) {
 }
 
 // 32 fp32 columns of one row per lane (a warp's 32 rows, `ld` elements apart from `row0` on, of which the
-// first `rows` are real), times f, stored as bf16.  A 4 x 4 transpose of 16-byte chunks inside each
-// group of four lanes lets four lanes cover 64 contiguous bytes of a row: a store then writes 16
-// whole sectors where a lane per row touched 32 halves (an item's epilogue took 4,900 cycles).
+// first `rows` are real), times f, stored as bf16, transposed so that four lanes cover 64 contiguous
+// bytes of a row: a store then writes 16 whole sectors where a lane per row touched 32 halves (an
+// item's epilogue took 4,900 cycles).
 __device__ __forceinline__ void store_cols32(uint16_t* row0, int64_t ld, int rows, const uint32_t (&o)[32], float f,
                                              int lane) {
   uint4 v[4];
@@ -178,22 +178,7 @@ __device__ __forceinline__ void store_cols32(uint16_t* row0, int64_t ld, int row
     v[p].z = pack2(__uint_as_float(o[8 * p + 4]) * f, __uint_as_float(o[8 * p + 5]) * f);
     v[p].w = pack2(__uint_as_float(o[8 * p + 6]) * f, __uint_as_float(o[8 * p + 7]) * f);
   }
-#pragma unroll
-  for (int k = 1; k <= 2; k <<= 1) {  // round k exchanges chunk pairs (p, p | k) with lane ^ k
-    const bool upper = (lane & k) != 0;
-#pragma unroll
-    for (int p = 0; p < 4; ++p) {
-      if (p & k) continue;
-      const uint4 send = upper ? v[p] : v[p | k];
-      uint4 got;
-      got.x = __shfl_xor_sync(0xffffffffu, send.x, k);
-      got.y = __shfl_xor_sync(0xffffffffu, send.y, k);
-      got.z = __shfl_xor_sync(0xffffffffu, send.z, k);
-      got.w = __shfl_xor_sync(0xffffffffu, send.w, k);
-      if (upper) v[p] = got;
-      else v[p | k] = got;
-    }
-  }
+  transpose_quads(v, lane);
   // lane 4a + i holds chunk i of rows 4a .. 4a + 3
 #pragma unroll
   for (int j = 0; j < 4; ++j) {

@@ -238,6 +238,37 @@ __device__ __forceinline__ void fence_proxy_async_smem() {
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
 }
 
+// 16 bytes of a CTA of this cluster (a shared::cluster address).
+__device__ __forceinline__ float4 ld_cluster_f4(uint32_t cluster_addr) {
+  float4 v;
+  asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
+               : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+               : "r"(cluster_addr)
+               : "memory");
+  return v;
+}
+
+// 4 x 4 transpose of 16-byte chunks inside each group of four lanes of a converged warp: from chunk p of
+// its own row in v[p], lane 4a + i comes to hold chunk i of the rows of lanes 4a .. 4a + 3 in v[0 .. 3].
+__device__ __forceinline__ void transpose_quads(uint4 (&v)[4], int lane) {
+#pragma unroll
+  for (int k = 1; k <= 2; k <<= 1) {  // round k exchanges chunk pairs (p, p | k) with lane ^ k
+    const bool upper = (lane & k) != 0;
+#pragma unroll
+    for (int p = 0; p < 4; ++p) {
+      if (p & k) continue;
+      const uint4 send = upper ? v[p] : v[p | k];
+      uint4 got;
+      got.x = __shfl_xor_sync(0xffffffffu, send.x, k);
+      got.y = __shfl_xor_sync(0xffffffffu, send.y, k);
+      got.z = __shfl_xor_sync(0xffffffffu, send.z, k);
+      got.w = __shfl_xor_sync(0xffffffffu, send.w, k);
+      if (upper) v[p] = got;
+      else v[p | k] = got;
+    }
+  }
+}
+
 // ------------------------------------------------------------------ tcgen05
 
 template <int CG>

@@ -72,15 +72,6 @@ __device__ __forceinline__ void load_run(const float* p, int64_t limit, bool vec
   for (int i = 0; i < N; ++i) v[i] = i < limit ? __ldg(p + i) : 0.0f;
 }
 
-__device__ __forceinline__ float4 ld_cluster4(uint32_t addr) {
-  float4 v;
-  asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
-               : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
-               : "r"(addr)
-               : "memory");
-  return v;
-}
-
 // Staging of one operand, R rows (the tile's i or j) x TK contraction columns, by 256 threads with V
 // consecutive values each.  C_MAJOR: memory runs along the rows (one run per contraction index),
 // otherwise along the contraction.
@@ -243,7 +234,7 @@ __global__ void __launch_bounds__(kThr, 2) simt_gemm_kernel(const __grid_constan
     if (r < r1) {
       const uint32_t at = smem_u32(&sm.out[r][tx * kMj]);
       for (int p = 0; p < S; ++p) {
-        const float4 q = S > 1 ? ld_cluster4(mapa_shared(at, p)) : *reinterpret_cast<const float4*>(&sm.out[r][tx * kMj]);
+        const float4 q = S > 1 ? ld_cluster_f4(mapa_shared(at, p)) : *reinterpret_cast<const float4*>(&sm.out[r][tx * kMj]);
         y[0] += q.x;
         y[1] += q.y;
         y[2] += q.z;

@@ -239,10 +239,8 @@ __device__ __forceinline__ bool mbar_wait_drain(uint32_t bar, uint32_t parity) {
 }
 
 // 32 fp32 accumulator columns of one row per lane (32 rows per warp, 32 consecutive columns
-// from `col`) stored as bf16.  A 4 x 4 transpose of 16-byte chunks inside each group of four
-// lanes (two xor-shuffle rounds) turns the lane-per-row layout into stores where four lanes
-// cover 64 contiguous bytes of one row, so each store instruction writes 8 row segments
-// instead of touching 32 rows.  ncols is a multiple of 8, so a chunk is wholly in or out.
+// from `col`) stored as bf16, transposed so that four lanes cover 64 contiguous bytes of one row:
+// each store instruction writes 8 row segments instead of touching 32 rows.  ncols is a multiple of 8, so a chunk is wholly in or out.
 __device__ __forceinline__ void store_rows_bf16x32(uint16_t* C, int64_t M, int64_t ncols, int64_t row0, int64_t col,
                                                    const uint32_t (&r)[32], int lane) {
   uint4 v[4];
@@ -253,24 +251,7 @@ __device__ __forceinline__ void store_rows_bf16x32(uint16_t* C, int64_t M, int64
     v[p].z = pack_bf16x2(__uint_as_float(r[8 * p + 4]), __uint_as_float(r[8 * p + 5]));
     v[p].w = pack_bf16x2(__uint_as_float(r[8 * p + 6]), __uint_as_float(r[8 * p + 7]));
   }
-  // Round k exchanges chunk pairs (p, p | k) with lane ^ k; afterwards lane 4a + i holds
-  // chunk i of rows 4a .. 4a + 3 in v[0 .. 3].
-#pragma unroll
-  for (int k = 1; k <= 2; k <<= 1) {
-    const bool upper = (lane & k) != 0;
-#pragma unroll
-    for (int p = 0; p < 4; ++p) {
-      if (p & k) continue;
-      const uint4 send = upper ? v[p] : v[p | k];
-      uint4 got;
-      got.x = __shfl_xor_sync(0xffffffffu, send.x, k);
-      got.y = __shfl_xor_sync(0xffffffffu, send.y, k);
-      got.z = __shfl_xor_sync(0xffffffffu, send.z, k);
-      got.w = __shfl_xor_sync(0xffffffffu, send.w, k);
-      if (upper) v[p] = got;
-      else v[p | k] = got;
-    }
-  }
+  transpose_quads(v, lane);  // lane 4a + i now holds chunk i of rows 4a .. 4a + 3
   const int64_t c = col + 8 * (lane & 3);
   if (c >= ncols) return;
 #pragma unroll
@@ -966,15 +947,6 @@ constexpr int kNarrowSmemMax = 227 * 1024 - kNarrowProdWarps * static_cast<int>(
 // Shared memory: rings, table (float4, then mu), barriers, 1 KB of alignment slack.
 __host__ __device__ constexpr int narrow_smem(int bn, int nacc, int sa, int sw, int entries, bool mu) {
   return sa * nacc * kNarrowABytes + sw * bn * BK * 2 + entries * (mu ? 20 : 16) + kNarrowBarBytes + 16 + 1024;
-}
-
-__device__ __forceinline__ float4 ld_cluster_f4(uint32_t cluster_addr) {
-  float4 v;
-  asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
-               : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
-               : "r"(cluster_addr)
-               : "memory");
-  return v;
 }
 
 // The options of the general epilogue for 8 consecutive finished columns of one row.
