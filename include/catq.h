@@ -176,9 +176,9 @@ catq_status catq_soft_ternary_linear_fwd_ex(const catq_layer* layer, catq_schedu
 /* How a bf16 layer's forward (dx 0) or dX (dx 1) is cut on a GPU of sm_count SMs, as the calls decide it.
  * Host only: touches no device.  fused_loss: the forward with the loss in its epilogue.  row_offsets:
  * NULL for a dense layer of M rows, else the n_experts + 1 host offsets of a grouped one (M is then
- * ignored).  form [7] = { CTA pairs per cluster (2 or 1; 0: the narrow kernel), and for the narrow
- * kernel its columns, 128-row accumulators and shares of the contraction, the slots of its A and W
- * rings and the entries of its constants' table (else 0) }.  N, K, g as a bf16 layer's (else
+ * ignored).  form [7] = { CTA pairs per cluster (2 or 1; -1: tiles of one CTA; 0: the narrow kernel), and
+ * for the narrow kernel its columns, 128-row accumulators and shares of the contraction, the slots of
+ * its A and W rings and the entries of its constants' table (else 0) }.  N, K, g as a bf16 layer's (else
  * CATQ_ERR_SHAPE), M >= 1 and at least one routed row, sm_count >= 1, 1 <= n_experts <= 128 when
  * grouped; other values and a null form: CATQ_ERR_INVALID_ARG. */
 catq_status catq_linear_form(int64_t N, int64_t K, int32_t g, int32_t recon, catq_schedule sched, int64_t M,

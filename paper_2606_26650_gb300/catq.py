@@ -344,8 +344,9 @@ def catq_soft_ternary_linear_fwd_loss(layer: Layer, sched: catq_schedule, X, Y_r
 
 def catq_linear_form(N: int, K: int, g: int, sched: catq_schedule, M: int = 0, row_offsets=None, dx: bool = False,
                      fused_loss: bool = False, recon: int = RECON_ALPHA_T, sm_count: int = 152) -> tuple:
-    """How a bf16 layer's forward or dX is cut: (CTA pairs per cluster or 0 for the narrow kernel, and the
-    narrow kernel's columns, accumulators, shares, A and W ring slots, table entries).  Host only."""
+    """How a bf16 layer's forward or dX is cut: (CTA pairs per cluster, -1 for tiles of one CTA or 0 for the
+    narrow kernel, and the narrow kernel's columns, accumulators, shares, A and W ring slots, table entries).
+    Host only."""
     form = (ctypes.c_int32 * 7)()
     off = None if row_offsets is None else _offsets(row_offsets)
     E = 0 if row_offsets is None else len(row_offsets) - 1

@@ -18,7 +18,8 @@
 //                    idle: one CTA per tile of up to 512 rows x 64 or 128 columns and share of
 //                    the contraction, the shares added up through distributed shared memory.
 //
-// CG = 1 (dw_kernel, narrow layers): one CTA per tile (MMA M = 128).  CG = 2: a CTA pair (cluster of 2) computes one
+// CG = 1 (dw_kernel on narrow layers, fused_gemm_kernel on grouped ones of few rows): one CTA per tile
+// (MMA M = 128).  CG = 2: a CTA pair (cluster of 2) computes one
 // tile with tcgen05 cta_group::2 (MMA M = 256), each CTA holding half of the operand
 // columns; only the even CTA issues MMAs.
 //
@@ -58,19 +59,20 @@ constexpr int gcd_c(int a, int b) { return b == 0 ? a : gcd_c(b, a % b); }
 // against the same produced operand tiles; each pair produces every other stage and sends
 // its transformed half-tiles to the other pair's CTAs through distributed shared memory,
 // which halves the per-SM transform work.
-template <int PAIRS>
+// CG == 1 is a tile of one CTA (256 rows), for grouped launches of few rows an expert.
+template <int CG, int PAIRS>
 struct FusedCfg {
-  static constexpr int CG = 2;  // CTAs per pair
+  static_assert(PAIRS == 1 || CG == 2, "pairs of pairs need CTA pairs");
   static constexpr int kClusterCtas = CG * PAIRS;
   static constexpr int kRowsPerAcc = 128 * CG;          // MMA M
   static constexpr int kTileRows = kRowsPerAcc * NACC;  // rows of C per pair per tile
   static constexpr int kBRows = BN / CG;                // 128-byte operand rows per CTA per stage
   static constexpr int kABytes = NACC * 128 * BK * 2;   // this CTA's A rows per stage
   static constexpr int kWBytes = kBRows * BK * 2;       // this CTA's operand rows per stage
-  static constexpr int kStagesA = 4;                    // A ring: TMA -> MMA
+  static constexpr int kStagesA = CG == 1 ? 3 : 4;      // A ring: TMA -> MMA
   // W ring: TMA -> producers (in place) -> MMA.  Even with two pairs, so every slot is always
   // produced by the same pair (and received by the other).
-  static constexpr int kStagesW = PAIRS == 2 ? 6 : 5;
+  static constexpr int kStagesW = PAIRS == 2 ? 6 : (CG == 1 ? 3 : 5);
   static constexpr int kEpiWarps = 4;
   // Two groups of 8 producer warps take alternate stages (of the ones this CTA produces), so
   // each group has two stage periods per operand tile and the groups' MUFU work interleaves.
@@ -78,7 +80,7 @@ struct FusedCfg {
   static constexpr int kGroupWarps = 8;
   static constexpr int kProdWarps = kProdGroups * kGroupWarps;
   static constexpr int kGroupThreads = 32 * kGroupWarps;
-  static constexpr int kThreadsPerRow = kGroupThreads / kBRows;  // 2
+  static constexpr int kThreadsPerRow = kGroupThreads / kBRows;  // 1 (CG 1) or 2
   static constexpr int kChunksPerThread = 8 / kThreadsPerRow;    // 16-byte chunks of a 128-byte row
   static constexpr int kThreads = 32 * (kEpiWarps + 3 + kProdWarps);
   // Stage q lands on the raw-W barrier of its producer group and slot; that barrier sees one
@@ -329,9 +331,9 @@ __device__ __forceinline__ void load_yref_bf16x16(const uint16_t* Yr, int64_t nc
 // CTA's tile sequence) and tracks which W row, K chunk and group its 128-byte operand row
 // holds, the group as its index into the [K/g][N] operand-constant array.  Divisions happen
 // once per tile; each stage step is a few integer adds.
-template <bool B_MN, int PAIRS>
+template <int CG, bool B_MN, int PAIRS>
 struct OperandRowIter {
-  using Cfg = FusedCfg<PAIRS>;
+  using Cfg = FusedCfg<CG, PAIRS>;
   int t, kb;      // tile index, k block
   int64_t n, kc;  // W row (within its expert), first K column of the 64-element chunk
   int64_t ci;     // operand-constant index of (n, kc): (kc / g) * N + n, in float4 units from
@@ -401,12 +403,12 @@ struct OperandRowIter {
 // kernel carries none of its work).  EPI: 0 stores C in bf16; 1 is the general epilogue
 // (row scale, fp32 C, fused loss), a separate instantiation so the plain forward and dX
 // keep their register allocation; 2 is a row scale on a bf16 C alone.
-template <bool B_MN, int PAIRS, bool MU, int EPI = 0>
-__global__ void __launch_bounds__(FusedCfg<PAIRS>::kThreads, 1)
+template <int CG, bool B_MN, int PAIRS, bool MU, int EPI = 0>
+__global__ void __launch_bounds__(FusedCfg<CG, PAIRS>::kThreads, 1)
     fused_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmW,
                       const FusedArgs args) {
-  using Cfg = FusedCfg<PAIRS>;
-  constexpr int SA = Cfg::kStagesA, SW = Cfg::kStagesW, CG = Cfg::CG;
+  using Cfg = FusedCfg<CG, PAIRS>;
+  constexpr int SA = Cfg::kStagesA, SW = Cfg::kStagesW;
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw_addr = smem_u32(smem_raw);
   const uint32_t base = (raw_addr + 1023u) & ~1023u;
@@ -478,9 +480,9 @@ __global__ void __launch_bounds__(FusedCfg<PAIRS>::kThreads, 1)
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
   // Barriers a whole pair signals live in the pair's even CTA.
-  const uint32_t leader_full_a0 = mapa_shared(full_a(0), leader);
-  const uint32_t leader_full_w0 = mapa_shared(full_w(0), leader);
-  const uint32_t leader_tmem_empty0 = mapa_shared(tmem_empty0, leader);
+  const uint32_t leader_full_a0 = CG == 2 ? mapa_shared(full_a(0), leader) : full_a(0);
+  const uint32_t leader_full_w0 = CG == 2 ? mapa_shared(full_w(0), leader) : full_w(0);
+  const uint32_t leader_tmem_empty0 = CG == 2 ? mapa_shared(tmem_empty0, leader) : tmem_empty0;
   const uint16_t pair_mask = static_cast<uint16_t>(3u << (2 * pair));
   const uint16_t all_mask = static_cast<uint16_t>((1u << Cfg::kClusterCtas) - 1u);
 
@@ -503,7 +505,8 @@ __global__ void __launch_bounds__(FusedCfg<PAIRS>::kThreads, 1)
 #pragma unroll
           for (int acc = 0; acc < NACC; ++acc) {
             const int32_t row = m0 + acc * Cfg::kRowsPerAcc + cta * 128;
-            tma_load_2d_pair_hint(dst + acc * (128 * BK * 2), &tmA, fb, kb * BK, row, pol_a);
+            if constexpr (CG == 1) tma_load_2d_hint(dst + acc * (128 * BK * 2), &tmA, fb, kb * BK, row, pol_a);
+            else tma_load_2d_pair_hint(dst + acc * (128 * BK * 2), &tmA, fb, kb * BK, row, pol_a);
           }
           issued_mask |= 1u << s;
           issued_phase = (issued_phase & ~(1u << s)) | (ph << s);
@@ -830,7 +833,7 @@ __global__ void __launch_bounds__(FusedCfg<PAIRS>::kThreads, 1)
     // `cur` is the stage being produced; `ahead` runs two of this thread's stages ahead and
     // requests that stage's operand constants (one 16-byte vector, precomputed per call), so
     // an L2 round trip is hidden behind two stages.
-    OperandRowIter<B_MN, PAIRS> cur, ahead;
+    OperandRowIter<CG, B_MN, PAIRS> cur, ahead;
     cur.init(args, cta, row, cluster, 0);
     cur.step(args, cta, row, nclusters, q0);
     ahead = cur;
@@ -839,7 +842,7 @@ __global__ void __launch_bounds__(FusedCfg<PAIRS>::kThreads, 1)
     float m0 = 0.0f, m1 = 0.0f;
     int64_t j0 = -1, j1 = -1;
     constexpr bool with_mu = MU;
-    auto request = [&](const OperandRowIter<B_MN, PAIRS>& it, float4& dst, float& dm, int64_t& jd,
+    auto request = [&](const OperandRowIter<CG, B_MN, PAIRS>& it, float4& dst, float& dm, int64_t& jd,
                        const float4& other, float om, int64_t jo) {
       if (transform && it.live(args, num_tiles) && it.valid(args)) {
         if (jo == it.ci) {
@@ -1921,10 +1924,10 @@ int64_t fill_groups(FusedArgs& args, const GroupSpec& grp, int64_t rows_per_tile
 
 // grp (nullable): a grouped launch over grp->E experts whose weights are stacked from L.W on
 // and whose rows of A and C are expert-sorted (host offsets grp->off).
-template <bool B_MN, int PAIRS, bool MU, int EPI = 0>
+template <int CG, bool B_MN, int PAIRS, bool MU, int EPI = 0>
 cudaError_t run_fused(const LayerDev& L, StepScalars sc, const void* A, int64_t M, int64_t depth, void* C,
                       int64_t ncols, cudaStream_t st, const GroupSpec* grp = nullptr, const EpiOpts* opts = nullptr) {
-  using Cfg = FusedCfg<PAIRS>;
+  using Cfg = FusedCfg<CG, PAIRS>;
   DeviceInfo& d = device_info();
   if (!d.ok) return cudaErrorInvalidDevice;
   if (grp && (grp->E < 1 || grp->E > kMaxGroupExperts)) return cudaErrorInvalidValue;
@@ -1959,7 +1962,7 @@ cudaError_t run_fused(const LayerDev& L, StepScalars sc, const void* A, int64_t 
     args.num_m_tiles = tiles / args.num_n_tiles;  // the kernel's tile count is M x N blocks
     if (tiles == 0) return cudaSuccess;
   }
-  auto kern = fused_gemm_kernel<B_MN, PAIRS, MU, EPI>;
+  auto kern = fused_gemm_kernel<CG, B_MN, PAIRS, MU, EPI>;
   const int fit = max_active_clusters(kern, Cfg::kClusterCtas, Cfg::kThreads, Cfg::kSmemBytes,
                                       d.sm_count / Cfg::kClusterCtas);
   const int clusters = std::min(tiles, fit);
@@ -2123,9 +2126,9 @@ int64_t count_tiles(int64_t M, int64_t ncols, const GroupSpec* grp, int64_t rows
   return m * ((ncols + cols - 1) / cols);
 }
 
-// How a fused launch is cut: pairs of pairs (4 CTAs, 1024 rows), pairs (2, 512 rows) or narrow (1).
-// Each form's time is estimated from what it measured per contraction block on one GB300 (g = 128,
-// SOFT; microseconds), and the least is taken:
+// How a fused launch is cut: pairs of pairs (4 CTAs, 1024 rows), pairs (2, 512 rows), in grouped launches
+// also single CTAs (256 rows), or narrow (1).  Each form's time is estimated from what it measured per
+// contraction block on one GB300 (g = 128, SOFT; microseconds), and the least is taken:
 //   pairs       8 + waves (0.62 T + 2), plus 3.5 for the launch that writes op_const,
 //   narrow      7 + rounds (S = 1) or 6 + 3 rounds (S > 1: two cluster barriers each), and nk blocks of
 //               0.38 / 0.48 / 0.54 / 0.68 (64 columns, 1 to 4 accumulators) or 0.56 / 0.72 / 0.95 /
@@ -2141,8 +2144,16 @@ int64_t count_tiles(int64_t M, int64_t ncols, const GroupSpec* grp, int64_t rows
 // instead of single CTAs or pairs of pairs: 64 x 4096 x 14336 77 -> 46, 1100 x 4096 x 14336 173 -> 134,
 // dX of 1500 x 6144 x 2048 51 -> 30.  Pairs of pairs are 3 to 5 % faster than pairs at equal waves,
 // and transform each weight half as often under the power cap: kept up to 10 % more.
+// A grouped launch runs many tiles one after the other, on weights that each is the only one to read:
+//   pairs       6 + waves (0.6 T + 4), plus 3.5 and 12 us a million groups for op_const,
+//   single      4 + waves (T + 6), plus the same,
+//   narrow      as above less 1, its blocks 1.07 (dX: 1.28) times; no such limit from HBM.
+// Over 60 grouped forwards and dX (4 to 64 experts of 768 x 2048 to 4096 x 1536, 122 to 12304 rows) this
+// is within 1.3 % of the best form; the dense estimates, which took pairs for few rows an expert, 13 %,
+// and single CTAs for all 16 %.  62 experts' 4096 x 1536 on 392 rows: forward 316 -> 273, dX 298 -> 278 us;
+// 64 experts' 768 x 2048 on 666: forward 88 -> 77, dX 97 -> 88.
 struct FusedPlan {
-  int pairs;      // 2, 1, or 0: narrow
+  int pairs;      // 2, 1, -1: single CTAs, or 0: narrow
   NarrowPlan np;
 };
 
@@ -2150,20 +2161,32 @@ FusedPlan plan_fused(int64_t M, int64_t depth, int64_t ncols, int32_t g, bool b_
                      bool loss, StepScalars sc, int sm_count) {
   const int64_t T = (depth + BK - 1) / BK;
   // two tanh a weight (s Delta < 6, reckoned at Delta = 0.5) cost the narrow dX a fifth more a block
-  const double wide_dx = b_mn && sc.phase == PHASE_SOFT && sc.s < 12.0f ? 1.2 : 1.0;
+  const double wide_dx = !grp && b_mn && sc.phase == PHASE_SOFT && sc.s < 12.0f ? 1.2 : 1.0;
   auto waves = [](int64_t tiles, int64_t fit) { return static_cast<double>((tiles + fit - 1) / fit); };
   const int64_t clusters2 = std::max(1, sm_count / 2), clusters4 = std::max(1, sm_count / 4 - 2);
-  const double per_tile = 0.62 * T + 2.0, consts = sc.phase == PHASE_TEACHER ? 0.0 : 3.5;
-  const double t2 = 8.0 + consts + waves(count_tiles(M, ncols, grp, 512, BN), clusters2) * per_tile;
-  const double t4 = 8.0 + consts + waves(count_tiles(M, ncols, grp, 1024, BN), clusters4) * per_tile;
+  const double groups = grp ? static_cast<double>(grp->E) * depth * ncols / g : 0.0;
+  const double before = sc.phase == PHASE_TEACHER ? 0.0 : 3.5 + 1.2e-5 * groups;
+  const double base = (grp ? 6.0 : 8.0) + before, per_tile = grp ? 0.6 * T + 4.0 : 0.62 * T + 2.0;
+  const double t2 = base + waves(count_tiles(M, ncols, grp, 512, BN), clusters2) * per_tile;
+  const double t4 = base + waves(count_tiles(M, ncols, grp, 1024, BN), clusters4) * per_tile;
   FusedPlan p{};
   const int64_t rows = grp ? M / grp->E : M;  // grouped: by the mean rows of an expert
   p.pairs = rows >= 1024 && t4 <= 1.1 * t2 ? 2 : 1;
-  const double pairs_best = 0.92 * (p.pairs == 2 ? t4 : t2);  // the estimates' own error
+  double pairs_best = p.pairs == 2 ? t4 : t2;
+  if (grp) {
+    const double t1 = 4.0 + before + waves(count_tiles(M, ncols, grp, 256, BN), sm_count) * (1.0 * T + 6.0);
+    if (t1 < pairs_best) {
+      pairs_best = t1;
+      p.pairs = -1;
+    }
+  } else {
+    pairs_best *= 0.92;  // the estimates' own error
+  }
   double best = pairs_best, best_paced = pairs_best;  // the narrow form's, as listed and paced by its rings
   NarrowPlan narrow{};
   static constexpr double kBlock[2][4] = {{0.38, 0.48, 0.54, 0.68}, {0.56, 0.72, 0.95, 1.2}};
-  const double w_us = static_cast<double>(grp ? grp->E : 1) * depth * ncols * 2 / 1.95e6;
+  const double w_us = grp ? 0.0 : static_cast<double>(depth) * ncols * 2 / 1.95e6;
+  const double scale = grp ? (b_mn ? 1.28 : 1.07) : 1.0;
   for (int bi = 0; bi < 2; ++bi)
     for (int nacc = 1; nacc <= 4; ++nacc) {
       if (nacc > 1 && 128 * (nacc - 1) >= M) break;
@@ -2172,11 +2195,11 @@ FusedPlan plan_fused(int64_t M, int64_t depth, int64_t ncols, int32_t g, bool b_
       for (int s = 1; s <= 8; s *= 2) {
         // clusters of s CTAs, one per SM, that a GPC layout leaves room for
         const int64_t fit = s == 8 ? sm_count / 8 - 5 : (s == 4 ? sm_count / 4 - 2 : sm_count / s);
-        if (s > T || fit < 1 || (loss && tiles * s > sm_count * FusedCfg<1>::kEpiWarps)) continue;
+        if (s > T || fit < 1 || (loss && tiles * s > sm_count * FusedCfg<2, 1>::kEpiWarps)) continue;
         const int64_t nk = (T + s - 1) / s;
-        const double over = s == 1 ? 7.0 + nacc : 6.0 + 3.0 * nacc;
+        const double over = (s == 1 ? 7.0 + nacc : 6.0 + 3.0 * nacc) - (grp ? 1.0 : 0.0);
         auto estimate = [&](double block) { return std::max(waves(tiles, fit) * (over + nk * block), 6.0 + w_us); };
-        const double block = kBlock[bi][nacc - 1], t = estimate(block);
+        const double block = scale * kBlock[bi][nacc - 1], t = estimate(block);
         if (t >= best) continue;
         NarrowPlan np{};
         np.bn = bn;
@@ -2222,10 +2245,14 @@ cudaError_t dispatch_fused_epi(const LayerDev& L, StepScalars sc, const void* A,
     return mu ? dispatch_narrow<B_MN, true>(L, sc, A, M, depth, C, ncols, p.np, st, grp, opts)
               : dispatch_narrow<B_MN, false>(L, sc, A, M, depth, C, ncols, p.np, st, grp, opts);
   if (p.pairs == 2)
-    return mu ? run_fused<B_MN, 2, true, EPI>(L, sc, A, M, depth, C, ncols, st, grp, opts)
-              : run_fused<B_MN, 2, false, EPI>(L, sc, A, M, depth, C, ncols, st, grp, opts);
-  return mu ? run_fused<B_MN, 1, true, EPI>(L, sc, A, M, depth, C, ncols, st, grp, opts)
-            : run_fused<B_MN, 1, false, EPI>(L, sc, A, M, depth, C, ncols, st, grp, opts);
+    return mu ? run_fused<2, B_MN, 2, true, EPI>(L, sc, A, M, depth, C, ncols, st, grp, opts)
+              : run_fused<2, B_MN, 2, false, EPI>(L, sc, A, M, depth, C, ncols, st, grp, opts);
+  constexpr int kEpiSingle = EPI == 0 ? 0 : 1;
+  if (p.pairs < 0)
+    return mu ? run_fused<1, B_MN, 1, true, kEpiSingle>(L, sc, A, M, depth, C, ncols, st, grp, opts)
+              : run_fused<1, B_MN, 1, false, kEpiSingle>(L, sc, A, M, depth, C, ncols, st, grp, opts);
+  return mu ? run_fused<2, B_MN, 1, true, EPI>(L, sc, A, M, depth, C, ncols, st, grp, opts)
+            : run_fused<2, B_MN, 1, false, EPI>(L, sc, A, M, depth, C, ncols, st, grp, opts);
 }
 
 bool only_row_scale(const EpiOpts& o, const void* C) { return o.row_scale && C && !o.y_f32 && !o.yref; }
@@ -2267,7 +2294,7 @@ void fused_form(int64_t N, int64_t K, int32_t g, bool mu, StepScalars sc, int64_
   std::copy(f, f + 7, form);
 }
 
-int fused_loss_max_parts(int sm_count) { return (sm_count > 0 ? sm_count : 1) * FusedCfg<1>::kEpiWarps; }
+int fused_loss_max_parts(int sm_count) { return (sm_count > 0 ? sm_count : 1) * FusedCfg<2, 1>::kEpiWarps; }
 
 cudaError_t launch_tc_dx_grouped(const LayerDev& L0, StepScalars sc, const void* dY, const GroupSpec& grp, void* dX,
                                  cudaStream_t st) {

@@ -1,5 +1,5 @@
 """GPU vs oracle parity of the fused forward and dX in every form that a call can take (pairs of CTAs, two
-pairs sharing each weight tile, the narrow kernel by columns, accumulators and shares), with every
+pairs sharing each weight tile, single CTAs, the narrow kernel by columns, accumulators and shares), with every
 epilogue.  catq_linear_form gives the form of a call, and each case asserts the one it is here for."""
 import numpy as np
 import pytest
@@ -22,7 +22,8 @@ def device():
 
 
 def _form(device, N, K, g, sched, **kw):
-    """Pairs per cluster, or (columns, accumulators, shares) of the narrow kernel, on this device."""
+    """Pairs per cluster, -1 for tiles of one CTA, or (columns, accumulators, shares) of the narrow kernel,
+    on this device."""
     import torch
 
     from paper_2606_26650_gb300 import catq as C
@@ -108,8 +109,12 @@ def test_form(device, M, N, K, g, recon, phase, s, what, fwd, dx):
     ([130, 0, 1, 257, 40], 192, 1024, 64, 0, SOFT, 30.0, (128, 1, 8), (64, 1, 1)),
     ([300, 5, 0, 700], 1032, 1152, 192, 1, SOFT, 30.0, (64, 2, 1), (64, 2, 1)),
     ([300, 5, 0, 700], 2056, 1152, 192, 0, HARD, 30.0, (64, 3, 1), (128, 3, 4)),
-    ([1100, 0, 900, 2100], 264, 1536, 192, 0, SOFT, 30.0, (64, 2, 1), (128, 3, 1)),
-    ([2100, 0, 1030, 1], 2056, 1152, 192, 1, SOFT, 30.0, 1, 1),
+    ([1100, 0, 900, 2100], 264, 1536, 192, 0, SOFT, 30.0, (128, 3, 4), (128, 3, 1)),
+    ([2100, 600, 1030, 1], 2056, 1152, 192, 1, SOFT, 30.0, 1, 1),
+    ([2100, 0, 1030, 1], 2056, 1152, 192, 1, SOFT, 30.0, -1, 1),
+    ([520, 513, 300, 0, 700, 600], 2056, 576, 64, 0, HARD, 30.0, -1, (128, 2, 2)),
+    ([2100, 0, 1030, 1], 1032, 2304, 192, 0, SOFT, 3.75, 1, -1),
+    ([520, 513, 300, 0, 700, 600], 1032, 2304, 192, 1, SOFT, 30.0, (128, 2, 1), -1),
     ([1100, 0, 900, 2100], 1032, 1152, 192, 0, SOFT, 30.0, 2, 2),
     ([1100, 0, 900, 2100], 1032, 1152, 192, 1, HARD, 30.0, 2, 2)])
 def test_grouped_form(device, rows, N, K, g, recon, phase, s, fwd, dx):
