@@ -82,6 +82,9 @@ struct Lay {
 };
 constexpr uint32_t kTmemCols = 512;
 constexpr float kLazy = 8.0f;                        // rescale only past this rise (log2 units)
+// A chain's maximum before it has seen a score above -inf: below every product of a score, and finite, so
+// that scores of -inf weigh 2^(-inf - kNoMax) = 0 and not 2^(-inf + inf).
+constexpr float kNoMax = -3e38f;
 
 struct TcAttnArgs {
   uint16_t* out;
@@ -108,6 +111,16 @@ __device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t (&r)[16
       "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]), "r"(r[9]),
       "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15])
       : "memory");
+}
+__device__ __forceinline__ void tmem_st4(uint32_t taddr, const uint32_t (&r)[4]) {
+  asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1,%2,%3,%4};" ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]),
+               "r"(r[3])
+               : "memory");
+}
+__device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&r)[8]) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+               : "r"(taddr));
 }
 __device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 
@@ -204,6 +217,31 @@ struct ItemOf {
     b = rem / nh;
   }
 };
+
+// The weights of one row's 128 scores (keys up to `last`) where its maximum m is 2^24 or more: there the
+// fused product's unrounded part could exceed the exponent's range (the maximum is a rounded product), so
+// the products are rounded first, like it.  A loop of few instructions, off the path of ordinary scores
+// (which took 4 to 10 % longer with this in line).  P goes over the scores as there; returns its sum.
+__device__ __forceinline__ float weigh_far(uint32_t sbuf, float scale_log2, float m, int last) {
+  float sum = 0.0f;
+#pragma unroll 1
+  for (int k = 0; k < kTk / 8; ++k) {
+    uint32_t s[8], pk[4];
+    tmem_ld8(sbuf + 8u * k, s);
+    tmem_ld_wait();
+    float p[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const float x = __fsub_rn(__fmul_rn(__uint_as_float(s[i]), scale_log2), m);
+      p[i] = 8 * k + i > last ? 0.0f : fast_exp2(x);
+      sum += p[i];
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) pk[i] = pack2(p[2 * i], p[2 * i + 1]);
+    tmem_st4(sbuf + 64u * (k >> 3) + 4u * (k & 7), pk);
+  }
+  return sum;
+}
 
 template <int HD>
 __global__ void __launch_bounds__(kThreadsTc, 1)
@@ -352,7 +390,7 @@ __global__ void __launch_bounds__(kThreadsTc, 1)
       int qt, h, b;
       item_of(it, qt, h, b);
       const int n = qt + 1;
-      float m = -INFINITY, l = 0.0f;
+      float m = kNoMax, l = 0.0f;
       for (int j = c; j < n; j += 2) {
         if (!mbar_wait_warp(s_full0 + 8u * c, sph, a.wc)) { ok = false; break; }
         sph ^= 1u;
@@ -391,31 +429,37 @@ __global__ void __launch_bounds__(kThreadsTc, 1)
           for (int i = 0; i < w; ++i) mv[i] = fmaxf(mv[i], mv[i + w]);
         const float mx = mv[0] * a.scale_log2;
         const bool raise = mx > m + kLazy;
-        // raise the maximum: O's row (after the chain's previous P V) and l scale by 2^(m - mx).  The
-        // warp goes together (tcgen05 loads and stores are the whole warp's): rows that keep their
-        // maximum scale by 1.
-        if (__any_sync(0xffffffffu, raise && m != -INFINITY)) {
-          const float f = raise && m != -INFINITY ? fast_exp2(m - mx) : 1.0f;
-          l *= f;
-          if (!mbar_wait_warp(pv_done0 + 8u * c, (done - 1) & 1, a.wc)) { ok = false; break; }
-          tc_fence_after();
+        const float base = raise ? mx : m;
+        const bool far = fabsf(base) >= 16777216.0f;  // (see weigh_far)
+        if (__any_sync(0xffffffffu, far || (raise && j != c))) {
+          // raise the maximum: past the item's first tile O's row (after the chain's previous P V) and l
+          // scale by 2^(m - mx).  The warp goes together (tcgen05 loads and stores are the whole warp's):
+          // rows that keep their maximum scale by 1.
+          if (j != c) {
+            const float f = raise ? fast_exp2(m - mx) : 1.0f;
+            l *= f;
+            if (!mbar_wait_warp(pv_done0 + 8u * c, (done - 1) & 1, a.wc)) { ok = false; break; }
+            tc_fence_after();
 #pragma unroll
-          for (int u = 0; u < HD / 32; ++u) {
-            uint32_t o[32];
-            tmem_ld32(orow + 32u * u, o);
-            tmem_ld_wait();
+            for (int u = 0; u < HD / 32; ++u) {
+              uint32_t o[32];
+              tmem_ld32(orow + 32u * u, o);
+              tmem_ld_wait();
 #pragma unroll
-            for (int i = 0; i < 32; ++i) o[i] = __float_as_uint(__uint_as_float(o[i]) * f);
-            tmem_st32(orow + 32u * u, o);
+              for (int i = 0; i < 32; ++i) o[i] = __float_as_uint(__uint_as_float(o[i]) * f);
+              tmem_st32(orow + 32u * u, o);
+            }
+          }
+          if (__any_sync(0xffffffffu, far)) {
+            m = base;
+            l += weigh_far(sbuf, a.scale_log2, m, diag ? r : kTk);
+            tmem_st_wait();
+            warp_arrive(p_full0 + 8u * c, lane);
+            ++done;
+            continue;
           }
         }
-        if (raise) m = mx;
-        // A chain that has seen only scores of -inf has no maximum yet: 0 in its place gives them weight 0.
-        // And from 2^24 on the fused product's unrounded part could exceed the exponent's range (the
-        // maximum is a rounded product): the products are then rounded first, like it.
-        const float mb = m == -INFINITY ? 0.0f : m;
-        const bool far = __any_sync(0xffffffffu, fabsf(mb) >= 16777216.0f);
-        const float p_scale = far ? 1.0f : a.scale_log2, p_base = far ? 0.0f : mb;
+        m = base;
         // P_j in bf16, each half over its own scores (the second half is still in registers)
         float ls[8];
 #pragma unroll
@@ -423,20 +467,13 @@ __global__ void __launch_bounds__(kThreadsTc, 1)
 #pragma unroll
         for (int hf = 1; hf >= 0; --hf) {
           if (hf == 0) load_half(0);
-          if (far) {
-#pragma unroll
-            for (int u = 0; u < 2; ++u)
-#pragma unroll
-              for (int i = 0; i < 32; ++i)
-                sr[u][i] = __float_as_uint(__fsub_rn(__fmul_rn(__uint_as_float(sr[u][i]), a.scale_log2), mb));
-          }
 #pragma unroll
           for (int u = 0; u < 2; ++u) {
             uint32_t pk[16];
 #pragma unroll
             for (int i = 0; i < 32; i += 2) {
-              const float p0 = fast_exp2(fmaf(__uint_as_float(sr[u][i]), p_scale, -p_base));
-              const float p1 = fast_exp2(fmaf(__uint_as_float(sr[u][i + 1]), p_scale, -p_base));
+              const float p0 = fast_exp2(fmaf(__uint_as_float(sr[u][i]), a.scale_log2, -m));
+              const float p1 = fast_exp2(fmaf(__uint_as_float(sr[u][i + 1]), a.scale_log2, -m));
               ls[(i >> 1) & 7] += p0 + p1;
               pk[i / 2] = pack2(p0, p1);
             }
@@ -461,7 +498,7 @@ __global__ void __launch_bounds__(kThreadsTc, 1)
       ok = bar_all(1, kElem, ok);
       if (!ok) break;
       tc_fence_after();
-      const float2 e0 = mine[r], e1 = mine[kTq + r];  // chain 1 of a one-tile item: (-inf, 0)
+      const float2 e0 = mine[r], e1 = mine[kTq + r];  // chain 1 of a one-tile item: (kNoMax, 0)
       const float mm = fmaxf(e0.x, e1.x);
       const float f0 = fast_exp2(e0.x - mm), f1 = fast_exp2(e1.x - mm);
       const float lt = fmaf(e0.y, f0, e1.y * f1);
