@@ -93,8 +93,25 @@ __device__ __forceinline__ void load_gamma8(const float* p, float (&f)[8]) {
     v.load(p);
     v.get(f);
   } else {
-#pragma unroll
-    for (int i = 0; i < 8; ++i) f[i] = __ldg(p + i);
+    // aligned vectors of the eight, the rest one by one: p is 4, 8 or 12 bytes past a 16-byte boundary, the
+    // same in every thread (8192 rows of 4096 in bf16: forward 43 -> 32 us with 8 loads as 3 or 4)
+    auto one = [&](int i) { f[i] = __ldg(p + i); };
+    auto two = [&](int i) {
+      const float2 v = __ldg(reinterpret_cast<const float2*>(p + i));
+      f[i] = v.x; f[i + 1] = v.y;
+    };
+    auto four = [&](int i) {
+      const float4 v = __ldg(reinterpret_cast<const float4*>(p + i));
+      f[i] = v.x; f[i + 1] = v.y; f[i + 2] = v.z; f[i + 3] = v.w;
+    };
+    const uint32_t off = (static_cast<uint32_t>(reinterpret_cast<uintptr_t>(p)) >> 2) & 3u;
+    if (off == 2) {
+      two(0); four(2); two(6);
+    } else if (off == 1) {
+      one(0); two(1); four(3); one(7);
+    } else {
+      one(0); four(1); two(5); one(7);
+    }
   }
 }
 
@@ -281,6 +298,16 @@ __global__ void __launch_bounds__(kRowThreads) rmsnorm_bwd_kernel(const TH* __re
 // lane, U rows of every team of a warp in flight at once.
 constexpr int kRowWarps = kRowThreads / 32;
 
+// Weights of less alignment pass through shared memory, loaded one by one but side by side (8 loads of a
+// lane's 8 neighbours touch 32 sectors each; 8192 rows of 1024, backward in bf16: 21.7 -> 10.8 us).
+template <bool GVEC, int CAP>
+__device__ __forceinline__ const float* stage_gamma(const float* gamma, int H, float* shared) {
+  if constexpr (GVEC) return gamma;
+  for (int i = threadIdx.x; i < CAP && i < H; i += kRowThreads) shared[i] = __ldg(gamma + i);
+  __syncthreads();
+  return shared;
+}
+
 template <typename TX, bool GVEC, int VPL, int U>
 __global__ void __launch_bounds__(kRowThreads) rmsnorm_fwd_team_kernel(const TX* __restrict__ x,
                                                                         const uint16_t* __restrict__ res,
@@ -291,6 +318,7 @@ __global__ void __launch_bounds__(kRowThreads) rmsnorm_fwd_team_kernel(const TX*
                                                                         float* __restrict__ r) {
   const int lane = threadIdx.x & 31, sub = lane & (team - 1), nvec = H / 8;
   const int per_warp = 32 / team;
+  __shared__ __align__(16) float gs[GVEC ? 1 : 256 * VPL];
   const int64_t t0 =
       (blockIdx.x * static_cast<int64_t>(kRowWarps) + (threadIdx.x >> 5)) * per_warp * U + lane / team;
   FwdVec<TX> q[U][VPL];
@@ -303,6 +331,7 @@ __global__ void __launch_bounds__(kRowThreads) rmsnorm_fwd_team_kernel(const TX*
       if (t < T && v < nvec) q[k][u].load(x, res, t * H + 8 * v);
     }
   }
+  const float* const g8 = stage_gamma<GVEC, 256 * VPL>(gamma, H, gs);
 #pragma unroll
   for (int k = 0; k < U; ++k) {
     const int64_t t = t0 + k * per_warp;
@@ -317,7 +346,7 @@ __global__ void __launch_bounds__(kRowThreads) rmsnorm_fwd_team_kernel(const TX*
 #pragma unroll
     for (int u = 0; u < VPL; ++u) {
       const int v = sub + u * team;
-      if (t < T && v < nvec) q[k][u].template store_z<GVEC>(res != nullptr, gamma, 8 * v, rr, z + t * H + 8 * v);
+      if (t < T && v < nvec) q[k][u].template store_z<true>(res != nullptr, g8, 8 * v, rr, z + t * H + 8 * v);
     }
   }
 }
@@ -331,6 +360,7 @@ __global__ void __launch_bounds__(kRowThreads) rmsnorm_bwd_team_kernel(const TH*
                                                                         int32_t team, uint16_t* dx) {
   const int lane = threadIdx.x & 31, sub = lane & (team - 1), nvec = H / 8;
   const int per_warp = 32 / team;
+  __shared__ __align__(16) float gs[GVEC ? 1 : 256 * VPL];
   const int64_t t0 =
       (blockIdx.x * static_cast<int64_t>(kRowWarps) + (threadIdx.x >> 5)) * per_warp * U + lane / team;
   const bool two = dy2 != nullptr, with_res = dres != nullptr;
@@ -346,6 +376,7 @@ __global__ void __launch_bounds__(kRowThreads) rmsnorm_bwd_team_kernel(const TH*
       if (t < T && v < nvec) q[k][u].load(x, dy, dy2, dres, t * H + 8 * v);
     }
   }
+  const float* const g8 = stage_gamma<GVEC, 256 * VPL>(gamma, H, gs);
 #pragma unroll
   for (int k = 0; k < U; ++k) {
     const int64_t t = t0 + k * per_warp;
@@ -353,13 +384,13 @@ __global__ void __launch_bounds__(kRowThreads) rmsnorm_bwd_team_kernel(const TH*
 #pragma unroll
     for (int u = 0; u < VPL; ++u) {
       const int v = sub + u * team;
-      if (t < T && v < nvec) sux = q[k][u].template dot<GVEC>(two, gamma, 8 * v, sux);
+      if (t < T && v < nvec) sux = q[k][u].template dot<true>(two, g8, 8 * v, sux);
     }
     const float c = team_sum(sux, team) / static_cast<float>(H) * rr[k] * rr[k] * rr[k];
 #pragma unroll
     for (int u = 0; u < VPL; ++u) {
       const int v = sub + u * team;
-      if (t < T && v < nvec) q[k][u].template store_dx<GVEC>(two, with_res, gamma, 8 * v, rr[k], c, dx + t * H + 8 * v);
+      if (t < T && v < nvec) q[k][u].template store_dx<true>(two, with_res, g8, 8 * v, rr[k], c, dx + t * H + 8 * v);
     }
   }
 }
@@ -599,7 +630,8 @@ namespace {
 bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
 // Lanes per row of the team kernels: one vector per lane up to 256 elements (four rows of a team in
-// flight, two of fp32 input), then 2 or 4 vectors per lane of a whole warp.
+// flight, two of fp32 input; one where a launch is of no more than two CTAs an SM even so, since the
+// shorter program starts sooner: 8 rows of 40, 2.9 -> 2.1 us), then 2 or 4 vectors per lane of a whole warp.
 int row_team(int64_t H) {
   int team = 1;
   while (team < 32 && team * 8 < H) team *= 2;
@@ -617,7 +649,10 @@ cudaError_t run_rmsnorm_fwd(const TX* x, const uint16_t* res, const float* gamma
   const int team = row_team(H), h32 = static_cast<int>(H);
   const unsigned rows = static_cast<unsigned>(T);
   constexpr int U = sizeof(TX) == 2 ? 4 : 2;
-  if (H <= 256)
+  if (H <= 256 && row_grid(T, team, 1) <= 2 * 152)
+    rmsnorm_fwd_team_kernel<TX, GVEC, 1, 1><<<row_grid(T, team, 1), kRowThreads, 0, st>>>(x, res, gamma, T, h32, team,
+                                                                                         eps, h_out, z, r);
+  else if (H <= 256)
     rmsnorm_fwd_team_kernel<TX, GVEC, 1, U><<<row_grid(T, team, U), kRowThreads, 0, st>>>(x, res, gamma, T, h32, team,
                                                                                          eps, h_out, z, r);
   else if (H <= 512)
@@ -641,7 +676,10 @@ cudaError_t run_rmsnorm_bwd(const TH* x, const float* gamma, const float* r, con
   const int team = row_team(H), h32 = static_cast<int>(H);
   const unsigned rows = static_cast<unsigned>(T);
   constexpr int U = sizeof(TH) == 2 ? 4 : 2;
-  if (H <= 256)
+  if (H <= 256 && row_grid(T, team, 1) <= 2 * 152)
+    rmsnorm_bwd_team_kernel<TH, GVEC, 1, 1><<<row_grid(T, team, 1), kRowThreads, 0, st>>>(x, gamma, r, dy, dy2, dres, T,
+                                                                                         h32, team, dx);
+  else if (H <= 256)
     rmsnorm_bwd_team_kernel<TH, GVEC, 1, U><<<row_grid(T, team, U), kRowThreads, 0, st>>>(x, gamma, r, dy, dy2, dres, T,
                                                                                          h32, team, dx);
   else if (H <= 512)

@@ -60,6 +60,33 @@ def test_row_norm_edges(device, H, gamma_offset):
     assert U.fro_rel(_f64(g), want) <= 4e-3
 
 
+# Weights 4, 8 and 12 bytes past a 16-byte boundary, in every kind of row: the arithmetic is the aligned one's,
+# bit for bit.  And launches of one row a team in flight beside those of two or four (3 and 9000 rows).
+@pytest.mark.parametrize("H,T", [(8, 3), (136, 9000), (256, 67), (520, 67), (1024, 67), (1032, 67), (2056, 67), (8200, 19)])
+def test_row_norm_weight_alignment(device, H, T):
+    import torch
+
+    from paper_2606_26650_gb300 import catq as C
+    gen = torch.Generator(device=device).manual_seed(H)
+    x = torch.randn(T, H, generator=gen, device=device)
+    dz = torch.randn(T, H, generator=gen, device=device).bfloat16()
+    buf = torch.rand(H + 4, generator=gen, device=device) + 0.5
+    first = None
+    for off in range(4):
+        g = torch.zeros(H + 4, device=device)[off:off + H]
+        g.copy_(buf[:H])
+        out = []
+        for a in (x, x.bfloat16()):
+            z, r, dx = torch.empty_like(dz), torch.empty(T, device=device), torch.empty_like(dz)
+            C.catq_rmsnorm_fwd(a, g, z, r, 1e-5)
+            C.catq_rmsnorm_bwd(a, g, r, dz, dx)
+            out += [z, r, dx]
+        first = first or out
+        assert all(torch.equal(a, b) for a, b in zip(first, out)), off
+    want, _ = O.rmsnorm(_f64(x), _f64(buf[:H]), 1e-5)
+    assert U.fro_rel(_f64(first[0]), want) <= 4e-3
+
+
 # Rotary embedding: runs of 1, 2, 4 and 8 heads per thread (by the size of the launch), head counts
 # that are no multiple of the run.
 @pytest.mark.parametrize("T,S,nh,d", [(3, 2, 1, 16), (65, 64, 9, 64), (1024, 512, 33, 128), (8192, 2048, 21, 128)])
