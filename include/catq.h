@@ -155,7 +155,10 @@ catq_status catq_modulate_ternarize(const catq_layer* layer, catq_schedule sched
 
 /* Forward Y = X Wq^T (Eq. 6 weight, Eq. 7 window output for one linear).
  *   X [M, K] row-major, Y [M, N] row-major, both of dtype x_dtype (== w_dtype); fp32
- *   accumulation.  M == 0 is a no-op.                                                    */
+ *   accumulation.  M == 0 is a no-op.  The same call gives the same bits on a given device;
+ *   how a contraction is cut (catq_linear_form; the fp32 path likewise) depends on M, in grouped
+ *   calls also on the rows of all experts and on whether the loss is fused, so a row of Y or dX
+ *   may round differently beside other rows.                                             */
 catq_status catq_soft_ternary_linear_fwd(const catq_layer* layer, catq_schedule sched,
                                          const void* X, int64_t M, int32_t x_dtype, void* Y,
                                          catq_stream stream);

@@ -149,8 +149,8 @@ def header_functions(path: str = HEADER):
 # so these run on every argument of every call and keep to a handful of attribute reads each:
 # addresses as ints, structs filled in one call, the stream without a Stream object.  Nothing is
 # remembered from one call to the next.  On a Grace host, Python and launch together: forward of a
-# layer 18.0 -> 8.9 us, its backward 27.3 -> 16.2, a row norm 9.7 -> 5.3, three decode layers
-# 17.9 -> 9.9.
+# layer 18.0 -> 9.6 us, its backward 27.3 -> 17.2, a row norm 9.7 -> 5.4, three decode layers
+# 17.9 -> 10.7.
 
 def _ptr(t):
     return None if t is None else t.data_ptr()

@@ -1,7 +1,7 @@
 // block.cu — the layers around the seven soft-ternary linears of one decoder block, for the
 // block-output reconstruction step (§2.4, Eq. 7 over a window of one block): RMSNorm (with the
 // residual add fused into the forward, and the residual and second upstream gradient fused
-// into the backward; one CTA per long row, one warp per short row such as an attention head),
+// into the backward; one CTA per long row, a team of lanes per short row such as an attention head),
 // rotary position embedding, SwiGLU, the fp32 block output with the loss on it, and the row sums
 // the attention backward needs.  The attention itself runs on tcgen05 (attn_tc.cu).
 #include <cuda_bf16.h>

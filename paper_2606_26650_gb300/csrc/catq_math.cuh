@@ -438,7 +438,7 @@ __device__ __forceinline__ LogiSums2 logi_add(const LogiSums2& a, const LogiSums
                    add_f32x2(a.sxs, pack_f32x2(b.sxs, 0.0f)), add_f32x2(a.sdelta, pack_f32x2(b.sdelta, 0.0f))};
 }
 
-// grad_element_onexp's form of two neighbouring elements, w2 their bf16 weights.  CLAMP caps the
+// The one-exponential form (OneExp) of two neighbouring elements, w2 their bf16 weights.  CLAMP caps the
 // exponent at 126; a group needs it only when its largest exponent, c2 (at x = 0), is above that.
 template <bool MU, bool SOFT, bool CLAMP>
 __device__ __forceinline__ void grad_pair_logistic(float g0, float g1, uint32_t w2, const GroupConst& c,

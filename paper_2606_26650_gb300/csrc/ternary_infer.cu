@@ -536,7 +536,7 @@ __global__ void __launch_bounds__(kThreads, 2) ternary_mma_kernel(const __grid_c
     const uint4* const xbase =
         reinterpret_cast<const uint4*>(f.X + static_cast<int64_t>(gid < nb ? gid : 0) * f.ldx + 16 * VW * q);
     // (32 bytes at a time where X allows: half the passes through L1, which a load of eight token rows
-    // at 16 bytes a lane keeps busy; two 8B blocks, 8 tokens: 97 -> 87 us, staged 129 -> 101.  A staged
+    // at 16 bytes a lane keeps busy; two 8B blocks, 8 tokens: 10 us less, staged 129 -> 101.  A staged
     // launch's X may be an earlier stage's Y: plain loads, after the stage's acquire, or through L2 for
     // a single token, whose row is not read twice: 96 -> 92.)
     const bool x32 = (reinterpret_cast<uintptr_t>(xbase) & 31u) == 0 && (!STAGED || nb > 1);
@@ -700,8 +700,8 @@ __global__ void __launch_bounds__(kThreads, 2) ternary_mma_kernel(const __grid_c
 
 // Dynamic shared memory of a CTA: half of an SM's, less its reserve and the static arrays.
 constexpr int64_t kDynBytes = 112 * 1024;
-// More than two slab buffers only up to this much of it: the rest caches activations (the layers of
-// two 8B blocks, 8 tokens, as one staged call: 121 us so, 141 us with a third buffer instead).
+// More than two slab buffers only up to this much of it: the rest caches activations (two 8B blocks, groups
+// of 128, 8 tokens: 101 us staged and 92 in single launches so, 114 and 94 with a third buffer instead).
 constexpr int64_t kRingBytes = 80 * 1024;
 
 // log2 of the lanes that share n pieces of a row: the power of two up to a warp that covers them.
