@@ -61,8 +61,9 @@ def test_row_norm_edges(device, H, gamma_offset):
 
 
 # Weights 4, 8 and 12 bytes past a 16-byte boundary, in every kind of row: the arithmetic is the aligned one's,
-# bit for bit.  And launches of one row a team in flight beside those of two or four (3 and 9000 rows).
-@pytest.mark.parametrize("H,T", [(8, 3), (136, 9000), (256, 67), (520, 67), (1024, 67), (1032, 67), (2056, 67), (8200, 19)])
+# bit for bit.  And launches of one row a team in flight beside those of two or four (9000
+# rows and more).
+@pytest.mark.parametrize("H,T", [(8, 3), (24, 40000), (128, 9000), (136, 9000), (256, 67), (520, 67), (1024, 67), (1032, 67), (2056, 67), (8200, 19)])
 def test_row_norm_weight_alignment(device, H, T):
     import torch
 
@@ -87,9 +88,10 @@ def test_row_norm_weight_alignment(device, H, T):
     assert U.fro_rel(_f64(first[0]), want) <= 4e-3
 
 
-# Rotary embedding: runs of 1, 2, 4 and 8 heads per thread (by the size of the launch), head counts
-# that are no multiple of the run.
-@pytest.mark.parametrize("T,S,nh,d", [(3, 2, 1, 16), (65, 64, 9, 64), (1024, 512, 33, 128), (8192, 2048, 21, 128)])
+# Rotary embedding: runs of 1, 2, 4 and 8 heads per thread (by the size of the launch: 1 in the first three
+# cases), head counts that are no multiple of the run.
+@pytest.mark.parametrize("T,S,nh,d", [(3, 2, 1, 16), (65, 64, 9, 64), (1024, 512, 33, 128), (8192, 2048, 13, 128),
+                                       (8192, 2048, 21, 128), (8192, 2048, 37, 128)])
 def test_rope_head_runs(device, T, S, nh, d):
     from paper_2606_26650_gb300 import catq as C
     r = syn.rng(301, f"rope/{T}/{nh}")
@@ -238,11 +240,13 @@ def test_attention_ragged_tiles(device, S, nh, nkv, d):
 
 
 # Inference on packed codes: one super-chunk for eight warps, groups longer and shorter than a slab, several
-# slabs with a remainder, both item heights with remainders, two token blocks, scales and
-# activations at their least alignment (no 16-byte scale copies, no 32-byte activation loads).
+# slabs of equal and (16 x 20608, 23 x 20160, 9720 x 6720) unequal length, items of 16 rows and (9720) of 32
+# with remainders, two token blocks, scales and activations at their least alignment (no 16-byte scale
+# copies, no 32-byte activation loads).
 @pytest.mark.parametrize("N,K,g,B,mu,shift", [
     (33, 64, 64, 1, False, 0), (40, 192, 192, 9, True, 1), (16, 20480, 256, 8, False, 0), (48, 24576, 24576, 3, True, 0),
-    (9744, 256, 128, 2, False, 1), (9744, 640, 64, 8, True, 0), (31, 17408, 128, 5, False, 1)])
+    (9744, 256, 128, 2, False, 1), (9744, 640, 64, 8, True, 0), (31, 17408, 128, 5, False, 1),
+    (9720, 256, 128, 2, False, 1), (9720, 6720, 64, 3, True, 0), (16, 20608, 128, 8, False, 0), (23, 20160, 192, 5, True, 1)])
 def test_ternary_infer_slabs(device, N, K, g, B, mu, shift):
     import torch
 
