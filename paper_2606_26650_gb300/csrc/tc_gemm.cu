@@ -2135,9 +2135,11 @@ int64_t count_tiles(int64_t M, int64_t ncols, const GroupSpec* grp, int64_t rows
 //               1.2 (128 columns), per wave; W from HBM at no more than 1.95 TB/s.
 // T contraction blocks of 64, nk a share's, rounds the accumulators with rows.  The narrow form found is
 // weighed against the pairs once more as its rings pace it: with only two slots of one beside the
-// table a block waits for its copy (no less than 2.0 / the A ring's slots or 2.9 / the W ring's), and in
-// dX two tanh a weight cost a fifth more.  Of 840 forwards and dX of drawn shapes 72 then ran 1.1 to 2.0
-// times faster, as pairs (654 x 14336 x 4096: 216 -> 135 us), and nine 1.05 to 1.23 times slower.
+// table a block waits for its copy (no less than 2.0 / the A ring's slots, 1.6 in a forward of 64 columns,
+// or 2.9 / the W ring's, 1.9 of 64 columns), and with deeper rings two tanh a weight cost a fifth more in
+// dX.  Of 840 forwards and dX of drawn shapes 67 then ran 1.1 to 2.0 times faster, as pairs
+// (654 x 14336 x 4096: 216 -> 135 us), and four 1.05 to 1.23 times slower, the worst of them dX of
+// 269 x 14336 x 4096 in mode mu (151 -> 186 us).
 // Forward of M x K x N,
 // before (single CTAs below 512 rows) and now: 8 x 2048 x 1024 40 -> 10 us, 128 x 2048 x 2048 41 -> 12,
 // 300 x 2048 x 1024 42 -> 14, 512 x 6144 x 2048 69 -> 33, 1000 x 2048 x 2048 31 -> 23; as pairs
@@ -2219,8 +2221,10 @@ FusedPlan plan_fused(int64_t M, int64_t depth, int64_t ncols, int32_t g, bool b_
         }
         if (depth_best < 2) continue;
         best = t;
-        best_paced = estimate(wide_dx * block);
-        if (depth_best == 2) best_paced = std::max(best_paced, estimate(std::max(2.0 / np.stages_a, 2.9 / np.stages_w)));
+        best_paced = depth_best > 2
+                         ? estimate(wide_dx * block)
+                         : estimate(std::max({block, (bn == 64 && !b_mn ? 1.6 : 2.0) / np.stages_a,
+                                              (bn == 64 ? 1.9 : 2.9) / np.stages_w}));
         narrow = np;
       }
     }
